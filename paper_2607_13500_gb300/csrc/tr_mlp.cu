@@ -555,17 +555,17 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
-    int stage = 0;
-    uint32_t phase = 0, filled = 0, last_parity = 0;
-    bool ok = true;
-    for (int tile = blockIdx.x; tile < g.tiles && ok; tile += gridDim.x) {
-      const int rb = tile / g.n_tiles, nt = tile - rb * g.n_tiles;
-      for (int kb = 0; kb < g.kblocks; ++kb) {
-        if (!tc::mbar_wait_warp(empty(stage), phase ^ 1u)) {
-          ok = false;
-          break;
-        }
-        if (lane == 0) {
+    if (tc::elect_one()) {
+      int stage = 0;
+      uint32_t phase = 0, filled = 0, last_parity = 0;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < g.tiles && ok; tile += gridDim.x) {
+        const int rb = tile / g.n_tiles, nt = tile - rb * g.n_tiles;
+        for (int kb = 0; kb < g.kblocks; ++kb) {
+          if (!tc::mbar_wait(empty(stage), phase ^ 1u)) {
+            ok = false;
+            break;
+          }
           if (kMode == kModeProject) {  // A comes from the row loaders
             tc::mbar_expect_tx(full(stage), kBTile);
           } else {
@@ -573,61 +573,59 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
             tc::tma_load_2d(sa(stage), &map_a, kb * kBK, rb * kBM, full(stage));
           }
           tc::tma_load_2d(sb(stage), &map_b, kb * kBK, nt * kBN, full(stage));
-        }
-        __syncwarp();
-        filled |= 1u << stage;
-        last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
-        if (++stage == kStages) {
-          stage = 0;
-          phase ^= 1u;
+          filled |= 1u << stage;
+          last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
+          if (++stage == kStages) {
+            stage = 0;
+            phase ^= 1u;
+          }
         }
       }
+      if (!ok) flag_error(g, 1);
+      // the loads already issued land before the CTA may exit
+      for (int s = 0; s < kStages; ++s)
+        if (filled & (1u << s)) tc::mbar_wait(full(s), (last_parity >> s) & 1u);
     }
-    if (!ok && lane == 0) flag_error(g, 1);
-    // the loads already issued land before the CTA may exit
-    for (int s = 0; s < kStages; ++s)
-      if (filled & (1u << s)) tc::mbar_wait_warp(full(s), (last_parity >> s) & 1u);
+    __syncwarp();
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    int stage = 0, acc = 0;
-    uint32_t phase = 0, acc_phase = 0;
-    bool ok = true;
-    for (int tile = blockIdx.x; tile < g.tiles && ok; tile += gridDim.x) {
-      if (!tc::mbar_wait_warp(tempty(acc), acc_phase ^ 1u)) {
-        ok = false;
-        break;
-      }
-      tc::fence_after_sync();
-      const uint32_t d = tmem + (uint32_t)(acc * kBN);
-      for (int kb = 0; kb < g.kblocks; ++kb) {
-        if (!tc::mbar_wait_warp(full(stage), phase)) {
+    if (tc::elect_one()) {
+      int stage = 0, acc = 0;
+      uint32_t phase = 0, acc_phase = 0;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < g.tiles && ok; tile += gridDim.x) {
+        if (!tc::mbar_wait(tempty(acc), acc_phase ^ 1u)) {
           ok = false;
           break;
         }
         tc::fence_after_sync();
-        if (lane == 0) {
+        const uint32_t d = tmem + (uint32_t)(acc * kBN);
+        for (int kb = 0; kb < g.kblocks; ++kb) {
+          if (!tc::mbar_wait(full(stage), phase)) {
+            ok = false;
+            break;
+          }
+          tc::fence_after_sync();
           const uint64_t da = tc::sw128_desc(sa(stage)), db = tc::sw128_desc(sb(stage));
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)  // 32 bytes further along K per step (start address >> 4: + 2)
             tc::mma_bf16(d, da + 2u * k, db + 2u * k, kIdesc, (kb | k) != 0);
           tc::mma_commit(empty(stage));  // the stage is free once these MMAs have read it
+          if (++stage == kStages) {
+            stage = 0;
+            phase ^= 1u;
+          }
         }
-        __syncwarp();
-        if (++stage == kStages) {
-          stage = 0;
-          phase ^= 1u;
-        }
+        if (!ok) break;
+        tc::mma_commit(tfull(acc));  // the accumulator is complete
+        acc ^= 1;
+        if (acc == 0) acc_phase ^= 1u;
       }
-      if (!ok) break;
-      if (lane == 0) tc::mma_commit(tfull(acc));  // the accumulator is complete
-      __syncwarp();
-      acc ^= 1;
-      if (acc == 0) acc_phase ^= 1u;
+      if (!ok) flag_error(g, 2);
+      tc::mma_commit(done);
     }
-    if (!ok && lane == 0) flag_error(g, 2);
-    // every MMA issued has completed before TMEM is released
-    if (lane == 0) tc::mma_commit(done);
     __syncwarp();
+    // every MMA issued has completed before TMEM is released
     tc::mbar_wait_warp(done, 0);
   } else if (kMode == kModeProject && warp >= 2 + epi_warps(kMode)) {
     // ---------------------------------------------------------------- A rows (projector mode)
@@ -789,80 +787,76 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer (both CTAs)
-    int stage = 0;
-    uint32_t phase = 0, filled = 0, last_parity = 0;
-    bool ok = true;
-    for (int tile = cluster; tile < tiles && ok; tile += clusters) {
-      const int rb = tile / g.n_tiles, nt = tile - rb * g.n_tiles;
-      for (int kb = 0; kb < g.kblocks; ++kb) {
-        if (!tc::mbar_wait_warp(empty(stage), phase ^ 1u)) {
-          ok = false;
-          break;
-        }
-        if (lane == 0) {
+    if (tc::elect_one()) {
+      int stage = 0;
+      uint32_t phase = 0, filled = 0, last_parity = 0;
+      bool ok = true;
+      for (int tile = cluster; tile < tiles && ok; tile += clusters) {
+        const int rb = tile / g.n_tiles, nt = tile - rb * g.n_tiles;
+        for (int kb = 0; kb < g.kblocks; ++kb) {
+          if (!tc::mbar_wait(empty(stage), phase ^ 1u)) {
+            ok = false;
+            break;
+          }
           const uint32_t bar = full_even(stage);
           if (leader) tc::mbar_expect_tx(full(stage), kTx);
           if (kMode != kModeProject)
             tc::tma_load_2d_pair(sa(stage), &map_a, kb * kBK, rb * 2 * kBM + (int)rank * kBM, bar);
           tc::tma_load_2d_pair(sb(stage), &map_b, kb * kBK, nt * kBN + (int)rank * 128, bar);
-        }
-        __syncwarp();
-        filled |= 1u << stage;
-        last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
-        if (++stage == kStagesP) {
-          stage = 0;
-          phase ^= 1u;
+          filled |= 1u << stage;
+          last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
+          if (++stage == kStagesP) {
+            stage = 0;
+            phase ^= 1u;
+          }
         }
       }
+      if (!ok) flag_error(g, 1);
+      // every load of either CTA lands on the even CTA's barriers: it waits for
+      // them before the final cluster barrier, so no CTA exits with loads in flight
+      if (leader)
+        for (int s = 0; s < kStagesP; ++s)
+          if (filled & (1u << s)) tc::mbar_wait(full(s), (last_parity >> s) & 1u);
     }
-    if (!ok && lane == 0) flag_error(g, 1);
-    // every load of either CTA lands on the even CTA's barriers: it waits for
-    // them before the final cluster barrier, so no CTA exits with loads in flight
-    if (leader)
-      for (int s = 0; s < kStagesP; ++s)
-        if (filled & (1u << s)) tc::mbar_wait_warp(full(s), (last_parity >> s) & 1u);
+    __syncwarp();
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer (even CTA)
-    if (leader) {
+    if (leader && tc::elect_one()) {
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
       for (int tile = cluster; tile < tiles && ok; tile += clusters) {
-        if (!tc::mbar_wait_warp(tempty(acc), acc_phase ^ 1u)) {
+        if (!tc::mbar_wait(tempty(acc), acc_phase ^ 1u)) {
           ok = false;
           break;
         }
         tc::fence_after_sync();
         const uint32_t d = tmem + (uint32_t)(acc * kBN);
         for (int kb = 0; kb < g.kblocks; ++kb) {
-          if (!tc::mbar_wait_warp(full(stage), phase)) {
+          if (!tc::mbar_wait(full(stage), phase)) {
             ok = false;
             break;
           }
           tc::fence_after_sync();
-          if (lane == 0) {
-            const uint64_t da = tc::sw128_desc(sa(stage)), db = tc::sw128_desc(sb(stage));
+          const uint64_t da = tc::sw128_desc(sa(stage)), db = tc::sw128_desc(sb(stage));
 #pragma unroll
-            for (int k = 0; k < kBK / 16; ++k)
-              tc::mma_bf16_pair(d, da + 2u * k, db + 2u * k, kIdescPair, (kb | k) != 0);
-            tc::mma_commit_pair(empty(stage), 0x3);  // both CTAs' stage is free once these MMAs read it
-          }
-          __syncwarp();
+          for (int k = 0; k < kBK / 16; ++k)
+            tc::mma_bf16_pair(d, da + 2u * k, db + 2u * k, kIdescPair, (kb | k) != 0);
+          tc::mma_commit_pair(empty(stage), 0x3);  // both CTAs' stage is free once these MMAs read it
           if (++stage == kStagesP) {
             stage = 0;
             phase ^= 1u;
           }
         }
         if (!ok) break;
-        if (lane == 0) tc::mma_commit_pair(tfull(acc), 0x3);
-        __syncwarp();
+        tc::mma_commit_pair(tfull(acc), 0x3);
         acc ^= 1;
         if (acc == 0) acc_phase ^= 1u;
       }
-      if (!ok && lane == 0) flag_error(g, 2);
-      if (lane == 0) tc::mma_commit_pair(done, 0x3);
-      __syncwarp();
+      if (!ok) flag_error(g, 2);
+      tc::mma_commit_pair(done, 0x3);
     }
+    __syncwarp();
     tc::mbar_wait_warp(done, 0);  // every pair MMA has completed (both CTAs' TMEM)
   } else if (kMode == kModeProject && warp >= 2 + epi_warps(kMode)) {
     // ---------------------------------------------------------------- A rows (projector mode)
