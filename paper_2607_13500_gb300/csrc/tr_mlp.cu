@@ -12,15 +12,17 @@
 // tensors.  The row records it writes are the ones tr_score writes.
 //
 // One kernel serves both GEMMs (C[m, n] = A[m, k] B[n, k]^T, bf16 operands,
-// fp32 accumulation): a persistent grid of one CTA per SM walks 128 x 256
-// output tiles (tile t: row block t / n_tiles, column block t % n_tiles,
-// so the CTAs running at one time share row blocks of A in L2).  Per CTA:
+// fp32 accumulation): a persistent grid of one CTA per SM, in pairs, walks
+// 256 x 256 output tiles (tile t: row block t / n_tiles, column block
+// t % n_tiles, so the pairs running at one time share row blocks of A in
+// L2).  Per CTA:
 //   warp 0      TMA producer: A and B k-blocks (64 wide, 128-byte swizzle)
-//               into a 4-stage shared-memory ring;
+//               into a 6-stage shared-memory ring;
 //   warp 1      allocates 512 TMEM columns (two 128 x 256 fp32
-//               accumulators) and issues tcgen05.mma (M 128, N 256, K 16)
-//               from one thread, committing each stage back to the
-//               producer and each finished accumulator to the epilogue;
+//               accumulators); in the pair's even CTA it issues tcgen05.mma
+//               (M 256, N 256, K 16) from one thread, committing each stage
+//               back to the producers and each finished accumulator to the
+//               epilogues;
 //   warps 2-    epilogue: one thread per accumulator row (TMEM lane: a
 //               warp reads the lane quarter warp % 4) and column part, 16
 //               columns per tcgen05.ld.  The score GEMM runs 8 warps (2-9,
@@ -71,10 +73,7 @@
 namespace tr {
 namespace {
 
-constexpr int kBM = 128, kBN = 256, kBK = 64, kStages = 4;
-constexpr int kATile = kBM * kBK * 2;             // bytes of one A k-block
-constexpr int kBTile = kBN * kBK * 2;             // bytes of one B k-block
-constexpr int kStageBytes = kATile + kBTile;      // 48 KiB
+constexpr int kBM = 128, kBN = 256, kBK = 64;  // a CTA's rows, a tile's columns, a k-block
 constexpr int kEpiWarps = 8;                      // score mode: two warpgroups, column halves of a tile
 enum { kModeHidden = 0, kModeScore = 1, kModeProject = 2 };
 // Epilogue warps per mode: the hidden GEMM's epilogue (activation and a TMA
@@ -97,14 +96,12 @@ __host__ __device__ constexpr int gemm_threads(int mode) {
 constexpr int kTmemCols = 2 * kBN;                // two accumulators
 constexpr int kChunk = 16;                        // columns per tcgen05.ld
 constexpr int kPartWords = 10;                    // hi, lo of L1, S2, A, B, P
-constexpr uint32_t kIdesc = tc::idesc_bf16(kBM, kBN);
 // Per epilogue warp of the hidden and projector modes, a 32-row bf16 output
 // block staged for a TMA store: 32 columns (64-byte rows, 64-byte swizzle)
 // with four column parts, 64 (128-byte rows and swizzle) with two; 32 KiB in
 // all either way.
 constexpr int kStageOutAll = 32 * 1024;
 __host__ __device__ constexpr int stage_out(int mode) { return kStageOutAll / epi_warps(mode); }
-constexpr size_t kGemmSmem = (size_t)kStages * kStageBytes + kStageOutAll + 1024 + 256;
 
 struct GemmArgs {
   int m, n, k;          // C[m, n] = A[m, k] B[n, k]^T
@@ -508,224 +505,22 @@ __device__ __forceinline__ long long kept_source_row(const GemmArgs &g, long lon
   return first + local;
 }
 
-template <int kMode>
-__global__ void __launch_bounds__(gemm_threads(kMode), 1)
-    k_mlp_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-               const __grid_constant__ CUtensorMap map_out, const GemmArgs g) {
-  extern __shared__ unsigned char smem_raw[];
-  // stage tiles at a 1024-byte boundary (the swizzle atom), barriers after them
-  unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                                          ~static_cast<uintptr_t>(1023));
-  const uint32_t out_stage = tc::smem_u32(smem + (size_t)kStages * kStageBytes);  // epilogue staging
-  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)kStages * kStageBytes + kStageOutAll);
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStages + 5);
-  const uint32_t sbase = tc::smem_u32(smem);
-  const uint32_t b0 = tc::smem_u32(bars);
-  auto full = [&](int s) { return b0 + 8u * s; };
-  auto empty = [&](int s) { return b0 + 8u * (kStages + s); };
-  auto tfull = [&](int a) { return b0 + 8u * (2 * kStages + a); };
-  auto tempty = [&](int a) { return b0 + 8u * (2 * kStages + 2 + a); };
-  const uint32_t done = b0 + 8u * (2 * kStages + 4);
-  auto sa = [&](int s) { return sbase + (uint32_t)(s * kStageBytes); };
-  auto sb = [&](int s) { return sbase + (uint32_t)(s * kStageBytes + kATile); };
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      tc::mbar_init(full(s), kMode == kModeProject ? 1 + kLoadWarps : 1);  // + one arrival per loader warp
-      tc::mbar_init(empty(s), 1);
-    }
-    for (int a = 0; a < 2; ++a) {
-      tc::mbar_init(tfull(a), 1);
-      tc::mbar_init(tempty(a), 32 * epi_warps(kMode));
-    }
-    tc::mbar_init(done, 1);
-    tc::mbar_fence_init();
-    tc::tma_prefetch_map(&map_a);
-    tc::tma_prefetch_map(&map_b);
-  }
-  if (warp == 1) {
-    tc::tmem_alloc(tc::smem_u32(tmem_slot), kTmemCols);
-    tc::tmem_relinquish();
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
-
-  if (warp == 0) {
-    // ---------------------------------------------------------------- TMA producer
-    if (tc::elect_one()) {
-      int stage = 0;
-      uint32_t phase = 0, filled = 0, last_parity = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < g.tiles && ok; tile += gridDim.x) {
-        const int rb = tile / g.n_tiles, nt = tile - rb * g.n_tiles;
-        for (int kb = 0; kb < g.kblocks; ++kb) {
-          if (!tc::mbar_wait(empty(stage), phase ^ 1u)) {
-            ok = false;
-            break;
-          }
-          if (kMode == kModeProject) {  // A comes from the row loaders
-            tc::mbar_expect_tx(full(stage), kBTile);
-          } else {
-            tc::mbar_expect_tx(full(stage), kStageBytes);
-            tc::tma_load_2d(sa(stage), &map_a, kb * kBK, rb * kBM, full(stage));
-          }
-          tc::tma_load_2d(sb(stage), &map_b, kb * kBK, nt * kBN, full(stage));
-          filled |= 1u << stage;
-          last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
-          if (++stage == kStages) {
-            stage = 0;
-            phase ^= 1u;
-          }
-        }
-      }
-      if (!ok) flag_error(g, 1);
-      // the loads already issued land before the CTA may exit
-      for (int s = 0; s < kStages; ++s)
-        if (filled & (1u << s)) tc::mbar_wait(full(s), (last_parity >> s) & 1u);
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    // ---------------------------------------------------------------- MMA issuer
-    if (tc::elect_one()) {
-      int stage = 0, acc = 0;
-      uint32_t phase = 0, acc_phase = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < g.tiles && ok; tile += gridDim.x) {
-        if (!tc::mbar_wait(tempty(acc), acc_phase ^ 1u)) {
-          ok = false;
-          break;
-        }
-        tc::fence_after_sync();
-        const uint32_t d = tmem + (uint32_t)(acc * kBN);
-        for (int kb = 0; kb < g.kblocks; ++kb) {
-          if (!tc::mbar_wait(full(stage), phase)) {
-            ok = false;
-            break;
-          }
-          tc::fence_after_sync();
-          const uint64_t da = tc::sw128_desc(sa(stage)), db = tc::sw128_desc(sb(stage));
-#pragma unroll
-          for (int k = 0; k < kBK / 16; ++k)  // 32 bytes further along K per step (start address >> 4: + 2)
-            tc::mma_bf16(d, da + 2u * k, db + 2u * k, kIdesc, (kb | k) != 0);
-          tc::mma_commit(empty(stage));  // the stage is free once these MMAs have read it
-          if (++stage == kStages) {
-            stage = 0;
-            phase ^= 1u;
-          }
-        }
-        if (!ok) break;
-        tc::mma_commit(tfull(acc));  // the accumulator is complete
-        acc ^= 1;
-        if (acc == 0) acc_phase ^= 1u;
-      }
-      if (!ok) flag_error(g, 2);
-      tc::mma_commit(done);
-    }
-    __syncwarp();
-    // every MMA issued has completed before TMEM is released
-    tc::mbar_wait_warp(done, 0);
-  } else if (kMode == kModeProject && warp >= 2 + epi_warps(kMode)) {
-    // ---------------------------------------------------------------- A rows (projector mode)
-    // lane l < kLoadLanes of loader warp w brings rows 4 j .. 4 j + 3 (j = w
-    // kLoadLanes + l) of each A k-block with one tile::gather4 load; a group
-    // with a row outside x (past the kept slots) or a k-block past x's
-    // columns takes four one-row loads instead, an outside row at coordinate
-    // -1, which reads zeros
-    const int j = (warp - 2 - epi_warps(kMode)) * kLoadLanes + lane;
-    const bool loads = lane < kLoadLanes;
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    for (int tile = blockIdx.x; tile < g.tiles && ok; tile += gridDim.x) {
-      const int rb = tile / g.n_tiles;
-      int srow[kLoadRows];
-      bool whole = true;
-#pragma unroll
-      for (int i = 0; i < kLoadRows; ++i) {
-        const long long src = loads ? kept_source_row(g, (long long)rb * kBM + kLoadRows * j + i) : -1;
-        srow[i] = src >= 0 ? (int)src : -1;
-        whole &= src >= 0;
-      }
-      for (int kb = 0; kb < g.kblocks; ++kb) {
-        if (!tc::mbar_wait_warp(empty(stage), phase ^ 1u)) {
-          ok = false;
-          break;
-        }
-        if (lane == 0) tc::mbar_expect_tx(full(stage), kATile / kLoadWarps);  // this warp's rows; one arrival
-        __syncwarp();
-        const uint32_t dst = sa(stage) + (uint32_t)(kLoadRows * j * kBK * 2);
-        if (loads) {
-          if (whole && (kb + 1) * kBK <= g.k) {  // rows and columns inside x
-            tc::tma_gather4(dst, &map_a, kb * kBK, srow[0], srow[1], srow[2], srow[3], full(stage));
-          } else {
-#pragma unroll
-            for (int i = 0; i < kLoadRows; ++i)
-              tc::tma_load_2d(dst + (uint32_t)(i * kBK * 2), &map_a, kb * kBK, srow[i], full(stage));
-          }
-        }
-        if (++stage == kStages) {
-          stage = 0;
-          phase ^= 1u;
-        }
-      }
-    }
-    if (!ok && lane == 0) flag_error(g, 8);
-  } else {
-    // ---------------------------------------------------------------- epilogue
-    const int q = warp & 3;            // TMEM lane quadrant this warp may read
-    const int half = (warp - 2) >> 2;  // column half (score) or quarter (hidden, projector) of the tile
-    int acc = 0;
-    uint32_t acc_phase = 0;
-    for (int tile = blockIdx.x; tile < g.tiles; tile += gridDim.x) {
-      const int rb = tile / g.n_tiles, nt = tile - rb * g.n_tiles;
-      if (!tc::mbar_wait_warp(tfull(acc), acc_phase)) {
-        if (lane == 0) flag_error(g, 4);
-        break;
-      }
-      tc::fence_after_sync();
-      const long long row = (long long)rb * kBM + 32 * q + lane;
-      const bool row_ok = row < g.m;
-      const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * kBN);
-      Acc sums{{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-      if (kMode == kModeScore)
-        drain_tile<kMode>(g, taddr, half, nt, row, row_ok, sums);
-      else
-        drain_tile_store<epi_parts(kMode)>(g, &map_out, out_stage + (uint32_t)((warp - 2) * stage_out(kMode)), taddr,
-                                           half, nt,
-                         row - lane);
-      tc::fence_before_sync();
-      tc::mbar_arrive(tempty(acc));  // the MMA warp may refill this accumulator
-      if (kMode == kModeScore) publish_rows(g, rb, nt, half, q, row, row_ok, sums);
-      acc ^= 1;
-      if (acc == 0) acc_phase ^= 1u;
-    }
-    if (kMode != kModeScore && lane == 0) tc::bulk_wait();  // this warp's output stores have completed
-  }
-
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 1) {
-    tc::fence_after_sync();
-    tc::tmem_dealloc(tmem, kTmemCols);
-  }
-}
-
 // ---------------------------------------------------------------- the SM-pair kernel
-// The same GEMM with tcgen05's 2-SM MMA: a cluster of two CTAs shares each
-// 256 x 256 output tile (tile t: row block t / n_tiles of 256 rows).  CTA
-// rank r loads A rows 128 r .. 128 r + 127 of the tile and B rows (output
-// columns) 128 r .. 128 r + 127 into its own shared memory -- 32 KiB per
-// k-block stage, six stages -- and both CTAs' loads complete on the even
-// CTA's stage barrier.  The even CTA alone issues the pair's MMAs (M 256,
-// N 256, K 16), which read both CTAs' stages and write each CTA's 128
-// accumulator rows into its own TMEM; its commits reach the same barriers
-// in both CTAs (multicast).  Each CTA's epilogue drains its own rows and
-// releases the accumulator on the even CTA's barrier.  Per SM a k-block
-// brings 32 KiB of operands for a 128 x 256 x 64 product, against 48 KiB on
-// one SM, so six stages in flight hide the load latency that four did not.
+// tcgen05's 2-SM MMA: a cluster of two CTAs shares each 256 x 256 output
+// tile (tile t: row block t / n_tiles of 256 rows).  CTA rank r loads A rows
+// 128 r .. 128 r + 127 of the tile and B rows (output columns) 128 r .. 128 r
+// + 127 into its own shared memory -- 32 KiB per k-block stage, six stages --
+// and both CTAs' loads complete on the even CTA's stage barrier.  The even
+// CTA alone issues the pair's MMAs (M 256, N 256, K 16), which read both
+// CTAs' stages and write each CTA's 128 accumulator rows into its own TMEM;
+// its commits reach the same barriers in both CTAs (multicast).  Each CTA's
+// epilogue drains its own rows and releases the accumulator on the even
+// CTA's barrier.  Per SM a k-block brings 32 KiB of operands for a
+// 128 x 256 x 64 product, against 48 KiB on one SM.  A batch of at most 128
+// rows runs here too, the odd CTA's rows read as zeros: what such a batch
+// waits for is W, and a pair brings each half of it into its own SM (128 rows,
+// D 1024, hidden 4096, both GEMMs: 57.4 us with an earlier one-SM kernel,
+// 55.3 here).
 constexpr int kStagesP = 6;
 constexpr int kHalfTile = 128 * kBK * 2;          // 128 rows of a k-block (A or B)
 constexpr int kStagePBytes = 2 * kHalfTile;       // this CTA's A rows + B rows
@@ -734,8 +529,8 @@ constexpr size_t kGemmPSmem = (size_t)kStagesP * kStagePBytes + kStageOutAll + 1
 
 template <int kMode>
 __global__ void __launch_bounds__(gemm_threads(kMode), 1)
-    k_mlp_gemm_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                    const __grid_constant__ CUtensorMap map_out, const GemmArgs g) {
+    k_mlp_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+               const __grid_constant__ CUtensorMap map_out, const GemmArgs g) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                           ~static_cast<uintptr_t>(1023));
@@ -860,9 +655,13 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
     tc::mbar_wait_warp(done, 0);  // every pair MMA has completed (both CTAs' TMEM)
   } else if (kMode == kModeProject && warp >= 2 + epi_warps(kMode)) {
     // ---------------------------------------------------------------- A rows (projector mode)
-    // as in the one-SM kernel, into this CTA's half of the pair's rows; the
-    // loads land on the even CTA's barrier, whose loader warps expect both
-    // CTAs' bytes (the odd CTA's loader warps do not arrive)
+    // lane l < kLoadLanes of loader warp w brings rows 4 j .. 4 j + 3 (j = w
+    // kLoadLanes + l) of this CTA's half of the pair's rows of each A k-block
+    // with one tile::gather4 load; a group with a row outside x (past the kept
+    // slots) or a k-block past x's columns takes four one-row loads instead, an
+    // outside row at coordinate -1, which reads zeros.  The loads land on the
+    // even CTA's barrier, whose loader warps expect both CTAs' bytes (the odd
+    // CTA's loader warps do not arrive)
     const int j = (warp - 2 - epi_warps(kMode)) * kLoadLanes + lane;
     const bool loads = lane < kLoadLanes;
     int stage = 0;
@@ -982,27 +781,8 @@ bool make_map(CUtensorMap *map, const void *base, long long rows, long long cols
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-std::atomic<int> g_gemm_smem_set[64];
-
 std::atomic<int> g_pair_smem_set[64];
 std::atomic<int> g_pair_clusters[64][3];
-
-template <int kMode>
-cudaError_t launch_single(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mo, const GemmArgs &g,
-                          cudaStream_t st, int dev) {
-  const int bit = 1 << kMode;
-  if (!(g_gemm_smem_set[dev & 63].load() & bit)) {
-    cudaError_t err =
-        cudaFuncSetAttribute(k_mlp_gemm<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem);
-    if (err != cudaSuccess) return err;
-    g_gemm_smem_set[dev & 63].fetch_or(bit);
-  }
-  const int sms = sm_count();
-  if (sms <= 0) return cudaErrorInvalidDevice;
-  const int grid = g.tiles < sms ? g.tiles : sms;
-  k_mlp_gemm<kMode><<<grid, gemm_threads(kMode), kGemmSmem, st>>>(ma, mb, mo, g);
-  return cudaGetLastError();
-}
 
 template <int kMode>
 cudaError_t launch_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mo, const GemmArgs &g,
@@ -1020,12 +800,12 @@ cudaError_t launch_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUte
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (!(g_pair_smem_set[dev & 63].load() & bit)) {
-    cudaError_t err = cudaFuncSetAttribute(k_mlp_gemm_pair<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t err = cudaFuncSetAttribute(k_mlp_gemm<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)kGemmPSmem);
     if (err != cudaSuccess) return err;
     int clusters = 0;
     cfg.gridDim = dim3(2 * 64);
-    err = cudaOccupancyMaxActiveClusters(&clusters, k_mlp_gemm_pair<kMode>, &cfg);
+    err = cudaOccupancyMaxActiveClusters(&clusters, k_mlp_gemm<kMode>, &cfg);
     if (err != cudaSuccess) return err;
     if (clusters <= 0) return cudaErrorInvalidConfiguration;
     g_pair_clusters[dev & 63][kMode].store(clusters);
@@ -1036,14 +816,8 @@ cudaError_t launch_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUte
   const int max_clusters = g_pair_clusters[dev & 63][kMode].load();
   const int clusters = tiles < max_clusters ? (int)tiles : max_clusters;
   cfg.gridDim = dim3(2 * clusters);
-  return cudaLaunchKernelEx(&cfg, k_mlp_gemm_pair<kMode>, ma, mb, mo, g);
+  return cudaLaunchKernelEx(&cfg, k_mlp_gemm<kMode>, ma, mb, mo, g);
 }
-
-// Batches of more than one 128-row block run on SM pairs (2-SM MMA); a
-// single row block on one SM.  The B operand's TMA box follows: 128 rows
-// per CTA in a pair, the whole 256-row tile on one SM.
-inline bool use_pair(int m) { return m > kBM; }
-inline int b_box_rows(int m) { return use_pair(m) ? 128 : kBN; }
 
 template <int kMode>
 cudaError_t launch_gemm(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mo, const GemmArgs &g,
@@ -1052,7 +826,7 @@ cudaError_t launch_gemm(const CUtensorMap &ma, const CUtensorMap &mb, const CUte
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
-  return use_pair(g.m) ? launch_pair<kMode>(ma, mb, mo, g, st, dev) : launch_single<kMode>(ma, mb, mo, g, st, dev);
+  return launch_pair<kMode>(ma, mb, mo, g, st, dev);
 }
 
 bool misaligned16(const void *p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
@@ -1102,7 +876,7 @@ tr_status dense_act_gemm(const void *a, int rows, int k, const void *w, const fl
   g.out = static_cast<uint16_t *>(out);
   g.err = d_error;
   CUtensorMap ma, mb, mo;
-  if (!make_map(&ma, a, rows, k, kBM) || !make_map(&mb, w, n, k, b_box_rows(g.m)) ||
+  if (!make_map(&ma, a, rows, k, kBM) || !make_map(&mb, w, n, k, kBN / 2) ||
       !make_map(&mo, out, rows, n, 32, 128 / epi_parts(kModeHidden),
                 epi_parts(kModeHidden) == 2 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
     return TR_ERR_CUDA;
@@ -1174,7 +948,7 @@ tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, fl
   g.s = s;
   g.err = d_error;
   CUtensorMap ma, mb;
-  if (!make_map(&ma, h, m->t, m->d_hidden, kBM) || !make_map(&mb, m->w2, m->d, m->d_hidden, b_box_rows(g.m)))
+  if (!make_map(&ma, h, m->t, m->d_hidden, kBM) || !make_map(&mb, m->w2, m->d, m->d_hidden, kBN / 2))
     return TR_ERR_CUDA;
   return launch_gemm<kModeScore>(ma, mb, mb, g, st) == cudaSuccess ? TR_OK : TR_ERR_CUDA;  // no output map
 }
@@ -1223,7 +997,7 @@ tr_status tr_project_kept(const tr_tokens *in, const int32_t *d_cu_k, const int3
   g.idx = idx;
   // A: x, one row per box (the loaders gather rows by kept index)
   CUtensorMap ma, mb, mo;
-  if (!make_map(&ma, in->x, total_rows, in->d, 1) || !make_map(&mb, w, d_out, in->d, b_box_rows(g.m)) ||
+  if (!make_map(&ma, in->x, total_rows, in->d, 1) || !make_map(&mb, w, d_out, in->d, kBN / 2) ||
       !make_map(&mo, z, total_k, d_out, 32, 128 / epi_parts(kModeProject),
                 epi_parts(kModeProject) == 2 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
     return TR_ERR_CUDA;
