@@ -102,25 +102,32 @@ constexpr int kPartWords = 10;                    // hi, lo of L1, S2, A, B, P
 // all either way.
 constexpr int kStageOutAll = 32 * 1024;
 __host__ __device__ constexpr int stage_out(int mode) { return kStageOutAll / epi_warps(mode); }
+// The score mode's epilogue staging: per warp two buffers of a 32 x 32 block
+// of x' and one of the residual (2 KiB each, 64-byte rows and swizzle),
+// loaded by TMA ahead of their use and overwritten in place by x'' and x.
+constexpr int kScoreBlk = 32;                         // columns per block
+constexpr int kScoreHalfBuf = 32 * kScoreBlk * 2;     // bytes of one tensor's block
+constexpr int kScoreBuf = 2 * kScoreHalfBuf;          // x' / x'' block, residual / x block
+constexpr int kScoreStageAll = 2 * kScoreBuf * kEpiWarps;
 
 struct GemmArgs {
   int m, n, k;          // C[m, n] = A[m, k] B[n, k]^T
   int n_tiles, tiles, kblocks;
   const float *bias;    // [n] or NULL
   int act;              // hidden GEMM: TR_ACT_*
-  uint16_t *out;        // hidden: H [m, n]; score: x'' [m, n] (bf16 bits)
-  const uint16_t *x_pre, *resid;  // score: x' [m, n], residual [m, n] or NULL
-  uint16_t *x;          // score: block output [m, n]
+  bool has_resid;       // score: x = x'' + residual
   float *part;          // score: [row blocks][n_tiles][2 halves][4][kPartWords][32] partial sums
-  int *arrivals;        // score: [row blocks][4], zero at launch
-  float4 *stats;        // score: [m] records (two float4 each)
-  float *h2, *s;        // score: optional outputs
   int32_t *err;         // optional: set when a pipeline wait timed out
   // projector mode: A row j = x[first row of the image owning kept slot j + idx[j]]
-  const uint16_t *gx;   // x [total_rows, k]
   long long total_rows;
   int batch, n_uniform;
   const int32_t *cu_seqlens, *cu_k, *idx;
+};
+
+// Tensor maps of one launch: the operands, the output (hidden, projector: the
+// activations; score: x''), and for the score mode x', the residual and x.
+struct GemmMaps {
+  CUtensorMap a, b, out, p, r, x;
 };
 
 __device__ __forceinline__ float bf16_val(uint32_t bits16) { return __uint_as_float(bits16 << 16); }
@@ -189,50 +196,6 @@ __device__ __forceinline__ void flag_error(const GemmArgs &g, int code) {
   if (g.err) atomicOr(g.err, code);
 }
 
-// Hidden GEMM epilogue for 16 columns of one row: H = bf16(act(acc + b1)).
-__device__ __forceinline__ void epi_hidden(const GemmArgs &g, long long row, int col0, const float (&v)[16]) {
-  float2 a[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) a[i] = make_float2(v[2 * i], v[2 * i + 1]);
-  if (g.bias) {  // the same 16 values in every lane: four broadcast loads
-    const float4 *bp = reinterpret_cast<const float4 *>(g.bias + col0);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float4 b = __ldg(bp + i);
-      a[2 * i] = __fadd2_rn(a[2 * i], make_float2(b.x, b.y));
-      a[2 * i + 1] = __fadd2_rn(a[2 * i + 1], make_float2(b.z, b.w));
-    }
-  }
-  uint32_t w[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float2 h = activate2(a[i], g.act);
-    w[i] = pack_bf16x2(h.x, h.y);
-  }
-  uint4 *dst = reinterpret_cast<uint4 *>(g.out + row * g.n + col0);
-  dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-  dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-}
-
-// The 16 columns of x' and of the residual that the score epilogue of one
-// chunk reads, loaded one chunk ahead of their use.
-struct ScoreIn {
-  uint4 p0, p1, r0, r1;
-};
-__device__ __forceinline__ void load_score_in(const GemmArgs &g, long long row, int col0, ScoreIn &in) {
-  const long long base = row * g.n + col0;
-  const uint4 *pp = reinterpret_cast<const uint4 *>(g.x_pre + base);
-  in.p0 = __ldg(pp);
-  in.p1 = __ldg(pp + 1);
-  if (g.resid) {
-    const uint4 *rp = reinterpret_cast<const uint4 *>(g.resid + base);
-    in.r0 = __ldg(rp);
-    in.r1 = __ldg(rp + 1);
-  } else {
-    in.r0 = in.r1 = make_uint4(0u, 0u, 0u, 0u);
-  }
-}
-
 // The score epilogue keeps its five double-float sums as fp32 pairs:
 // component x takes the even columns, component y the odd ones, merged once
 // per tile.
@@ -272,18 +235,23 @@ __device__ __forceinline__ void df2_fold(DF &out, const DF2 &in) {  // even + od
 }
 
 // Score GEMM epilogue for 16 columns of one row: x'' = bf16(acc + b2),
-// x = bf16(resid + x''), both stored; the five sums take the stored values
-// (products and squares of bf16 values are exact in fp32; each term enters
-// its double-float sum through TwoSum).
-__device__ __forceinline__ void epi_score(const GemmArgs &g, long long row, int col0, const float (&v)[16],
-                                          const ScoreIn &in, Acc2 &acc) {
-  const long long base = row * g.n + col0;
-  const uint32_t pw[8] = {in.p0.x, in.p0.y, in.p0.z, in.p0.w, in.p1.x, in.p1.y, in.p1.z, in.p1.w};
-  const uint32_t rw[8] = {in.r0.x, in.r0.y, in.r0.z, in.r0.w, in.r1.x, in.r1.y, in.r1.z, in.r1.w};
+// x = bf16(resid + x''); the five sums take the rounded values (products and
+// squares of bf16 values are exact in fp32; each term enters its double-float
+// sum through TwoSum).  x' and the residual come from this warp's staged
+// block (units u0, u0 + 1 of the lane's row) and x'' and x take their places.
+__device__ __forceinline__ void epi_score(const GemmArgs &g, int col0, const uint32_t (&v)[16], uint32_t rowbuf,
+                                          uint32_t u0, uint32_t u1, Acc2 &acc) {
+  uint32_t pw[8], rw[8], qo[8], xo[8];
+  tc::ld_shared_v4(rowbuf + u0, pw[0], pw[1], pw[2], pw[3]);
+  tc::ld_shared_v4(rowbuf + u1, pw[4], pw[5], pw[6], pw[7]);
+  if (g.has_resid) {
+    tc::ld_shared_v4(rowbuf + kScoreHalfBuf + u0, rw[0], rw[1], rw[2], rw[3]);
+    tc::ld_shared_v4(rowbuf + kScoreHalfBuf + u1, rw[4], rw[5], rw[6], rw[7]);
+  }
   float2 a[8];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) a[i] = make_float2(v[2 * i], v[2 * i + 1]);
-  if (g.bias) {
+  for (int i = 0; i < 8; ++i) a[i] = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+  if (g.bias) {  // the same 16 values in every lane: four broadcast loads
     const float4 *bp = reinterpret_cast<const float4 *>(g.bias + col0);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -292,12 +260,11 @@ __device__ __forceinline__ void epi_score(const GemmArgs &g, long long row, int 
       a[2 * i + 1] = __fadd2_rn(a[2 * i + 1], make_float2(b.z, b.w));
     }
   }
-  uint32_t qo[8], xo[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     qo[i] = pack_bf16x2(a[i].x, a[i].y);  // x''
     const float2 q = bf16x2_f2(qo[i]);
-    if (g.resid) {
+    if (g.has_resid) {
       const float2 xs = __fadd2_rn(bf16x2_f2(rw[i]), q);
       xo[i] = pack_bf16x2(xs.x, xs.y);
     } else {
@@ -311,18 +278,118 @@ __device__ __forceinline__ void epi_score(const GemmArgs &g, long long row, int 
     df2_add_prod(acc.b, q, q);
     df2_add_prod(acc.p, p, q);
   }
-  uint4 *dq = reinterpret_cast<uint4 *>(g.out + base);
-  dq[0] = make_uint4(qo[0], qo[1], qo[2], qo[3]);
-  dq[1] = make_uint4(qo[4], qo[5], qo[6], qo[7]);
-  uint4 *dx = reinterpret_cast<uint4 *>(g.x + base);
-  dx[0] = make_uint4(xo[0], xo[1], xo[2], xo[3]);
-  dx[1] = make_uint4(xo[4], xo[5], xo[6], xo[7]);
+  tc::st_shared_v4(rowbuf + u0, qo[0], qo[1], qo[2], qo[3]);
+  tc::st_shared_v4(rowbuf + u1, qo[4], qo[5], qo[6], qo[7]);
+  tc::st_shared_v4(rowbuf + kScoreHalfBuf + u0, xo[0], xo[1], xo[2], xo[3]);
+  tc::st_shared_v4(rowbuf + kScoreHalfBuf + u1, xo[4], xo[5], xo[6], xo[7]);
 }
 
-// Score epilogue of one tile half for this warp: the 8 chunks of 16 columns
-// of its column half, each chunk's TMEM load (and its x' and residual
-// loads) issued while the chunk before it is processed.
-//
+// The stream of staged blocks of one score-epilogue warp: its column half's
+// 32-column blocks of each of the CTA's tiles in turn, block j in buffer
+// j % 2.  load_next issues the TMA loads of the next block not yet requested;
+// the buffer's previous stores must have been read (bulk_wait_read).
+struct ScoreStream {
+  uint32_t buf, bar;   // two buffers of kScoreBuf bytes, two mbarriers
+  int tile, blk;       // next block to request
+  uint32_t requested, used;
+  __device__ __forceinline__ uint32_t buffer(uint32_t j) const { return buf + (j & 1u) * (uint32_t)kScoreBuf; }
+  __device__ __forceinline__ uint32_t barrier(uint32_t j) const { return bar + 8u * (j & 1u); }
+  // Blocks of column half `half` of column tile nt that lie inside the output.
+  static __device__ __forceinline__ int blocks(const GemmArgs &g, int nt, int half) {
+    const int left = g.n - (nt * kBN + half * (kBN / 2));
+    return left <= 0 ? 0 : min(kBN / 2 / kScoreBlk, (left + kScoreBlk - 1) / kScoreBlk);
+  }
+  // Every lane keeps the place; lane 0 issues.  row_of(row tile) = first of
+  // this warp's 32 rows.
+  template <typename RowOf>
+  __device__ __forceinline__ void load_next(const GemmArgs &g, const GemmMaps &maps, int half, int tiles, int step,
+                                            RowOf row_of) {
+    int nt = 0;
+    while (tile < tiles) {
+      nt = tile % g.n_tiles;
+      if (blk < blocks(g, nt, half)) break;
+      tile += step;
+      blk = 0;
+    }
+    if (tile >= tiles) return;
+    if ((threadIdx.x & 31) == 0) {
+      const int col = nt * kBN + half * (kBN / 2) + blk * kScoreBlk, row = row_of(tile / g.n_tiles);
+      const uint32_t dst = buffer(requested), b = barrier(requested);
+      tc::mbar_expect_tx(b, g.has_resid ? kScoreBuf : kScoreHalfBuf);
+      tc::tma_load_2d(dst, &maps.p, col, row, b);
+      if (g.has_resid) tc::tma_load_2d(dst + kScoreHalfBuf, &maps.r, col, row, b);
+    }
+    ++requested;
+    ++blk;
+  }
+};
+
+// Score epilogue of one tile half for this warp (32 rows): 32-column blocks,
+// x' and the residual staged by TMA up to two blocks ahead, x'' and x written
+// over them and stored by TMA, so that global memory sees whole row segments
+// and no thread waits for a load that its next instruction needs (with loads
+// straight from global memory, one 16-column chunk ahead, a tile's epilogue
+// took 24,000-33,000 clocks).  False when a block's loads timed out.
+template <typename RowOf>
+__device__ __forceinline__ bool drain_tile_score(const GemmArgs &g, const GemmMaps &maps, ScoreStream &st,
+                                                 uint32_t taddr, int half, int nt, int row0, int tiles, int step,
+                                                 RowOf row_of, Acc &sums) {
+  const int lane = threadIdx.x & 31;
+  const int col_first = nt * kBN + half * (kBN / 2);
+  const int nblk = ScoreStream::blocks(g, nt, half);
+  if (nblk == 0) return true;
+  const int chunks = min(kBN / 2, g.n - col_first) / kChunk;  // n is a multiple of 16
+  const uint32_t tcol = taddr + (uint32_t)(half * (kBN / 2));
+  const uint32_t sw = (uint32_t)((lane >> 1) & 3);  // the 64-byte swizzle's row term
+  Acc2 acc2{};
+  uint32_t cur[16], nxt[16];
+  tc::tmem_ld16_issue(tcol, cur);
+  for (int b = 0; b < nblk; ++b) {
+    const uint32_t buf = st.buffer(st.used);
+    const bool ok = tc::mbar_wait(st.barrier(st.used), (st.used >> 1) & 1u);
+    ++st.used;
+    if (!__all_sync(0xffffffffu, ok)) {
+      tc::tmem_ld_wait(cur);
+      return false;
+    }
+    const uint32_t rowbuf = buf + (uint32_t)(lane * kScoreBlk * 2);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = 2 * b + h;
+      if (c < chunks) {  // uniform
+        tc::tmem_ld_wait(cur);
+        const bool more = c + 1 < chunks;
+        if (more) tc::tmem_ld16_issue(tcol + (uint32_t)((c + 1) * kChunk), nxt);
+        epi_score(g, col_first + c * kChunk, cur, rowbuf, ((2u * h) ^ sw) << 4, ((2u * h + 1u) ^ sw) << 4, acc2);
+        if (more) {
+          tc::tmem_ld_wait(nxt);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) cur[i] = nxt[i];
+        }
+      }
+    }
+    tc::fence_async_shared();
+    __syncwarp();
+    if (lane == 0) {
+      if (row0 < g.m) {  // rows and columns past the output are clipped by the store
+        const int col = col_first + b * kScoreBlk;
+        tc::tma_store_2d(&maps.out, col, row0, buf);
+        tc::tma_store_2d(&maps.x, col, row0, buf + kScoreHalfBuf);
+      }
+      tc::bulk_commit();
+      tc::bulk_wait_read();
+    }
+    __syncwarp();
+    st.load_next(g, maps, half, tiles, step, row_of);
+  }
+  df2_fold(sums.l1, acc2.l1);
+  df2_fold(sums.s2, acc2.s2);
+  df2_fold(sums.a, acc2.a);
+  df2_fold(sums.b, acc2.b);
+  df2_fold(sums.p, acc2.p);
+  return true;
+}
+
 // Hidden / projector epilogue of one of a tile's kParts column parts for
 // this warp: chunks of 16 columns, H = bf16(act(acc + bias)), staged in this
 // warp's 32-row block of kBlk = 64 / (kParts / 2) columns, whose rows are
@@ -403,75 +470,33 @@ __device__ __forceinline__ void drain_tile_store(const GemmArgs &g, const CUtens
   __syncwarp();
 }
 
-template <int kMode>
-__device__ __forceinline__ void drain_tile(const GemmArgs &g, uint32_t taddr, int half, int nt, long long row,
-                                           bool row_ok, Acc &sums) {
-  constexpr int kChunks = kBN / 2 / kChunk;
-  int chunks = 0;  // chunks of this half inside the output (uniform across the warp)
-  while (chunks < kChunks && nt * kBN + half * (kBN / 2) + chunks * kChunk < g.n) ++chunks;
-  if (chunks == 0) return;
-  uint32_t cur[16], nxt[16];
-  ScoreIn in_cur{}, in_nxt{};
-  Acc2 acc2{};
-  const int col_first = nt * kBN + half * (kBN / 2);
-  tc::tmem_ld16_issue(taddr + (uint32_t)(half * (kBN / 2)), cur);
-  if (kMode == kModeScore && row_ok) load_score_in(g, row, col_first, in_cur);
-  tc::tmem_ld_wait(cur);
-  for (int c = 0; c < chunks; ++c) {
-    const int col0 = col_first + c * kChunk;
-    const bool more = c + 1 < chunks;
-    if (more) {
-      tc::tmem_ld16_issue(taddr + (uint32_t)(half * (kBN / 2) + (c + 1) * kChunk), nxt);
-      if (kMode == kModeScore && row_ok) load_score_in(g, row, col0 + kChunk, in_nxt);
-    }
-    if (row_ok) {
-      float v[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(cur[i]);
-      if (kMode == kModeScore)
-        epi_score(g, row, col0, v, in_cur, acc2);
-      else
-        epi_hidden(g, row, col0, v);
-    }
-    if (more) {
-      tc::tmem_ld_wait(nxt);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) cur[i] = nxt[i];
-      in_cur = in_nxt;
-    }
-  }
-  if (kMode == kModeScore) {
-    df2_fold(sums.l1, acc2.l1);
-    df2_fold(sums.s2, acc2.s2);
-    df2_fold(sums.a, acc2.a);
-    df2_fold(sums.b, acc2.b);
-    df2_fold(sums.p, acc2.p);
-  }
-}
-
-// This warp's 32 rows of one tile half are done: publish their partial
-// sums; the warp that completes a row block's quadrant (the last of its
-// 2 n_tiles column halves to arrive) merges the partials in column order
-// and writes the rows' records.
+// This warp's 32 rows of one tile half are done: their partial sums go to
+// the scratch; k_score_rows merges them once the GEMM has finished.
 __device__ __forceinline__ long long part_slot(const GemmArgs &g, int rb, int nt, int half, int q) {
   return (((long long)(rb * g.n_tiles + nt) * 2 + half) * 4 + q) * (kPartWords * 32);
 }
-__device__ __forceinline__ void publish_rows(const GemmArgs &g, int rb, int nt, int half, int q, long long row,
-                                             bool row_ok, const Acc &acc) {
-  const int lane = threadIdx.x & 31;
-  float *dst = g.part + part_slot(g, rb, nt, half, q) + lane;
+__device__ __forceinline__ void publish_rows(const GemmArgs &g, int rb, int nt, int half, int q, const Acc &acc) {
+  float *dst = g.part + part_slot(g, rb, nt, half, q) + (threadIdx.x & 31);
   const float vals[kPartWords] = {acc.l1.hi, acc.l1.lo, acc.s2.hi, acc.s2.lo, acc.a.hi,
                                   acc.a.lo,  acc.b.hi,  acc.b.lo,  acc.p.hi,  acc.p.lo};
 #pragma unroll
   for (int j = 0; j < kPartWords; ++j) __stcg(dst + 32 * j, vals[j]);
-  __threadfence();
-  __syncwarp();
-  int last = 0;
-  if (lane == 0) last = atomicAdd(g.arrivals + rb * 4 + q, 1) == 2 * g.n_tiles - 1;
-  last = __shfl_sync(0xffffffffu, last, 0);
-  if (!last) return;
-  __threadfence();
+}
+
+// The rows' records from the partial sums the score GEMM left: one warp per
+// 32 rows, the 2 n_tiles column halves merged in column order (the record
+// does not depend on which CTA made which part).  A kernel of its own, begun
+// while the GEMM drains: arrival counters inside the GEMM cost each tile a
+// fence over its stores, an atomic and, for the last warp, this same merge in
+// series (about 5,000 clocks a tile, and a memset before every launch).
+__global__ void __launch_bounds__(kBM) k_score_rows(const GemmArgs g, float4 *__restrict__ stats,
+                                                    float *__restrict__ h2, float *__restrict__ s_out) {
+  pdl_trigger();
+  pdl_wait();  // the partial sums come from the GEMM before this kernel
+  const int rb = blockIdx.x, q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long long row = (long long)rb * kBM + threadIdx.x;
   Acc tot{{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll 4
   for (int t = 0; t < 2 * g.n_tiles; ++t) {
     const float *src = g.part + part_slot(g, rb, t >> 1, t & 1, q) + lane;
     float w[kPartWords];
@@ -483,8 +508,7 @@ __device__ __forceinline__ void publish_rows(const GemmArgs &g, int rb, int nt, 
     df_merge(tot.b, w[6], w[7]);
     df_merge(tot.p, w[8], w[9]);
   }
-  if (row_ok) write_record(tot, row, g.stats, g.h2, g.s);
-  if (lane == 0) g.arrivals[rb * 4 + q] = 0;  // ready for the next launch
+  if (row < g.m) write_record(tot, row, stats, h2, s_out);
 }
 
 // Row of x that kept slot j names (projector mode), or -1: the image b with
@@ -519,24 +543,31 @@ __device__ __forceinline__ long long kept_source_row(const GemmArgs &g, long lon
 // 128 x 256 x 64 product, against 48 KiB on one SM.  A batch of at most 128
 // rows runs here too, the odd CTA's rows read as zeros: what such a batch
 // waits for is W, and a pair brings each half of it into its own SM (128 rows,
-// D 1024, hidden 4096, both GEMMs: 57.4 us with an earlier one-SM kernel,
-// 55.3 here).
-constexpr int kStagesP = 6;
+// D 1024, hidden 4096, both GEMMs: 57.4 us with a one-SM kernel, 55.3 here).
+// The score mode gives one stage to its epilogue's staging.
+__host__ __device__ constexpr int gemm_stages(int mode) { return mode == kModeScore ? 5 : 6; }
+__host__ __device__ constexpr int out_stage_bytes(int mode) {
+  return mode == kModeScore ? kScoreStageAll : kStageOutAll;
+}
 constexpr int kHalfTile = 128 * kBK * 2;          // 128 rows of a k-block (A or B)
 constexpr int kStagePBytes = 2 * kHalfTile;       // this CTA's A rows + B rows
 constexpr uint32_t kIdescPair = tc::idesc_bf16(2 * kBM, kBN);
-constexpr size_t kGemmPSmem = (size_t)kStagesP * kStagePBytes + kStageOutAll + 1024 + 256;
+__host__ __device__ constexpr int gemm_smem(int mode) {  // + alignment, barriers
+  return gemm_stages(mode) * kStagePBytes + out_stage_bytes(mode) + 1024 + 512;
+}
 
 template <int kMode>
 __global__ void __launch_bounds__(gemm_threads(kMode), 1)
-    k_mlp_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-               const __grid_constant__ CUtensorMap map_out, const GemmArgs g) {
+    k_mlp_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
+  constexpr int kStagesP = gemm_stages(kMode);
+  pdl_trigger();
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                           ~static_cast<uintptr_t>(1023));
   const uint32_t out_stage = tc::smem_u32(smem + (size_t)kStagesP * kStagePBytes);  // epilogue staging
-  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)kStagesP * kStagePBytes + kStageOutAll);
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStagesP + 5);
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)kStagesP * kStagePBytes + out_stage_bytes(kMode));
+  constexpr int kBlkBars = kMode == kModeScore ? 2 * kEpiWarps : 0;  // the score epilogue's staged blocks
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStagesP + 5 + kBlkBars);
   const uint32_t sbase = tc::smem_u32(smem);
   const uint32_t b0 = tc::smem_u32(bars);
   auto full = [&](int s) { return b0 + 8u * s; };
@@ -544,6 +575,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
   auto tfull = [&](int a) { return b0 + 8u * (2 * kStagesP + a); };
   auto tempty = [&](int a) { return b0 + 8u * (2 * kStagesP + 2 + a); };
   const uint32_t done = b0 + 8u * (2 * kStagesP + 4);
+  auto blk_bar = [&](int w) { return b0 + 8u * (2 * kStagesP + 5 + 2 * w); };  // two of epilogue warp w
   auto sa = [&](int s) { return sbase + (uint32_t)(s * kStagePBytes); };
   auto sb = [&](int s) { return sbase + (uint32_t)(s * kStagePBytes + kHalfTile); };
 
@@ -563,9 +595,10 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
       tc::mbar_init(tempty(a), 2 * epi_warps(kMode));  // one arrival per epilogue warp of either CTA
     }
     tc::mbar_init(done, 1);
+    for (int i = 0; i < kBlkBars; ++i) tc::mbar_init(blk_bar(0) + 8u * i, 1);
     tc::mbar_fence_init();
-    tc::tma_prefetch_map(&map_a);
-    tc::tma_prefetch_map(&map_b);
+    tc::tma_prefetch_map(&maps.a);
+    tc::tma_prefetch_map(&maps.b);
   }
   if (warp == 1) {
     tc::tmem_alloc_pair(tc::smem_u32(tmem_slot), kTmemCols);
@@ -577,8 +610,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
   const uint32_t tmem = *tmem_slot;
   auto full_even = [&](int s) { return tc::map_shared(full(s), 0); };
   auto tempty_even = [&](int a) { return tc::map_shared(tempty(a), 0); };
-  const int row_tiles = (g.m + 2 * kBM - 1) / (2 * kBM);
-  const int tiles = row_tiles * g.n_tiles;
+  const int tiles = g.tiles;
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer (both CTAs)
@@ -596,8 +628,8 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
           const uint32_t bar = full_even(stage);
           if (leader) tc::mbar_expect_tx(full(stage), kTx);
           if (kMode != kModeProject)
-            tc::tma_load_2d_pair(sa(stage), &map_a, kb * kBK, rb * 2 * kBM + (int)rank * kBM, bar);
-          tc::tma_load_2d_pair(sb(stage), &map_b, kb * kBK, nt * kBN + (int)rank * 128, bar);
+            tc::tma_load_2d_pair(sa(stage), &maps.a, kb * kBK, rb * 2 * kBM + (int)rank * kBM, bar);
+          tc::tma_load_2d_pair(sb(stage), &maps.b, kb * kBK, nt * kBN + (int)rank * 128, bar);
           filled |= 1u << stage;
           last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
           if (++stage == kStagesP) {
@@ -688,11 +720,11 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
         const uint32_t dst = sa(stage) + (uint32_t)(kLoadRows * j * kBK * 2);
         if (loads) {
           if (whole && (kb + 1) * kBK <= g.k) {  // rows and columns inside x
-            tc::tma_gather4_pair(dst, &map_a, kb * kBK, srow[0], srow[1], srow[2], srow[3], full_even(stage));
+            tc::tma_gather4_pair(dst, &maps.a, kb * kBK, srow[0], srow[1], srow[2], srow[3], full_even(stage));
           } else {
 #pragma unroll
             for (int i = 0; i < kLoadRows; ++i)
-              tc::tma_load_2d_pair(dst + (uint32_t)(i * kBK * 2), &map_a, kb * kBK, srow[i], full_even(stage));
+              tc::tma_load_2d_pair(dst + (uint32_t)(i * kBK * 2), &maps.a, kb * kBK, srow[i], full_even(stage));
           }
         }
         if (++stage == kStagesP) {
@@ -704,8 +736,13 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
     if (!ok && lane == 0) flag_error(g, 8);
   } else {
     // ---------------------------------------------------------------- epilogue (both CTAs)
-    const int q = warp & 3;
-    const int half = (warp - 2) >> 2;  // column half (score) or quarter of the tile
+    const int q = warp & 3;            // TMEM lane quadrant this warp may read
+    const int part = (warp - 2) >> 2;  // column half (score, projector) or quarter (hidden) of the tile
+    // first of this warp's 32 rows in a tile of row block rb
+    auto row_of = [&](int rb) { return (2 * rb + (int)rank) * kBM + 32 * q; };
+    ScoreStream st{out_stage + (uint32_t)((warp - 2) * 2 * kScoreBuf), blk_bar(warp - 2), cluster, 0, 0u, 0u};
+    if (kMode == kModeScore)
+      for (int i = 0; i < 2; ++i) st.load_next(g, maps, part, tiles, clusters, row_of);
     int acc = 0;
     uint32_t acc_phase = 0;
     for (int tile = cluster; tile < tiles; tile += clusters) {
@@ -715,25 +752,31 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
         break;
       }
       tc::fence_after_sync();
-      const int rb128 = 2 * rb + (int)rank;  // this CTA's 128-row block
-      const long long row = (long long)rb128 * kBM + 32 * q + lane;
-      const bool row_ok = row < g.m;
       const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * kBN);
       Acc sums{{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-      if (kMode == kModeScore)
-        drain_tile<kMode>(g, taddr, half, nt, row, row_ok, sums);
-      else
-        drain_tile_store<epi_parts(kMode)>(g, &map_out, out_stage + (uint32_t)((warp - 2) * stage_out(kMode)), taddr,
-                                           half, nt,
-                         row - lane);
+      if (kMode == kModeScore) {
+        if (!drain_tile_score(g, maps, st, taddr, part, nt, row_of(rb), tiles, clusters, row_of, sums)) {
+          if (lane == 0) flag_error(g, 16);
+          break;
+        }
+      } else {
+        drain_tile_store<epi_parts(kMode)>(g, &maps.out, out_stage + (uint32_t)((warp - 2) * stage_out(kMode)), taddr,
+                                           part, nt, row_of(rb));
+      }
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive_cluster(tempty_even(acc));  // this warp is done with the accumulator
-      if (kMode == kModeScore && rb128 * kBM < g.m) publish_rows(g, rb128, nt, half, q, row, row_ok, sums);
+      const int rb128 = 2 * rb + (int)rank;
+      if (kMode == kModeScore && rb128 * kBM < g.m) publish_rows(g, rb128, nt, part, q, sums);
       acc ^= 1;
       if (acc == 0) acc_phase ^= 1u;
     }
-    if (kMode != kModeScore && lane == 0) tc::bulk_wait();  // this warp's output stores have completed
+    if (lane == 0) {
+      if (kMode == kModeScore)  // blocks requested and not used (after a timeout) land before the CTA may exit
+        for (; st.used < st.requested; ++st.used) tc::mbar_wait(st.barrier(st.used), (st.used >> 1) & 1u);
+      tc::bulk_wait();  // this warp's output stores have completed
+    }
+    __syncwarp();
   }
 
   tc::fence_before_sync();
@@ -781,16 +824,18 @@ bool make_map(CUtensorMap *map, const void *base, long long rows, long long cols
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-std::atomic<int> g_pair_smem_set[64];
-std::atomic<int> g_pair_clusters[64][3];
+std::atomic<int> g_gemm_set[64];
+std::atomic<int> g_gemm_clusters[64][3];
 
 template <int kMode>
-cudaError_t launch_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mo, const GemmArgs &g,
-                        cudaStream_t st, int dev) {
+cudaError_t launch_gemm(const GemmMaps &maps, const GemmArgs &g, cudaStream_t st) {
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
   const int bit = 1 << kMode;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(gemm_threads(kMode));
-  cfg.dynamicSmemBytes = kGemmPSmem;
+  cfg.dynamicSmemBytes = gemm_smem(kMode);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -799,34 +844,21 @@ cudaError_t launch_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUte
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (!(g_pair_smem_set[dev & 63].load() & bit)) {
-    cudaError_t err = cudaFuncSetAttribute(k_mlp_gemm<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)kGemmPSmem);
+  if (!(g_gemm_set[dev & 63].load() & bit)) {
+    err = cudaFuncSetAttribute(k_mlp_gemm<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(kMode));
     if (err != cudaSuccess) return err;
     int clusters = 0;
     cfg.gridDim = dim3(2 * 64);
     err = cudaOccupancyMaxActiveClusters(&clusters, k_mlp_gemm<kMode>, &cfg);
     if (err != cudaSuccess) return err;
     if (clusters <= 0) return cudaErrorInvalidConfiguration;
-    g_pair_clusters[dev & 63][kMode].store(clusters);
-    g_pair_smem_set[dev & 63].fetch_or(bit);
+    g_gemm_clusters[dev & 63][kMode].store(clusters);
+    g_gemm_set[dev & 63].fetch_or(bit);
   }
-  const int row_tiles = (g.m + 2 * kBM - 1) / (2 * kBM);
-  const long long tiles = (long long)row_tiles * g.n_tiles;
-  const int max_clusters = g_pair_clusters[dev & 63][kMode].load();
-  const int clusters = tiles < max_clusters ? (int)tiles : max_clusters;
+  const int max_clusters = g_gemm_clusters[dev & 63][kMode].load();
+  const int clusters = g.tiles < max_clusters ? g.tiles : max_clusters;
   cfg.gridDim = dim3(2 * clusters);
-  return cudaLaunchKernelEx(&cfg, k_mlp_gemm<kMode>, ma, mb, mo, g);
-}
-
-template <int kMode>
-cudaError_t launch_gemm(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mo, const GemmArgs &g,
-                        cudaStream_t st) {
-  if (g.tiles == 0) return cudaSuccess;
-  int dev = 0;
-  cudaError_t err = cudaGetDevice(&dev);
-  if (err != cudaSuccess) return err;
-  return launch_pair<kMode>(ma, mb, mo, g, st, dev);
+  return cudaLaunchKernelEx(&cfg, k_mlp_gemm<kMode>, maps, g);
 }
 
 bool misaligned16(const void *p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
@@ -846,15 +878,14 @@ tr_status check_mlp(const tr_mlp *m) {
 }
 
 struct MlpWs {
-  size_t part, arrivals, total;
+  size_t part, total;
 };
 MlpWs mlp_ws(const tr_mlp *m) {
   const long long rblocks = ((long long)m->t + kBM - 1) / kBM;
   const long long n_tiles = (m->d + kBN - 1) / kBN;
   MlpWs w;
   w.part = 0;
-  w.arrivals = align_up((size_t)rblocks * n_tiles * 2 * 4 * kPartWords * 32 * sizeof(float), 256);
-  w.total = align_up(w.arrivals + (size_t)rblocks * 4 * sizeof(int), 256);
+  w.total = align_up((size_t)rblocks * n_tiles * 2 * 4 * kPartWords * 32 * sizeof(float), 256);
   return w;
 }
 
@@ -869,18 +900,17 @@ tr_status dense_act_gemm(const void *a, int rows, int k, const void *w, const fl
   g.n = n;
   g.k = k;
   g.n_tiles = (g.n + kBN - 1) / kBN;
-  g.tiles = ((g.m + kBM - 1) / kBM) * g.n_tiles;
+  g.tiles = (g.m + 2 * kBM - 1) / (2 * kBM) * g.n_tiles;
   g.kblocks = (g.k + kBK - 1) / kBK;
   g.bias = bias;
   g.act = act;
-  g.out = static_cast<uint16_t *>(out);
   g.err = d_error;
-  CUtensorMap ma, mb, mo;
-  if (!make_map(&ma, a, rows, k, kBM) || !make_map(&mb, w, n, k, kBN / 2) ||
-      !make_map(&mo, out, rows, n, 32, 128 / epi_parts(kModeHidden),
+  GemmMaps maps{};
+  if (!make_map(&maps.a, a, rows, k, kBM) || !make_map(&maps.b, w, n, k, kBN / 2) ||
+      !make_map(&maps.out, out, rows, n, 32, 128 / epi_parts(kModeHidden),
                 epi_parts(kModeHidden) == 2 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
     return TR_ERR_CUDA;
-  return launch_gemm<kModeHidden>(ma, mb, mo, g, st) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
+  return launch_gemm<kModeHidden>(maps, g, st) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 
 }  // namespace
@@ -928,29 +958,29 @@ tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, fl
   if (m->t == 0) return TR_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char *wsb = static_cast<char *>(ws);
-  if (cudaMemsetAsync(wsb + w.arrivals, 0, w.total - w.arrivals, st) != cudaSuccess) return TR_ERR_CUDA;
   GemmArgs g{};
   g.m = m->t;
   g.n = m->d;
   g.k = m->d_hidden;
   g.n_tiles = (g.n + kBN - 1) / kBN;
-  g.tiles = ((g.m + kBM - 1) / kBM) * g.n_tiles;
+  g.tiles = (g.m + 2 * kBM - 1) / (2 * kBM) * g.n_tiles;
   g.kblocks = (g.k + kBK - 1) / kBK;
   g.bias = m->b2;
-  g.out = static_cast<uint16_t *>(x_post);
-  g.x_pre = static_cast<const uint16_t *>(m->x_pre);
-  g.resid = static_cast<const uint16_t *>(m->resid);
-  g.x = static_cast<uint16_t *>(x);
+  g.has_resid = m->resid != nullptr;
   g.part = reinterpret_cast<float *>(wsb + w.part);
-  g.arrivals = reinterpret_cast<int *>(wsb + w.arrivals);
-  g.stats = reinterpret_cast<float4 *>(stats);
-  g.h2 = h2;
-  g.s = s;
   g.err = d_error;
-  CUtensorMap ma, mb;
-  if (!make_map(&ma, h, m->t, m->d_hidden, kBM) || !make_map(&mb, m->w2, m->d, m->d_hidden, kBN / 2))
+  GemmMaps maps{};
+  auto block_map = [&](CUtensorMap *map, const void *p) {  // the epilogue's 32 x 32 blocks
+    return make_map(map, p, m->t, m->d, 32, kScoreBlk, CU_TENSOR_MAP_SWIZZLE_64B);
+  };
+  if (!make_map(&maps.a, h, m->t, m->d_hidden, kBM) || !make_map(&maps.b, m->w2, m->d, m->d_hidden, kBN / 2) ||
+      !block_map(&maps.p, m->x_pre) || (m->resid && !block_map(&maps.r, m->resid)) || !block_map(&maps.out, x_post) ||
+      !block_map(&maps.x, x))
     return TR_ERR_CUDA;
-  return launch_gemm<kModeScore>(ma, mb, mb, g, st) == cudaSuccess ? TR_OK : TR_ERR_CUDA;  // no output map
+  if (launch_gemm<kModeScore>(maps, g, st) != cudaSuccess) return TR_ERR_CUDA;
+  const cudaError_t err = launch_kernel(k_score_rows, dim3((g.m + kBM - 1) / kBM), dim3(kBM), 0, st, true, g,
+                                        reinterpret_cast<float4 *>(stats), h2, s);
+  return err == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 
 tr_status tr_project_kept(const tr_tokens *in, const int32_t *d_cu_k, const int32_t *idx, int32_t total_k,
@@ -982,13 +1012,11 @@ tr_status tr_project_kept(const tr_tokens *in, const int32_t *d_cu_k, const int3
   g.n = d_out;
   g.k = in->d;
   g.n_tiles = (g.n + kBN - 1) / kBN;
-  g.tiles = (int)rblocks * g.n_tiles;
+  g.tiles = (g.m + 2 * kBM - 1) / (2 * kBM) * g.n_tiles;
   g.kblocks = (g.k + kBK - 1) / kBK;
   g.bias = bias;
   g.act = act;
-  g.out = static_cast<uint16_t *>(z);
   g.err = d_error;
-  g.gx = static_cast<const uint16_t *>(in->x);
   g.total_rows = total_rows;
   g.batch = in->batch;
   g.n_uniform = in->cu_seqlens ? 0 : in->n;
@@ -996,13 +1024,12 @@ tr_status tr_project_kept(const tr_tokens *in, const int32_t *d_cu_k, const int3
   g.cu_k = d_cu_k;
   g.idx = idx;
   // A: x, one row per box (the loaders gather rows by kept index)
-  CUtensorMap ma, mb, mo;
-  if (!make_map(&ma, in->x, total_rows, in->d, 1) || !make_map(&mb, w, d_out, in->d, kBN / 2) ||
-      !make_map(&mo, z, total_k, d_out, 32, 128 / epi_parts(kModeProject),
+  GemmMaps maps{};
+  if (!make_map(&maps.a, in->x, total_rows, in->d, 1) || !make_map(&maps.b, w, d_out, in->d, kBN / 2) ||
+      !make_map(&maps.out, z, total_k, d_out, 32, 128 / epi_parts(kModeProject),
                 epi_parts(kModeProject) == 2 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
     return TR_ERR_CUDA;
-  return launch_gemm<kModeProject>(ma, mb, mo, g, static_cast<cudaStream_t>(stream)) == cudaSuccess ? TR_OK
-                                                                                                     : TR_ERR_CUDA;
+  return launch_gemm<kModeProject>(maps, g, static_cast<cudaStream_t>(stream)) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 
 }  // extern "C"
