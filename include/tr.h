@@ -35,8 +35,9 @@
  *    synchronisation or copies), so they can be captured into a CUDA graph
  *    and replayed; make one call on the device outside the capture first
  *    (it raises the kernels' shared-memory limit once).
- *  - tr_select, tr_gather, tr_select_gather and tr_reduce launch their
- *    kernels with programmatic dependent launch: a kernel may be scheduled
+ *  - tr_select, tr_gather, tr_select_gather, tr_reduce, tr_mlp_hidden,
+ *    tr_mlp_score, tr_project_kept and tr_project launch their kernels with
+ *    programmatic dependent launch: a kernel may be scheduled
  *    while the kernel before it on the stream finishes, and waits in
  *    hardware for that kernel's completion before it reads anything, so
  *    stream order is kept (tr_score's kernel lets such a successor in as

@@ -100,15 +100,15 @@ inline Bounds certification_bounds(int d, int dtype) {
   if (dtype == TR_F32) ep *= 2.0;  // bf16 and fp16 products are exact in fp32
   // The encoder-MLP GEMM's epilogue (tr_mlp_score, bf16) writes the same
   // records: each term enters its double-float sum through TwoSum, over at
-  // most 128 columns per partial (low-part roundings below
-  // u^2 128 * 129 / 2 of the partial's sum|x'x''|), and the 2 ceil(d / 256)
-  // partials are merged (2 roundings of at most u^2 129 of the total each);
-  // the bound below, written for partials of up to 256 columns, covers that.
-  // The bounds cover both producers of a record.  Its L1, S2, A and B are
-  // within that same tiny relative error, far inside g below.
+  // most c = 128 columns per partial (low-part roundings below u^2 c (c + 1) /
+  // 2 of the partial's sum|x'x''|), and at most j = 8 ceil(d / 256) partials
+  // are merged, each merge two low-part additions whose sums stay below
+  // (c + j) u of the total: 2 j (c + j) u^2.  The bounds cover both producers
+  // of a record.  Its L1, S2, A and B are within that same tiny relative
+  // error, far inside g above.
   if (dtype == TR_BF16) {
-    const double col_blocks = (double)((d + 255) / 256);
-    const double ep_mlp = u * u * (256.0 * 257.0 / 2.0 + 2.0 * 257.0 * col_blocks) + 0x1p-52;
+    const double c = 128.0, j = 8.0 * (double)((d + 255) / 256);
+    const double ep_mlp = u * u * (c * (c + 1.0) / 2.0 + 2.0 * j * (c + j)) + 0x1p-52;
     if (ep_mlp > ep) ep = ep_mlp;
   }
   Bounds b;

@@ -24,41 +24,27 @@
 //               back to the producers and each finished accumulator to the
 //               epilogues;
 //   warps 2-    epilogue: one thread per accumulator row (TMEM lane: a
-//               warp reads the lane quarter warp % 4) and column part, 16
-//               columns per tcgen05.ld.  The score GEMM runs 8 warps (2-9,
-//               column halves): it stores x'' and x and accumulates the row
-//               sums.  The hidden GEMM runs 16 (2-17, column quarters):
-//               bias + activation, and H through TMA stores of 32 x 32
-//               blocks; the projector 8 (halves, 32 x 64 blocks).
+//               warp reads the lane quarter warp % 4); the tile's eight
+//               32-column blocks are dealt to the two or four warps of each
+//               quarter in turn.  Outputs leave through TMA stores of 32 x 32 blocks
+//               staged in shared memory; the score mode's x' and residual
+//               come in the same way.
+// When the tiles are few, clusters of two or four pairs share each tile's K
+// range and exchange the partial accumulators (kSplit, see below).
 // The projector mode (tr_project_kept) is the hidden GEMM with its A rows
 // gathered: A row j is token idx[j] of the image that owns kept slot j, so
 // the first projector layer reads X* = X_imp union X_div (Eq. 7) straight
-// from x without a gathered copy.  Four more warps (10-13) bring those
-// rows: lanes 0-7 of each load four rows of each A k-block with one TMA
-// tile::gather4 load (four 64-element rows of x by index, one-row box,
-// 128-byte swizzle -- the rows land in the layout the tensor cores read: the
-// swizzle follows the shared-memory address); a group with a row past the
-// kept slots (or a k-block past x's columns) takes four one-row tiled loads
-// instead, an outside row at coordinate -1, which reads zeros.  Each loader
-// warp's lane 0 adds its rows' bytes to the stage's transaction count and
-// arrives once.  The rate at which one warp issues TMA loads sets the pace:
-// 128 one-row loads per stage took 769 us from one warp and 273 us from
-// four, the gather4 loads 314 us from one warp and 200 us from four.  The
-// same layer on the gathered copy (tr_project: the hidden mode, plain tile
-// loads) is faster -- 86 us against 182 us on 12288 kept rows, 1024 -> 4096,
-// plus 12 us for the gather that writes the copy -- and gives the same z.
+// from x without a gathered copy.  It runs 8 epilogue warps, and four more
+// (10-13) bring those rows with TMA tile::gather4 loads (four 64-element rows
+// of x by index, one-row box, 128-byte swizzle -- the rows land in the layout
+// the tensor cores read: the swizzle follows the shared-memory address); a
+// group with a row past the kept slots (or a k-block past x's columns) takes
+// four one-row tiled loads instead, an outside row at coordinate -1, which
+// reads zeros.
 //
 // The epilogue of tile i overlaps the main loop of tile i + 1 (two TMEM
-// accumulators), but not for free: epilogue arithmetic on the SM
-// sub-partitions that also hold the producer and MMA warps slows the main
-// loop.  In a modified copy of the score GEMM with the sums' arithmetic
-// skipped on sub-partitions 0-1 it took 224 us, on 2-3 254 us, on all four
-// 193 us, against 257 us with none skipped.  So the epilogues do their fp32
-// arithmetic on packed pairs (add / mul / fma.f32x2, one instruction per two
-// columns): 6-7 % off all three modes.  A row's sums over its 2 n_tiles
-// column halves are combined by the last of the warps that worked on them
-// (an arrival counter; no warp or CTA waits for another), in column order,
-// so the record does not depend on which finished first.
+// accumulators).  It does its fp32 arithmetic on packed pairs (add / mul /
+// fma.f32x2, one instruction per two columns).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -74,41 +60,47 @@ namespace tr {
 namespace {
 
 constexpr int kBM = 128, kBN = 256, kBK = 64;  // a CTA's rows, a tile's columns, a k-block
-constexpr int kEpiWarps = 8;                      // score mode: two warpgroups, column halves of a tile
 enum { kModeHidden = 0, kModeScore = 1, kModeProject = 2 };
-// Epilogue warps per mode: the hidden GEMM's epilogue (activation and a TMA
-// store) runs four warpgroups, one per column quarter, so that more warps
-// hide the latencies of its TMEM loads and activation arithmetic; the score
-// and projector epilogues run two (column halves) -- the projector's
-// threads also include its four row-loader warps (measured on clip_mlp576's
-// projector: four loader warps with 8 epilogue warps 200 us, with 16 195 us
-// but spilling; two loader warps with 16, 226 us; eight with 8, 212 us).
-__host__ __device__ constexpr int epi_warps(int mode) { return mode == kModeHidden ? 2 * kEpiWarps : kEpiWarps; }
-__host__ __device__ constexpr int epi_parts(int mode) { return epi_warps(mode) / 4; }  // column parts of a tile
+// Epilogue warps per mode: four per lane quarter where the epilogue is on the
+// critical path (the hidden GEMM, whose main loop is short, and split tiles),
+// so that they hide the latencies of one another's TMEM loads and arithmetic;
+// two for the score GEMM's unsplit tiles (64 images x 576 tokens, D 1024,
+// hidden 4096, both GEMMs: 437 us, with four 446 us -- the main loop covers
+// this epilogue, and the staging it saves is a sixth operand stage) and for
+// the projector, whose threads include its row loaders.
+__host__ __device__ constexpr int epi_warps(int mode, int split) {
+  return mode == kModeHidden || (mode == kModeScore && split > 1) ? 16 : 8;
+}
+__host__ __device__ constexpr int epi_parts(int mode, int split) { return epi_warps(mode, split) / 4; }
 // producer, MMA issuer, epilogue (+ the A-row loader warps of the projector mode)
-constexpr int kLoadRows = 4;   // projector: rows per loader lane and k-block, one tile::gather4
-constexpr int kLoadWarps = 4;  // projector: loader warps, kBM / (kLoadRows kLoadWarps) lanes each
-constexpr int kLoadLanes = kBM / (kLoadRows * kLoadWarps);
-static_assert(kLoadLanes * kLoadRows * kLoadWarps == kBM && kLoadLanes <= 32, "the loaders cover a tile's rows");
-__host__ __device__ constexpr int gemm_threads(int mode) {
-  return 64 + 32 * epi_warps(mode) + (mode == kModeProject ? 32 * kLoadWarps : 0);
+constexpr int kLoadWarps = 4;  // projector: loader warps, 32 of a CTA's 128 rows each
+__host__ __device__ constexpr int gemm_threads(int mode, int split) {
+  return 64 + 32 * epi_warps(mode, split) + (mode == kModeProject ? 32 * kLoadWarps : 0);
 }
 constexpr int kTmemCols = 2 * kBN;                // two accumulators
-constexpr int kChunk = 16;                        // columns per tcgen05.ld
 constexpr int kPartWords = 10;                    // hi, lo of L1, S2, A, B, P
-// Per epilogue warp of the hidden and projector modes, a 32-row bf16 output
-// block staged for a TMA store: 32 columns (64-byte rows, 64-byte swizzle)
-// with four column parts, 64 (128-byte rows and swizzle) with two; 32 KiB in
-// all either way.
-constexpr int kStageOutAll = 32 * 1024;
-__host__ __device__ constexpr int stage_out(int mode) { return kStageOutAll / epi_warps(mode); }
-// The score mode's epilogue staging: per warp two buffers of a 32 x 32 block
-// of x' and one of the residual (2 KiB each, 64-byte rows and swizzle),
-// loaded by TMA ahead of their use and overwritten in place by x'' and x.
-constexpr int kScoreBlk = 32;                         // columns per block
-constexpr int kScoreHalfBuf = 32 * kScoreBlk * 2;     // bytes of one tensor's block
-constexpr int kScoreBuf = 2 * kScoreHalfBuf;          // x' / x'' block, residual / x block
-constexpr int kScoreStageAll = 2 * kScoreBuf * kEpiWarps;
+// The epilogue's unit: a block of 32 rows (one warp's TMEM lanes) x 32
+// columns in bf16, 2 KiB with 64-byte rows and the 64-byte swizzle (16-byte
+// unit u of row r at r * 64 + ((u ^ (r / 2 % 4)) << 4): the 32 lanes' 16-byte
+// accesses take the fewest shared-memory wavefronts).
+constexpr int kBlk = 32;
+constexpr int kTileBlks = kBN / kBlk;
+constexpr int kBlkBytes = 32 * kBlk * 2;
+// Staging per epilogue warp: the output block (the projector's warps two of
+// them); the score mode's blocks of x' and of the residual, loaded by TMA
+// ahead of their use and overwritten in place by x'' and x.
+__host__ __device__ constexpr int stage_blks(int mode) { return mode == kModeHidden ? 1 : 2; }
+__host__ __device__ constexpr int stage_bytes(int mode) { return stage_blks(mode) * kBlkBytes; }
+// Splits of K over the pairs of a cluster: pair p of kSplit sums its k-blocks
+// into its own accumulators and finishes the tile's blocks [p, p + 1) * 8 /
+// kSplit, whose partial sums the other pairs send it.
+__host__ __device__ constexpr int owned_blks(int split) { return kTileBlks / split; }
+// Warps per lane quarter with blocks of their own, and the score mode's
+// partial row sums per tile and lane quarter.
+__host__ __device__ constexpr int active_parts(int mode, int split) {
+  return owned_blks(split) < epi_parts(mode, split) ? owned_blks(split) : epi_parts(mode, split);
+}
+__host__ __device__ constexpr int row_parts(int split) { return split * active_parts(kModeScore, split); }
 
 struct GemmArgs {
   int m, n, k;          // C[m, n] = A[m, k] B[n, k]^T
@@ -116,7 +108,7 @@ struct GemmArgs {
   const float *bias;    // [n] or NULL
   int act;              // hidden GEMM: TR_ACT_*
   bool has_resid;       // score: x = x'' + residual
-  float *part;          // score: [row blocks][n_tiles][2 halves][4][kPartWords][32] partial sums
+  float *part;          // score: [row blocks][n_tiles][row parts][4][kPartWords][32] partial sums
   int32_t *err;         // optional: set when a pipeline wait timed out
   // projector mode: A row j = x[first row of the image owning kept slot j + idx[j]]
   long long total_rows;
@@ -234,34 +226,54 @@ __device__ __forceinline__ void df2_fold(DF &out, const DF2 &in) {  // even + od
   df_merge(out, in.hi.y, in.lo.y);
 }
 
-// Score GEMM epilogue for 16 columns of one row: x'' = bf16(acc + b2),
-// x = bf16(resid + x''); the five sums take the rounded values (products and
-// squares of bf16 values are exact in fp32; each term enters its double-float
-// sum through TwoSum).  x' and the residual come from this warp's staged
-// block (units u0, u0 + 1 of the lane's row) and x'' and x take their places.
-__device__ __forceinline__ void epi_score(const GemmArgs &g, int col0, const uint32_t (&v)[16], uint32_t rowbuf,
-                                          uint32_t u0, uint32_t u1, Acc2 &acc) {
-  uint32_t pw[8], rw[8], qo[8], xo[8];
-  tc::ld_shared_v4(rowbuf + u0, pw[0], pw[1], pw[2], pw[3]);
-  tc::ld_shared_v4(rowbuf + u1, pw[4], pw[5], pw[6], pw[7]);
-  if (g.has_resid) {
-    tc::ld_shared_v4(rowbuf + kScoreHalfBuf + u0, rw[0], rw[1], rw[2], rw[3]);
-    tc::ld_shared_v4(rowbuf + kScoreHalfBuf + u1, rw[4], rw[5], rw[6], rw[7]);
-  }
-  float2 a[8];
+// The epilogues work on one 16-byte unit (8 columns) of a lane's row at a
+// time, in loops that stay rolled: a tile's epilogue is short beside what it
+// takes to fetch its code (unrolled over a block, the scoring arithmetic ran
+// 17,000 clocks however few blocks a warp had).
+// acc + bias of 8 columns, as pairs.
+__device__ __forceinline__ void add_bias(const GemmArgs &g, int col0, const uint32_t (&v)[8], float2 (&a)[4]) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) a[i] = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
-  if (g.bias) {  // the same 16 values in every lane: four broadcast loads
+  for (int i = 0; i < 4; ++i) a[i] = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+  if (g.bias) {  // the same 8 values in every lane: two broadcast loads
     const float4 *bp = reinterpret_cast<const float4 *>(g.bias + col0);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 2; ++i) {
       const float4 b = __ldg(bp + i);
       a[2 * i] = __fadd2_rn(a[2 * i], make_float2(b.x, b.y));
       a[2 * i + 1] = __fadd2_rn(a[2 * i + 1], make_float2(b.z, b.w));
     }
   }
+}
+
+// Hidden / projector epilogue for 8 columns of one row: bf16(act(acc + bias))
+// to the staged unit at `addr`.
+__device__ __forceinline__ void epi_act(const GemmArgs &g, int col0, const uint32_t (&v)[8], uint32_t addr) {
+  float2 a[4];
+  add_bias(g, col0, v, a);
+  uint32_t w[4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < 4; ++i) {
+    const float2 h = activate2(a[i], g.act);
+    w[i] = pack_bf16x2(h.x, h.y);
+  }
+  tc::st_shared_v4(addr, w[0], w[1], w[2], w[3]);
+}
+
+// Score epilogue for 8 columns of one row: x'' = bf16(acc + b2),
+// x = bf16(resid + x''); the five sums take the rounded values (products and
+// squares of bf16 values are exact in fp32; each term enters its double-float
+// sum through TwoSum).  x' and the residual come from this warp's staged
+// blocks (the unit at `addr` and kBlkBytes further) and x'' and x take their
+// places.
+__device__ __forceinline__ void epi_score(const GemmArgs &g, int col0, const uint32_t (&v)[8], uint32_t addr,
+                                          Acc2 &acc) {
+  uint32_t pw[4], rw[4], qo[4], xo[4];
+  tc::ld_shared_v4(addr, pw[0], pw[1], pw[2], pw[3]);
+  if (g.has_resid) tc::ld_shared_v4(addr + kBlkBytes, rw[0], rw[1], rw[2], rw[3]);
+  float2 a[4];
+  add_bias(g, col0, v, a);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
     qo[i] = pack_bf16x2(a[i].x, a[i].y);  // x''
     const float2 q = bf16x2_f2(qo[i]);
     if (g.has_resid) {
@@ -278,236 +290,240 @@ __device__ __forceinline__ void epi_score(const GemmArgs &g, int col0, const uin
     df2_add_prod(acc.b, q, q);
     df2_add_prod(acc.p, p, q);
   }
-  tc::st_shared_v4(rowbuf + u0, qo[0], qo[1], qo[2], qo[3]);
-  tc::st_shared_v4(rowbuf + u1, qo[4], qo[5], qo[6], qo[7]);
-  tc::st_shared_v4(rowbuf + kScoreHalfBuf + u0, xo[0], xo[1], xo[2], xo[3]);
-  tc::st_shared_v4(rowbuf + kScoreHalfBuf + u1, xo[4], xo[5], xo[6], xo[7]);
+  tc::st_shared_v4(addr, qo[0], qo[1], qo[2], qo[3]);
+  tc::st_shared_v4(addr + kBlkBytes, xo[0], xo[1], xo[2], xo[3]);
 }
 
-// The stream of staged blocks of one score-epilogue warp: its column half's
-// 32-column blocks of each of the CTA's tiles in turn, block j in buffer
-// j % 2.  load_next issues the TMA loads of the next block not yet requested;
-// the buffer's previous stores must have been read (bulk_wait_read).
-struct ScoreStream {
-  uint32_t buf, bar;   // two buffers of kScoreBuf bytes, two mbarriers
-  int tile, blk;       // next block to request
-  uint32_t requested, used;
-  __device__ __forceinline__ uint32_t buffer(uint32_t j) const { return buf + (j & 1u) * (uint32_t)kScoreBuf; }
-  __device__ __forceinline__ uint32_t barrier(uint32_t j) const { return bar + 8u * (j & 1u); }
-  // Blocks of column half `half` of column tile nt that lie inside the output.
-  static __device__ __forceinline__ int blocks(const GemmArgs &g, int nt, int half) {
-    const int left = g.n - (nt * kBN + half * (kBN / 2));
-    return left <= 0 ? 0 : min(kBN / 2 / kScoreBlk, (left + kScoreBlk - 1) / kScoreBlk);
-  }
-  // Every lane keeps the place; lane 0 issues.  row_of(row tile) = first of
-  // this warp's 32 rows.
-  template <typename RowOf>
-  __device__ __forceinline__ void load_next(const GemmArgs &g, const GemmMaps &maps, int half, int tiles, int step,
-                                            RowOf row_of) {
-    int nt = 0;
-    while (tile < tiles) {
-      nt = tile % g.n_tiles;
-      if (blk < blocks(g, nt, half)) break;
-      tile += step;
-      blk = 0;
-    }
-    if (tile >= tiles) return;
-    if ((threadIdx.x & 31) == 0) {
-      const int col = nt * kBN + half * (kBN / 2) + blk * kScoreBlk, row = row_of(tile / g.n_tiles);
-      const uint32_t dst = buffer(requested), b = barrier(requested);
-      tc::mbar_expect_tx(b, g.has_resid ? kScoreBuf : kScoreHalfBuf);
-      tc::tma_load_2d(dst, &maps.p, col, row, b);
-      if (g.has_resid) tc::tma_load_2d(dst + kScoreHalfBuf, &maps.r, col, row, b);
-    }
-    ++requested;
-    ++blk;
-  }
+// One epilogue warp's place: its lane quarter, its blocks of a tile (first,
+// first + parts, ... below end) and its staging.
+struct EpiWarp {
+  int first, end;      // blocks of a tile (end: past the blocks this CTA finishes)
+  uint32_t buf, bar;   // staging, and the score mode's mbarrier of its loads
+  uint32_t loads;      // score: blocks requested so far
+  uint32_t used;       // score: blocks waited for so far
+  int tile, blk;       // score: the next block to request
 };
 
-// Score epilogue of one tile half for this warp (32 rows): 32-column blocks,
-// x' and the residual staged by TMA up to two blocks ahead, x'' and x written
-// over them and stored by TMA, so that global memory sees whole row segments
-// and no thread waits for a load that its next instruction needs (with loads
-// straight from global memory, one 16-column chunk ahead, a tile's epilogue
-// took 24,000-33,000 clocks).  False when a block's loads timed out.
-template <typename RowOf>
-__device__ __forceinline__ bool drain_tile_score(const GemmArgs &g, const GemmMaps &maps, ScoreStream &st,
-                                                 uint32_t taddr, int half, int nt, int row0, int tiles, int step,
-                                                 RowOf row_of, Acc &sums) {
-  const int lane = threadIdx.x & 31;
-  const int col_first = nt * kBN + half * (kBN / 2);
-  const int nblk = ScoreStream::blocks(g, nt, half);
-  if (nblk == 0) return true;
-  const int chunks = min(kBN / 2, g.n - col_first) / kChunk;  // n is a multiple of 16
-  const uint32_t tcol = taddr + (uint32_t)(half * (kBN / 2));
-  const uint32_t sw = (uint32_t)((lane >> 1) & 3);  // the 64-byte swizzle's row term
-  Acc2 acc2{};
-  uint32_t cur[16], nxt[16];
-  tc::tmem_ld16_issue(tcol, cur);
-  for (int b = 0; b < nblk; ++b) {
-    const uint32_t buf = st.buffer(st.used);
-    const bool ok = tc::mbar_wait(st.barrier(st.used), (st.used >> 1) & 1u);
-    ++st.used;
-    if (!__all_sync(0xffffffffu, ok)) {
-      tc::tmem_ld_wait(cur);
-      return false;
+// Score mode: requests the x' and residual blocks of the warp's next block
+// (every lane keeps the place; lane 0 issues).  The staged block must have
+// been stored (bulk_wait_read).  row_of(rb): first of this warp's 32 rows in
+// row tile rb.
+template <int kParts, typename RowOf>
+__device__ __forceinline__ void score_load_next(const GemmArgs &g, const GemmMaps &maps, EpiWarp &w, int step,
+                                                RowOf row_of) {
+  int nt = 0;
+  while (w.tile < g.tiles) {
+    nt = w.tile % g.n_tiles;
+    if (w.blk < w.end && nt * kBN + w.blk * kBlk < g.n) break;
+    w.tile += step;
+    w.blk = w.first;
+  }
+  if (w.tile >= g.tiles) return;
+  if ((threadIdx.x & 31) == 0) {
+    const int col = nt * kBN + w.blk * kBlk, row = row_of(w.tile / g.n_tiles);
+    tc::mbar_expect_tx(w.bar, g.has_resid ? 2 * kBlkBytes : kBlkBytes);
+    tc::tma_load_2d(w.buf, &maps.p, col, row, w.bar);
+    if (g.has_resid) tc::tma_load_2d(w.buf + kBlkBytes, &maps.r, col, row, w.bar);
+  }
+  ++w.loads;
+  w.blk += kParts;
+}
+
+// The partial sums of the other pairs for 8 columns are added to this pair's
+// (v), in the order of the pairs whatever pair this is, so that the result
+// does not depend on which pair owns the block.  slots: received partials,
+// [other pair][four-column unit of the owned columns][128 rows].
+template <int kSplit>
+__device__ __forceinline__ void add_partials(uint32_t slots, int pair, int unit, int row, uint32_t (&v)[8]) {
+  constexpr uint32_t kSlot = 128u * 4u * kBN / kSplit;
+  float sum[8];
+#pragma unroll
+  for (int o = 0; o < kSplit; ++o) {
+    float t[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) t[i] = __uint_as_float(v[i]);
+    if (o != pair) {
+      const uint32_t src = slots + (uint32_t)(o < pair ? o : o - 1) * kSlot + (uint32_t)(unit * 128 + row) * 16u;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        uint32_t r[4];
+        tc::ld_shared_v4(src + (uint32_t)u * 2048u, r[0], r[1], r[2], r[3]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) t[4 * u + i] = __uint_as_float(r[i]);
+      }
     }
-    const uint32_t rowbuf = buf + (uint32_t)(lane * kScoreBlk * 2);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int c = 2 * b + h;
-      if (c < chunks) {  // uniform
-        tc::tmem_ld_wait(cur);
-        const bool more = c + 1 < chunks;
-        if (more) tc::tmem_ld16_issue(tcol + (uint32_t)((c + 1) * kChunk), nxt);
-        epi_score(g, col_first + c * kChunk, cur, rowbuf, ((2u * h) ^ sw) << 4, ((2u * h + 1u) ^ sw) << 4, acc2);
-        if (more) {
-          tc::tmem_ld_wait(nxt);
+    for (int i = 0; i < 8; ++i) sum[i] = o == 0 ? t[i] : __fadd_rn(sum[i], t[i]);
+  }
 #pragma unroll
-          for (int i = 0; i < 16; ++i) cur[i] = nxt[i];
-        }
+  for (int i = 0; i < 8; ++i) v[i] = __float_as_uint(sum[i]);
+}
+
+// The epilogue of one tile for this warp: for each of its blocks, the
+// accumulator columns from TMEM, the mode's arithmetic into the staged block
+// and the TMA store(s).  Rows and columns past the output are computed from
+// zero operands and clipped by the store.  False when the score mode's loads
+// timed out.  (Score: with x' and the residual loaded straight from global
+// memory, 32 rows per warp load and one chunk ahead, a tile's epilogue took
+// 24,000-33,000 clocks.)
+template <int kMode, int kSplit, typename RowOf>
+__device__ __forceinline__ bool epilogue_tile(const GemmArgs &g, const GemmMaps &maps, EpiWarp &w, uint32_t taddr,
+                                              int nt, int row0, int step, RowOf row_of, uint32_t slots, int pair,
+                                              int row_in_tile, Acc2 &acc2) {
+  constexpr int kParts = epi_parts(kMode, kSplit);
+  constexpr int kUnits = kMode == kModeScore && kSplit > 1 ? 1 : 2;  // 8-column units in flight
+  const int lane = threadIdx.x & 31;
+  const uint32_t sw = (uint32_t)((lane >> 1) & 3);  // the 64-byte swizzle's row term
+  for (int blk = w.first; blk < w.end; blk += kParts) {
+    const int col = nt * kBN + blk * kBlk;
+    if (col >= g.n) break;
+    uint32_t buf = w.buf;
+    if (kMode == kModeScore) {
+      const bool ok = tc::mbar_wait(w.bar, w.used & 1u);
+      ++w.used;
+      if (!__all_sync(0xffffffffu, ok)) return false;
+    } else {  // the block's previous store must have been read
+      buf += (w.used % stage_blks(kMode)) * kBlkBytes;
+      ++w.used;
+      if (lane == 0) tc::bulk_wait_read<stage_blks(kMode) - 1>();
+      __syncwarp();
+    }
+    const uint32_t rowbuf = buf + (uint32_t)(lane * kBlk * 2);
+#pragma unroll 1
+    for (int u0 = 0; u0 < kBlk / 8; u0 += kUnits) {
+      if (col + 8 * u0 >= g.n) break;  // n is a multiple of 16
+      uint32_t v[kUnits][8];
+#pragma unroll
+      for (int i = 0; i < kUnits; ++i) tc::tmem_ld8(taddr + (uint32_t)(blk * kBlk + 8 * (u0 + i)), v[i]);
+#pragma unroll
+      for (int i = 0; i < kUnits; ++i) {
+        const int u = u0 + i;
+        if (kSplit > 1)
+          add_partials<kSplit>(slots, pair, (blk - pair * owned_blks(kSplit)) * 8 + 2 * u, row_in_tile, v[i]);
+        const uint32_t addr = rowbuf + (((uint32_t)u ^ sw) << 4);
+        if (kMode == kModeScore)
+          epi_score(g, col + 8 * u, v[i], addr, acc2);
+        else
+          epi_act(g, col + 8 * u, v[i], addr);
       }
     }
     tc::fence_async_shared();
     __syncwarp();
     if (lane == 0) {
-      if (row0 < g.m) {  // rows and columns past the output are clipped by the store
-        const int col = col_first + b * kScoreBlk;
+      if (row0 < g.m) {  // a block wholly past the last row is not stored
         tc::tma_store_2d(&maps.out, col, row0, buf);
-        tc::tma_store_2d(&maps.x, col, row0, buf + kScoreHalfBuf);
+        if (kMode == kModeScore) tc::tma_store_2d(&maps.x, col, row0, buf + kBlkBytes);
       }
       tc::bulk_commit();
-      tc::bulk_wait_read();
+      if (kMode == kModeScore) tc::bulk_wait_read<0>();  // the next loads overwrite the block
     }
-    __syncwarp();
-    st.load_next(g, maps, half, tiles, step, row_of);
+    if (kMode == kModeScore) {
+      __syncwarp();
+      score_load_next<kParts>(g, maps, w, step, row_of);
+    }
   }
-  df2_fold(sums.l1, acc2.l1);
-  df2_fold(sums.s2, acc2.s2);
-  df2_fold(sums.a, acc2.a);
-  df2_fold(sums.b, acc2.b);
-  df2_fold(sums.p, acc2.p);
   return true;
 }
 
-// Hidden / projector epilogue of one of a tile's kParts column parts for
-// this warp: chunks of 16 columns, H = bf16(act(acc + bias)), staged in this
-// warp's 32-row block of kBlk = 64 / (kParts / 2) columns, whose rows are
-// kBlk * 2 bytes with the swizzle of that span (unit u of row r at
-// r * 2 kBlk + ((u ^ ((r / (8 / (kBlk / 8))) % (kBlk / 8))) << 4): the 32
-// lanes' 16-byte writes take the fewest shared-memory wavefronts), and
-// written by one TMA store per block, so global memory sees whole row
-// segments.  The next chunk's TMEM load and bias are in flight while a chunk
-// is processed; the block is rewritten only after its previous store has
-// read it.  Rows and columns past the output are computed from zero operands
-// and clipped by the store.
-template <int kParts>
-__device__ __forceinline__ void drain_tile_store(const GemmArgs &g, const CUtensorMap *map_out, uint32_t buf,
-                                                 uint32_t taddr, int part, int nt, long long row0) {
-  constexpr int kChunks = kBN / kParts / kChunk;  // 8 (halves) or 4 (quarters)
-  constexpr int kBlk = 128 / kParts;              // block columns: 64 or 32
-  constexpr int kUnits = kBlk / 8;                // 16-byte units per block row: 8 or 4
-  constexpr int kPerBlk = kBlk / kChunk;          // chunks per block: 4 or 2
-  const int lane = threadIdx.x & 31;
-  const int col_first = nt * kBN + part * (kBN / kParts);
-  int chunks = 0;
-  while (chunks < kChunks && col_first + chunks * kChunk < g.n) ++chunks;
-  if (chunks == 0) return;
-  uint32_t cur[16], nxt[16];
-  float4 bc[4];
-  auto load_bias = [&](int col0, float4 (&b)[4]) {
-    if (g.bias) {
-      const float4 *bp = reinterpret_cast<const float4 *>(g.bias + col0);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) b[i] = __ldg(bp + i);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) b[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  };
-  const uint32_t tcol = taddr + (uint32_t)(part * (kBN / kParts));
-  tc::tmem_ld16_issue(tcol, cur);
-  tc::tmem_ld_wait(cur);
-  const uint32_t rowbuf = buf + (uint32_t)(lane * kBlk * 2);
-  const uint32_t sw = (uint32_t)((lane / (8 / kUnits)) % kUnits);  // the swizzle's row term
-  for (int c = 0; c < chunks; ++c) {
-    const int col0 = col_first + c * kChunk;
-    const bool more = c + 1 < chunks;
-    if (more) tc::tmem_ld16_issue(tcol + (uint32_t)((c + 1) * kChunk), nxt);
-    load_bias(col0, bc);  // the same 16 values in every lane (broadcast loads, cached)
-    const float bias[16] = {bc[0].x, bc[0].y, bc[0].z, bc[0].w, bc[1].x, bc[1].y, bc[1].z, bc[1].w,
-                            bc[2].x, bc[2].y, bc[2].z, bc[2].w, bc[3].x, bc[3].y, bc[3].z, bc[3].w};
-    uint32_t w[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float2 h = activate2(__fadd2_rn(make_float2(__uint_as_float(cur[2 * i]), __uint_as_float(cur[2 * i + 1])),
-                                            make_float2(bias[2 * i], bias[2 * i + 1])),
-                                 g.act);
-      w[i] = pack_bf16x2(h.x, h.y);
-    }
-    if (c % kPerBlk == 0 && c > 0) {  // the block's previous store must have read it
-      if (lane == 0) tc::bulk_wait_read();
-      __syncwarp();
-    }
-    const uint32_t u = 2u * (uint32_t)(c % kPerBlk);
-    tc::st_shared_v4(rowbuf + ((u ^ sw) << 4), w[0], w[1], w[2], w[3]);
-    tc::st_shared_v4(rowbuf + (((u + 1u) ^ sw) << 4), w[4], w[5], w[6], w[7]);
-    if (c % kPerBlk == kPerBlk - 1 || !more) {  // a block is complete: one TMA store for the warp's 32 rows
-      tc::fence_async_shared();
-      __syncwarp();
-      if (lane == 0 && row0 < g.m) {  // a block wholly past the last row is not stored
-        tc::tma_store_2d(map_out, col_first + kBlk * (c / kPerBlk), (int)row0, buf);
-        tc::bulk_commit();
-      }
-    }
-    if (more) {
-      tc::tmem_ld_wait(nxt);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) cur[i] = nxt[i];
+// Split tiles: this pair's partial sums of the blocks the other pairs finish
+// go to them (16-byte stores into the owner's shared memory, whose operand
+// ring is idle by then; 32 lanes write 512 consecutive bytes).
+template <int kMode, int kSplit>
+__device__ __forceinline__ void send_partials(uint32_t slots, uint32_t taddr, int pair, uint32_t rank, int part,
+                                              int row_in_tile) {
+  constexpr uint32_t kSlot = 128u * 4u * kBN / kSplit;
+  for (int blk = part; blk < kTileBlks; blk += epi_parts(kMode, kSplit)) {
+    const int owner = blk / owned_blks(kSplit);
+    if (owner == pair) continue;
+    const int unit = (blk - owner * owned_blks(kSplit)) * 8;
+    const uint32_t dst = tc::map_shared(slots + (uint32_t)(pair < owner ? pair : pair - 1) * kSlot +
+                                            (uint32_t)(unit * 128 + row_in_tile) * 16u,
+                                        2u * (uint32_t)owner + (rank & 1u));
+#pragma unroll 1
+    for (int u = 0; u < kBlk / 8; ++u) {
+      uint32_t v[8];
+      tc::tmem_ld8(taddr + (uint32_t)(blk * kBlk + 8 * u), v);
+      tc::st_cluster_v4(dst + (uint32_t)(2 * u) * 2048u, v[0], v[1], v[2], v[3]);
+      tc::st_cluster_v4(dst + (uint32_t)(2 * u + 1) * 2048u, v[4], v[5], v[6], v[7]);
     }
   }
-  if (lane == 0) tc::bulk_wait_read();  // the block may be rewritten by the next tile
-  __syncwarp();
 }
 
-// This warp's 32 rows of one tile half are done: their partial sums go to
-// the scratch; k_score_rows merges them once the GEMM has finished.
-__device__ __forceinline__ long long part_slot(const GemmArgs &g, int rb, int nt, int half, int q) {
-  return (((long long)(rb * g.n_tiles + nt) * 2 + half) * 4 + q) * (kPartWords * 32);
+// This warp's 32 rows are done for its blocks of a tile: their partial sums
+// go to the scratch; k_score_rows merges them once the GEMM has finished.
+__device__ __forceinline__ long long part_slot(const GemmArgs &g, int parts, int rb, int nt, int part, int q) {
+  return (((long long)(rb * g.n_tiles + nt) * parts + part) * 4 + q) * (kPartWords * 32);
 }
-__device__ __forceinline__ void publish_rows(const GemmArgs &g, int rb, int nt, int half, int q, const Acc &acc) {
-  float *dst = g.part + part_slot(g, rb, nt, half, q) + (threadIdx.x & 31);
+__device__ __forceinline__ void publish_rows(float *dst, const Acc2 &acc2) {
+  Acc acc{{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+  df2_fold(acc.l1, acc2.l1);
+  df2_fold(acc.s2, acc2.s2);
+  df2_fold(acc.a, acc2.a);
+  df2_fold(acc.b, acc2.b);
+  df2_fold(acc.p, acc2.p);
   const float vals[kPartWords] = {acc.l1.hi, acc.l1.lo, acc.s2.hi, acc.s2.lo, acc.a.hi,
                                   acc.a.lo,  acc.b.hi,  acc.b.lo,  acc.p.hi,  acc.p.lo};
 #pragma unroll
   for (int j = 0; j < kPartWords; ++j) __stcg(dst + 32 * j, vals[j]);
 }
 
-// The rows' records from the partial sums the score GEMM left: one warp per
-// 32 rows, the 2 n_tiles column halves merged in column order (the record
-// does not depend on which CTA made which part).  A kernel of its own, begun
-// while the GEMM drains: arrival counters inside the GEMM cost each tile a
-// fence over its stores, an atomic and, for the last warp, this same merge in
-// series (about 5,000 clocks a tile, and a memset before every launch).
-__global__ void __launch_bounds__(kBM) k_score_rows(const GemmArgs g, float4 *__restrict__ stats,
-                                                    float *__restrict__ h2, float *__restrict__ s_out) {
+// The rows' records from the partial sums the score GEMM left: a CTA per 32
+// rows, warp w of its kRowWarps merging parts w, w + kRowWarps, ... in turn
+// and warp 0 then the warps' sums, so that the record does not depend on
+// which CTA made which part; four parts' loads are in flight at a time (one
+// warp walking all parts with its loads one part ahead of their use took 19 us on
+// 36,864 rows and 34 us on 576 rows of a split GEMM).  A kernel of its own,
+// begun while the GEMM drains: arrival counters inside the GEMM cost each
+// tile a fence over its stores, an atomic and, for the last warp, this same
+// merge in series (about 5,000 clocks a tile, and a memset before every
+// launch).
+constexpr int kRowWarps = 8;
+__device__ __forceinline__ void merge_part(Acc &tot, const float (&w)[kPartWords]) {
+  df_merge(tot.l1, w[0], w[1]);
+  df_merge(tot.s2, w[2], w[3]);
+  df_merge(tot.a, w[4], w[5]);
+  df_merge(tot.b, w[6], w[7]);
+  df_merge(tot.p, w[8], w[9]);
+}
+__global__ void __launch_bounds__(kRowWarps * 32) k_score_rows(const GemmArgs g, const int parts,
+                                                               float4 *__restrict__ stats, float *__restrict__ h2,
+                                                               float *__restrict__ s_out) {
+  __shared__ float sh[kRowWarps][kPartWords][32];
   pdl_trigger();
   pdl_wait();  // the partial sums come from the GEMM before this kernel
-  const int rb = blockIdx.x, q = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long row = (long long)rb * kBM + threadIdx.x;
+  const int rb = blockIdx.x >> 2, q = blockIdx.x & 3, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int total = parts * g.n_tiles;
+  const float *src = g.part + part_slot(g, parts, rb, 0, 0, q) + lane;
+  constexpr int kStep = 4 * kPartWords * 32;  // floats from one part to the next (the four quarters between)
+  constexpr int kU = 4;
   Acc tot{{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-#pragma unroll 4
-  for (int t = 0; t < 2 * g.n_tiles; ++t) {
-    const float *src = g.part + part_slot(g, rb, t >> 1, t & 1, q) + lane;
-    float w[kPartWords];
+  for (int t0 = warp; t0 < total; t0 += kU * kRowWarps) {
+    float w[kU][kPartWords];
 #pragma unroll
-    for (int j = 0; j < kPartWords; ++j) w[j] = __ldcg(src + 32 * j);
-    df_merge(tot.l1, w[0], w[1]);
-    df_merge(tot.s2, w[2], w[3]);
-    df_merge(tot.a, w[4], w[5]);
-    df_merge(tot.b, w[6], w[7]);
-    df_merge(tot.p, w[8], w[9]);
+    for (int u = 0; u < kU; ++u) {
+      const int t = t0 + u * kRowWarps;
+      // past the last part: its values again, dropped below (no branch holds up the loads)
+      const float *p = src + (long long)(t < total ? t : t0) * kStep;
+#pragma unroll
+      for (int j = 0; j < kPartWords; ++j) w[u][j] = __ldcg(p + 32 * j);
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (t0 + u * kRowWarps < total) merge_part(tot, w[u]);  // uniform
   }
+  const float vals[kPartWords] = {tot.l1.hi, tot.l1.lo, tot.s2.hi, tot.s2.lo, tot.a.hi,
+                                  tot.a.lo,  tot.b.hi,  tot.b.lo,  tot.p.hi,  tot.p.lo};
+#pragma unroll
+  for (int j = 0; j < kPartWords; ++j) sh[warp][j][lane] = vals[j];
+  __syncthreads();
+  if (warp) return;
+  for (int w = 1; w < kRowWarps; ++w) {
+    float v[kPartWords];
+#pragma unroll
+    for (int j = 0; j < kPartWords; ++j) v[j] = sh[w][j][lane];
+    merge_part(tot, v);
+  }
+  const long long row = (long long)rb * kBM + 32 * q + lane;
   if (row < g.m) write_record(tot, row, stats, h2, s_out);
 }
 
@@ -544,29 +560,32 @@ __device__ __forceinline__ long long kept_source_row(const GemmArgs &g, long lon
 // rows runs here too, the odd CTA's rows read as zeros: what such a batch
 // waits for is W, and a pair brings each half of it into its own SM (128 rows,
 // D 1024, hidden 4096, both GEMMs: 57.4 us with a one-SM kernel, 55.3 here).
-// The score mode gives one stage to its epilogue's staging.
-__host__ __device__ constexpr int gemm_stages(int mode) { return mode == kModeScore ? 5 : 6; }
-__host__ __device__ constexpr int out_stage_bytes(int mode) {
-  return mode == kModeScore ? kScoreStageAll : kStageOutAll;
-}
+//
+// Splits: with few tiles most SMs would idle while a pair runs through all of
+// K, so a cluster of kSplit pairs shares a tile: pair p takes the k-blocks
+// [p, p + 1) * kblocks / kSplit, then the pairs exchange their partial sums
+// through distributed shared memory, each finishing 256 / kSplit of the
+// tile's columns.  One tile per cluster.
+// A split score GEMM gives one stage to its epilogue's staging.
+__host__ __device__ constexpr int gemm_stages(int mode, int split) { return mode == kModeScore && split > 1 ? 5 : 6; }
 constexpr int kHalfTile = 128 * kBK * 2;          // 128 rows of a k-block (A or B)
 constexpr int kStagePBytes = 2 * kHalfTile;       // this CTA's A rows + B rows
 constexpr uint32_t kIdescPair = tc::idesc_bf16(2 * kBM, kBN);
-__host__ __device__ constexpr int gemm_smem(int mode) {  // + alignment, barriers
-  return gemm_stages(mode) * kStagePBytes + out_stage_bytes(mode) + 1024 + 512;
+__host__ __device__ constexpr int gemm_smem(int mode, int split) {  // + alignment, barriers
+  return gemm_stages(mode, split) * kStagePBytes + epi_warps(mode, split) * stage_bytes(mode) + 1024 + 512;
 }
 
-template <int kMode>
-__global__ void __launch_bounds__(gemm_threads(kMode), 1)
+template <int kMode, int kSplit>
+__global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
     k_mlp_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
-  constexpr int kStagesP = gemm_stages(kMode);
+  constexpr int kStagesP = gemm_stages(kMode, kSplit);
   pdl_trigger();
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                           ~static_cast<uintptr_t>(1023));
   const uint32_t out_stage = tc::smem_u32(smem + (size_t)kStagesP * kStagePBytes);  // epilogue staging
-  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)kStagesP * kStagePBytes + out_stage_bytes(kMode));
-  constexpr int kBlkBars = kMode == kModeScore ? 2 * kEpiWarps : 0;  // the score epilogue's staged blocks
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)kStagesP * kStagePBytes + epi_warps(kMode, kSplit) * stage_bytes(kMode));
+  constexpr int kBlkBars = kMode == kModeScore ? epi_warps(kMode, kSplit) : 0;  // the score epilogue's staged blocks
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStagesP + 5 + kBlkBars);
   const uint32_t sbase = tc::smem_u32(smem);
   const uint32_t b0 = tc::smem_u32(bars);
@@ -575,14 +594,17 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
   auto tfull = [&](int a) { return b0 + 8u * (2 * kStagesP + a); };
   auto tempty = [&](int a) { return b0 + 8u * (2 * kStagesP + 2 + a); };
   const uint32_t done = b0 + 8u * (2 * kStagesP + 4);
-  auto blk_bar = [&](int w) { return b0 + 8u * (2 * kStagesP + 5 + 2 * w); };  // two of epilogue warp w
+  auto blk_bar = [&](int w) { return b0 + 8u * (2 * kStagesP + 5 + w); };  // of epilogue warp w
   auto sa = [&](int s) { return sbase + (uint32_t)(s * kStagePBytes); };
   auto sb = [&](int s) { return sbase + (uint32_t)(s * kStagePBytes + kHalfTile); };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = tc::cluster_rank();
+  const uint32_t crank = tc::cluster_rank();   // pair (split) crank / 2, CTA crank % 2 of it
+  const uint32_t rank = crank & 1u;
+  const int pair = kSplit > 1 ? (int)(crank >> 1) : 0;
   const bool leader = rank == 0;
-  const int cluster = blockIdx.x >> 1, clusters = gridDim.x >> 1;
+  const int cluster = blockIdx.x / (2 * kSplit), clusters = gridDim.x / (2 * kSplit);
+  const int kb_first = pair * g.kblocks / kSplit, kb_end = (pair + 1) * g.kblocks / kSplit;
   // operand bytes landing on the even CTA's stage barrier per k-block (both CTAs)
   constexpr uint32_t kTx = kMode == kModeProject ? 2 * kHalfTile : 2 * kStagePBytes;
   if (threadIdx.x == 0) {
@@ -592,10 +614,10 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
     }
     for (int a = 0; a < 2; ++a) {
       tc::mbar_init(tfull(a), 1);
-      tc::mbar_init(tempty(a), 2 * epi_warps(kMode));  // one arrival per epilogue warp of either CTA
+      tc::mbar_init(tempty(a), 2 * epi_warps(kMode, kSplit));  // one arrival per epilogue warp of either CTA
     }
     tc::mbar_init(done, 1);
-    for (int i = 0; i < kBlkBars; ++i) tc::mbar_init(blk_bar(0) + 8u * i, 1);
+    for (int i = 0; i < kBlkBars; ++i) tc::mbar_init(blk_bar(i), 1);
     tc::mbar_fence_init();
     tc::tma_prefetch_map(&maps.a);
     tc::tma_prefetch_map(&maps.b);
@@ -608,8 +630,11 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
   tc::cluster_sync();  // barriers initialised and TMEM allocated in both CTAs
   tc::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  auto full_even = [&](int s) { return tc::map_shared(full(s), 0); };
-  auto tempty_even = [&](int a) { return tc::map_shared(tempty(a), 0); };
+  pdl_wait();  // operands come from, and outputs may still be read by, the kernels before this one
+  const uint32_t even = crank & ~1u;           // the pair's even CTA in the cluster
+  const uint16_t both = (uint16_t)(0x3u << even);
+  auto full_even = [&](int s) { return tc::map_shared(full(s), even); };
+  auto tempty_even = [&](int a) { return tc::map_shared(tempty(a), even); };
   const int tiles = g.tiles;
 
   if (warp == 0) {
@@ -620,7 +645,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
       bool ok = true;
       for (int tile = cluster; tile < tiles && ok; tile += clusters) {
         const int rb = tile / g.n_tiles, nt = tile - rb * g.n_tiles;
-        for (int kb = 0; kb < g.kblocks; ++kb) {
+        for (int kb = kb_first; kb < kb_end; ++kb) {
           if (!tc::mbar_wait(empty(stage), phase ^ 1u)) {
             ok = false;
             break;
@@ -659,7 +684,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
         }
         tc::fence_after_sync();
         const uint32_t d = tmem + (uint32_t)(acc * kBN);
-        for (int kb = 0; kb < g.kblocks; ++kb) {
+        for (int kb = kb_first; kb < kb_end; ++kb) {
           if (!tc::mbar_wait(full(stage), phase)) {
             ok = false;
             break;
@@ -668,117 +693,130 @@ __global__ void __launch_bounds__(gemm_threads(kMode), 1)
           const uint64_t da = tc::sw128_desc(sa(stage)), db = tc::sw128_desc(sb(stage));
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
-            tc::mma_bf16_pair(d, da + 2u * k, db + 2u * k, kIdescPair, (kb | k) != 0);
-          tc::mma_commit_pair(empty(stage), 0x3);  // both CTAs' stage is free once these MMAs read it
+            tc::mma_bf16_pair(d, da + 2u * k, db + 2u * k, kIdescPair, kb != kb_first || k != 0);
+          tc::mma_commit_pair(empty(stage), both);  // both CTAs' stage is free once these MMAs read it
           if (++stage == kStagesP) {
             stage = 0;
             phase ^= 1u;
           }
         }
         if (!ok) break;
-        tc::mma_commit_pair(tfull(acc), 0x3);
+        tc::mma_commit_pair(tfull(acc), both);
         acc ^= 1;
         if (acc == 0) acc_phase ^= 1u;
       }
       if (!ok) flag_error(g, 2);
-      tc::mma_commit_pair(done, 0x3);
+      tc::mma_commit_pair(done, both);
     }
     __syncwarp();
     tc::mbar_wait_warp(done, 0);  // every pair MMA has completed (both CTAs' TMEM)
-  } else if (kMode == kModeProject && warp >= 2 + epi_warps(kMode)) {
+  } else if (kMode == kModeProject && warp >= 2 + epi_warps(kMode, kSplit)) {
     // ---------------------------------------------------------------- A rows (projector mode)
-    // lane l < kLoadLanes of loader warp w brings rows 4 j .. 4 j + 3 (j = w
-    // kLoadLanes + l) of this CTA's half of the pair's rows of each A k-block
-    // with one tile::gather4 load; a group with a row outside x (past the kept
-    // slots) or a k-block past x's columns takes four one-row loads instead, an
-    // outside row at coordinate -1, which reads zeros.  The loads land on the
-    // even CTA's barrier, whose loader warps expect both CTAs' bytes (the odd
-    // CTA's loader warps do not arrive)
-    const int j = (warp - 2 - epi_warps(kMode)) * kLoadLanes + lane;
-    const bool loads = lane < kLoadLanes;
+    // loader warp w brings rows 32 w .. 32 w + 31 of this CTA's half of the
+    // pair's rows of each A k-block with eight tile::gather4 loads; a group
+    // with a row outside x (past the kept slots) or a k-block past x's
+    // columns takes four one-row loads instead, an outside row at coordinate
+    // -1, which reads zeros.  The loads land on the even CTA's barrier, whose
+    // loader warps expect both CTAs' bytes (the odd CTA's loader warps do not
+    // arrive).  Each lane looks up one row; one thread issues.
+    const int lw = warp - 2 - epi_warps(kMode, kSplit);
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
     for (int tile = cluster; tile < tiles && ok; tile += clusters) {
       const int rb = tile / g.n_tiles;
-      int srow[kLoadRows];
-      bool whole = true;
+      const long long src = kept_source_row(g, (long long)rb * 2 * kBM + (long long)rank * kBM + 32 * lw + lane);
+      const int mine = src >= 0 ? (int)src : -1;
+      const uint32_t inside = __ballot_sync(0xffffffffu, mine >= 0);
+      int srow[32];
 #pragma unroll
-      for (int i = 0; i < kLoadRows; ++i) {
-        const long long src =
-            loads ? kept_source_row(g, (long long)rb * 2 * kBM + (long long)rank * kBM + kLoadRows * j + i) : -1;
-        srow[i] = src >= 0 ? (int)src : -1;
-        whole &= src >= 0;
-      }
-      for (int kb = 0; kb < g.kblocks; ++kb) {
-        if (!tc::mbar_wait_warp(empty(stage), phase ^ 1u)) {
-          ok = false;
-          break;
-        }
-        if (lane == 0 && leader) tc::mbar_expect_tx(full(stage), 2 * kHalfTile / kLoadWarps);
-        __syncwarp();
-        const uint32_t dst = sa(stage) + (uint32_t)(kLoadRows * j * kBK * 2);
-        if (loads) {
-          if (whole && (kb + 1) * kBK <= g.k) {  // rows and columns inside x
-            tc::tma_gather4_pair(dst, &maps.a, kb * kBK, srow[0], srow[1], srow[2], srow[3], full_even(stage));
-          } else {
+      for (int i = 0; i < 32; ++i) srow[i] = __shfl_sync(0xffffffffu, mine, i);
+      if (tc::elect_one()) {
+        for (int kb = kb_first; kb < kb_end; ++kb) {
+          if (!tc::mbar_wait(empty(stage), phase ^ 1u)) {
+            ok = false;
+            break;
+          }
+          if (leader) tc::mbar_expect_tx(full(stage), 2 * kHalfTile / kLoadWarps);
+          const uint32_t dst = sa(stage) + (uint32_t)(32 * lw * kBK * 2);
+          const uint32_t bar = full_even(stage);
+          const bool cols = (kb + 1) * kBK <= g.k;  // the k-block lies inside x's columns
 #pragma unroll
-            for (int i = 0; i < kLoadRows; ++i)
-              tc::tma_load_2d_pair(dst + (uint32_t)(i * kBK * 2), &maps.a, kb * kBK, srow[i], full_even(stage));
+          for (int j = 0; j < 8; ++j) {
+            if (cols && ((inside >> (4 * j)) & 0xfu) == 0xfu) {
+              tc::tma_gather4_pair(dst + (uint32_t)(4 * j * kBK * 2), &maps.a, kb * kBK, srow[4 * j], srow[4 * j + 1],
+                                   srow[4 * j + 2], srow[4 * j + 3], bar);
+            } else {
+#pragma unroll
+              for (int i = 4 * j; i < 4 * j + 4; ++i)
+                tc::tma_load_2d_pair(dst + (uint32_t)(i * kBK * 2), &maps.a, kb * kBK, srow[i], bar);
+            }
+          }
+          if (++stage == gemm_stages(kMode, kSplit)) {
+            stage = 0;
+            phase ^= 1u;
           }
         }
-        if (++stage == kStagesP) {
-          stage = 0;
-          phase ^= 1u;
-        }
+        if (!ok) flag_error(g, 8);
       }
+      ok = __all_sync(0xffffffffu, ok) != 0;  // (stage and phase live in the elected thread, the same one every time)
     }
-    if (!ok && lane == 0) flag_error(g, 8);
   } else {
     // ---------------------------------------------------------------- epilogue (both CTAs)
     const int q = warp & 3;            // TMEM lane quadrant this warp may read
-    const int part = (warp - 2) >> 2;  // column half (score, projector) or quarter (hidden) of the tile
-    // first of this warp's 32 rows in a tile of row block rb
+    const int part = (warp - 2) >> 2;  // which of the quadrant's warps
+    // first of this warp's 32 rows in row tile rb
     auto row_of = [&](int rb) { return (2 * rb + (int)rank) * kBM + 32 * q; };
-    ScoreStream st{out_stage + (uint32_t)((warp - 2) * 2 * kScoreBuf), blk_bar(warp - 2), cluster, 0, 0u, 0u};
-    if (kMode == kModeScore)
-      for (int i = 0; i < 2; ++i) st.load_next(g, maps, part, tiles, clusters, row_of);
+    const int own = pair * owned_blks(kSplit);
+    EpiWarp w{own + part, own + owned_blks(kSplit), out_stage + (uint32_t)((warp - 2) * stage_bytes(kMode)),
+              blk_bar(warp - 2), 0u, 0u, cluster, own + part};
+    if (kMode == kModeScore) score_load_next<epi_parts(kMode, kSplit)>(g, maps, w, clusters, row_of);
     int acc = 0;
     uint32_t acc_phase = 0;
     for (int tile = cluster; tile < tiles; tile += clusters) {
       const int rb = tile / g.n_tiles, nt = tile - rb * g.n_tiles;
-      if (!tc::mbar_wait_warp(tfull(acc), acc_phase)) {
-        if (lane == 0) flag_error(g, 4);
-        break;
-      }
+      if (g.bias)  // the first blocks' bias on its way to L1 while the main loop runs
+        for (int blk = w.first; blk < w.end; blk += epi_parts(kMode, kSplit))
+          if (nt * kBN + blk * kBlk + lane < g.n) tc::touch(g.bias + nt * kBN + blk * kBlk + lane);
+      bool ok = tc::mbar_wait_warp(tfull(acc), acc_phase);
+      if (!ok && lane == 0) flag_error(g, 4);
       tc::fence_after_sync();
       const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * kBN);
-      Acc sums{{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-      if (kMode == kModeScore) {
-        if (!drain_tile_score(g, maps, st, taddr, part, nt, row_of(rb), tiles, clusters, row_of, sums)) {
-          if (lane == 0) flag_error(g, 16);
-          break;
-        }
-      } else {
-        drain_tile_store<epi_parts(kMode)>(g, &maps.out, out_stage + (uint32_t)((warp - 2) * stage_out(kMode)), taddr,
-                                           part, nt, row_of(rb));
+      if (kSplit > 1) {  // every pair's MMAs are done: the operand rings may take the partial sums
+        tc::cluster_sync();
+        if (ok) send_partials<kMode, kSplit>(sbase, taddr, pair, rank, part, 32 * q + lane);
+        tc::cluster_sync();
       }
+      Acc2 sums{};
+      if (ok && !epilogue_tile<kMode, kSplit>(g, maps, w, taddr, nt, row_of(rb), clusters, row_of, sbase, pair,
+                                              32 * q + lane, sums)) {
+        ok = false;
+        if (lane == 0) flag_error(g, 16);
+      }
+      if (!ok) break;
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive_cluster(tempty_even(acc));  // this warp is done with the accumulator
       const int rb128 = 2 * rb + (int)rank;
-      if (kMode == kModeScore && rb128 * kBM < g.m) publish_rows(g, rb128, nt, part, q, sums);
+      if (kMode == kModeScore && rb128 * kBM < g.m && part < active_parts(kMode, kSplit))
+        publish_rows(g.part + part_slot(g, row_parts(kSplit), rb128, nt, pair * active_parts(kMode, kSplit) + part, q) +
+                         lane,
+                     sums);
       acc ^= 1;
       if (acc == 0) acc_phase ^= 1u;
     }
     if (lane == 0) {
-      if (kMode == kModeScore)  // blocks requested and not used (after a timeout) land before the CTA may exit
-        for (; st.used < st.requested; ++st.used) tc::mbar_wait(st.barrier(st.used), (st.used >> 1) & 1u);
+      if (kMode == kModeScore && w.used != w.loads)  // a block requested and not used (after a timeout) lands first
+        tc::mbar_wait(w.bar, w.used & 1u);
       tc::bulk_wait();  // this warp's output stores have completed
     }
     __syncwarp();
   }
 
+  if (kSplit > 1 && (warp < 2 || warp >= 2 + epi_warps(kMode, kSplit))) {  // the two barriers around the exchange
+    tc::cluster_sync();
+    tc::cluster_sync();
+  }
   tc::fence_before_sync();
   tc::cluster_sync();  // neither CTA leaves while the other may still signal its barriers
   if (warp == 1) {
@@ -824,42 +862,74 @@ bool make_map(CUtensorMap *map, const void *base, long long rows, long long cols
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Per device (index & 63): bit mode * 3 + log2(split) set once the variant's
+// shared-memory limit is raised and its co-resident clusters are counted.
 std::atomic<int> g_gemm_set[64];
-std::atomic<int> g_gemm_clusters[64][3];
+std::atomic<int> g_gemm_clusters[64][9];
 
-template <int kMode>
+template <int kMode, int kSplit>
 cudaError_t launch_gemm(const GemmMaps &maps, const GemmArgs &g, cudaStream_t st) {
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
-  const int bit = 1 << kMode;
+  constexpr int kVariant = kMode * 3 + (kSplit == 4 ? 2 : kSplit - 1);
   cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(gemm_threads(kMode));
-  cfg.dynamicSmemBytes = gemm_smem(kMode);
+  cfg.blockDim = dim3(gemm_threads(kMode, kSplit));
+  cfg.dynamicSmemBytes = gemm_smem(kMode, kSplit);
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.x = 2 * kSplit;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (!(g_gemm_set[dev & 63].load() & bit)) {
-    err = cudaFuncSetAttribute(k_mlp_gemm<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(kMode));
+  if (!(g_gemm_set[dev & 63].load() & (1 << kVariant))) {
+    err = cudaFuncSetAttribute(k_mlp_gemm<kMode, kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               gemm_smem(kMode, kSplit));
     if (err != cudaSuccess) return err;
     int clusters = 0;
-    cfg.gridDim = dim3(2 * 64);
-    err = cudaOccupancyMaxActiveClusters(&clusters, k_mlp_gemm<kMode>, &cfg);
+    cfg.gridDim = dim3(2 * kSplit * 64);
+    err = cudaOccupancyMaxActiveClusters(&clusters, k_mlp_gemm<kMode, kSplit>, &cfg);
     if (err != cudaSuccess) return err;
     if (clusters <= 0) return cudaErrorInvalidConfiguration;
-    g_gemm_clusters[dev & 63][kMode].store(clusters);
-    g_gemm_set[dev & 63].fetch_or(bit);
+    g_gemm_clusters[dev & 63][kVariant].store(clusters);
+    g_gemm_set[dev & 63].fetch_or(1 << kVariant);
   }
-  const int max_clusters = g_gemm_clusters[dev & 63][kMode].load();
-  const int clusters = g.tiles < max_clusters ? g.tiles : max_clusters;
-  cfg.gridDim = dim3(2 * clusters);
-  return cudaLaunchKernelEx(&cfg, k_mlp_gemm<kMode>, maps, g);
+  const int max_clusters = g_gemm_clusters[dev & 63][kVariant].load();
+  // split tiles: one per cluster (the grid may be larger than what runs at once)
+  const int clusters = kSplit > 1 || g.tiles < max_clusters ? g.tiles : max_clusters;
+  cfg.gridDim = dim3(2 * kSplit * clusters);
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, k_mlp_gemm<kMode, kSplit>, maps, g);
 }
+
+// Splits of K for a GEMM of `tiles` output tiles and `kblocks` k-blocks: four
+// (or two) while the clusters all run at once -- 16 clusters of eight SMs, 32
+// of four -- and the main loop is long enough: a k-block takes about 520
+// clocks, the exchange 4,500 (two pairs) to 7,000 (four; 96 KiB into each
+// SM).  576 rows, D 1024, hidden 4096: the score GEMM (12 tiles of 64
+// k-blocks) 45 us unsplit, 21 in four; a 192-row, 1024 -> 4096 layer (16
+// tiles of 16 k-blocks) 16.6 us unsplit, 24 in four.  The sums of a tile are
+// the same for every mode (tr_project and tr_project_kept agree bit for bit).
+inline int gemm_split(int tiles, int kblocks) {
+  if (tiles <= 16 && kblocks >= 32) return 4;
+  if (tiles <= 32 && kblocks >= 24) return 2;
+  return 1;
+}
+
+template <int kMode>
+cudaError_t launch_split(const GemmMaps &maps, const GemmArgs &g, cudaStream_t st) {
+  switch (gemm_split(g.tiles, g.kblocks)) {
+    case 4: return launch_gemm<kMode, 4>(maps, g, st);
+    case 2: return launch_gemm<kMode, 2>(maps, g, st);
+    default: return launch_gemm<kMode, 1>(maps, g, st);
+  }
+}
+
+inline int row_tiles(int m) { return (int)(((long long)m + 2 * kBM - 1) / (2 * kBM)); }
 
 bool misaligned16(const void *p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
 
@@ -882,10 +952,11 @@ struct MlpWs {
 };
 MlpWs mlp_ws(const tr_mlp *m) {
   const long long rblocks = ((long long)m->t + kBM - 1) / kBM;
-  const long long n_tiles = (m->d + kBN - 1) / kBN;
+  const int n_tiles = (m->d + kBN - 1) / kBN;
+  const int parts = row_parts(gemm_split(row_tiles(m->t) * n_tiles, (m->d_hidden + kBK - 1) / kBK));
   MlpWs w;
   w.part = 0;
-  w.total = align_up((size_t)rblocks * n_tiles * 2 * 4 * kPartWords * 32 * sizeof(float), 256);
+  w.total = align_up((size_t)rblocks * n_tiles * parts * 4 * kPartWords * 32 * sizeof(float), 256);
   return w;
 }
 
@@ -900,17 +971,16 @@ tr_status dense_act_gemm(const void *a, int rows, int k, const void *w, const fl
   g.n = n;
   g.k = k;
   g.n_tiles = (g.n + kBN - 1) / kBN;
-  g.tiles = (g.m + 2 * kBM - 1) / (2 * kBM) * g.n_tiles;
+  g.tiles = row_tiles(g.m) * g.n_tiles;
   g.kblocks = (g.k + kBK - 1) / kBK;
   g.bias = bias;
   g.act = act;
   g.err = d_error;
   GemmMaps maps{};
   if (!make_map(&maps.a, a, rows, k, kBM) || !make_map(&maps.b, w, n, k, kBN / 2) ||
-      !make_map(&maps.out, out, rows, n, 32, 128 / epi_parts(kModeHidden),
-                epi_parts(kModeHidden) == 2 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
+      !make_map(&maps.out, out, rows, n, 32, kBlk, CU_TENSOR_MAP_SWIZZLE_64B))
     return TR_ERR_CUDA;
-  return launch_gemm<kModeHidden>(maps, g, st) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
+  return launch_split<kModeHidden>(maps, g, st) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 
 }  // namespace
@@ -963,7 +1033,7 @@ tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, fl
   g.n = m->d;
   g.k = m->d_hidden;
   g.n_tiles = (g.n + kBN - 1) / kBN;
-  g.tiles = (g.m + 2 * kBM - 1) / (2 * kBM) * g.n_tiles;
+  g.tiles = row_tiles(g.m) * g.n_tiles;
   g.kblocks = (g.k + kBK - 1) / kBK;
   g.bias = m->b2;
   g.has_resid = m->resid != nullptr;
@@ -971,14 +1041,15 @@ tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, fl
   g.err = d_error;
   GemmMaps maps{};
   auto block_map = [&](CUtensorMap *map, const void *p) {  // the epilogue's 32 x 32 blocks
-    return make_map(map, p, m->t, m->d, 32, kScoreBlk, CU_TENSOR_MAP_SWIZZLE_64B);
+    return make_map(map, p, m->t, m->d, 32, kBlk, CU_TENSOR_MAP_SWIZZLE_64B);
   };
   if (!make_map(&maps.a, h, m->t, m->d_hidden, kBM) || !make_map(&maps.b, m->w2, m->d, m->d_hidden, kBN / 2) ||
       !block_map(&maps.p, m->x_pre) || (m->resid && !block_map(&maps.r, m->resid)) || !block_map(&maps.out, x_post) ||
       !block_map(&maps.x, x))
     return TR_ERR_CUDA;
-  if (launch_gemm<kModeScore>(maps, g, st) != cudaSuccess) return TR_ERR_CUDA;
-  const cudaError_t err = launch_kernel(k_score_rows, dim3((g.m + kBM - 1) / kBM), dim3(kBM), 0, st, true, g,
+  if (launch_split<kModeScore>(maps, g, st) != cudaSuccess) return TR_ERR_CUDA;
+  const int parts = row_parts(gemm_split(g.tiles, g.kblocks));
+  const cudaError_t err = launch_kernel(k_score_rows, dim3((g.m + kBM - 1) / kBM * 4), dim3(kRowWarps * 32), 0, st, true, g, parts,
                                         reinterpret_cast<float4 *>(stats), h2, s);
   return err == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
@@ -1012,7 +1083,7 @@ tr_status tr_project_kept(const tr_tokens *in, const int32_t *d_cu_k, const int3
   g.n = d_out;
   g.k = in->d;
   g.n_tiles = (g.n + kBN - 1) / kBN;
-  g.tiles = (g.m + 2 * kBM - 1) / (2 * kBM) * g.n_tiles;
+  g.tiles = row_tiles(g.m) * g.n_tiles;
   g.kblocks = (g.k + kBK - 1) / kBK;
   g.bias = bias;
   g.act = act;
@@ -1026,10 +1097,9 @@ tr_status tr_project_kept(const tr_tokens *in, const int32_t *d_cu_k, const int3
   // A: x, one row per box (the loaders gather rows by kept index)
   GemmMaps maps{};
   if (!make_map(&maps.a, in->x, total_rows, in->d, 1) || !make_map(&maps.b, w, d_out, in->d, kBN / 2) ||
-      !make_map(&maps.out, z, total_k, d_out, 32, 128 / epi_parts(kModeProject),
-                epi_parts(kModeProject) == 2 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
+      !make_map(&maps.out, z, total_k, d_out, 32, kBlk, CU_TENSOR_MAP_SWIZZLE_64B))
     return TR_ERR_CUDA;
-  return launch_gemm<kModeProject>(maps, g, static_cast<cudaStream_t>(stream)) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
+  return launch_split<kModeProject>(maps, g, static_cast<cudaStream_t>(stream)) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 
 }  // extern "C"

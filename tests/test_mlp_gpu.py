@@ -240,3 +240,53 @@ def test_project_kept_index_outside_its_image():
         rows[slot] = x[row]
     v, mag = _gemm_ref(rows, w, bias)
     _check_close(z, _sigma(v, "gelu"), mag, slope=1.13)
+
+
+# GEMMs whose K is split over the pairs of a cluster: 256 x 256 tiles and
+# 64-wide k-blocks at the edges of the rule (16 / 32 tiles, 32 / 24 k-blocks),
+# with ragged rows, columns and k-blocks and k-blocks that do not divide evenly.
+SPLIT_CASES = [
+    ("four_one_row", 1, 256, 2048, "none", False, True),         # 1 tile, 32 k-blocks
+    ("four_uneven_k", 300, 528, 2224, "gelu", True, True),       # 6 tiles, 34.75 k-blocks
+    ("four_most_tiles", 1000, 1024, 2112, "quick_gelu", True, False),  # 16 tiles, 33 k-blocks
+    ("two_few_k", 257, 272, 1552, "gelu", True, True),           # 4 tiles, 24.25 k-blocks
+    ("two_most_tiles", 2048, 784, 2064, "gelu", False, True),    # 32 tiles, 32.25 k-blocks
+    ("none_few_k", 129, 1056, 1472, "gelu", True, True),         # 5 tiles, 23 k-blocks
+    ("none_more_tiles", 2049, 784, 1600, "none", True, True),    # 36 tiles, 25 k-blocks
+]
+
+
+@pytest.mark.parametrize("name,t,d,dh,act,resid,bias", SPLIT_CASES, ids=[c[0] for c in SPLIT_CASES])
+def test_mlp_split(name, t, d, dh, act, resid, bias):
+    test_mlp_outputs_and_records(name, t, d, dh, act, resid, bias)
+    # a second call reproduces every bit: the partial sums are added in a fixed order
+    altr = _alt()
+    xp, w1, w2, b1, b2, r = _inputs(t, d, dh, seed=3, resid=resid, bias=bias)
+    m = altr.Mlp(t, w1, w2, b1, b2, act=act)
+    first = [v.clone() for v in (lambda o: (o.h, o.x_post, o.x, o.stats))(m.run(xp, r))]
+    again = (lambda o: (o.h, o.x_post, o.x, o.stats))(m.run(xp, r))
+    torch.cuda.synchronize()
+    for u, v in zip(first, again):
+        assert torch.equal(u.view(torch.int16), v.view(torch.int16))
+
+
+@pytest.mark.parametrize("d,d_out,k", [(2064, 528, 40), (1600, 1280, 200)], ids=["four", "two"])
+def test_project_split(d, d_out, k):
+    # K split: the dense projector within the GEMM tolerance of float64, and the
+    # rows read by index bit for bit the same
+    altr = _alt()
+    g = torch.Generator(device="cuda").manual_seed(9)
+    n, b = 300, 3
+    x = torch.randn(b * n, d, generator=g, device="cuda").to(torch.bfloat16)
+    idx = torch.rand(b, n, generator=g, device="cuda").argsort(1)[:, :k].sort(1).values.to(torch.int32)
+    w = (torch.randn(d_out, d, generator=g, device="cuda") / math.sqrt(d)).to(torch.bfloat16)
+    bias = 0.05 * torch.randn(d_out, generator=g, device="cuda")
+    y = torch.cat([x[i * n:(i + 1) * n][idx[i].long()] for i in range(b)]).contiguous()
+    z, err = altr.project(y, w, bias, act="gelu")
+    zk, err_k = altr.project_kept(x, idx.reshape(-1).contiguous(), [i * k for i in range(b + 1)], w, bias, act="gelu",
+                                  seqlens=[n] * b)
+    torch.cuda.synchronize()
+    assert err.item() == 0 and err_k.item() == 0
+    assert torch.equal(z.view(torch.int16), zk.view(torch.int16))
+    v, mag = _gemm_ref(y, w, bias)
+    _check_close(z, _sigma(v, "gelu"), mag, slope=1.13)
