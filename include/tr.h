@@ -183,12 +183,14 @@ tr_status tr_gather(const tr_tokens *in, const int32_t *d_cu_k, const int32_t *i
                     void *stream);
 
 /*
- * Selection and gather in one launch, from the statistics of tr_score: the
+ * Selection and gather in one call, from the statistics of tr_score: the
  * result of tr_select (idx, optional H2 / s fix-ups, status) plus the kept
- * rows y as tr_gather would copy them.  When there are fewer images than
- * SMs, each image's selection is run by several CTAs at once and each copies
- * its share of the kept rows (the selection is deterministic, so all reach
- * the same indices; only one writes idx and the status words).
+ * rows y as tr_gather would copy them.  Large images of a small batch: the
+ * launches of tr_select and tr_gather.  Otherwise one launch; when there are
+ * fewer images than SMs, each image's selection is run by several CTAs at
+ * once and each copies its share of the kept rows (the selection is
+ * deterministic, so all reach the same indices; only one writes idx and the
+ * status words).
  *   total_k:  host int, = cu_k[batch]; y: device [total_k, d], 16-byte aligned.
  *   Other arguments as in tr_select (role is not produced).
  */
@@ -199,7 +201,8 @@ tr_status tr_select_gather(const tr_tokens *in, const float *stats, const int32_
 /*
  * The whole path in one call on `stream`, with the statistics kept in the
  * workspace: tr_score then tr_select_gather for a uniform batch (two kernel
- * launches); tr_score, tr_select and tr_gather for a ragged one (three).
+ * launches, three for large images of a small batch); tr_score, tr_select and
+ * tr_gather for a ragged one (three).
  *   total_k:  host int, = cu_k[batch] (the number of output rows).
  *   y:        device [total_k, d] in the input dtype, 16-byte aligned.
  *   idx, h2, s, d_status: as in tr_select (role is not produced); h2 and s

@@ -180,6 +180,10 @@ tr_status tr_select_gather(const tr_tokens *in, const float *stats, const int32_
   if (in->batch > 0 && (!stats || !d_k || !d_k1 || !d_cu_k || !idx || (total_k > 0 && !y))) return TR_ERR_ARG;
   if (misaligned(stats, 16) || misaligned(y, 16)) return TR_ERR_ALIGN;
   if ((rc = check_ws(sh, ws, ws_bytes)) != TR_OK) return rc;
+  if (select_cluster_ctas(in->batch, sh.max_n) > 1) {  // a cluster per image, then the grid-wide copy
+    rc = tr_select(in, stats, d_k, d_k1, d_cu_k, idx, nullptr, h2, s, ws, ws_bytes, d_status, stream);
+    return rc == TR_OK ? tr_gather(in, d_cu_k, idx, total_k, y, stream) : rc;
+  }
   SelectArgs a = select_args(in, sh, stats, d_k, d_k1, d_cu_k, idx, nullptr, h2, s, ws, d_status);
   cudaError_t err = launch_select_gather(a, y, static_cast<cudaStream_t>(stream), true);
   return err == cudaSuccess ? TR_OK : TR_ERR_CUDA;

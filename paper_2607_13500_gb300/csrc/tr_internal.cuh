@@ -202,6 +202,26 @@ cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
   cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
+// The same with clusters of `cluster` CTAs.
+template <typename... P, typename... A>
+cudaError_t launch_kernel_cluster(void (*kernel)(P...), dim3 grid, dim3 block, int cluster, size_t smem,
+                                  cudaStream_t st, bool pdl, A &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // ---------------------------------------------------------------- launchers
 struct SelectArgs {
@@ -224,6 +244,9 @@ struct SelectArgs {
 size_t select_smem_bytes(int max_n);  // dynamic shared memory of one select CTA
 cudaError_t launch_score(const void *x, const void *x_pre, const void *x_post, int dtype, int d, long long total,
                          float *stats, float *h2, float *s, cudaStream_t st);
+// CTAs per image of an uncapped selection: more than one (a cluster) for
+// large images of a small batch.
+int select_cluster_ctas(int batch, int max_n);
 // max_ctas > 0 caps the grid (each CTA then selects several images in turn);
 // pdl: programmatic dependent launch after the kernel before it on st.
 cudaError_t launch_select(const SelectArgs &a, cudaStream_t st, int max_ctas, bool pdl);

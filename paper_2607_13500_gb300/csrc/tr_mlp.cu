@@ -783,8 +783,10 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
       tc::fence_after_sync();
       const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * kBN);
       if (kSplit > 1) {  // every pair's MMAs are done: the operand rings may take the partial sums
+        __syncwarp();
         tc::cluster_sync();
         if (ok) send_partials<kMode, kSplit>(sbase, taddr, pair, rank, part, 32 * q + lane);
+        __syncwarp();
         tc::cluster_sync();
       }
       Acc2 sums{};

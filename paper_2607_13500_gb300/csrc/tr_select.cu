@@ -8,8 +8,10 @@
 // the same deterministic selection (only replica 0 writes idx and the status
 // words) and copies its 1/R share of the image's kept rows, so the copies of
 // one image overlap the selections of the others on SMs that would be idle.
+#include <algorithm>
 #include <atomic>
 
+#include "tr_select_cluster.cuh"
 #include "tr_select_dev.cuh"
 
 namespace tr {
@@ -22,6 +24,17 @@ __global__ void __launch_bounds__(kSelectThreads, 1) k_select(const SelectArgs a
   pdl_trigger();
   pdl_wait();  // the statistics come from the kernel before this one
   for (int b = blockIdx.x; b < a.batch; b += gridDim.x) select_image(a, b, smem);
+}
+
+// A cluster of c CTAs per image (large images of small batches).
+__global__ void __launch_bounds__(kSelectThreads, 1) k_select_cluster(const SelectArgs a, const int c) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  pdl_trigger();
+  pdl_wait();  // the statistics come from the kernel before this one
+  const int b = blockIdx.x / c, rank = (int)tc::cluster_rank();
+  if (select_image_cluster(a, b, c, rank, smem)) return;
+  cluster_barrier();  // nobody reads this CTA's shared memory any more
+  if (rank == 0) select_image(a, b, smem);
 }
 
 __device__ __forceinline__ uint4 ld_nc16(const uint4 *p) {
@@ -84,7 +97,7 @@ __global__ void __launch_bounds__(kSelectThreads, 1)
 }
 
 // Per device (index & 63): dynamic shared memory limit already raised (bit 0
-// k_select, bit 1 k_select_gather), and the SM count.  Atomic so that first
+// k_select, bit 1 k_select_gather, bit 2 k_select_cluster), and the SM count.  Atomic so that first
 // calls from several host threads are well defined (raising the limit twice
 // is harmless).
 std::atomic<int> g_smem_set[64];
@@ -108,11 +121,34 @@ cudaError_t raise_smem_limit(K kernel, int dev) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
+// A cluster per image pays from about 2500 tokens on (below, its barriers
+// cost what the split passes save) and while the clusters run at once; more
+// CTAs than that only queue.  Reduction of B images, us with 1 / 2 / 4 / 8
+// CTAs per image (bf16, D 512, K = N / 8):
+//   N 2048:  B 1   20.9 /  22.7 /  22.0 /  22.6
+//   N 2880:  B 1   26.7 /  24.7 /  24.4 /  23.5   B 64  195 / 189 / 203 / 244
+//   N 6272:  B 1   40.7 /  34.6 /  30.8 /  28.7   B 8   96.4 / 85.4 / 81.5 / 80.2
+//            B 16  138 / 127 / 123 / 132          B 32  220 / 210 / 207 / 231
+//   N 16384: B 1    103 /  76.0 /  61.5 /  53.7   B 16  331 / 285 / 272 / 289
+int select_cluster_ctas(int batch, int max_n) {
+  if (batch <= 0 || max_n < 2560) return 1;
+  return batch <= 12 ? 8 : (batch <= 36 ? 4 : (batch <= 72 ? 2 : 1));
+}
+
 cudaError_t launch_select(const SelectArgs &a, cudaStream_t st, int max_ctas, bool pdl) {
   if (a.batch == 0) return cudaSuccess;
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
+  const int c = max_ctas > 0 ? 1 : select_cluster_ctas(a.batch, a.max_n);
+  if (c > 1) {
+    if (!(g_smem_set[dev & 63].load() & 4)) {
+      if ((err = raise_smem_limit(k_select_cluster, dev)) != cudaSuccess) return err;
+      g_smem_set[dev & 63].fetch_or(4);
+    }
+    const size_t need = std::max(cluster_smem_bytes(a.max_n, c), select_smem_bytes(a.max_n));
+    return launch_kernel_cluster(k_select_cluster, dim3(a.batch * c), dim3(kSelectThreads), c, need, st, pdl, a, c);
+  }
   const size_t smem = select_smem_bytes(a.max_n);
   if (!(g_smem_set[dev & 63].load() & 1)) {
     if ((err = raise_smem_limit(k_select, dev)) != cudaSuccess) return err;

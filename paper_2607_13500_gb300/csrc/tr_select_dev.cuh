@@ -638,20 +638,17 @@ __device__ __forceinline__ void exact_row_any(const SelectArgs &a, long long row
 // Runs longer than this skip the tier: long runs are exact ties in practice.
 constexpr int kDfRunMax = 32;
 
-// Value of element i of a 16-byte chunk as fp32 (exact for all three types).
+// The elements of one 32-bit word as fp32 (exact for all three types; one
+// element for fp32, two otherwise).
 template <int kDt>
-__device__ __forceinline__ void unpack_f32(const uint4 &v, float *out) {
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+__device__ __forceinline__ void unpack_word(uint32_t w, float (&out)[2]) {
   if (kDt == TR_BF16) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      out[2 * i] = __uint_as_float(w[i] << 16);
-      out[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-    }
+    out[0] = __uint_as_float(w << 16);
+    out[1] = __uint_as_float(w & 0xffff0000u);
   } else if (kDt == TR_F16) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint32_t h = (w[i >> 1] >> (16 * (i & 1))) & 0xffffu;
+    for (int i = 0; i < 2; ++i) {
+      const uint32_t h = (w >> (16 * i)) & 0xffffu;
       const uint32_t sg = (h & 0x8000u) << 16, ex = (h >> 10) & 0x1fu, mant = h & 0x3ffu;
       float f;
       if (ex == 0x1fu)
@@ -663,8 +660,8 @@ __device__ __forceinline__ void unpack_f32(const uint4 &v, float *out) {
       out[i] = f;
     }
   } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) out[i] = __uint_as_float(w[i]);
+    out[0] = __uint_as_float(w);
+    out[1] = 0.f;
   }
 }
 
@@ -686,14 +683,6 @@ __device__ __forceinline__ void df_join(float &hi, float &lo, float h2, float l2
   hi = r.h;
   lo = __fadd_rn(__fadd_rn(lo, l2), r.l);
 }
-__device__ __forceinline__ void df_warp_join(float &hi, float &lo) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-    df_join(hi, lo, h2, l2);
-  }
-}
-
 struct PartDf {
   float h[kWarps * 3], l[kWarps * 3];
   int ok[4];  // per group: the row's keys were written
@@ -703,73 +692,70 @@ struct PartDf {
 // A, B, P of x', x'') by a group of warps; writes rec->r_* or rec->s_* and
 // returns true, uniformly across the group, or false when the row is not
 // eligible (nothing written).
+//
+// The code is kept small on purpose: a CTA comes here once or twice per launch
+// and for a few rows, so fetching the instructions is a good part of what it
+// costs.  (With two chunks' elements unrolled, settling the pick runs of a
+// 6272-token clip took 9.8 us of its selection's 29.5; with two elements per
+// iteration 8.9.)
 template <int kDt>
 __device__ __noinline__ bool df_row_block(const SelectArgs &a, long long row, int mode, ExactRec *rec, PartDf &part,
                                           const Group g) {
   constexpr int kPer = kDt == TR_F32 ? 4 : 8;  // elements per 16-byte chunk
-  constexpr int kLoads = 2;                    // chunks per stream in flight per thread
   const int nchunks = a.d / kPer;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   bool ok = true;
   float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
   const uint4 *p0 = static_cast<const uint4 *>(mode == 0 ? a.x : (a.x_pre ? a.x_pre : a.x)) + row * nchunks;
-  const uint4 *p1 = static_cast<const uint4 *>(a.x_post) + row * nchunks;
-  for (int c0 = g.tid(); c0 < nchunks; c0 += kLoads * g.size) {
-    uint4 u0[kLoads], u1[kLoads];
-#pragma unroll
-    for (int j = 0; j < kLoads; ++j) {  // every load of the round first
-      const int c = c0 + j * g.size;
-      if (c < nchunks) {
-        u0[j] = __ldg(p0 + c);
-        if (mode != 0) u1[j] = __ldg(p1 + c);
-      }
+  const uint4 *p1 = mode == 0 ? p0 : static_cast<const uint4 *>(a.x_post) + row * nchunks;
+  uint4 n0 = make_uint4(0u, 0u, 0u, 0u), n1 = n0;
+  if (g.tid() < nchunks) {
+    n0 = __ldg(p0 + g.tid());
+    n1 = __ldg(p1 + g.tid());
+  }
+#pragma unroll 1
+  for (int c = g.tid(); c < nchunks; c += g.size) {
+    uint4 u0 = n0, u1 = n1;
+    if (c + g.size < nchunks) {  // the next chunk's loads are in flight meanwhile
+      n0 = __ldg(p0 + c + g.size);
+      n1 = __ldg(p1 + c + g.size);
     }
+#pragma unroll 1
+    for (int w = 0; w < 4; ++w) {
+      float v0[2], v1[2];
+      unpack_word<kDt>(u0.x, v0);
+      unpack_word<kDt>(u1.x, v1);
 #pragma unroll
-    for (int j = 0; j < kLoads; ++j) {
-      if (c0 + j * g.size >= nchunks) break;
-      float v0[kPer], v1[kPer];
-      unpack_f32<kDt>(u0[j], v0);
-      if (mode == 0) {
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-          const float x = v0[i];
-          ok &= df_value_ok(x);
-          df_term(h0, l0, fabsf(x));
-          if (kDt == TR_F32) {
-            const df::F2 q = df::two_prod(x, x);
-            df_term(h1, l1, q.h);
-            l1 = __fadd_rn(l1, q.l);
-          } else {
-            df_term(h1, l1, __fmul_rn(x, x));
-          }
+      for (int i = 0; i < (kDt == TR_F32 ? 1 : 2); ++i) {
+        const float p = v0[i], q = v1[i];  // mode 0: both x
+        ok &= df_value_ok(p) && df_value_ok(q);
+        // the terms |x|, x^2 (mode 0) or x'^2, x''^2, x'x'', products exact
+        // (fp32: as TwoProd pairs)
+        const df::F2 pp = kDt == TR_F32 ? df::two_prod(p, p) : df::F2{__fmul_rn(p, p), 0.f};
+        const df::F2 qq = kDt == TR_F32 ? df::two_prod(q, q) : df::F2{__fmul_rn(q, q), 0.f};
+        df_term(h0, l0, mode == 0 ? fabsf(p) : pp.h);
+        df_term(h1, l1, qq.h);
+        if (kDt == TR_F32) {
+          if (mode != 0) l0 = __fadd_rn(l0, pp.l);
+          l1 = __fadd_rn(l1, qq.l);
         }
-      } else {
-        unpack_f32<kDt>(u1[j], v1);
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-          const float p = v0[i], q = v1[i];
-          ok &= df_value_ok(p) && df_value_ok(q);
-          if (kDt == TR_F32) {
-            const df::F2 pp2 = df::two_prod(p, p), qq2 = df::two_prod(q, q), pq2 = df::two_prod(p, q);
-            df_term(h0, l0, pp2.h);
-            l0 = __fadd_rn(l0, pp2.l);
-            df_term(h1, l1, qq2.h);
-            l1 = __fadd_rn(l1, qq2.l);
-            df_term(h2, l2, pq2.h);
-            l2 = __fadd_rn(l2, pq2.l);
-          } else {
-            df_term(h0, l0, __fmul_rn(p, p));
-            df_term(h1, l1, __fmul_rn(q, q));
-            df_term(h2, l2, __fmul_rn(p, q));
-          }
+        if (mode != 0) {
+          const df::F2 pq = kDt == TR_F32 ? df::two_prod(p, q) : df::F2{__fmul_rn(p, q), 0.f};
+          df_term(h2, l2, pq.h);
+          if (kDt == TR_F32) l2 = __fadd_rn(l2, pq.l);
         }
       }
+      u0 = make_uint4(u0.y, u0.z, u0.w, 0u);  // the next word
+      u1 = make_uint4(u1.y, u1.z, u1.w, 0u);
     }
   }
   if (!g.all(ok)) return false;
-  df_warp_join(h0, l0);
-  df_warp_join(h1, l1);
-  if (mode != 0) df_warp_join(h2, l2);
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) {
+    df_join(h0, l0, __shfl_xor_sync(0xffffffffu, h0, o), __shfl_xor_sync(0xffffffffu, l0, o));
+    df_join(h1, l1, __shfl_xor_sync(0xffffffffu, h1, o), __shfl_xor_sync(0xffffffffu, l1, o));
+    df_join(h2, l2, __shfl_xor_sync(0xffffffffu, h2, o), __shfl_xor_sync(0xffffffffu, l2, o));
+  }
   if (lane == 0) {
     part.h[warp * 3 + 0] = h0;
     part.l[warp * 3 + 0] = l0;

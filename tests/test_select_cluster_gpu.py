@@ -1,0 +1,124 @@
+"""The selection of large images by a cluster of CTAs (k_select_cluster)
+against the oracle: the edges of its rule (2560 tokens; 12, 36 and 72 images
+for eight, four and two CTAs), images much smaller than the batch's largest,
+near-ties at the cut and at the picks, and the inputs it leaves to the
+one-CTA selection (exact ties, crowded keys, rows outside the fp32 model).
+Kept indices and rows are compared bit for bit.
+"""
+import pytest
+import torch
+
+from test_parity_gpu import _near_tie_triples, _rows, check_reduce
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_2607_13500_gb300 import _build
+    _build.build()
+
+
+def _budget(ks, k1s):
+    cu = [0]
+    for k in ks:
+        cu.append(cu[-1] + k)
+    return list(ks), list(k1s), cu
+
+
+@pytest.mark.parametrize("batch,n,d,dtype", [
+    (1, 2559, 128, torch.bfloat16), (1, 2560, 128, torch.bfloat16), (1, 2561, 64, torch.float32),
+    (3, 4099, 64, torch.float16), (12, 2563, 64, torch.bfloat16), (13, 2816, 64, torch.bfloat16),
+    (36, 2560, 32, torch.float32), (37, 2600, 64, torch.bfloat16), (72, 2560, 64, torch.bfloat16),
+    (73, 2560, 64, torch.bfloat16), (1, 16384, 64, torch.bfloat16), (2, 16383, 32, torch.float32),
+])
+def test_sizes(batch, n, d, dtype):
+    x, xp, xq = _rows(batch * n, d, 7 * n + batch, dtype)
+    images = sorted({0, batch // 2, batch - 1})
+    for k, k1, stride in [(n // 9, n // 27, "alg1"), (n // 3 + 1, n // 10, "interval")]:
+        check_reduce(x, xp, xq, [n] * batch, _budget([k] * batch, [k1] * batch), images=images, stride=stride)
+
+
+def test_ragged_sizes():
+    seqlens = [2560, 1, 16384, 255, 0, 7000, 16, 513]
+    x, xp, xq = _rows(sum(seqlens), 64, 5, torch.bfloat16)
+    ks = [max(1, 2 * n // 9) if n else 0 for n in seqlens]
+    check_reduce(x, xp, xq, seqlens, _budget(ks, [k // 3 for k in ks]))
+
+
+@pytest.mark.parametrize("k,k1", [(1, 0), (1, 1), (2, 1), (3000, 1000), (3000, 0), (2999, 2999), (1500, 1500),
+                                  (2999, 1), (700, 0)])
+def test_budgets(k, k1):
+    n = 3000
+    x, xp, xq = _rows(n, 128, 11, torch.bfloat16)
+    check_reduce(x, xp, xq, [n], _budget([k], [k1]))
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "f32"])
+def test_near_ties(dtype):
+    # triples that the fp32 keys leave uncertain and the double-float keys
+    # separate, among ordinary rows: no exact sums are needed, wherever the cut
+    # splits a triple and for dense and sparse picks
+    d = 1024
+    tx, tp, tq, *_ = _near_tie_triples(32, d, dtype, 3)
+    x, xp, xq = (torch.cat([a, b]) for a, b in zip((tx, tp, tq), _rows(2500, d, 4, dtype)))
+    perm = torch.randperm(x.shape[0], generator=torch.Generator().manual_seed(6))
+    x, xp, xq = x[perm], xp[perm], xq[perm]
+    n = x.shape[0]
+    v = x.double()
+    order = torch.argsort(v.abs().sum(1) ** 2 / (v * v).sum(1), descending=True)
+    members = (perm[order] < 96).nonzero()[:, 0]  # places of the triples' rows by R
+    for k1, k2, stride in [(int(members[31]), 400, "alg1"), (int(members[34]) + 1, 1200, "alg1"),
+                           (int(members[60]), 701, "interval"), (0, 900, "interval")]:
+        st = check_reduce(x, xp, xq, [n], _budget([k1 + k2], [k1]), stride=stride)
+        assert st[2] == 0, st
+
+    # exact ties: a few rows twice, one pair at the cut; their runs, and only
+    # they, take exact sums
+    pairs = [(int(order[members[20]]), 5)] + [(i, n - 1 - i) for i in range(40, 60)]
+    for i, j in pairs:
+        x[j], xp[j], xq[j] = x[i], xp[i], xq[i]
+    v = x.double()
+    r = v.abs().sum(1) ** 2 / (v * v).sum(1)
+    place = int((r > r[5]).sum())  # the tied pair at the cut holds places `place` and `place` + 1 (in its run)
+    for k1, k2 in [(place + 1, 1000), (0, n - 1)]:
+        st = check_reduce(x, xp, xq, [n], _budget([k1 + k2], [k1]))
+        assert 0 < st[2] <= 4 * len(pairs) + 8, st
+
+
+def test_left_to_one_cta():
+    n, d = 2600, 64
+    base, bp, bq = _rows(n, d, 21, torch.bfloat16)
+
+    def run(edit, k=600, k1=200, **kw):
+        x, xp, xq = base.clone(), bp.clone(), bq.clone()
+        edit(x, xp, xq)
+        return check_reduce(x, xp, xq, [n], _budget([k], [k1]), **kw)
+
+    def ties(x, xp, xq):  # every row four times, far apart
+        for v in (x, xp, xq):
+            v.copy_(v[:n // 4].repeat(4, 1))
+
+    def equal(x, xp, xq):
+        for v in (x, xp, xq):
+            v.copy_(v[:1].expand(n, d).clone())
+
+    def crowded(x, xp, xq):  # one far outlier: nearly all keys fall into one bucket
+        x[7] = 0
+        x[7, 0] = 1
+        xq[9] = -xp[9]
+        x[100:2400] = x[100:101] + 0.01 * torch.randn(2300, d, generator=torch.Generator().manual_seed(1)).to(x.dtype)
+
+    def outside(x, xp, xq):
+        x[3, 1] = float("nan")
+        x[5] = 0
+        xq[11, 0] = float("inf")
+        xp[12] = 0
+        x[13] = x[13] * 2.0 ** 70
+
+    assert run(ties)[2] > 0
+    run(equal)
+    run(crowded)
+    run(outside, expect_nonfinite=True)
