@@ -123,6 +123,14 @@ const char *tr_version(void);
 tr_status tr_budgets(int32_t batch, const int32_t *h_seqlens, int32_t k, int32_t r_num, int32_t r_den,
                      int32_t lam_num, int32_t lam_den, int32_t *h_k, int32_t *h_k1, int32_t *h_cu_k);
 
+/*
+ * d_dst[0..n) = h_src[0..n): budgets and offsets (n small) from the host to
+ * the device in stream order, carried by the parameters of a kernel (up to
+ * 1000 words a launch).  h_src may be reused at return; nothing is copied
+ * or synchronised, and a captured call replays the same words.
+ */
+tr_status tr_put_words(int32_t *d_dst, const int32_t *h_src, int32_t n, void *stream);
+
 /* Device workspace bytes that tr_select and tr_reduce need for `in`
  * (0 on invalid input).  The workspace must be 256-byte aligned. */
 size_t tr_workspace_bytes(const tr_tokens *in);

@@ -78,6 +78,7 @@ def load() -> ctypes.CDLL:
     lib.tr_version.argtypes, lib.tr_version.restype = [], ctypes.c_char_p
     lib.tr_budgets.argtypes = [I32, P(I32), I32, I32, I32, I32, I32, P(I32), P(I32), P(I32)]
     lib.tr_budgets.restype = I32
+    lib.tr_put_words.argtypes, lib.tr_put_words.restype = [VP, VP, I32, VP], I32
     lib.tr_workspace_bytes.argtypes, lib.tr_workspace_bytes.restype = [tok], SZ
     lib.tr_score.argtypes, lib.tr_score.restype = [tok, VP, VP, VP, VP], I32
     lib.tr_select.argtypes = [tok, VP, VP, VP, VP, VP, VP, VP, VP, VP, SZ, VP, VP]

@@ -6,6 +6,7 @@ when libtr.so is missing or a tensor is not on a CUDA device.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 from dataclasses import dataclass
 
@@ -29,7 +30,7 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _check_buf(t, device, dtype, min_numel, name):
@@ -41,8 +42,31 @@ def _check_buf(t, device, dtype, min_numel, name):
         raise ValueError(f"{name} must be a contiguous {dtype} tensor of at least {min_numel} elements on {device}")
 
 
-def _stream(device) -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+def _stream(device) -> int:
+    """The raw handle of torch's current stream on ``device``."""
+    index = device.index
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if index is None else index)
+
+
+# A kernel launch carries this many words; longer arrays go up by copy.
+_MAX_PUT_WORDS = 4 * 1000
+
+
+def _device_words(words, device) -> torch.Tensor:
+    """int32 device tensor of a host sequence, written by a kernel that carries
+    the words as its parameters: in stream order on the current stream, with
+    no host buffer to keep, no copy and no synchronisation (a pageable copy,
+    torch.tensor(..., device=...), waits for the stream to drain).  For use on
+    that stream."""
+    if device.type == "cuda" and 0 < len(words) <= _MAX_PUT_WORDS:
+        try:
+            buf = array.array("i", words)
+        except (TypeError, OverflowError):  # not plain int32 values: torch's conversions and errors
+            return torch.tensor(words, dtype=torch.int32, device=device)
+        t = torch.empty(len(buf), dtype=torch.int32, device=device)
+        check("tr_put_words", load().tr_put_words(t.data_ptr(), buf.buffer_info()[0], len(buf), _stream(device)))
+        return t
+    return torch.tensor(words, dtype=torch.int32, device=device)
 
 
 def _flatten(x, x_pre, x_post, seqlens):
@@ -61,41 +85,114 @@ def _flatten(x, x_pre, x_post, seqlens):
             raise ValueError("seqlens must sum to the number of rows of x")
     else:
         raise ValueError("x must be [B, N, D] or [T, D]")
-    for t in (x, x_pre, x_post):
-        if t is None:
-            continue
-        if t.shape != x.shape or t.dtype != x.dtype or t.device != x.device:
-            raise ValueError("x, x_pre and x_post must share shape, dtype and device")
-        if not t.is_contiguous():
-            raise ValueError("token tensors must be contiguous")
-    if x.device.type != "cuda":
-        raise ValueError("token tensors must live on a CUDA device (libtr has no CPU path)")
+    _check_tokens(x, x_pre, x_post)
     return x, x_pre, x_post, seqlens
 
 
-class _Tokens:
-    """A TrTokens struct plus the device tensors it points into."""
+def _check_tokens(x, x_pre, x_post):
+    shape, dtype, device = x.shape, x.dtype, x.device
+    if not x.is_contiguous():
+        raise ValueError("token tensors must be contiguous")
+    for t in (x_pre, x_post):
+        if t is None:
+            continue
+        if t.shape != shape or t.dtype != dtype or t.device != device:
+            raise ValueError("x, x_pre and x_post must share shape, dtype and device")
+        if not t.is_contiguous():
+            raise ValueError("token tensors must be contiguous")
+    if device.type != "cuda":
+        raise ValueError("token tensors must live on a CUDA device (libtr has no CPU path)")
 
-    def __init__(self, x, x_pre, x_post, seqlens, stride="alg1"):
+
+def _cu_seqlens(seqlens):
+    """Row offsets of the images, or None when they all have the same size."""
+    if len(set(seqlens)) <= 1:
+        return None
+    cu = [0]
+    for n in seqlens:
+        cu.append(cu[-1] + n)
+    return cu
+
+
+class _Tokens:
+    """A TrTokens struct plus the device tensors it points into.  ``cu``: the
+    row offsets on the device, where the caller keeps them."""
+
+    def __init__(self, x, x_pre, x_post, seqlens, stride="alg1", cu=None):
         self.x, self.x_pre, self.x_post, self.seqlens = x, x_pre, x_post, seqlens
         if stride not in STRIDE_MODES:
             raise ValueError(f"stride must be one of {sorted(STRIDE_MODES)}")
-        uniform = len(set(seqlens)) <= 1
-        self.cu = None
-        if not uniform:
-            cu = [0]
-            for n in seqlens:
-                cu.append(cu[-1] + n)
-            self.cu = torch.tensor(cu, dtype=torch.int32, device=x.device)
+        self.cu = cu
+        if cu is None:
+            offsets = _cu_seqlens(seqlens)
+            if offsets is not None:
+                self.cu = _device_words(offsets, x.device)
         self.s = TrTokens(
             x=x.data_ptr(), x_pre=None if x_pre is None else x_pre.data_ptr(), x_post=x_post.data_ptr(),
             dtype=_dtype_code(x), d=x.shape[1], batch=len(seqlens),
-            n=seqlens[0] if (uniform and seqlens) else 0,
+            n=seqlens[0] if (self.cu is None and seqlens) else 0,
             cu_seqlens=None if self.cu is None else self.cu.data_ptr(),
             total=x.shape[0], max_n=max(seqlens) if seqlens else 0, flags=STRIDE_MODES[stride])
+        self._ref = ctypes.byref(self.s)
+
+    def rebind(self, x, x_pre, x_post):
+        """The same images in other tensors."""
+        self.x, self.x_pre, self.x_post = x, x_pre, x_post
+        s = self.s
+        s.x, s.x_post = x.data_ptr(), x_post.data_ptr()
+        s.x_pre = None if x_pre is None else x_pre.data_ptr()
+        s.dtype, s.d, s.total = _dtype_code(x), x.shape[1], x.shape[0]
+        return self
 
     def ref(self):
-        return ctypes.byref(self.s)
+        return self._ref
+
+
+class _Bound:
+    """What Reducer and Pipeline share: the images of a fixed batch shape and
+    their budgets, kept on the device, and the token struct of the tensors of
+    the call at hand."""
+
+    def _setup(self, seqlens, d, dtype, device, k, ratio, lam, alias_pre, budget, stride, sync):
+        self.lib = load()
+        self.seqlens = [int(v) for v in seqlens]
+        self.device = torch.device(device)
+        self.d, self.dtype, self.alias_pre, self.stride = d, dtype, alias_pre, stride
+        self.ks, self.k1s, self.cu_k = budget if budget is not None else budgets(self.seqlens, k, ratio, lam)
+        self.total_k = self.cu_k[-1]
+        self._total = sum(self.seqlens)
+        self._tok = None
+        dev = self.device
+        offsets = _cu_seqlens(self.seqlens)
+        if sync:  # complete at return, whatever stream the object is used on
+            mk = lambda v: torch.tensor(v, dtype=torch.int32, device=dev)
+            self.d_k, self.d_k1, self.d_cu = mk(self.ks), mk(self.k1s), mk(self.cu_k)
+            self._cu = None if offsets is None else mk(offsets)
+            return torch.zeros(TR_STATUS_WORDS, dtype=torch.int32, device=dev)
+        # used on the current stream only: one launch writes everything
+        b = len(self.seqlens)
+        parts = [[0] * TR_STATUS_WORDS, self.ks, self.k1s, self.cu_k] + ([] if offsets is None else [offsets])
+        if len(self.ks) != b or len(self.k1s) != b or len(self.cu_k) != b + 1:
+            mk = lambda v: torch.tensor(v, dtype=torch.int32, device=dev)
+            views = [mk(v) for v in parts]
+        else:
+            views = _device_words([w for v in parts for w in v], dev).split([len(v) for v in parts])
+        self.d_k, self.d_k1, self.d_cu = views[1:4]
+        self._cu = None if offsets is None else views[4]
+        return views[0]
+
+    def _bind(self, x, x_pre, x_post):
+        if x.dim() == 2:
+            if x.shape[0] != self._total:
+                raise ValueError("seqlens must sum to the number of rows of x")
+            _check_tokens(x, x_pre, x_post)
+        else:
+            x, x_pre, x_post, _ = _flatten(x, x_pre, x_post, self.seqlens)
+        if self._tok is None:
+            self._tok = _Tokens(x, x_pre, x_post, self.seqlens, self.stride, self._cu)
+        else:
+            self._tok.rebind(x, x_pre, x_post)
+        return self._tok
 
 
 def budgets(seqlens, k=None, ratio=None, lam=(1, 3)):
@@ -151,9 +248,7 @@ def select(x, x_pre, x_post, stats, k=None, ratio=None, lam=(1, 3), seqlens=None
     tok = _Tokens(x, x_pre, x_post, seqlens, stride)
     ks, k1s, cu_k = budget if budget is not None else budgets(seqlens, k, ratio, lam)
     dev = x.device
-    d_k = torch.tensor(ks, dtype=torch.int32, device=dev)
-    d_k1 = torch.tensor(k1s, dtype=torch.int32, device=dev)
-    d_cu = torch.tensor(cu_k, dtype=torch.int32, device=dev)
+    d_k, d_k1, d_cu = _device_words(ks, dev), _device_words(k1s, dev), _device_words(cu_k, dev)
     idx = torch.empty(max(cu_k[-1], 1), dtype=torch.int32, device=dev)
     role = torch.empty(x.shape[0], dtype=torch.uint8, device=dev)
     status = torch.zeros(TR_STATUS_WORDS, dtype=torch.int32, device=dev)
@@ -174,7 +269,7 @@ class ReduceResult:
     status: torch.Tensor   # int32[4], see include/tr.h
 
 
-class Reducer:
+class Reducer(_Bound):
     """tr_reduce with buffers allocated once for a fixed batch shape.
 
     ``run`` takes device tensors (inputs already in HBM); ``run_host`` takes
@@ -182,45 +277,34 @@ class Reducer:
     """
 
     def __init__(self, seqlens, d, dtype, device, k=None, ratio=None, lam=(1, 3), alias_pre=False, scores=False,
-                 budget=None, stride="alg1"):
-        self.lib = load()
-        self.seqlens = [int(v) for v in seqlens]
-        self.device = torch.device(device)
-        self.d, self.dtype, self.alias_pre, self.stride = d, dtype, alias_pre, stride
-        self.ks, self.k1s, self.cu_k = budget if budget is not None else budgets(self.seqlens, k, ratio, lam)
-        self.total_k = self.cu_k[-1]
-        t = sum(self.seqlens)
-        dev = self.device
-        self.d_k = torch.tensor(self.ks, dtype=torch.int32, device=dev)
-        self.d_k1 = torch.tensor(self.k1s, dtype=torch.int32, device=dev)
-        self.d_cu = torch.tensor(self.cu_k, dtype=torch.int32, device=dev)
+                 budget=None, stride="alg1", _sync=True):
+        self.status = self._setup(seqlens, d, dtype, device, k, ratio, lam, alias_pre, budget, stride, _sync)
+        t, dev = self._total, self.device
         self.y = torch.empty(max(self.total_k, 1), d, dtype=dtype, device=dev)
         self.idx = torch.empty(max(self.total_k, 1), dtype=torch.int32, device=dev)
         self.h2 = torch.empty(t, dtype=torch.float32, device=dev) if scores else None
         self.s = torch.empty(t, dtype=torch.float32, device=dev) if scores else None
-        self.status = torch.zeros(TR_STATUS_WORDS, dtype=torch.int32, device=dev)
-        self._tok = None
         self._ws = None
-        self._in = None
 
     def _bind(self, x, x_pre, x_post):
-        x, x_pre, x_post, _ = _flatten(x, x_pre, x_post, self.seqlens)
-        key = (x.data_ptr(), None if x_pre is None else x_pre.data_ptr(), x_post.data_ptr())
-        if self._tok is None or self._in != key:
-            self._tok = _Tokens(x, x_pre, x_post, self.seqlens, self.stride)
-            self._in = key
-            if self._ws is None:
-                self._ws, self._ws_bytes = _workspace(self.lib, self._tok, self.device)
-        return self._tok
+        tok = super()._bind(x, x_pre, x_post)
+        if self._ws is None:
+            self._ws, self._ws_bytes = _workspace(self.lib, tok, self.device)
+        return tok
+
+    def _result(self) -> ReduceResult:
+        y, idx = (self.y, self.idx) if self.total_k else (self.y[:0], self.idx[:0])
+        return ReduceResult(y, idx, self.cu_k, self.h2, self.s, self.status)
 
     def run(self, x, x_pre, x_post) -> ReduceResult:
-        tok = self._bind(x, x_pre, x_post)
+        return self._run(self._bind(x, x_pre, x_post))
+
+    def _run(self, tok) -> ReduceResult:
         check("tr_reduce", self.lib.tr_reduce(
             tok.ref(), _ptr(self.d_k), _ptr(self.d_k1), _ptr(self.d_cu), self.total_k, _ptr(self.y),
             _ptr(self.idx), _ptr(self.h2), _ptr(self.s), _ptr(self._ws), self._ws_bytes, _ptr(self.status),
             _stream(self.device)))
-        return ReduceResult(self.y[:self.total_k], self.idx[:self.total_k], self.cu_k, self.h2, self.s,
-                            self.status)
+        return self._result()
 
     def graph(self, x, x_pre, x_post) -> "torch.cuda.CUDAGraph":
         """``run`` (with the status words zeroed first) captured into a CUDA
@@ -253,8 +337,7 @@ class Reducer:
             _ptr(self.idx), _ptr(self.h2), _ptr(self.s), _ptr(self._ws), self._ws_bytes, _ptr(self.status), st))
         if events:
             events[2].record()
-        return ReduceResult(self.y[:self.total_k], self.idx[:self.total_k], self.cu_k, self.h2, self.s,
-                            self.status)
+        return self._result()
 
     def run_select_gather(self, x, x_pre, x_post, stats, events=None):
         """tr_select then tr_gather on statistics records made elsewhere (e.g.
@@ -275,8 +358,7 @@ class Reducer:
         check("tr_gather", lib.tr_gather(tok.ref(), _ptr(self.d_cu), _ptr(self.idx), self.total_k, _ptr(self.y), st))
         if events:
             events[2].record()
-        return ReduceResult(self.y[:self.total_k], self.idx[:self.total_k], self.cu_k, self.h2, self.s,
-                            self.status)
+        return self._result()
 
     def run_separate(self, x, x_pre, x_post, events=None):
         """The three kernels the pipeline launches, tr_score, tr_select and
@@ -299,8 +381,7 @@ class Reducer:
         check("tr_gather", lib.tr_gather(tok.ref(), _ptr(self.d_cu), _ptr(self.idx), self.total_k, _ptr(self.y), st))
         if events:
             events[3].record()
-        return ReduceResult(self.y[:self.total_k], self.idx[:self.total_k], self.cu_k, self.h2, self.s,
-                            self.status)
+        return self._result()
 
     def _stats_view(self):
         # tr_reduce keeps the statistics at the start of the workspace; the
@@ -326,7 +407,7 @@ class Reducer:
         return r
 
 
-class Pipeline:
+class Pipeline(_Bound):
     """tr_pipeline: successive batches of one shape, each scored on its slot's
     stream of ``score_streams`` and then selected and gathered on
     ``select_stream`` (higher priority), so that the selection and gather of
@@ -339,17 +420,9 @@ class Pipeline:
 
     def __init__(self, seqlens, d, dtype, device, k=None, ratio=None, lam=(1, 3), alias_pre=False, scores=False,
                  budget=None, slots=2, stride="alg1", score_streams=None):
-        self.lib = load()
-        self.seqlens = [int(v) for v in seqlens]
-        self.device = torch.device(device)
-        self.d, self.dtype, self.alias_pre, self.slots, self.stride = d, dtype, alias_pre, int(slots), stride
-        self.ks, self.k1s, self.cu_k = budget if budget is not None else budgets(self.seqlens, k, ratio, lam)
-        self.total_k = self.cu_k[-1]
-        t = sum(self.seqlens)
-        dev = self.device
-        self.d_k = torch.tensor(self.ks, dtype=torch.int32, device=dev)
-        self.d_k1 = torch.tensor(self.k1s, dtype=torch.int32, device=dev)
-        self.d_cu = torch.tensor(self.cu_k, dtype=torch.int32, device=dev)
+        self.slots = int(slots)
+        self._setup(seqlens, d, dtype, device, k, ratio, lam, alias_pre, budget, stride, True)
+        t, dev = self._total, self.device
         mk = lambda *shape, dt: torch.empty(*shape, dtype=dt, device=dev)
         self.outs = [dict(y=mk(max(self.total_k, 1), d, dt=dtype), idx=mk(max(self.total_k, 1), dt=torch.int32),
                           h2=mk(t, dt=torch.float32) if scores else None, s=mk(t, dt=torch.float32) if scores else None,
@@ -362,17 +435,11 @@ class Pipeline:
         self._host = None  # submit_host: per-slot device inputs, copy streams and reuse events
         self._ws = None
         self._handle = None
-        self._tok = None
-        self._in = None
         self._graphed = False
         self.submitted = 0
 
     def _bind(self, x, x_pre, x_post):
-        x, x_pre, x_post, _ = _flatten(x, x_pre, x_post, self.seqlens)
-        key = (x.data_ptr(), None if x_pre is None else x_pre.data_ptr(), x_post.data_ptr())
-        if self._tok is None or self._in != key:
-            self._tok = _Tokens(x, x_pre, x_post, self.seqlens, self.stride)
-            self._in = key
+        super()._bind(x, x_pre, x_post)
         if self._handle is None:
             nbytes = self.lib.tr_workspace_bytes(self._tok.ref())
             if nbytes == 0:
@@ -414,7 +481,8 @@ class Pipeline:
             self._handle, tok.ref(), _ptr(self.d_k), _ptr(self.d_k1), _ptr(self.d_cu), self.total_k, _ptr(o["y"]),
             _ptr(o["idx"]), _ptr(o["h2"]), _ptr(o["s"]), _ptr(o["status"]), ev[0], ev[1]))
         self.submitted += 1
-        return ReduceResult(o["y"][:self.total_k], o["idx"][:self.total_k], self.cu_k, o["h2"], o["s"], o["status"])
+        y, idx = (o["y"], o["idx"]) if self.total_k else (o["y"][:0], o["idx"][:0])
+        return ReduceResult(y, idx, self.cu_k, o["h2"], o["s"], o["status"])
 
     def submit_host(self, x_h, x_pre_h, x_post_h, y_h, idx_h) -> ReduceResult:
         """End to end from pinned host memory: copies this batch's inputs into
@@ -565,9 +633,8 @@ def reduce(x, x_pre, x_post, k=None, ratio=None, lam=(1, 3), seqlens=None, score
     ``stride`` is "alg1" (Algorithm 1) or "interval" (Section IV-B)."""
     x2, p2, q2, seqlens = _flatten(x, x_pre, x_post, seqlens)
     r = Reducer(seqlens, x2.shape[1], x2.dtype, x2.device, k=k, ratio=ratio, lam=lam, alias_pre=p2 is None,
-                scores=scores, budget=budget, stride=stride)
-    out = r.run(x2, p2, q2)
-    return out
+                scores=scores, budget=budget, stride=stride, _sync=False)
+    return r.run(x2, p2, q2)
 
 
 # ---------------------------------------------------------------- encoder MLP with fused scoring
@@ -616,20 +683,18 @@ class Mlp:
         self.s = torch.empty(max(self.t, 1), dtype=torch.float32, device=dev) if scores else None
         self.error = torch.zeros(1, dtype=torch.int32, device=dev)
         self._ws = None
+        self._shape = torch.Size((self.t, self.d))
 
     def _struct(self, x_pre, resid):
         for t in (x_pre, resid):
             if t is None:
                 continue
-            if t.dtype != torch.bfloat16 or tuple(t.shape) != (self.t, self.d) or not t.is_contiguous():
+            if t.dtype != torch.bfloat16 or t.shape != self._shape or not t.is_contiguous():
                 raise ValueError(f"x_pre / resid must be contiguous bf16 [{self.t}, {self.d}]")
             if t.device != self.device:
                 raise ValueError("x_pre / resid must be on the weights' device")
-        return TrMlp(x_pre=x_pre.data_ptr(), resid=None if resid is None else resid.data_ptr(),
-                     w1=self.w1.data_ptr(), w2=self.w2.data_ptr(),
-                     b1=None if self.b1 is None else self.b1.data_ptr(),
-                     b2=None if self.b2 is None else self.b2.data_ptr(),
-                     t=self.t, d=self.d, d_hidden=self.dh, act=TR_ACT[self.act])
+        return TrMlp(x_pre.data_ptr(), _ptr(resid), self.w1.data_ptr(), self.w2.data_ptr(), _ptr(self.b1),
+                     _ptr(self.b2), self.t, self.d, self.dh, TR_ACT[self.act])
 
     def run(self, x_pre, resid=None, events=None) -> MlpResult:
         """Both GEMMs on the current stream; ``events`` (three torch.cuda.Event
@@ -651,10 +716,10 @@ class Mlp:
                                                     self._ws_bytes, _ptr(self.error), st))
         if events:
             events[2].record()
-        t = self.t
-        return MlpResult(self.h[:t], self.x_post[:t], self.x[:t], self.stats[:t],
-                         None if self.h2 is None else self.h2[:t], None if self.s is None else self.s[:t],
-                         self.error)
+        outs = (self.h, self.x_post, self.x, self.stats, self.h2, self.s)
+        if self.t == 0:  # the buffers hold a row more
+            outs = tuple(None if v is None else v[:0] for v in outs)
+        return MlpResult(*outs, self.error)
 
 
 def mlp(x_pre, w1, w2, b1=None, b2=None, resid=None, act="gelu", scores=False) -> MlpResult:
@@ -681,13 +746,13 @@ def project_kept(x, idx, cu_k, w, bias=None, act="gelu", seqlens=None, error=Non
     total_k = int(cu_k[-1])
     d_out = int(w.shape[0])
     dev = x2.device
-    d_cu = torch.tensor(list(cu_k), dtype=torch.int32, device=dev)
+    d_cu = _device_words(list(cu_k), dev)
     b = None if bias is None else bias.float().contiguous()
     z = torch.empty(max(total_k, 1), d_out, dtype=torch.bfloat16, device=dev)
     err = torch.zeros(1, dtype=torch.int32, device=dev) if error is None else error
     check("tr_project_kept", lib.tr_project_kept(tok.ref(), _ptr(d_cu), _ptr(idx), total_k, _ptr(w.contiguous()),
                                                  _ptr(b), d_out, TR_ACT[act], _ptr(z), _ptr(err), _stream(dev)))
-    return z[:total_k], err
+    return z if total_k else z[:0], err
 
 
 def project(y, w, bias=None, act="gelu", error=None, out=None):
@@ -714,4 +779,4 @@ def project(y, w, bias=None, act="gelu", error=None, out=None):
     err = torch.zeros(1, dtype=torch.int32, device=dev) if error is None else error
     check("tr_project", lib.tr_project(_ptr(y), rows, d, _ptr(w.contiguous()), _ptr(b), d_out, TR_ACT[act], _ptr(z),
                                        _ptr(err), _stream(dev)))
-    return z[:rows], err
+    return z if z.shape[0] == rows else z[:rows], err
