@@ -48,6 +48,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <atomic>
 #include <climits>
 #include <mutex>
@@ -59,7 +60,7 @@
 namespace tr {
 namespace {
 
-constexpr int kBM = 128, kBN = 256, kBK = 64;  // a CTA's rows, a tile's columns, a k-block
+constexpr int kBM = 128, kBN = 256, kBK = 64;  // a CTA's rows, a tile's columns at most, a k-block
 enum { kModeHidden = 0, kModeScore = 1, kModeProject = 2 };
 // Epilogue warps per mode: four per lane quarter where the epilogue is on the
 // critical path (the hidden GEMM, whose main loop is short, and split tiles),
@@ -104,6 +105,7 @@ __host__ __device__ constexpr int row_parts(int split) { return split * active_p
 
 struct GemmArgs {
   int m, n, k;          // C[m, n] = A[m, k] B[n, k]^T
+  int bn;               // tile columns: 256, 192, 128 or 64 (256 when K is split)
   int n_tiles, tiles, kblocks;
   const float *bias;    // [n] or NULL
   int act;              // hidden GEMM: TR_ACT_*
@@ -314,13 +316,13 @@ __device__ __forceinline__ void score_load_next(const GemmArgs &g, const GemmMap
   int nt = 0;
   while (w.tile < g.tiles) {
     nt = w.tile % g.n_tiles;
-    if (w.blk < w.end && nt * kBN + w.blk * kBlk < g.n) break;
+    if (w.blk < w.end && nt * g.bn + w.blk * kBlk < g.n) break;
     w.tile += step;
     w.blk = w.first;
   }
   if (w.tile >= g.tiles) return;
   if ((threadIdx.x & 31) == 0) {
-    const int col = nt * kBN + w.blk * kBlk, row = row_of(w.tile / g.n_tiles);
+    const int col = nt * g.bn + w.blk * kBlk, row = row_of(w.tile / g.n_tiles);
     tc::mbar_expect_tx(w.bar, g.has_resid ? 2 * kBlkBytes : kBlkBytes);
     tc::tma_load_2d(w.buf, &maps.p, col, row, w.bar);
     if (g.has_resid) tc::tma_load_2d(w.buf + kBlkBytes, &maps.r, col, row, w.bar);
@@ -375,7 +377,7 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs &g, const GemmMaps 
   const int lane = threadIdx.x & 31;
   const uint32_t sw = (uint32_t)((lane >> 1) & 3);  // the 64-byte swizzle's row term
   for (int blk = w.first; blk < w.end; blk += kParts) {
-    const int col = nt * kBN + blk * kBlk;
+    const int col = nt * g.bn + blk * kBlk;
     if (col >= g.n) break;
     uint32_t buf = w.buf;
     if (kMode == kModeScore) {
@@ -570,7 +572,6 @@ __device__ __forceinline__ long long kept_source_row(const GemmArgs &g, long lon
 __host__ __device__ constexpr int gemm_stages(int mode, int split) { return mode == kModeScore && split > 1 ? 5 : 6; }
 constexpr int kHalfTile = 128 * kBK * 2;          // 128 rows of a k-block (A or B)
 constexpr int kStagePBytes = 2 * kHalfTile;       // this CTA's A rows + B rows
-constexpr uint32_t kIdescPair = tc::idesc_bf16(2 * kBM, kBN);
 __host__ __device__ constexpr int gemm_smem(int mode, int split) {  // + alignment, barriers
   return gemm_stages(mode, split) * kStagePBytes + epi_warps(mode, split) * stage_bytes(mode) + 1024 + 512;
 }
@@ -606,7 +607,9 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
   const int cluster = blockIdx.x / (2 * kSplit), clusters = gridDim.x / (2 * kSplit);
   const int kb_first = pair * g.kblocks / kSplit, kb_end = (pair + 1) * g.kblocks / kSplit;
   // operand bytes landing on the even CTA's stage barrier per k-block (both CTAs)
-  constexpr uint32_t kTx = kMode == kModeProject ? 2 * kHalfTile : 2 * kStagePBytes;
+  const uint32_t b_bytes = (uint32_t)g.bn * kBK * 2u;  // of B per k-block, both CTAs
+  const uint32_t tx = b_bytes + (kMode == kModeProject ? 0u : 2u * kHalfTile);
+  const uint32_t idesc = tc::idesc_bf16(2 * kBM, g.bn);
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStagesP; ++s) {
       tc::mbar_init(full(s), kMode == kModeProject ? 1 + kLoadWarps : 1);  // + the even CTA's loader warps
@@ -651,10 +654,10 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
             break;
           }
           const uint32_t bar = full_even(stage);
-          if (leader) tc::mbar_expect_tx(full(stage), kTx);
+          if (leader) tc::mbar_expect_tx(full(stage), tx);
           if (kMode != kModeProject)
             tc::tma_load_2d_pair(sa(stage), &maps.a, kb * kBK, rb * 2 * kBM + (int)rank * kBM, bar);
-          tc::tma_load_2d_pair(sb(stage), &maps.b, kb * kBK, nt * kBN + (int)rank * 128, bar);
+          tc::tma_load_2d_pair(sb(stage), &maps.b, kb * kBK, nt * g.bn + (int)rank * (g.bn / 2), bar);
           filled |= 1u << stage;
           last_parity = (last_parity & ~(1u << stage)) | (phase << stage);
           if (++stage == kStagesP) {
@@ -693,7 +696,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
           const uint64_t da = tc::sw128_desc(sa(stage)), db = tc::sw128_desc(sb(stage));
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
-            tc::mma_bf16_pair(d, da + 2u * k, db + 2u * k, kIdescPair, kb != kb_first || k != 0);
+            tc::mma_bf16_pair(d, da + 2u * k, db + 2u * k, idesc, kb != kb_first || k != 0);
           tc::mma_commit_pair(empty(stage), both);  // both CTAs' stage is free once these MMAs read it
           if (++stage == kStagesP) {
             stage = 0;
@@ -768,7 +771,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
     // first of this warp's 32 rows in row tile rb
     auto row_of = [&](int rb) { return (2 * rb + (int)rank) * kBM + 32 * q; };
     const int own = pair * owned_blks(kSplit);
-    EpiWarp w{own + part, own + owned_blks(kSplit), out_stage + (uint32_t)((warp - 2) * stage_bytes(kMode)),
+    EpiWarp w{own + part, own + (kSplit > 1 ? owned_blks(kSplit) : g.bn / kBlk), out_stage + (uint32_t)((warp - 2) * stage_bytes(kMode)),
               blk_bar(warp - 2), 0u, 0u, cluster, own + part};
     if (kMode == kModeScore) score_load_next<epi_parts(kMode, kSplit)>(g, maps, w, clusters, row_of);
     int acc = 0;
@@ -777,7 +780,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
       const int rb = tile / g.n_tiles, nt = tile - rb * g.n_tiles;
       if (g.bias)  // the first blocks' bias on its way to L1 while the main loop runs
         for (int blk = w.first; blk < w.end; blk += epi_parts(kMode, kSplit))
-          if (nt * kBN + blk * kBlk + lane < g.n) tc::touch(g.bias + nt * kBN + blk * kBlk + lane);
+          if (nt * g.bn + blk * kBlk + lane < g.n) tc::touch(g.bias + nt * g.bn + blk * kBlk + lane);
       bool ok = tc::mbar_wait_warp(tfull(acc), acc_phase);
       if (!ok && lane == 0) flag_error(g, 4);
       tc::fence_after_sync();
@@ -908,30 +911,80 @@ cudaError_t launch_gemm(const GemmMaps &maps, const GemmArgs &g, cudaStream_t st
   return cudaLaunchKernelEx(&cfg, k_mlp_gemm<kMode, kSplit>, maps, g);
 }
 
-// Splits of K for a GEMM of `tiles` output tiles and `kblocks` k-blocks: four
-// (or two) while the clusters all run at once -- 16 clusters of eight SMs, 32
-// of four -- and the main loop is long enough: a k-block takes about 520
-// clocks, the exchange 4,500 (two pairs) to 7,000 (four; 96 KiB into each
-// SM).  576 rows, D 1024, hidden 4096: the score GEMM (12 tiles of 64
-// k-blocks) 45 us unsplit, 21 in four; a 192-row, 1024 -> 4096 layer (16
-// tiles of 16 k-blocks) 16.6 us unsplit, 24 in four.  The sums of a tile are
-// the same for every mode (tr_project and tr_project_kept agree bit for bit).
-inline int gemm_split(int tiles, int kblocks) {
-  if (tiles <= 16 && kblocks >= 32) return 4;
-  if (tiles <= 32 && kblocks >= 24) return 2;
-  return 1;
+inline int row_tiles(int m) { return (int)(((long long)m + 2 * kBM - 1) / (2 * kBM)); }
+
+// How a GEMM is laid out on the 76 SM pairs: tile columns and splits of K.
+struct GemmShape {
+  int bn, split, n_tiles, kblocks;
+};
+// The cheapest of the layouts by a model in clocks, fitted to the measured
+// kernels; a function of the sizes alone (it also sizes tr_mlp_score's
+// scratch), whatever the device has free.
+//   A k-block takes the larger of its MMAs (2 clocks a column) and the operands
+//   into each SM at 63 bytes a clock, A's 16 KiB and B's 64 bytes a column:
+//   520 clocks for 256 columns, 455, 390 and 325 for 192, 128 and 64; the
+//   projector's row gather 1065 whatever the columns.  A tile's epilogue takes
+//   80 (score), 30 (hidden) or 65 (projector) clocks a column, overlapped with
+//   the next tile's main loop where there is one.
+//   Splitting K over two or four pairs (256 columns, only while all clusters
+//   run at once: 32 of four SMs, 16 of eight) divides the main loop and the
+//   epilogue and adds the exchange, 4500 or 7000 clocks (96 KiB into each SM).
+// Measured: 192 rows, 1024 -> 4096, 16 tiles of 256 columns 12.3 us a pass, 64
+// of 64 columns 8.4; both GEMMs of 2885 rows, 1152 -> 4304 -> 1152, 63.4 us
+// with 60 score tiles of 256 columns, 58.9 with 72 of 192; the score GEMM of
+// 576 rows, 4096 -> 1024, 45 us unsplit, 21 split in four.
+// The sums of an output element are the same for every mode (tr_project and
+// tr_project_kept agree bit for bit): they depend on the split alone.
+inline GemmShape gemm_shape(int m, int n, int k, bool score, bool gather) {
+  constexpr long long kPairs = 76;
+  const int kb = (k + kBK - 1) / kBK;
+  const long long rows = row_tiles(m);
+  auto tiles_of = [&](int bn) { return (n + bn - 1) / bn; };
+  auto epi = [&](int bn, bool g) { return (long long)bn * (score ? 80 : (g ? 65 : 30)); };
+  auto cost = [&](int bn, bool g) {
+    const long long waves = (rows * tiles_of(bn) + kPairs - 1) / kPairs;
+    const long long main = (long long)kb * (g ? 1065 : std::max(2 * bn + 8, (16384 + 64 * bn) / 63));
+    return waves * std::max(main, epi(bn, g)) + epi(bn, g);
+  };
+  auto narrowest = [&](bool g, long long *least) {  // the cheapest width
+    int best = kBN;
+    *least = cost(kBN, g);
+    for (const int bn : {192, 128, 64})
+      if (cost(bn, g) < *least) {
+        *least = cost(bn, g);
+        best = bn;
+      }
+    return best;
+  };
+  long long least = 0;
+  int bn = narrowest(false, &least), split = 1;
+  for (const int s : {2, 4})  // the same for gathered rows
+    if (kb >= 4 * s && rows * tiles_of(kBN) * s <= 64) {
+      const long long c = (long long)(kb + s - 1) / s * 520 + epi(kBN, false) / s + (s == 2 ? 4500 : 7000);
+      if (c < least) {
+        least = c;
+        bn = kBN;
+        split = s;
+      }
+    }
+  if (gather && split == 1) bn = narrowest(true, &least);
+  return GemmShape{bn, split, tiles_of(bn), kb};
 }
 
 template <int kMode>
-cudaError_t launch_split(const GemmMaps &maps, const GemmArgs &g, cudaStream_t st) {
-  switch (gemm_split(g.tiles, g.kblocks)) {
+cudaError_t launch_shape(const GemmMaps &maps, const GemmArgs &g, int split, cudaStream_t st) {
+  switch (split) {
     case 4: return launch_gemm<kMode, 4>(maps, g, st);
     case 2: return launch_gemm<kMode, 2>(maps, g, st);
     default: return launch_gemm<kMode, 1>(maps, g, st);
   }
 }
-
-inline int row_tiles(int m) { return (int)(((long long)m + 2 * kBM - 1) / (2 * kBM)); }
+inline void set_shape(GemmArgs &g, const GemmShape &sh) {
+  g.bn = sh.bn;
+  g.n_tiles = sh.n_tiles;
+  g.tiles = row_tiles(g.m) * sh.n_tiles;
+  g.kblocks = sh.kblocks;
+}
 
 bool misaligned16(const void *p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
 
@@ -954,11 +1007,10 @@ struct MlpWs {
 };
 MlpWs mlp_ws(const tr_mlp *m) {
   const long long rblocks = ((long long)m->t + kBM - 1) / kBM;
-  const int n_tiles = (m->d + kBN - 1) / kBN;
-  const int parts = row_parts(gemm_split(row_tiles(m->t) * n_tiles, (m->d_hidden + kBK - 1) / kBK));
+  const GemmShape sh = gemm_shape(m->t, m->d, m->d_hidden, true, false);
   MlpWs w;
   w.part = 0;
-  w.total = align_up((size_t)rblocks * n_tiles * parts * 4 * kPartWords * 32 * sizeof(float), 256);
+  w.total = align_up((size_t)rblocks * sh.n_tiles * row_parts(sh.split) * 4 * kPartWords * 32 * sizeof(float), 256);
   return w;
 }
 
@@ -972,17 +1024,16 @@ tr_status dense_act_gemm(const void *a, int rows, int k, const void *w, const fl
   g.m = rows;
   g.n = n;
   g.k = k;
-  g.n_tiles = (g.n + kBN - 1) / kBN;
-  g.tiles = row_tiles(g.m) * g.n_tiles;
-  g.kblocks = (g.k + kBK - 1) / kBK;
+  const GemmShape sh = gemm_shape(g.m, g.n, g.k, false, false);
+  set_shape(g, sh);
   g.bias = bias;
   g.act = act;
   g.err = d_error;
   GemmMaps maps{};
-  if (!make_map(&maps.a, a, rows, k, kBM) || !make_map(&maps.b, w, n, k, kBN / 2) ||
+  if (!make_map(&maps.a, a, rows, k, kBM) || !make_map(&maps.b, w, n, k, sh.bn / 2) ||
       !make_map(&maps.out, out, rows, n, 32, kBlk, CU_TENSOR_MAP_SWIZZLE_64B))
     return TR_ERR_CUDA;
-  return launch_split<kModeHidden>(maps, g, st) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
+  return launch_shape<kModeHidden>(maps, g, sh.split, st) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 
 }  // namespace
@@ -1034,9 +1085,8 @@ tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, fl
   g.m = m->t;
   g.n = m->d;
   g.k = m->d_hidden;
-  g.n_tiles = (g.n + kBN - 1) / kBN;
-  g.tiles = row_tiles(g.m) * g.n_tiles;
-  g.kblocks = (g.k + kBK - 1) / kBK;
+  const GemmShape sh = gemm_shape(g.m, g.n, g.k, true, false);
+  set_shape(g, sh);
   g.bias = m->b2;
   g.has_resid = m->resid != nullptr;
   g.part = reinterpret_cast<float *>(wsb + w.part);
@@ -1045,12 +1095,12 @@ tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, fl
   auto block_map = [&](CUtensorMap *map, const void *p) {  // the epilogue's 32 x 32 blocks
     return make_map(map, p, m->t, m->d, 32, kBlk, CU_TENSOR_MAP_SWIZZLE_64B);
   };
-  if (!make_map(&maps.a, h, m->t, m->d_hidden, kBM) || !make_map(&maps.b, m->w2, m->d, m->d_hidden, kBN / 2) ||
+  if (!make_map(&maps.a, h, m->t, m->d_hidden, kBM) || !make_map(&maps.b, m->w2, m->d, m->d_hidden, sh.bn / 2) ||
       !block_map(&maps.p, m->x_pre) || (m->resid && !block_map(&maps.r, m->resid)) || !block_map(&maps.out, x_post) ||
       !block_map(&maps.x, x))
     return TR_ERR_CUDA;
-  if (launch_split<kModeScore>(maps, g, st) != cudaSuccess) return TR_ERR_CUDA;
-  const int parts = row_parts(gemm_split(g.tiles, g.kblocks));
+  if (launch_shape<kModeScore>(maps, g, sh.split, st) != cudaSuccess) return TR_ERR_CUDA;
+  const int parts = row_parts(sh.split);
   const cudaError_t err = launch_kernel(k_score_rows, dim3((g.m + kBM - 1) / kBM * 4), dim3(kRowWarps * 32), 0, st, true, g, parts,
                                         reinterpret_cast<float4 *>(stats), h2, s);
   return err == cudaSuccess ? TR_OK : TR_ERR_CUDA;
@@ -1084,9 +1134,8 @@ tr_status tr_project_kept(const tr_tokens *in, const int32_t *d_cu_k, const int3
   g.m = total_k;
   g.n = d_out;
   g.k = in->d;
-  g.n_tiles = (g.n + kBN - 1) / kBN;
-  g.tiles = row_tiles(g.m) * g.n_tiles;
-  g.kblocks = (g.k + kBK - 1) / kBK;
+  const GemmShape sh = gemm_shape(g.m, g.n, g.k, false, true);
+  set_shape(g, sh);
   g.bias = bias;
   g.act = act;
   g.err = d_error;
@@ -1098,10 +1147,10 @@ tr_status tr_project_kept(const tr_tokens *in, const int32_t *d_cu_k, const int3
   g.idx = idx;
   // A: x, one row per box (the loaders gather rows by kept index)
   GemmMaps maps{};
-  if (!make_map(&maps.a, in->x, total_rows, in->d, 1) || !make_map(&maps.b, w, d_out, in->d, kBN / 2) ||
+  if (!make_map(&maps.a, in->x, total_rows, in->d, 1) || !make_map(&maps.b, w, d_out, in->d, sh.bn / 2) ||
       !make_map(&maps.out, z, total_k, d_out, 32, kBlk, CU_TENSOR_MAP_SWIZZLE_64B))
     return TR_ERR_CUDA;
-  return launch_split<kModeProject>(maps, g, static_cast<cudaStream_t>(stream)) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
+  return launch_shape<kModeProject>(maps, g, sh.split, static_cast<cudaStream_t>(stream)) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 
 }  // extern "C"

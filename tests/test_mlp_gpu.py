@@ -242,17 +242,18 @@ def test_project_kept_index_outside_its_image():
     _check_close(z, _sigma(v, "gelu"), mag, slope=1.13)
 
 
-# GEMMs whose K is split over the pairs of a cluster: 256 x 256 tiles and
-# 64-wide k-blocks at the edges of the rule (16 / 32 tiles, 32 / 24 k-blocks),
-# with ragged rows, columns and k-blocks and k-blocks that do not divide evenly.
+# The layouts a GEMM may take (gemm_shape): K split over two or four pairs of a
+# cluster, and 192-, 128- and 64-column tiles, with ragged rows, columns and
+# k-blocks and k-blocks that do not divide evenly.  Named by the score GEMM's.
 SPLIT_CASES = [
-    ("four_one_row", 1, 256, 2048, "none", False, True),         # 1 tile, 32 k-blocks
-    ("four_uneven_k", 300, 528, 2224, "gelu", True, True),       # 6 tiles, 34.75 k-blocks
-    ("four_most_tiles", 1000, 1024, 2112, "quick_gelu", True, False),  # 16 tiles, 33 k-blocks
-    ("two_few_k", 257, 272, 1552, "gelu", True, True),           # 4 tiles, 24.25 k-blocks
-    ("two_most_tiles", 2048, 784, 2064, "gelu", False, True),    # 32 tiles, 32.25 k-blocks
-    ("none_few_k", 129, 1056, 1472, "gelu", True, True),         # 5 tiles, 23 k-blocks
-    ("none_more_tiles", 2049, 784, 1600, "none", True, True),    # 36 tiles, 25 k-blocks
+    ("four_one_row", 1, 256, 6144, "none", False, True),         # 1 tile, 96 k-blocks
+    ("four_uneven_k", 300, 528, 4464, "gelu", True, True),       # 6 tiles, 69.75 k-blocks
+    ("four_most_tiles", 1000, 1024, 4160, "quick_gelu", True, False),  # 16 tiles, 65 k-blocks
+    ("two_uneven_k", 1500, 1024, 4400, "gelu", True, True),      # 24 tiles, 68.75 k-blocks
+    ("two_most_tiles", 2048, 784, 4112, "gelu", False, True),    # 32 tiles, 64.25 k-blocks
+    ("narrow_192", 2049, 1152, 1600, "none", True, True),        # 9 x 6 tiles
+    ("narrow_128", 2048, 784, 2064, "gelu", False, True),        # 8 x 7 tiles, the last 16 columns
+    ("narrow_64", 129, 1056, 1472, "quick_gelu", True, True),    # 1 x 17 tiles, the last half empty
 ]
 
 
@@ -270,10 +271,11 @@ def test_mlp_split(name, t, d, dh, act, resid, bias):
         assert torch.equal(u.view(torch.int16), v.view(torch.int16))
 
 
-@pytest.mark.parametrize("d,d_out,k", [(2064, 528, 40), (1600, 1280, 200)], ids=["four", "two"])
+@pytest.mark.parametrize("d,d_out,k", [(8208, 528, 40), (4096, 2560, 200), (784, 1296, 50)],
+                         ids=["four", "two", "narrow"])
 def test_project_split(d, d_out, k):
-    # K split: the dense projector within the GEMM tolerance of float64, and the
-    # rows read by index bit for bit the same
+    # K split, or narrow tiles: the dense projector within the GEMM tolerance
+    # of float64, and the rows read by index bit for bit the same
     altr = _alt()
     g = torch.Generator(device="cuda").manual_seed(9)
     n, b = 300, 3
