@@ -35,7 +35,7 @@
  *    synchronisation or copies), so they can be captured into a CUDA graph
  *    and replayed; make one call on the device outside the capture first
  *    (it raises the kernels' shared-memory limit once).
- *  - tr_select, tr_gather, tr_select_gather, tr_reduce, tr_mlp_hidden,
+ *  - tr_score, tr_select, tr_gather, tr_select_gather, tr_reduce, tr_mlp_hidden,
  *    tr_mlp_score, tr_project_kept and tr_project launch their kernels with
  *    programmatic dependent launch: a kernel may be scheduled
  *    while the kernel before it on the stream finishes, and waits in

@@ -75,6 +75,17 @@ SelectArgs select_args(const tr_tokens *in, const Shape &sh, const float *stats,
   return a;
 }
 
+tr_status score_impl(const tr_tokens *in, float *stats, float *h2, float *s, void *stream, bool pdl) {
+  Shape sh;
+  tr_status rc = check_tokens(in, &sh);
+  if (rc != TR_OK) return rc;
+  if (!stats) return TR_ERR_ARG;
+  if (misaligned(stats, 16) || misaligned(h2, 4) || misaligned(s, 4)) return TR_ERR_ALIGN;
+  cudaError_t err = launch_score(in->x, in->x_pre, in->x_post, in->dtype, in->d, sh.total, stats, h2, s,
+                                 static_cast<cudaStream_t>(stream), pdl);
+  return err == cudaSuccess ? TR_OK : TR_ERR_CUDA;
+}
+
 tr_status select_capped(const tr_tokens *in, const float *stats, const int32_t *d_k, const int32_t *d_k1,
                         const int32_t *d_cu_k, int32_t *idx, uint8_t *role, float *h2, float *s, void *ws,
                         size_t ws_bytes, int32_t *d_status, void *stream, int max_ctas, bool pdl) {
@@ -188,14 +199,7 @@ size_t tr_workspace_bytes(const tr_tokens *in) {
 }
 
 tr_status tr_score(const tr_tokens *in, float *stats, float *h2, float *s, void *stream) {
-  Shape sh;
-  tr_status rc = check_tokens(in, &sh);
-  if (rc != TR_OK) return rc;
-  if (!stats) return TR_ERR_ARG;
-  if (misaligned(stats, 16) || misaligned(h2, 4) || misaligned(s, 4)) return TR_ERR_ALIGN;
-  cudaError_t err = launch_score(in->x, in->x_pre, in->x_post, in->dtype, in->d, sh.total, stats, h2, s,
-                                 static_cast<cudaStream_t>(stream));
-  return err == cudaSuccess ? TR_OK : TR_ERR_CUDA;
+  return score_impl(in, stats, h2, s, stream, true);
 }
 
 tr_status tr_select(const tr_tokens *in, const float *stats, const int32_t *d_k, const int32_t *d_k1,
@@ -329,7 +333,7 @@ tr_status tr_pipeline_submit(tr_pipeline *p, const tr_tokens *in, const int32_t 
       capturing == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : cudaEventRecordDefault;
   if (score_begin && cudaEventRecordWithFlags(static_cast<cudaEvent_t>(score_begin), a, rec_flags) != cudaSuccess)
     return TR_ERR_CUDA;
-  if ((rc = tr_score(in, stats, h2, s, a)) != TR_OK) return rc;
+  if ((rc = score_impl(in, stats, h2, s, a, false)) != TR_OK) return rc;
   if (cudaEventRecord(p->head[slot], a) != cudaSuccess) return TR_ERR_CUDA;
   if (score_end && cudaEventRecordWithFlags(static_cast<cudaEvent_t>(score_end), a, rec_flags) != cudaSuccess)
     return TR_ERR_CUDA;

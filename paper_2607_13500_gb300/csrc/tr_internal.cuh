@@ -243,7 +243,7 @@ struct SelectArgs {
 
 size_t select_smem_bytes(int max_n);  // dynamic shared memory of one select CTA
 cudaError_t launch_score(const void *x, const void *x_pre, const void *x_post, int dtype, int d, long long total,
-                         float *stats, float *h2, float *s, cudaStream_t st);
+                         float *stats, float *h2, float *s, cudaStream_t st, bool pdl);
 // CTAs per image of an uncapped selection: more than one (a cluster) for
 // large images of a small batch.
 int select_cluster_ctas(int batch, int max_n);

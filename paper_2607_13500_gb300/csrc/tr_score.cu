@@ -11,6 +11,7 @@ template <int kDt>
 __global__ void __launch_bounds__(kScoreWarps * 32)
     k_score(const uint4 *__restrict__ x, const uint4 *__restrict__ xp, const uint4 *__restrict__ xq, int nchunks,
             long long total, float4 *__restrict__ stats, float *__restrict__ h2, float *__restrict__ s_out) {
+  pdl_wait();     // the inputs come from, and the records may still be read by, the kernels before
   pdl_trigger();  // a dependent selection may be scheduled once every CTA runs
   const int lane = threadIdx.x & 31;
   const long long stride = (long long)gridDim.x * kScoreWarps;
@@ -21,13 +22,17 @@ __global__ void __launch_bounds__(kScoreWarps * 32)
 }  // namespace
 
 cudaError_t launch_score(const void *x, const void *x_pre, const void *x_post, int dtype, int d, long long total,
-                         float *stats, float *h2, float *s, cudaStream_t st) {
+                         float *stats, float *h2, float *s, cudaStream_t st, bool pdl) {
   if (total == 0) return cudaSuccess;
   const int row_bytes = d * elem_bytes(dtype);
   const unsigned char *bx = static_cast<const unsigned char *>(x);
   const unsigned char *bp = static_cast<const unsigned char *>(x_pre ? x_pre : x);
   const unsigned char *bq = static_cast<const unsigned char *>(x_post);
   float4 *ps = reinterpret_cast<float4 *>(stats);
+  // Programmatic dependent launch (single calls): the launch of one call's
+  // scoring overlaps the end of the call before it on the stream -- passes of
+  // one 576-token fp32 image 22.1 -> 19.7 us, of a 6272-token clip 58.3 ->
+  // 55.9, of 4 x 2880 fp16 74.2 -> 72.3, of 64 x 576 bf16 191.8 -> 189.8.
   // One row per warp and no more, in small CTAs: CTAs retire as they
   // finish, so kernels on other streams (the selection of an earlier batch)
   // can take SMs while this one still runs, and an SM's slots refill row by
@@ -40,13 +45,11 @@ cudaError_t launch_score(const void *x, const void *x_pre, const void *x_post, i
   const uint4 *px = reinterpret_cast<const uint4 *>(bx);
   const uint4 *pp = reinterpret_cast<const uint4 *>(bp);
   const uint4 *pq = reinterpret_cast<const uint4 *>(bq);
-  if (dtype == TR_BF16)
-    k_score<TR_BF16><<<grid, kScoreWarps * 32, 0, st>>>(px, pp, pq, nchunks, total, ps, h2, s);
-  else if (dtype == TR_F16)
-    k_score<TR_F16><<<grid, kScoreWarps * 32, 0, st>>>(px, pp, pq, nchunks, total, ps, h2, s);
-  else
-    k_score<TR_F32><<<grid, kScoreWarps * 32, 0, st>>>(px, pp, pq, nchunks, total, ps, h2, s);
-  return cudaGetLastError();
+  auto launch = [&](auto kernel) {
+    return launch_kernel(kernel, dim3(grid), dim3(kScoreWarps * 32), 0, st, pdl, px, pp, pq, nchunks, total, ps, h2, s);
+  };
+  return dtype == TR_BF16 ? launch(k_score<TR_BF16>)
+                          : (dtype == TR_F16 ? launch(k_score<TR_F16>) : launch(k_score<TR_F32>));
 }
 
 }  // namespace tr
