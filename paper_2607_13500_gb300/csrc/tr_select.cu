@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(kSelectThreads, 1) k_select(const SelectArgs a
   extern __shared__ __align__(16) unsigned char smem[];
   pdl_trigger();
   pdl_wait();  // the statistics come from the kernel before this one
-  for (int b = blockIdx.x; b < a.batch; b += gridDim.x) select_image(a, b, smem);
+  for (int b = blockIdx.x; b < a.batch; b += gridDim.x) select_image_solo(a, b, smem, true);
 }
 
 // A cluster of c CTAs per image (large images of small batches).
@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(kSelectThreads, 1) k_select_cluster(const Sele
   pdl_trigger();
   pdl_wait();  // the statistics come from the kernel before this one
   const int b = blockIdx.x / c, rank = (int)tc::cluster_rank();
-  if (select_image_cluster(a, b, c, rank, smem)) return;
+  if (select_image_cluster<true>(a, b, c, rank, smem, true, nullptr)) return;
   cluster_barrier();  // nobody reads this CTA's shared memory any more
   if (rank == 0) select_image(a, b, smem);
 }
@@ -48,7 +48,7 @@ __device__ __forceinline__ uint4 ld_nc16(const uint4 *p) {
 // Replica r of `replicas` copies its share of image b's kept rows, whose
 // local indices select_image left in this CTA's shared memory.
 __device__ __forceinline__ void copy_kept(const SelectArgs &a, const int b, const int r, const int replicas,
-                                          const int nchunks, uint4 *__restrict__ y, unsigned char *smem) {
+                                          const int nchunks, uint4 *__restrict__ y, const uint16_t *kept) {
   long long off;
   int n;
   if (a.cu_seqlens) {
@@ -62,7 +62,6 @@ __device__ __forceinline__ void copy_kept(const SelectArgs &a, const int b, cons
   if (n <= 0 || n > a.max_n || off < 0 || off + n > a.total_rows || k < 0 || k > n || k1 < 0 || k1 > k)
     return;  // counted by select_image
   // this replica's share of the image's kept rows
-  const uint16_t *kept = kept_rows(a, smem);
   const int j0 = (int)((long long)r * k / replicas), j1 = (int)((long long)(r + 1) * k / replicas);
   const uint4 *x = static_cast<const uint4 *>(a.x);
   // one warp per row, eight 16-byte loads in flight per lane, streaming stores
@@ -92,8 +91,8 @@ __global__ void __launch_bounds__(kSelectThreads, 1)
   extern __shared__ __align__(16) unsigned char smem[];
   pdl_wait();  // the statistics come from the kernel before this one
   const int b = blockIdx.x / replicas, r = blockIdx.x % replicas;
-  select_image(a, b, smem, r == 0);
-  copy_kept(a, b, r, replicas, nchunks, y, smem);
+  const uint16_t *kept = select_image_solo(a, b, smem, r == 0);
+  copy_kept(a, b, r, replicas, nchunks, y, kept);
 }
 
 // Per device (index & 63): dynamic shared memory limit already raised (bit 0
@@ -110,6 +109,12 @@ size_t select_smem_bytes(int max_n) {
   return cap * (sizeof(uint32_t) + 3 * sizeof(uint16_t) + sizeof(uint8_t)) + kWarps * 256 * sizeof(uint32_t);
 }
 
+// Dynamic shared memory of one CTA per image: both its paths.
+size_t solo_smem_bytes(int max_n) {
+  const size_t general = select_smem_bytes(max_n);
+  return max_n <= kSoloMaxN ? std::max(general, cluster_smem_bytes(max_n > 0 ? max_n : 1, 1)) : general;
+}
+
 template <typename K>
 cudaError_t raise_smem_limit(K kernel, int dev) {
   int optin = 0;
@@ -121,18 +126,21 @@ cudaError_t raise_smem_limit(K kernel, int dev) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
-// A cluster per image pays from about 2500 tokens on (below, its barriers
-// cost what the split passes save) and while the clusters run at once; more
-// CTAs than that only queue.  Reduction of B images, us with 1 / 2 / 4 / 8
-// CTAs per image (bf16, D 512, K = N / 8):
-//   N 2048:  B 1   20.9 /  22.7 /  22.0 /  22.6
-//   N 2880:  B 1   26.7 /  24.7 /  24.4 /  23.5   B 64  195 / 189 / 203 / 244
-//   N 6272:  B 1   40.7 /  34.6 /  30.8 /  28.7   B 8   96.4 / 85.4 / 81.5 / 80.2
-//            B 16  138 / 127 / 123 / 132          B 32  220 / 210 / 207 / 231
-//   N 16384: B 1    103 /  76.0 /  61.5 /  53.7   B 16  331 / 285 / 272 / 289
+// A cluster per image pays from about 5000 tokens on (below, its barriers
+// cost more than the split passes save) and while the clusters run at once;
+// more CTAs than that only queue, and two pay only where one CTA is left with
+// select_image.  Reduction of B images, us with 1 / 2 / 4 / 8 CTAs per image
+// (bf16, D 512, K = N / 8):
+//   N 2880:  B 1   19.8 / 22.9 / 21.8 / 21.5     B 64  179 / 186 / 201 / 243
+//   N 4096:  B 1   23.5 / 26.0 / 23.9 / 23.3     B 16  80.9 / 86.0 / 84.0 / 91.5
+//   N 6272:  B 1   32.4 / 32.3 / 28.3 / 26.9     B 12  101 / 104 / 100 / 99.0
+//            B 16  122 / 125 / 121 / 129         B 32  205 / 208 / 205 / 230
+//   N 8192:  B 1   45.9 / 44.5 / 39.7 / 37.3     B 32  264 / 263 / 258 / 285
+//   N 16384: B 1    100 / 72.1 / 58.2 / 51.5     B 16  324 / 282 / 268 / 288
 int select_cluster_ctas(int batch, int max_n) {
-  if (batch <= 0 || max_n < 2560) return 1;
-  return batch <= 12 ? 8 : (batch <= 36 ? 4 : (batch <= 72 ? 2 : 1));
+  if (batch <= 0 || max_n < 5120) return 1;
+  if (batch <= 36) return batch <= 12 ? 8 : 4;
+  return batch <= 72 && max_n > kSoloMaxN ? 2 : 1;
 }
 
 cudaError_t launch_select(const SelectArgs &a, cudaStream_t st, int max_ctas, bool pdl) {
@@ -149,7 +157,7 @@ cudaError_t launch_select(const SelectArgs &a, cudaStream_t st, int max_ctas, bo
     const size_t need = std::max(cluster_smem_bytes(a.max_n, c), select_smem_bytes(a.max_n));
     return launch_kernel_cluster(k_select_cluster, dim3(a.batch * c), dim3(kSelectThreads), c, need, st, pdl, a, c);
   }
-  const size_t smem = select_smem_bytes(a.max_n);
+  const size_t smem = solo_smem_bytes(a.max_n);
   if (!(g_smem_set[dev & 63].load() & 1)) {
     if ((err = raise_smem_limit(k_select, dev)) != cudaSuccess) return err;
     g_smem_set[dev & 63].fetch_or(1);
@@ -179,7 +187,7 @@ cudaError_t launch_select_gather(const SelectArgs &a, void *y, cudaStream_t st, 
   }
   const int sms = sm_count();
   if (sms <= 0) return cudaErrorInvalidDevice;
-  const size_t smem = select_smem_bytes(a.max_n);
+  const size_t smem = solo_smem_bytes(a.max_n);
   const int nchunks = a.d * elem_bytes(a.dtype) / 16;
   const int replicas = max(1, min(16, sms / a.batch));
   return launch_kernel(k_select_gather, dim3(a.batch * replicas), dim3(kSelectThreads), smem, st, pdl, a, replicas,

@@ -1,8 +1,8 @@
-// The selection of one image by a thread-block cluster of C CTAs (2, 4 or 8),
-// for large images: CTA r holds rows [r cap, (r + 1) cap) of the image, and
-// every pass over the rows is split over the cluster.  What one CTA does in
-// tr_select_dev.cuh in passes over n rows is, per CTA, a pass over n / C rows
-// between cluster barriers:
+// The fast path of the selection, over one CTA or a thread-block cluster of C
+// CTAs (2, 4 or 8; large images).  In a cluster CTA r holds rows [r cap,
+// (r + 1) cap) of the image, and every pass over the rows is split over the
+// cluster.  What select_image does in passes over n rows is, per CTA, a pass
+// over n / C rows between cluster barriers:
 //
 //   keys      range of R and of s over the image (each CTA sends its own to
 //             all);
@@ -24,6 +24,13 @@
 // rows outside the fp32 error model, values crowded into one bucket, long or
 // very many runs -- is decided by the whole cluster alike (flags exchanged
 // before a barrier), and CTA 0 then makes the selection anew.
+//
+// With one CTA the same code runs without the exchanges (block barriers, plain
+// shared memory): the selection of every image up to kSoloMaxN tokens that no
+// cluster takes.  It beats select_image's fast path by keeping the s keys from
+// the one load of the records, by ranking buckets instead of sorting, and by
+// fewer passes: passes of one 576-token fp32 image 19.5 -> 14.7 us, k_select on
+// 64 x 576 tokens 25.6 -> 20.5, a 2880-token image (bf16, D 512) 26.7 -> 19.8.
 //
 // What bounds it: a chain of about ten short phases, each ending in a cluster
 // barrier (0.5-0.6 us) and spending as much on its own latencies; a run to
@@ -139,7 +146,7 @@ __device__ __noinline__ bool refine_df(const SelectArgs &a, long long off, const
 // (mode 0) or s (mode 1) outputs rewritten from them; false (block-uniform)
 // when a row's sums do not fit the exact representation.
 __device__ __noinline__ bool refine_exact(const SelectArgs &a, long long off, const uint16_t *rows, int cnt, int mode,
-                                          ExactRec *rec) {
+                                          ExactRec *rec, const bool primary) {
   __shared__ Part128 part;
   const int groups = cnt >= 4 ? 4 : (cnt >= 2 ? 2 : 1);
   const int gsize = (int)blockDim.x / groups;
@@ -156,35 +163,71 @@ __device__ __noinline__ bool refine_exact(const SelectArgs &a, long long off, co
     const ExactRec &r = rec[rows[i]];
     const bool fine = (mode == 0 ? r.flags_l : r.flags_s) == 0u;
     ok &= fine;
-    if (fine && mode == 0 && a.h2) a.h2[off + rows[i]] = exact_h2(r);
-    if (fine && mode == 1 && a.s) a.s[off + rows[i]] = exact_s_key(r);
+    if (fine && primary && mode == 0 && a.h2) a.h2[off + rows[i]] = exact_h2(r);
+    if (fine && primary && mode == 1 && a.s) a.s[off + rows[i]] = exact_s_key(r);
   }
   return !__syncthreads_or(!ok);
 }
 
-// What a CTA of the cluster knows of its image.
-struct ClusterImage {
+// What a CTA knows of its image, and the cluster's memory: with kMany = false
+// one CTA has the image to itself.
+template <bool kMany>
+struct SplitImage {
   long long off;
   int n, k, k1, k2, ko;
   int c, rank;            // CTAs of the cluster, this one
   int cap, first, rows;   // rows per CTA; this CTA's first row and number of rows
+  bool primary;           // writes the outputs
   uint32_t *keyr, *keys, *sk, *sk2;
   uint16_t *sr, *sr2;
   uint8_t *fl;
   ExactRec *rec;
-  __device__ __forceinline__ uint32_t remote(const void *p, int cta) const {
+  static __device__ __forceinline__ void barrier() {
+    if (kMany)
+      cluster_barrier();
+    else
+      __syncthreads();
+  }
+  static __device__ __forceinline__ uint32_t at(const void *p, int cta) {
     return tc::map_shared(tc::smem_u32(p), (uint32_t)cta);
   }
+  // *p in CTA `cta`
+  static __device__ __forceinline__ void put(uint32_t *p, int cta, uint32_t v) {
+    if (kMany)
+      st_cl_u32(at(p, cta), v);
+    else
+      *p = v;
+  }
+  static __device__ __forceinline__ void put(uint16_t *p, int cta, uint32_t v) {
+    if (kMany)
+      st_cl_u16(at(p, cta), v);
+    else
+      *p = (uint16_t)v;
+  }
+  static __device__ __forceinline__ uint32_t add(uint32_t *p, int cta, uint32_t v) {
+    return kMany ? atom_cl_add(at(p, cta), v) : atomicAdd(p, v);
+  }
+  __device__ __forceinline__ int ctas() const { return kMany ? c : 1; }
   // marks image row `row` in its CTA's flags
   __device__ __forceinline__ void mark(int row, uint32_t f) const {
-    const int o = row / cap;
-    st_cl_u8(remote(fl + (row - o * cap), o), f);
+    if (kMany) {
+      const int o = row / cap;
+      st_cl_u8(at(fl + (row - o * cap), o), f);
+    } else {
+      fl[row] = (uint8_t)f;
+    }
   }
 };
 
 // Sums the cluster's histogram word `w` (this thread's two buckets) over the
 // CTAs; *mine: the part of the CTAs before this one.
-__device__ __forceinline__ uint32_t sum_words(const ClusterImage &im, const uint32_t *hist, int w, uint32_t *mine) {
+template <bool kMany>
+__device__ __forceinline__ uint32_t sum_words(const SplitImage<kMany> &im, const uint32_t *hist, int w,
+                                              uint32_t *mine) {
+  if (!kMany) {
+    *mine = 0u;
+    return hist[w];
+  }
   const uint32_t local = tc::smem_u32(hist + w);
   uint32_t v[kClMax], total = 0u, before = 0u;
 #pragma unroll
@@ -217,7 +260,8 @@ __device__ __forceinline__ bool bucket_map(float vmin, float vmax, bool compleme
 // Stage I across the cluster; marks X_imp in the rows' flags.  False
 // (cluster-uniform) when it is left to select_image.  On return the marks of
 // every CTA are in place.
-__device__ __forceinline__ bool cluster_stage_one(const SelectArgs &a, const ClusterImage &im, ClusterShared &sh,
+template <bool kMany>
+__device__ __forceinline__ bool cluster_stage_one(const SelectArgs &a, const SplitImage<kMany> &im, ClusterShared &sh,
                                                   float vmin, float vmax) {
   const int tid = threadIdx.x, nthr = blockDim.x;
   BucketMap map;
@@ -226,7 +270,7 @@ __device__ __forceinline__ bool cluster_stage_one(const SelectArgs &a, const Clu
     const int b = map(im.keyr[i]);
     atomicAdd(&sh.hist_r[b >> 1], 1u << (16 * (b & 1)));
   }
-  cluster_barrier();
+  im.barrier();
   uint32_t unused;
   const uint32_t w = sum_words(im, sh.hist_r, tid, &unused);
   const int c0 = (int)(w & 0xffffu), c1 = (int)(w >> 16);
@@ -268,14 +312,14 @@ __device__ __forceinline__ bool cluster_stage_one(const SelectArgs &a, const Clu
     if (b < wlo) {
       im.fl[i] = F_IMP;  // R above the whole window's
     } else if (b <= whi) {
-      const uint32_t slot = atom_cl_add(im.remote(&sh.win_count, 0), 1u);
+      const uint32_t slot = im.add(&sh.win_count, 0, 1u);
       if (slot < (uint32_t)kClWindow) {
-        st_cl_u32(im.remote(&sh.win_key[slot], 0), key);
-        st_cl_u16(im.remote(&sh.win_row[slot], 0), (uint32_t)(im.first + i));
+        im.put(&sh.win_key[slot], 0, key);
+        im.put(&sh.win_row[slot], 0, (uint32_t)(im.first + i));
       }
     }
   }
-  cluster_barrier();
+  im.barrier();
   if (im.rank == 0) {
     // sorted by key (equal keys in any order: they are never certified)
     for (int i = tid; i < len; i += nthr) sh.win_ord[i] = (uint16_t)i;
@@ -323,7 +367,7 @@ __device__ __forceinline__ bool cluster_stage_one(const SelectArgs &a, const Clu
           open = __syncthreads_or(open) != 0;
         }
         if (open) {
-          ok = refine_exact(a, im.off, sh.list, len, 0, im.rec);
+          ok = refine_exact(a, im.off, sh.list, len, 0, im.rec, im.primary);
           rank = 0;
           if (ok && tid < len) {
             const int r = sh.list[tid];
@@ -339,9 +383,9 @@ __device__ __forceinline__ bool cluster_stage_one(const SelectArgs &a, const Clu
         __syncthreads();
       }
     }
-    if (!ok && tid < im.c) st_cl_u32(im.remote(&sh.fail[kFailCut], tid), 1u);
+    if (!ok && tid < im.ctas()) im.put(&sh.fail[kFailCut], tid, 1u);
   }
-  cluster_barrier();
+  im.barrier();
   return sh.fail[kFailCut] == 0u;
 }
 
@@ -350,7 +394,9 @@ struct SortedRow {
   float s;
   int row;
 };
-__device__ __forceinline__ SortedRow sorted_row(const ClusterImage &im, const ClusterShared &sh, int q) {
+template <bool kMany>
+__device__ __forceinline__ SortedRow sorted_row(const SplitImage<kMany> &im, const ClusterShared &sh, int q) {
+  if (!kMany) return SortedRow{unord32(im.sk2[q]), im.sr2[q]};
   int o = im.rank;
   if (q < sh.own[o] || q >= sh.own[o + 1]) {
     o = 0;
@@ -358,10 +404,11 @@ __device__ __forceinline__ SortedRow sorted_row(const ClusterImage &im, const Cl
   }
   const int i = q - sh.own[o];
   if (o == im.rank) return SortedRow{unord32(im.sk2[i]), im.sr2[i]};
-  return SortedRow{unord32(ld_cl_u32(im.remote(im.sk2 + i, o))), (int)ld_cl_u16(im.remote(im.sr2 + i, o))};
+  return SortedRow{unord32(ld_cl_u32(im.at(im.sk2 + i, o))), (int)ld_cl_u16(im.at(im.sr2 + i, o))};
 }
 // Cut between sorted positions q - 1 and q certain (as cert_s).
-__device__ __forceinline__ bool cluster_cert_s(const ClusterImage &im, const ClusterShared &sh, int q,
+template <bool kMany>
+__device__ __forceinline__ bool cluster_cert_s(const SplitImage<kMany> &im, const ClusterShared &sh, int q,
                                                const Bounds &bd) {
   const float sa = sorted_row(im, sh, q - 1).s, sb = sorted_row(im, sh, q).s;
   const float hi_a = __fadd_ru(sa, __fmaf_ru(bd.s_rel, fabsf(sa), bd.s_abs));
@@ -371,7 +418,8 @@ __device__ __forceinline__ bool cluster_cert_s(const ClusterImage &im, const Clu
 
 // Stage II across the cluster: marks X_div.  False (cluster-uniform) when it
 // is left to select_image.
-__device__ __forceinline__ bool cluster_stage_two(const SelectArgs &a, const ClusterImage &im, ClusterShared &sh,
+template <bool kMany>
+__device__ __forceinline__ bool cluster_stage_two(const SelectArgs &a, const SplitImage<kMany> &im, ClusterShared &sh,
                                                   float vmin, float vmax, int slots) {
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int m = im.n - im.k1, t = max(1, m / im.k2);
@@ -382,8 +430,9 @@ __device__ __forceinline__ bool cluster_stage_two(const SelectArgs &a, const Clu
       const int b = map(im.keys[i]);
       atomicAdd(&sh.hist_s[b >> 1], 1u << (16 * (b & 1)));
     }
-  if (tid <= im.c) sh.own[tid] = m;
-  cluster_barrier();
+  const int nc = im.ctas();
+  if (tid <= nc) sh.own[tid] = tid < nc && !kMany ? 0 : m;
+  im.barrier();
   uint32_t mine;
   const uint32_t w = sum_words(im, sh.hist_s, tid, &mine);
   const int c0 = (int)(w & 0xffffu), c1 = (int)(w >> 16);
@@ -395,24 +444,26 @@ __device__ __forceinline__ bool cluster_stage_two(const SelectArgs &a, const Clu
   sh.base[2 * tid + 1] = (uint32_t)(pre + c0) + (mine >> 16);
   if (tid == 0) sh.start[kClBuckets] = (uint32_t)m;
   // a bucket belongs to the CTA whose m / C stretch its start lies in
-  if (c0) atomicMin(&sh.own[pre * im.c / m], pre);
-  if (c1) atomicMin(&sh.own[(pre + c0) * im.c / m], pre + c0);
+  if (kMany && c0) atomicMin(&sh.own[pre * nc / m], pre);
+  if (kMany && c1) atomicMin(&sh.own[(pre + c0) * nc / m], pre + c0);
   if (__syncthreads_or(max(c0, c1) > kClBucketMax)) return false;  // the same in every CTA
-  if (tid == 0)
-    for (int o = im.c - 1; o >= 0; --o) sh.own[o] = min(sh.own[o], sh.own[o + 1]);
-  __syncthreads();
+  if (kMany) {
+    if (tid == 0)
+      for (int o = nc - 1; o >= 0; --o) sh.own[o] = min(sh.own[o], sh.own[o + 1]);
+    __syncthreads();
+  }
   for (int i = tid; i < im.rows; i += nthr)
     if (!(im.fl[i] & F_IMP)) {
       const uint32_t key = im.keys[i];
       const int b = map(key);
-      const int o = (int)sh.start[b] * im.c / m;
+      const int o = kMany ? (int)sh.start[b] * nc / m : 0;
       const int at = (int)atomicAdd(&sh.base[b], 1u) - sh.own[o];
       if (at < slots) {  // always: a stretch is at most m / C + kClBucketMax rows
-        st_cl_u32(im.remote(im.sk + at, o), key);
-        st_cl_u16(im.remote(im.sr + at, o), (uint32_t)(im.first + i));
+        im.put(im.sk + at, o, key);
+        im.put(im.sr + at, o, (uint32_t)(im.first + i));
       }
     }
-  cluster_barrier();
+  im.barrier();
   const int q0 = sh.own[im.rank], q1 = sh.own[im.rank + 1];
   for (int i = tid; i < q1 - q0; i += nthr) {
     const uint32_t key = im.sk[i];
@@ -425,7 +476,7 @@ __device__ __forceinline__ bool cluster_stage_two(const SelectArgs &a, const Clu
     im.sk2[lo + rank] = key;
     im.sr2[lo + rank] = row;
   }
-  cluster_barrier();
+  im.barrier();
   // the picks inside this CTA's stretch
   bool bad = false, marked = false;
   for (int j = tid; j < im.k2; j += nthr) {
@@ -477,7 +528,7 @@ __device__ __forceinline__ bool cluster_stage_two(const SelectArgs &a, const Clu
       }
     }
     __syncthreads();
-    if (sh.exact_rows > 0) bad = !refine_exact(a, im.off, sh.xlist, sh.exact_rows, 1, im.rec);
+    if (sh.exact_rows > 0) bad = !refine_exact(a, im.off, sh.xlist, sh.exact_rows, 1, im.rec, im.primary);
     if (!bad) {
       for (int r = tid; r < runs; r += nthr) {
         const int lo = (int)(sh.run[r] >> 16), len = (int)(sh.run[r] & 0xffffu) - lo;
@@ -497,19 +548,22 @@ __device__ __forceinline__ bool cluster_stage_two(const SelectArgs &a, const Clu
     }
     if (tid == 0) sh.exact_total += sh.exact_rows;
   }
-  if (bad && tid < im.c) st_cl_u32(im.remote(&sh.fail[kFailPicks], tid), 1u);
-  cluster_barrier();
+  if (bad && tid < im.ctas()) im.put(&sh.fail[kFailPicks], tid, 1u);
+  im.barrier();
   return sh.fail[kFailPicks] == 0u;
 }
 
-// Selection of image b by a cluster of c CTAs (this one: rank).  False
-// (cluster-uniform, nothing written) when the image is left to select_image:
-// another barrier is then due before a CTA's shared memory is reused or gone.
+// Selection of image b by a cluster of c CTAs (kMany; this one: rank) or by
+// this CTA.  False (cluster-uniform, nothing written) when the image is left
+// to select_image: another barrier is then due before a CTA's shared memory is
+// reused or gone.  Only a primary CTA writes outputs; *kept (one CTA): the kept
+// local indices in shared memory.
+template <bool kMany>
 __device__ bool select_image_cluster(const SelectArgs &a, const int b, const int c, const int rank,
-                                     unsigned char *smem) {
+                                     unsigned char *smem, const bool primary, const uint16_t **kept) {
   __shared__ ClusterShared sh;
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  ClusterImage im;
+  SplitImage<kMany> im;
   if (a.cu_seqlens) {
     im.off = a.cu_seqlens[b];
     im.n = a.cu_seqlens[b + 1] - a.cu_seqlens[b];
@@ -526,9 +580,10 @@ __device__ bool select_image_cluster(const SelectArgs &a, const int b, const int
   im.k2 = im.k - im.k1;
   im.ko = a.cu_k[b];
   im.c = c;
-  im.rank = rank;
+  im.rank = kMany ? rank : 0;
+  im.primary = primary;
   im.cap = cluster_rows(a.max_n, c);
-  im.first = rank * im.cap;
+  im.first = im.rank * im.cap;
   im.rows = max(0, min(im.cap, im.n - im.first));
   const int slots = cluster_slots(a.max_n, c);
   im.keyr = reinterpret_cast<uint32_t *>(smem);
@@ -545,7 +600,7 @@ __device__ bool select_image_cluster(const SelectArgs &a, const int b, const int
     sh.win_count = 0u;
     sh.runs = sh.run_rows = sh.exact_rows = sh.exact_total = 0;
   }
-  cluster_arrive();  // this CTA runs and has its counters cleared
+  if (kMany) cluster_arrive();  // this CTA runs and has its counters cleared
   const bool need_r = im.k1 > 0 && im.k1 < im.n, need_s = im.k2 > 0;
   const float *st = a.stats + (im.off + im.first) * TR_STATS_WORDS;
   float4 range = make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY);
@@ -586,8 +641,8 @@ __device__ bool select_image_cluster(const SelectArgs &a, const int b, const int
     sh.wr[warp][3] = range.w;
   }
   bad = __syncthreads_or(bad) != 0;
-  cluster_wait();  // and so do the others: their shared memory may be written
-  if (tid < c) {
+  if (kMany) cluster_wait();  // and so do the others: their shared memory may be written
+  if (tid < im.ctas()) {
     range = make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY);
     for (int w = 0; w < kWarps; ++w) {
       range.x = fminf(range.x, sh.wr[w][0]);
@@ -595,14 +650,17 @@ __device__ bool select_image_cluster(const SelectArgs &a, const int b, const int
       range.z = fminf(range.z, sh.wr[w][2]);
       range.w = fmaxf(range.w, sh.wr[w][3]);
     }
-    tc::st_cluster_v4(im.remote(&sh.range[rank], tid), __float_as_uint(range.x), __float_as_uint(range.y),
-                      __float_as_uint(range.z), __float_as_uint(range.w));
-    if (bad) st_cl_u32(im.remote(&sh.fail[kFailKeys], tid), 1u);
+    if (kMany)
+      tc::st_cluster_v4(im.at(&sh.range[rank], tid), __float_as_uint(range.x), __float_as_uint(range.y),
+                        __float_as_uint(range.z), __float_as_uint(range.w));
+    else
+      sh.range[0] = range;
+    if (bad) im.put(&sh.fail[kFailKeys], tid, 1u);
   }
-  cluster_barrier();
+  im.barrier();
   if (sh.fail[kFailKeys]) return false;
   range = sh.range[0];
-  for (int o = 1; o < c; ++o) {
+  for (int o = 1; o < im.ctas(); ++o) {
     const float4 v = sh.range[o];
     range.x = fminf(range.x, v.x);
     range.y = fmaxf(range.y, v.y);
@@ -618,23 +676,51 @@ __device__ bool select_image_cluster(const SelectArgs &a, const int b, const int
   for (int i = i0; i < i1; ++i) cnt += (im.fl[i] & (F_IMP | F_DIV)) != 0;
   int total = 0;
   int pos = block_exclusive_scan(cnt, &total);
-  if (tid < c) st_cl_u32(im.remote(&sh.kept[rank], tid), (uint32_t)total);
-  cluster_barrier();
-  int all = 0;
-  for (int o = 0; o < c; ++o) {
-    if (o < rank) pos += (int)sh.kept[o];
-    all += (int)sh.kept[o];
+  int all = total;
+  if (kMany) {
+    if (tid < c) im.put(&sh.kept[rank], tid, (uint32_t)total);
+    im.barrier();
+    all = 0;
+    for (int o = 0; o < c; ++o) {
+      if (o < rank) pos += (int)sh.kept[o];
+      all += (int)sh.kept[o];
+    }
   }
   for (int i = i0; i < i1; ++i) {
     const uint8_t f = im.fl[i];
-    if ((f & (F_IMP | F_DIV)) && pos < im.k) a.idx[im.ko + pos++] = im.first + i;  // never past this image's slots
-    if (a.role) a.role[im.off + im.first + i] = (f & F_IMP) ? 1 : ((f & F_DIV) ? 2 : 0);
+    if ((f & (F_IMP | F_DIV)) && pos < im.k) {  // never past this image's slots
+      if (primary) a.idx[im.ko + pos] = im.first + i;
+      if (!kMany) im.sr[pos] = (uint16_t)i;
+      ++pos;
+    }
+    if (primary && a.role) a.role[im.off + im.first + i] = (f & F_IMP) ? 1 : ((f & F_DIV) ? 2 : 0);
   }
-  if (tid == 0 && a.status) {
-    if (rank == 0 && all != im.k) atomicAdd(&a.status[3], 1);
+  if (tid == 0 && primary && a.status) {
+    if (im.rank == 0 && all != im.k) atomicAdd(&a.status[3], 1);
     if (sh.exact_total) atomicAdd(&a.status[2], sh.exact_total);
   }
+  if (!kMany) {
+    *kept = im.sr;
+    __syncthreads();  // the list is complete, and the arrays may serve the next image
+  }
   return true;
+}
+
+// Images up to this size take the fast path in one CTA (its arrays fit beside
+// what select_image needs).
+constexpr int kSoloMaxN = 8192;
+
+// The selection of image b by this CTA; returns the kept local indices in
+// shared memory.
+__device__ __forceinline__ const uint16_t *select_image_solo(const SelectArgs &a, const int b, unsigned char *smem,
+                                                             const bool primary) {
+  const uint16_t *kept = kept_rows(a, smem);
+  if (a.max_n <= kSoloMaxN) {
+    if (select_image_cluster<false>(a, b, 1, 0, smem, primary, &kept)) return kept;
+    __syncthreads();
+  }
+  select_image(a, b, smem, primary);
+  return kept_rows(a, smem);
 }
 
 }  // namespace

@@ -1,9 +1,9 @@
-"""The selection of large images by a cluster of CTAs (k_select_cluster)
-against the oracle: the edges of its rule (2560 tokens; 12, 36 and 72 images
-for eight, four and two CTAs), images much smaller than the batch's largest,
-near-ties at the cut and at the picks, and the inputs it leaves to the
-one-CTA selection (exact ties, crowded keys, rows outside the fp32 model).
-Kept indices and rows are compared bit for bit.
+"""The selection's fast path, in one CTA and in a cluster of CTAs per image,
+against the oracle: the edges of its rules (5120 and 8192 tokens; 12, 36 and
+72 images), images much smaller than the batch's largest, near-ties at the
+cut and at the picks, and the inputs it leaves to select_image (exact ties
+in numbers, crowded keys, rows outside the fp32 model).  Kept indices and
+rows are compared bit for bit.
 """
 import pytest
 import torch
@@ -29,41 +29,52 @@ def _budget(ks, k1s):
 
 
 @pytest.mark.parametrize("batch,n,d,dtype", [
-    (1, 2559, 128, torch.bfloat16), (1, 2560, 128, torch.bfloat16), (1, 2561, 64, torch.float32),
-    (3, 4099, 64, torch.float16), (12, 2563, 64, torch.bfloat16), (13, 2816, 64, torch.bfloat16),
-    (36, 2560, 32, torch.float32), (37, 2600, 64, torch.bfloat16), (72, 2560, 64, torch.bfloat16),
-    (73, 2560, 64, torch.bfloat16), (1, 16384, 64, torch.bfloat16), (2, 16383, 32, torch.float32),
+    # one CTA per image, up to 8192 tokens
+    (3, 1, 64, torch.bfloat16), (3, 2, 64, torch.float16), (2, 511, 64, torch.bfloat16), (5, 513, 64, torch.float32),
+    (200, 1025, 32, torch.bfloat16), (1, 5119, 128, torch.bfloat16), (37, 8192, 32, torch.bfloat16),
+    # clusters
+    (1, 5120, 128, torch.bfloat16), (1, 5121, 64, torch.float32), (3, 7001, 64, torch.float16),
+    (12, 5123, 64, torch.bfloat16), (13, 5200, 64, torch.bfloat16), (36, 5120, 32, torch.float32),
+    (37, 8193, 32, torch.bfloat16), (72, 8200, 32, torch.bfloat16), (1, 16384, 64, torch.bfloat16),
+    (2, 16383, 32, torch.float32),
+    # neither
+    (73, 8193, 32, torch.bfloat16),
 ])
 def test_sizes(batch, n, d, dtype):
     x, xp, xq = _rows(batch * n, d, 7 * n + batch, dtype)
     images = sorted({0, batch // 2, batch - 1})
-    for k, k1, stride in [(n // 9, n // 27, "alg1"), (n // 3 + 1, n // 10, "interval")]:
+    for k, k1, stride in [(max(1, n // 9), n // 27, "alg1"), (min(n, n // 3 + 1), n // 10, "interval")]:
         check_reduce(x, xp, xq, [n] * batch, _budget([k] * batch, [k1] * batch), images=images, stride=stride)
 
 
 def test_ragged_sizes():
-    seqlens = [2560, 1, 16384, 255, 0, 7000, 16, 513]
+    for seqlens in ([2560, 1, 16384, 255, 0, 7000, 16, 513], [600, 1, 4000, 0, 17]):
+        _ragged(seqlens)
+
+
+def _ragged(seqlens):
     x, xp, xq = _rows(sum(seqlens), 64, 5, torch.bfloat16)
     ks = [max(1, 2 * n // 9) if n else 0 for n in seqlens]
     check_reduce(x, xp, xq, seqlens, _budget(ks, [k // 3 for k in ks]))
 
 
-@pytest.mark.parametrize("k,k1", [(1, 0), (1, 1), (2, 1), (3000, 1000), (3000, 0), (2999, 2999), (1500, 1500),
-                                  (2999, 1), (700, 0)])
-def test_budgets(k, k1):
-    n = 3000
+@pytest.mark.parametrize("n", [700, 6000])
+def test_budgets(n):
     x, xp, xq = _rows(n, 128, 11, torch.bfloat16)
-    check_reduce(x, xp, xq, [n], _budget([k], [k1]))
+    for k, k1 in [(1, 0), (1, 1), (2, 1), (n, n // 3), (n, 0), (n, n), (n - 1, n - 1), (n // 2, n // 2), (n - 1, 1),
+                  (n // 4, 0)]:
+        check_reduce(x, xp, xq, [n], _budget([k], [k1]))
 
 
+@pytest.mark.parametrize("rows", [2500, 5500])
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "f32"])
-def test_near_ties(dtype):
+def test_near_ties(dtype, rows):
     # triples that the fp32 keys leave uncertain and the double-float keys
     # separate, among ordinary rows: no exact sums are needed, wherever the cut
     # splits a triple and for dense and sparse picks
     d = 1024
     tx, tp, tq, *_ = _near_tie_triples(32, d, dtype, 3)
-    x, xp, xq = (torch.cat([a, b]) for a, b in zip((tx, tp, tq), _rows(2500, d, 4, dtype)))
+    x, xp, xq = (torch.cat([a, b]) for a, b in zip((tx, tp, tq), _rows(rows, d, 4, dtype)))
     perm = torch.randperm(x.shape[0], generator=torch.Generator().manual_seed(6))
     x, xp, xq = x[perm], xp[perm], xq[perm]
     n = x.shape[0]
@@ -88,8 +99,9 @@ def test_near_ties(dtype):
         assert 0 < st[2] <= 4 * len(pairs) + 8, st
 
 
-def test_left_to_one_cta():
-    n, d = 2600, 64
+@pytest.mark.parametrize("n", [2600, 6000])
+def test_left_to_select_image(n):
+    d = 64
     base, bp, bq = _rows(n, d, 21, torch.bfloat16)
 
     def run(edit, k=600, k1=200, **kw):
