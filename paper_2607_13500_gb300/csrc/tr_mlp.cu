@@ -85,7 +85,6 @@ constexpr int kPartWords = 10;                    // hi, lo of L1, S2, A, B, P
 // unit u of row r at r * 64 + ((u ^ (r / 2 % 4)) << 4): the 32 lanes' 16-byte
 // accesses take the fewest shared-memory wavefronts).
 constexpr int kBlk = 32;
-constexpr int kTileBlks = kBN / kBlk;
 constexpr int kBlkBytes = 32 * kBlk * 2;
 // Staging per epilogue warp: the output block (the projector's warps two of
 // them); the score mode's blocks of x' and of the residual, loaded by TMA
@@ -93,19 +92,20 @@ constexpr int kBlkBytes = 32 * kBlk * 2;
 __host__ __device__ constexpr int stage_blks(int mode) { return mode == kModeHidden ? 1 : 2; }
 __host__ __device__ constexpr int stage_bytes(int mode) { return stage_blks(mode) * kBlkBytes; }
 // Splits of K over the pairs of a cluster: pair p of kSplit sums its k-blocks
-// into its own accumulators and finishes the tile's blocks [p, p + 1) * 8 /
-// kSplit, whose partial sums the other pairs send it.
-__host__ __device__ constexpr int owned_blks(int split) { return kTileBlks / split; }
-// Warps per lane quarter with blocks of their own, and the score mode's
-// partial row sums per tile and lane quarter.
-__host__ __device__ constexpr int active_parts(int mode, int split) {
-  return owned_blks(split) < epi_parts(mode, split) ? owned_blks(split) : epi_parts(mode, split);
+// into its own accumulators and finishes the tile's blocks [p, p + 1) * own,
+// own = tile blocks / kSplit, whose partial sums the other pairs send it.
+// The score mode's partial row sums per tile and lane quarter: one for each
+// warp that has blocks.
+__host__ __device__ constexpr int active_parts(int own, int split) {
+  return own < epi_parts(kModeScore, split) ? own : epi_parts(kModeScore, split);
 }
-__host__ __device__ constexpr int row_parts(int split) { return split * active_parts(kModeScore, split); }
+__host__ __device__ constexpr int row_parts(int bn, int split) {
+  return split * active_parts(bn / kBlk / split, split);
+}
 
 struct GemmArgs {
   int m, n, k;          // C[m, n] = A[m, k] B[n, k]^T
-  int bn;               // tile columns: 256, 192, 128 or 64 (256 when K is split)
+  int bn;               // tile columns: 256, 192, 128 or 64
   int n_tiles, tiles, kblocks;
   const float *bias;    // [n] or NULL
   int act;              // hidden GEMM: TR_ACT_*
@@ -336,8 +336,8 @@ __device__ __forceinline__ void score_load_next(const GemmArgs &g, const GemmMap
 // does not depend on which pair owns the block.  slots: received partials,
 // [other pair][four-column unit of the owned columns][128 rows].
 template <int kSplit>
-__device__ __forceinline__ void add_partials(uint32_t slots, int pair, int unit, int row, uint32_t (&v)[8]) {
-  constexpr uint32_t kSlot = 128u * 4u * kBN / kSplit;
+__device__ __forceinline__ void add_partials(uint32_t slots, uint32_t slot_bytes, int pair, int unit, int row,
+                                             uint32_t (&v)[8]) {
   float sum[8];
 #pragma unroll
   for (int o = 0; o < kSplit; ++o) {
@@ -345,7 +345,7 @@ __device__ __forceinline__ void add_partials(uint32_t slots, int pair, int unit,
 #pragma unroll
     for (int i = 0; i < 8; ++i) t[i] = __uint_as_float(v[i]);
     if (o != pair) {
-      const uint32_t src = slots + (uint32_t)(o < pair ? o : o - 1) * kSlot + (uint32_t)(unit * 128 + row) * 16u;
+      const uint32_t src = slots + (uint32_t)(o < pair ? o : o - 1) * slot_bytes + (uint32_t)(unit * 128 + row) * 16u;
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         uint32_t r[4];
@@ -376,6 +376,7 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs &g, const GemmMaps 
   constexpr int kUnits = kMode == kModeScore && kSplit > 1 ? 1 : 2;  // 8-column units in flight
   const int lane = threadIdx.x & 31;
   const uint32_t sw = (uint32_t)((lane >> 1) & 3);  // the 64-byte swizzle's row term
+  const int own = g.bn / kBlk / kSplit;             // blocks that each pair finishes
   for (int blk = w.first; blk < w.end; blk += kParts) {
     const int col = nt * g.bn + blk * kBlk;
     if (col >= g.n) break;
@@ -401,7 +402,8 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs &g, const GemmMaps 
       for (int i = 0; i < kUnits; ++i) {
         const int u = u0 + i;
         if (kSplit > 1)
-          add_partials<kSplit>(slots, pair, (blk - pair * owned_blks(kSplit)) * 8 + 2 * u, row_in_tile, v[i]);
+          add_partials<kSplit>(slots, 512u * (uint32_t)(own * kBlk), pair, (blk - pair * own) * 8 + 2 * u, row_in_tile,
+                               v[i]);
         const uint32_t addr = rowbuf + (((uint32_t)u ^ sw) << 4);
         if (kMode == kModeScore)
           epi_score(g, col + 8 * u, v[i], addr, acc2);
@@ -431,16 +433,16 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs &g, const GemmMaps 
 // go to them (16-byte stores into the owner's shared memory, whose operand
 // ring is idle by then; 32 lanes write 512 consecutive bytes).
 template <int kMode, int kSplit>
-__device__ __forceinline__ void send_partials(uint32_t slots, uint32_t taddr, int pair, uint32_t rank, int part,
-                                              int row_in_tile) {
-  constexpr uint32_t kSlot = 128u * 4u * kBN / kSplit;
-  for (int blk = part; blk < kTileBlks; blk += epi_parts(kMode, kSplit)) {
-    const int owner = blk / owned_blks(kSplit);
+__device__ __forceinline__ void send_partials(const GemmArgs &g, uint32_t slots, uint32_t taddr, int pair,
+                                              uint32_t rank, int part, int row_in_tile) {
+  const int own = g.bn / kBlk / kSplit;
+  for (int blk = part; blk < g.bn / kBlk; blk += epi_parts(kMode, kSplit)) {
+    const int owner = blk / own;
     if (owner == pair) continue;
-    const int unit = (blk - owner * owned_blks(kSplit)) * 8;
-    const uint32_t dst = tc::map_shared(slots + (uint32_t)(pair < owner ? pair : pair - 1) * kSlot +
-                                            (uint32_t)(unit * 128 + row_in_tile) * 16u,
-                                        2u * (uint32_t)owner + (rank & 1u));
+    const uint32_t dst =
+        tc::map_shared(slots + (uint32_t)(pair < owner ? pair : pair - 1) * 512u * (uint32_t)(own * kBlk) +
+                           (uint32_t)((blk - owner * own) * 8 * 128 + row_in_tile) * 16u,
+                       2u * (uint32_t)owner + (rank & 1u));
 #pragma unroll 1
     for (int u = 0; u < kBlk / 8; ++u) {
       uint32_t v[8];
@@ -770,9 +772,9 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
     const int part = (warp - 2) >> 2;  // which of the quadrant's warps
     // first of this warp's 32 rows in row tile rb
     auto row_of = [&](int rb) { return (2 * rb + (int)rank) * kBM + 32 * q; };
-    const int own = pair * owned_blks(kSplit);
-    EpiWarp w{own + part, own + (kSplit > 1 ? owned_blks(kSplit) : g.bn / kBlk), out_stage + (uint32_t)((warp - 2) * stage_bytes(kMode)),
-              blk_bar(warp - 2), 0u, 0u, cluster, own + part};
+    const int own = g.bn / kBlk / kSplit, own0 = pair * own;
+    EpiWarp w{own0 + part, own0 + own, out_stage + (uint32_t)((warp - 2) * stage_bytes(kMode)),
+              blk_bar(warp - 2), 0u, 0u, cluster, own0 + part};
     if (kMode == kModeScore) score_load_next<epi_parts(kMode, kSplit)>(g, maps, w, clusters, row_of);
     int acc = 0;
     uint32_t acc_phase = 0;
@@ -788,7 +790,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
       if (kSplit > 1) {  // every pair's MMAs are done: the operand rings may take the partial sums
         __syncwarp();
         tc::cluster_sync();
-        if (ok) send_partials<kMode, kSplit>(sbase, taddr, pair, rank, part, 32 * q + lane);
+        if (ok) send_partials<kMode, kSplit>(g, sbase, taddr, pair, rank, part, 32 * q + lane);
         __syncwarp();
         tc::cluster_sync();
       }
@@ -803,10 +805,9 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
       __syncwarp();
       if (lane == 0) tc::mbar_arrive_cluster(tempty_even(acc));  // this warp is done with the accumulator
       const int rb128 = 2 * rb + (int)rank;
-      if (kMode == kModeScore && rb128 * kBM < g.m && part < active_parts(kMode, kSplit))
-        publish_rows(g.part + part_slot(g, row_parts(kSplit), rb128, nt, pair * active_parts(kMode, kSplit) + part, q) +
-                         lane,
-                     sums);
+      const int active = active_parts(own, kSplit);
+      if (kMode == kModeScore && rb128 * kBM < g.m && part < active)
+        publish_rows(g.part + part_slot(g, kSplit * active, rb128, nt, pair * active + part, q) + lane, sums);
       acc ^= 1;
       if (acc == 0) acc_phase ^= 1u;
     }
@@ -926,13 +927,16 @@ struct GemmShape {
 //   projector's row gather 1065 whatever the columns.  A tile's epilogue takes
 //   80 (score), 30 (hidden) or 65 (projector) clocks a column, overlapped with
 //   the next tile's main loop where there is one.
-//   Splitting K over two or four pairs (256 columns, only while all clusters
-//   run at once: 32 of four SMs, 16 of eight) divides the main loop and the
-//   epilogue and adds the exchange, 4500 or 7000 clocks (96 KiB into each SM).
+//   Splitting K over two or four pairs (while all clusters run at once: 64
+//   pairs) divides the main loop and the epilogue and adds the exchange: two
+//   cluster barriers and the partial sums into each SM at 14 bytes a clock (96
+//   KiB for 256 columns in four, 7,000 clocks in all).
 // Measured: 192 rows, 1024 -> 4096, 16 tiles of 256 columns 12.3 us a pass, 64
 // of 64 columns 8.4; both GEMMs of 2885 rows, 1152 -> 4304 -> 1152, 63.4 us
 // with 60 score tiles of 256 columns, 58.9 with 72 of 192; the score GEMM of
-// 576 rows, 4096 -> 1024, 45 us unsplit, 21 split in four.
+// 576 rows, 4096 -> 1024, 45 us in 256 columns, 21 with K split in four; both
+// GEMMs of 48 and 128 rows (1024 -> 4096 -> 1024) 28.7 and 27.0 us with 256
+// columns in four, 25.2 and 23.5 with 128.
 // The sums of an output element are the same for every mode (tr_project and
 // tr_project_kept agree bit for bit): they depend on the split alone.
 inline GemmShape gemm_shape(int m, int n, int k, bool score, bool gather) {
@@ -959,14 +963,16 @@ inline GemmShape gemm_shape(int m, int n, int k, bool score, bool gather) {
   long long least = 0;
   int bn = narrowest(false, &least), split = 1;
   for (const int s : {2, 4})  // the same for gathered rows
-    if (kb >= 4 * s && rows * tiles_of(kBN) * s <= 64) {
-      const long long c = (long long)(kb + s - 1) / s * 520 + epi(kBN, false) / s + (s == 2 ? 4500 : 7000);
-      if (c < least) {
-        least = c;
-        bn = kBN;
-        split = s;
+    for (const int w : {256, 192, 128, 64})
+      if (w / kBlk % s == 0 && kb >= 4 * s && rows * tiles_of(w) * s <= 64) {
+        const long long c = (long long)((kb + s - 1) / s) * std::max(2 * w + 8, (16384 + 64 * w) / 63) +
+                            std::max(2500LL, epi(w, false) / s) + 1000 + 512LL * (s - 1) * (w / s) / 14;
+        if (c < least) {
+          least = c;
+          bn = w;
+          split = s;
+        }
       }
-    }
   if (gather && split == 1) bn = narrowest(true, &least);
   return GemmShape{bn, split, tiles_of(bn), kb};
 }
@@ -1010,7 +1016,7 @@ MlpWs mlp_ws(const tr_mlp *m) {
   const GemmShape sh = gemm_shape(m->t, m->d, m->d_hidden, true, false);
   MlpWs w;
   w.part = 0;
-  w.total = align_up((size_t)rblocks * sh.n_tiles * row_parts(sh.split) * 4 * kPartWords * 32 * sizeof(float), 256);
+  w.total = align_up((size_t)rblocks * sh.n_tiles * row_parts(sh.bn, sh.split) * 4 * kPartWords * 32 * sizeof(float), 256);
   return w;
 }
 
@@ -1100,7 +1106,7 @@ tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, fl
       !block_map(&maps.x, x))
     return TR_ERR_CUDA;
   if (launch_shape<kModeScore>(maps, g, sh.split, st) != cudaSuccess) return TR_ERR_CUDA;
-  const int parts = row_parts(sh.split);
+  const int parts = row_parts(sh.bn, sh.split);
   const cudaError_t err = launch_kernel(k_score_rows, dim3((g.m + kBM - 1) / kBM * 4), dim3(kRowWarps * 32), 0, st, true, g, parts,
                                         reinterpret_cast<float4 *>(stats), h2, s);
   return err == cudaSuccess ? TR_OK : TR_ERR_CUDA;

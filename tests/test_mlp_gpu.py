@@ -242,18 +242,21 @@ def test_project_kept_index_outside_its_image():
     _check_close(z, _sigma(v, "gelu"), mag, slope=1.13)
 
 
-# The layouts a GEMM may take (gemm_shape): K split over two or four pairs of a
-# cluster, and 192-, 128- and 64-column tiles, with ragged rows, columns and
-# k-blocks and k-blocks that do not divide evenly.  Named by the score GEMM's.
+# The layouts a GEMM may take (gemm_shape): tile columns x pairs that split K,
+# with ragged rows, columns and k-blocks and k-blocks that do not divide
+# evenly.  Named by the score GEMM's layout.
 SPLIT_CASES = [
-    ("four_one_row", 1, 256, 6144, "none", False, True),         # 1 tile, 96 k-blocks
-    ("four_uneven_k", 300, 528, 4464, "gelu", True, True),       # 6 tiles, 69.75 k-blocks
-    ("four_most_tiles", 1000, 1024, 4160, "quick_gelu", True, False),  # 16 tiles, 65 k-blocks
-    ("two_uneven_k", 1500, 1024, 4400, "gelu", True, True),      # 24 tiles, 68.75 k-blocks
-    ("two_most_tiles", 2048, 784, 4112, "gelu", False, True),    # 32 tiles, 64.25 k-blocks
-    ("narrow_192", 2049, 1152, 1600, "none", True, True),        # 9 x 6 tiles
-    ("narrow_128", 2048, 784, 2064, "gelu", False, True),        # 8 x 7 tiles, the last 16 columns
-    ("narrow_64", 129, 1056, 1472, "quick_gelu", True, True),    # 1 x 17 tiles, the last half empty
+    ("256x4", 1000, 1024, 16400, "none", True, True),            # 16 tiles, 256.25 k-blocks
+    ("128x4_one_row", 1, 256, 6144, "none", False, True),        # 2 tiles, 96 k-blocks
+    ("128x4_uneven_k", 300, 528, 4464, "gelu", True, True),      # 10 tiles, 69.75 k-blocks
+    ("256x2_uneven_k", 1500, 1024, 4400, "gelu", True, True),    # 24 tiles, 68.75 k-blocks
+    ("256x2_most_tiles", 2048, 784, 4112, "gelu", False, True),  # 32 tiles, 64.25 k-blocks
+    ("192x2", 1200, 1024, 4096, "quick_gelu", True, True),       # 5 x 6 tiles, the last 64 columns
+    ("128x2", 1000, 1024, 4160, "quick_gelu", True, False),      # 32 tiles, 65 k-blocks
+    ("64x2", 129, 1056, 1472, "quick_gelu", True, True),         # 17 tiles, the last half empty
+    ("192x1", 2885, 1152, 4304, "gelu", True, True),             # 12 x 6 tiles
+    ("128x1", 2048, 784, 2064, "gelu", False, True),             # 8 x 7 tiles, the last 16 columns
+    ("64x1", 2049, 1152, 1600, "none", True, True),              # 9 x 18 tiles
 ]
 
 
@@ -271,24 +274,55 @@ def test_mlp_split(name, t, d, dh, act, resid, bias):
         assert torch.equal(u.view(torch.int16), v.view(torch.int16))
 
 
-@pytest.mark.parametrize("d,d_out,k", [(8208, 528, 40), (4096, 2560, 200), (784, 1296, 50)],
-                         ids=["four", "two", "narrow"])
-def test_project_split(d, d_out, k):
+def _project_direct(x, idx, cu_k, w, bias, seqlens):
+    """tr_project_kept itself, which the binding's project_kept calls for few
+    rows and for images above 16384 tokens."""
+    from paper_2607_13500_gb300 import _lib
+    from paper_2607_13500_gb300.api import _Tokens, _ptr, _stream
+    tok = _Tokens(x, None, x, seqlens)
+    z = torch.empty(cu_k[-1], w.shape[0], dtype=torch.bfloat16, device=x.device)
+    err = torch.zeros(1, dtype=torch.int32, device=x.device)
+    d_cu = torch.tensor(cu_k, dtype=torch.int32, device=x.device)
+    _lib.check("tr_project_kept", _lib.load().tr_project_kept(
+        tok.ref(), _ptr(d_cu), _ptr(idx), cu_k[-1], _ptr(w), _ptr(bias), w.shape[0], 0, _ptr(z), _ptr(err),
+        _stream(x.device)))
+    return z, err
+
+
+@pytest.mark.parametrize("d,d_out,k,n,b", [(8208, 528, 40, 300, 3), (4096, 2560, 200, 300, 3), (784, 1296, 50, 300, 3),
+                                           (272, 528, 200, 300, 16), (256, 272, 1025, 1300, 3)],
+                         ids=["128x4", "256x2", "64x1", "gathered", "gathered_few"])
+def test_project_split(d, d_out, k, n, b):
     # K split, or narrow tiles: the dense projector within the GEMM tolerance
     # of float64, and the rows read by index bit for bit the same
     altr = _alt()
     g = torch.Generator(device="cuda").manual_seed(9)
-    n, b = 300, 3
     x = torch.randn(b * n, d, generator=g, device="cuda").to(torch.bfloat16)
     idx = torch.rand(b, n, generator=g, device="cuda").argsort(1)[:, :k].sort(1).values.to(torch.int32)
     w = (torch.randn(d_out, d, generator=g, device="cuda") / math.sqrt(d)).to(torch.bfloat16)
     bias = 0.05 * torch.randn(d_out, generator=g, device="cuda")
     y = torch.cat([x[i * n:(i + 1) * n][idx[i].long()] for i in range(b)]).contiguous()
+    idx, cu_k = idx.reshape(-1).contiguous(), [i * k for i in range(b + 1)]
     z, err = altr.project(y, w, bias, act="gelu")
-    zk, err_k = altr.project_kept(x, idx.reshape(-1).contiguous(), [i * k for i in range(b + 1)], w, bias, act="gelu",
-                                  seqlens=[n] * b)
+    zk, err_k = altr.project_kept(x, idx, cu_k, w, bias, act="gelu", seqlens=[n] * b)
+    zd, err_d = _project_direct(x, idx, cu_k, w, bias, [n] * b)
     torch.cuda.synchronize()
-    assert err.item() == 0 and err_k.item() == 0
+    assert err.item() == 0 and err_k.item() == 0 and err_d.item() == 0
     assert torch.equal(z.view(torch.int16), zk.view(torch.int16))
+    assert torch.equal(z.view(torch.int16), zd.view(torch.int16))
     v, mag = _gemm_ref(y, w, bias)
     _check_close(z, _sigma(v, "gelu"), mag, slope=1.13)
+
+
+def test_project_kept_of_an_image_past_the_gather_limit():
+    # more tokens in an image than tr_gather takes: the direct kernel
+    altr = _alt()
+    g = torch.Generator(device="cuda").manual_seed(2)
+    n, d, d_out, k = 20000, 64, 96, 4000
+    x = torch.randn(n, d, generator=g, device="cuda").to(torch.bfloat16)
+    idx = torch.randperm(n, generator=g, device="cuda")[:k].sort().values.to(torch.int32)
+    w = (torch.randn(d_out, d, generator=g, device="cuda") / 8).to(torch.bfloat16)
+    z, err = altr.project_kept(x, idx, [0, k], w, act="none", seqlens=[n])
+    zd, err_d = altr.project(x[idx.long()].contiguous(), w, act="none")
+    torch.cuda.synchronize()
+    assert err.item() == 0 and err_d.item() == 0 and torch.equal(z.view(torch.int16), zd.view(torch.int16))
