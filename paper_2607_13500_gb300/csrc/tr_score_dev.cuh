@@ -216,10 +216,13 @@ __device__ __forceinline__ void accumulate_round(const uint4 *__restrict__ rx, c
 }
 
 // Partial sums of chunks [c0, c1) of one row, read straight from global
-// memory in rounds of kB chunks per lane and stream.  When the row's chunks
-// are a multiple of 32 (every lane has the same count) the last round is cut
-// to the chunks that remain (6, 4 or 2 per lane, fewer than a full round), so
-// no lane works on padding.
+// memory in rounds of kB chunks per lane and stream.  The last round is cut to
+// the chunks that remain: 6, 4 or 2 per lane exactly when they are a multiple
+// of 64, else the smallest of 2, 4, 6, kB that holds them, its missing chunks
+// read as zeros (a full round for any other rest made the arithmetic on the
+// zeros the bound: passes of 48 x 1000 tokens of 776 bf16 channels 92.4 us
+// against 75.2, 24 x 1000 of 3000 fp16 channels 99.1 against 87.7, 48 x 576 of
+// 2824 bf16 channels 110.9 against 103.5).
 template <int kDt>
 __device__ __forceinline__ void accumulate_global(const uint4 *__restrict__ rx, const uint4 *__restrict__ rp,
                                                   const uint4 *__restrict__ rq, int c0, int c1, Acc &acc,
@@ -237,6 +240,12 @@ __device__ __forceinline__ void accumulate_global(const uint4 *__restrict__ rx, 
       accumulate_round<kDt, 4, false>(rx, rp, rq, base, c1, acc, acc2, lane);
     else if (rest == 32 * 2)
       accumulate_round<kDt, 2, false>(rx, rp, rq, base, c1, acc, acc2, lane);
+    else if (rest <= 32 * 2)
+      accumulate_round<kDt, 2, true>(rx, rp, rq, base, c1, acc, acc2, lane);
+    else if (rest <= 32 * 4)
+      accumulate_round<kDt, 4, true>(rx, rp, rq, base, c1, acc, acc2, lane);
+    else if (rest <= 32 * 6)
+      accumulate_round<kDt, 6, true>(rx, rp, rq, base, c1, acc, acc2, lane);
     else
       accumulate_round<kDt, kB, true>(rx, rp, rq, base, c1, acc, acc2, lane);
   }
