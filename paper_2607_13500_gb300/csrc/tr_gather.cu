@@ -77,9 +77,13 @@ cudaError_t launch_gather(const void *x, long long total_rows, int dtype, int d,
   // (14 per lane: two of seven), none alone: what a round costs is its latency.
   // (Four a round and the rest one by one took 55.5 us on 12 ragged images of
   // 3584 bf16 channels, 322 MB, against 51.8, and 10.2 against 8.2 for a clip's
-  // 784 rows, launch included.)
+  // 784 rows, launch included.)  Beside another batch's scoring (the pipeline,
+  // pdl false) four loads a round: there its own latency is hidden and its
+  // bursts hold the scoring up (64 images of 576 x 4096 bf16, a third kept,
+  // 168.2 us a batch against 168.6; 32 images, a third kept, 85.6 against 85.9).
   const int per_lane = (nchunks + 31) / 32;
-  const int rounds = (per_lane + 7) / 8;
+  const int most = pdl ? 8 : 4;
+  const int rounds = (per_lane + most - 1) / most;
   switch ((per_lane + rounds - 1) / rounds) {
     case 1: return launch(k_gather<1>);
     case 2: return launch(k_gather<2>);
