@@ -352,7 +352,12 @@ typedef struct {
 /* H = sigma(x' W1^T + b1): h is device bf16 [t, d_hidden]. */
 tr_status tr_mlp_hidden(const tr_mlp *m, void *h, int32_t *d_error, void *stream);
 
-/* Scratch bytes of tr_mlp_score (256-byte aligned device memory); 0 on invalid input. */
+/*
+ * Scratch bytes of tr_mlp_score (256-byte aligned device memory); 0 on invalid
+ * input.  A call given fewer (scratch sized for a larger t, whose GEMM is laid
+ * out differently) still runs, in 256-column tiles, from 10 KiB per 128 rows
+ * and 256 channels (begun ones counted whole) on.
+ */
 size_t tr_mlp_workspace_bytes(const tr_mlp *m);
 
 /*

@@ -1008,16 +1008,17 @@ tr_status check_mlp(const tr_mlp *m) {
   return TR_OK;
 }
 
-struct MlpWs {
-  size_t part, total;
-};
-MlpWs mlp_ws(const tr_mlp *m) {
+// Bytes of the score mode's partial sums in one layout, and the layout that
+// tr_mlp_score takes with `bytes` of them: the one gemm_shape chooses, or with
+// fewer (a workspace sized for another batch: a split or narrow layout of few
+// rows may want more than 256-column tiles of many) 256-column tiles.
+size_t part_bytes(const tr_mlp *m, const GemmShape &sh) {
   const long long rblocks = ((long long)m->t + kBM - 1) / kBM;
+  return align_up((size_t)rblocks * sh.n_tiles * row_parts(sh.bn, sh.split) * 4 * kPartWords * 32 * sizeof(float), 256);
+}
+GemmShape score_shape(const tr_mlp *m, size_t bytes) {
   const GemmShape sh = gemm_shape(m->t, m->d, m->d_hidden, true, false);
-  MlpWs w;
-  w.part = 0;
-  w.total = align_up((size_t)rblocks * sh.n_tiles * row_parts(sh.bn, sh.split) * 4 * kPartWords * 32 * sizeof(float), 256);
-  return w;
+  return part_bytes(m, sh) <= bytes ? sh : GemmShape{kBN, 1, (m->d + kBN - 1) / kBN, sh.kblocks};
 }
 
 // out = act(a W^T + bias) for dense bf16 rows a [rows, k] and W [n, k]: the
@@ -1071,7 +1072,7 @@ tr_status tr_project(const void *y, int32_t rows, int32_t d, const void *w, cons
 
 size_t tr_mlp_workspace_bytes(const tr_mlp *m) {
   if (check_mlp(m) != TR_OK) return 0;
-  return mlp_ws(m).total;
+  return part_bytes(m, score_shape(m, SIZE_MAX));
 }
 
 tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, float *stats, float *h2, float *s,
@@ -1082,20 +1083,18 @@ tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, fl
   if (misaligned16(h) || misaligned16(x_post) || misaligned16(x) || misaligned16(stats) ||
       (reinterpret_cast<uintptr_t>(h2) & 3u) || (reinterpret_cast<uintptr_t>(s) & 3u))
     return TR_ERR_ALIGN;
-  const MlpWs w = mlp_ws(m);
-  if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < w.total) return TR_ERR_WORKSPACE;
+  const GemmShape sh = score_shape(m, ws_bytes);
+  if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) || ws_bytes < part_bytes(m, sh)) return TR_ERR_WORKSPACE;
   if (m->t == 0) return TR_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  char *wsb = static_cast<char *>(ws);
   GemmArgs g{};
   g.m = m->t;
   g.n = m->d;
   g.k = m->d_hidden;
-  const GemmShape sh = gemm_shape(g.m, g.n, g.k, true, false);
   set_shape(g, sh);
   g.bias = m->b2;
   g.has_resid = m->resid != nullptr;
-  g.part = reinterpret_cast<float *>(wsb + w.part);
+  g.part = static_cast<float *>(ws);
   g.err = d_error;
   GemmMaps maps{};
   auto block_map = [&](CUtensorMap *map, const void *p) {  // the epilogue's 32 x 32 blocks
@@ -1107,8 +1106,8 @@ tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, fl
     return TR_ERR_CUDA;
   if (launch_shape<kModeScore>(maps, g, sh.split, st) != cudaSuccess) return TR_ERR_CUDA;
   const int parts = row_parts(sh.bn, sh.split);
-  const cudaError_t err = launch_kernel(k_score_rows, dim3((g.m + kBM - 1) / kBM * 4), dim3(kRowWarps * 32), 0, st, true, g, parts,
-                                        reinterpret_cast<float4 *>(stats), h2, s);
+  const cudaError_t err = launch_kernel(k_score_rows, dim3((g.m + kBM - 1) / kBM * 4), dim3(kRowWarps * 32), 0, st, true,
+                                        g, parts, reinterpret_cast<float4 *>(stats), h2, s);
   return err == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 

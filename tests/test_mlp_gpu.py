@@ -326,3 +326,27 @@ def test_project_kept_of_an_image_past_the_gather_limit():
     zd, err_d = altr.project(x[idx.long()].contiguous(), w, act="none")
     torch.cuda.synchronize()
     assert err.item() == 0 and err_d.item() == 0 and torch.equal(z.view(torch.int16), zd.view(torch.int16))
+
+
+@pytest.mark.parametrize("t,d,dh", [(2048, 1024, 4096), (192, 1024, 256), (1, 272, 512)])
+def test_mlp_score_with_a_smaller_workspace(t, d, dh):
+    # what 256-column tiles need, less than the layout chosen otherwise, is
+    # enough; a block fewer is refused
+    altr = _alt()
+    xp, w1, w2, b1, b2, r = _inputs(t, d, dh, seed=4)
+    m = altr.Mlp(t, w1, w2, b1, b2, act="gelu", scores=True)
+    m.run(xp, r)
+    least = -(-t // 128) * -(-d // 256) * 10240
+    assert m._ws_bytes > least
+    m._ws = torch.full((least + 4096,), 0xff, dtype=torch.uint8, device="cuda")
+    m._ws_bytes = least
+    o = m.run(xp, r)
+    v, mag = _gemm_ref(o.h, w2, b2)
+    _check_close(o.x_post, v, mag)
+    assert o.error.item() == 0 and bool((m._ws[least:] == 0xff).all())
+    st, h2, s = altr.score(o.x, xp, o.x_post)
+    assert torch.allclose(o.stats[:, :4], st[:, :4], rtol=2.0 ** -21, atol=0)
+    assert torch.allclose(o.h2, h2, rtol=1e-5, atol=2e-6) and torch.allclose(o.s, s, rtol=0, atol=1e-5)
+    m._ws_bytes = least - 256
+    with pytest.raises(Exception, match="tr_mlp_score"):
+        m.run(xp, r)
