@@ -1,9 +1,13 @@
-// The selection kernels: a CTA runs select_image (Algorithm 1, see
-// tr_select_dev.cuh) on statistics left by the scoring kernel, one image at
-// a time (k_select: one image per CTA, or several in turn when the launch
-// caps the grid, as the pipeline does).
+// The selection kernels (Algorithm 1) on statistics left by the scoring kernel:
+// k_select runs one CTA per image (or several images in turn when the launch
+// caps the grid, as the pipeline does), by the fast path of
+// tr_select_cluster.cuh up to kSoloMaxN tokens and by select_image
+// (tr_select_dev.cuh) above and for what that path leaves open;
+// k_select_cluster shares each image among the CTAs of a cluster
+// (select_cluster_ctas: large images of small batches).
 //
-// k_select_gather (tr_reduce on uniform batches) also copies the kept rows.
+// k_select_gather (tr_reduce on uniform batches that take no clusters) also
+// copies the kept rows.
 // With fewer images than SMs it runs R replica CTAs per image: each makes
 // the same deterministic selection (only replica 0 writes idx and the status
 // words) and copies its 1/R share of the image's kept rows, so the copies of
@@ -96,9 +100,9 @@ __global__ void __launch_bounds__(kSelectThreads, 1)
 }
 
 // Per device (index & 63): dynamic shared memory limit already raised (bit 0
-// k_select, bit 1 k_select_gather, bit 2 k_select_cluster), and the SM count.  Atomic so that first
-// calls from several host threads are well defined (raising the limit twice
-// is harmless).
+// k_select, bit 1 k_select_gather, bit 2 k_select_cluster), and the SM count.
+// Atomic so that first calls from several host threads are well defined
+// (raising the limit twice is harmless).
 std::atomic<int> g_smem_set[64];
 std::atomic<int> g_sms[64];
 
