@@ -473,8 +473,9 @@ __device__ __forceinline__ void publish_rows(float *dst, const Acc2 &acc2) {
 
 // The rows' records from the partial sums the score GEMM left: a CTA per 32
 // rows, warp w of its kRowWarps merging parts w, w + kRowWarps, ... in turn
-// and warp 0 then the warps' sums, so that the record does not depend on
-// which CTA made which part; four parts' loads are in flight at a time (one
+// and a warp for each of the five sums then the warps' (one warp for all five:
+// passes of 576 rows 32.06 us against 31.78), so that the record does not
+// depend on which CTA made which part; four parts' loads are in flight at a time (one
 // warp walking all parts with its loads one part ahead of their use took 19 us on
 // 36,864 rows and 34 us on 576 rows of a split GEMM).  A kernel of its own,
 // begun while the GEMM drains: arrival counters inside the GEMM cost each
@@ -520,13 +521,23 @@ __global__ void __launch_bounds__(kRowWarps * 32) k_score_rows(const GemmArgs g,
 #pragma unroll
   for (int j = 0; j < kPartWords; ++j) sh[warp][j][lane] = vals[j];
   __syncthreads();
-  if (warp) return;
-  for (int w = 1; w < kRowWarps; ++w) {
-    float v[kPartWords];
+  if (warp < kPartWords / 2) {  // sum number `warp` of the five, over the warps
+    DF v{sh[0][2 * warp][lane], sh[0][2 * warp + 1][lane]};
 #pragma unroll
-    for (int j = 0; j < kPartWords; ++j) v[j] = sh[w][j][lane];
-    merge_part(tot, v);
+    for (int w = 1; w < kRowWarps; ++w) df_merge(v, sh[w][2 * warp][lane], sh[w][2 * warp + 1][lane]);
+    if (warp) {
+      sh[0][2 * warp][lane] = v.hi;  // read by this warp alone until here
+      sh[0][2 * warp + 1][lane] = v.lo;
+    } else {
+      tot.l1 = v;
+    }
   }
+  __syncthreads();
+  if (warp) return;
+  tot.s2 = DF{sh[0][2][lane], sh[0][3][lane]};
+  tot.a = DF{sh[0][4][lane], sh[0][5][lane]};
+  tot.b = DF{sh[0][6][lane], sh[0][7][lane]};
+  tot.p = DF{sh[0][8][lane], sh[0][9][lane]};
   const long long row = (long long)rb * kBM + 32 * q + lane;
   if (row < g.m) write_record(tot, row, stats, h2, s_out);
 }
