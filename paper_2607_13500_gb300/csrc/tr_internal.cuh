@@ -134,7 +134,8 @@ inline Bounds certification_bounds(int d, int dtype) {
   // elements per chunk, doubled for fp32, whose squares and products enter as
   // TwoProd pairs) into a double-float by TwoSum, so hi + (the exact errors)
   // is the exact partial sum and only the low part's additions round: at most
-  // k^2 u^2 of the sum of |terms| T.  Merging two partials (TwoSum of the high
+  // k^2 u^2 of the sum of |terms| T (it keeps two such sums of k / 2 terms and
+  // merges them: k^2 / 4 + k + 1, less).  Merging two partials (TwoSum of the high
   // parts, two low-part additions) rounds by at most (2 j + 1) u^2 T at a
   // merge whose inputs carry low parts below j u T: the five shuffle levels
   // inside a warp add at most (10 k + 35) u^2 T, and merging at most 16 warp

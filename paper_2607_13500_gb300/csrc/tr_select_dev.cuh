@@ -638,45 +638,88 @@ __device__ __forceinline__ void exact_row_any(const SelectArgs &a, long long row
 // Runs longer than this skip the tier: long runs are exact ties in practice.
 constexpr int kDfRunMax = 32;
 
-// The elements of one 32-bit word as fp32 (exact for all three types; one
-// element for fp32, two otherwise).
+// The first two elements of a chunk as fp32 (exact for all three types), and
+// the chunk without them.
 template <int kDt>
-__device__ __forceinline__ void unpack_word(uint32_t w, float (&out)[2]) {
-  if (kDt == TR_BF16) {
-    out[0] = __uint_as_float(w << 16);
-    out[1] = __uint_as_float(w & 0xffff0000u);
-  } else if (kDt == TR_F16) {
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const uint32_t h = (w >> (16 * i)) & 0xffffu;
-      const uint32_t sg = (h & 0x8000u) << 16, ex = (h >> 10) & 0x1fu, mant = h & 0x3ffu;
-      float f;
-      if (ex == 0x1fu)
-        f = __uint_as_float(sg | 0x7f800000u | (mant << 13));
-      else if (ex == 0u)
-        f = __uint_as_float(sg | __float_as_uint(__uint2float_rn(mant) * 0x1p-24f));
-      else
-        f = __uint_as_float(sg | ((ex + 112u) << 23) | (mant << 13));
-      out[i] = f;
+__device__ __forceinline__ float2 first_pair(const uint4 &u) {
+  if (kDt == TR_BF16) return make_float2(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u));
+  if (kDt == TR_F32) return make_float2(__uint_as_float(u.x), __uint_as_float(u.y));
+  float2 v;
+  asm("{\n .reg .f16 l, h;\n mov.b32 {l, h}, %2;\n cvt.f32.f16 %0, l;\n cvt.f32.f16 %1, h;\n}"
+      : "=f"(v.x), "=f"(v.y)
+      : "r"(u.x));
+  return v;
+}
+template <int kDt>
+__device__ __forceinline__ uint4 after_pair(const uint4 &u) {
+  return kDt == TR_F32 ? make_uint4(u.z, u.w, 0u, 0u) : make_uint4(u.y, u.z, u.w, 0u);
+}
+
+// Whether all values seen are ones whose squares (and whose products with
+// other such values) are exact normal fp32 numbers or zero: 0, or 2^-50 <= |v|
+// <= 2^50.  Kept on the bit patterns, two 16-bit values at a time: with the
+// sign bit set and 1 taken away, zero becomes the largest signed value and
+// every other one, by magnitude, a negative one, so the signed minimum is the
+// least non-zero magnitude and the unsigned maximum the greatest (a
+// non-finite value lies above the limit).
+template <int kDt>
+struct ValueRange {
+  static constexpr uint32_t kSign = kDt == TR_F32 ? 0x80000000u : 0x80008000u;
+  static constexpr uint32_t kOne = kDt == TR_F32 ? 1u : 0x00010001u;
+  uint32_t least = kSign - kOne, most = kSign - kOne;  // as after a zero
+  __device__ __forceinline__ void add_word(uint32_t w) {
+    const uint32_t t = (w | kSign) - kOne;
+    if (kDt == TR_F32) {
+      least = (uint32_t)min((int)least, (int)t);
+      most = max(most, t);
+    } else {
+      asm("min.s16x2 %0, %0, %1;" : "+r"(least) : "r"(t));
+      asm("max.u16x2 %0, %0, %1;" : "+r"(most) : "r"(t));
     }
-  } else {
-    out[0] = __uint_as_float(w);
-    out[1] = 0.f;
   }
-}
+  __device__ __forceinline__ void add_pair(const uint4 &u) {
+    add_word(u.x);
+    if (kDt == TR_F32) add_word(u.y);
+  }
+  __device__ __forceinline__ bool ok() const {
+    if (kDt == TR_F32)  // 2^-50 and 2^50
+      return (int)least >= (int)(kSign + (77u << 23) - 1u) && most <= kSign + (177u << 23) - 1u;
+    // fp16: any finite value (0x7bff is the greatest)
+    const uint32_t lo = kDt == TR_BF16 ? 77u << 7 : 1u, hi = kDt == TR_BF16 ? 177u << 7 : 0x7bffu;
+    bool fine = true;
+#pragma unroll
+    for (int i = 0; i < 32; i += 16)
+      fine &= (int16_t)(least >> i) >= (int16_t)(0x8000u + lo - 1u) && (uint16_t)(most >> i) <= 0x8000u + hi - 1u;
+    return fine;
+  }
+};
 
-// A value whose square (and whose products with other such values) is an
-// exact normal fp32 number or zero: 0, or 2^-50 <= |v| <= 2^50.
-__device__ __forceinline__ bool df_value_ok(float v) {
-  const float m = fabsf(v);
-  return m == 0.f || (m >= 0x1p-50f && m <= 0x1p+50f);
+// A pair of double-floats, one per component: hi + lo += t, or += u v, with hi
+// + (exact errors) the exact running sum (Knuth's TwoSum; nb = hi - s).
+struct DfPair {
+  float2 hi{0.f, 0.f}, lo{0.f, 0.f};
+};
+__device__ __forceinline__ float2 pair_sub(float2 a, float2 b) {  // a - b, one rounding
+  return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
 }
-
-// hi + lo += t with hi + (exact errors) the exact running sum.
-__device__ __forceinline__ void df_term(float &hi, float &lo, float t) {
-  const df::F2 r = df::two_sum(hi, t);
-  hi = r.h;
-  lo = __fadd_rn(lo, r.l);
+__device__ __forceinline__ void df_term(DfPair &a, float2 t) {
+  const float2 s = __fadd2_rn(a.hi, t);
+  const float2 nb = pair_sub(a.hi, s);
+  a.lo = __fadd2_rn(a.lo, __fadd2_rn(pair_sub(a.hi, __fadd2_rn(s, nb)), __fadd2_rn(t, nb)));
+  a.hi = s;
+}
+template <int kDt>
+__device__ __forceinline__ void df_product(DfPair &a, float2 u, float2 v) {
+  if (kDt == TR_F32) {  // a TwoProd pair
+    const float2 t = __fmul2_rn(u, v);
+    df_term(a, t);
+    a.lo = __fadd2_rn(a.lo, __ffma2_rn(u, v, make_float2(-t.x, -t.y)));
+  } else {  // exact: the fused operations round as the ones on the product would
+    const float2 s = __ffma2_rn(u, v, a.hi);
+    const float2 nb = pair_sub(a.hi, s);
+    a.lo = __fadd2_rn(a.lo, __fadd2_rn(pair_sub(a.hi, __fadd2_rn(s, nb)), __ffma2_rn(u, v, nb)));
+    a.hi = s;
+  }
 }
 __device__ __forceinline__ void df_join(float &hi, float &lo, float h2, float l2) {
   const df::F2 r = df::two_sum(hi, h2);
@@ -697,15 +740,18 @@ struct PartDf {
 // and for a few rows, so fetching the instructions is a good part of what it
 // costs.  (With two chunks' elements unrolled, settling the pick runs of a
 // 6272-token clip took 9.8 us of its selection's 29.5; with two elements per
-// iteration 8.9.)
+// iteration 8.9.)  The two go through packed fp32 instructions, about half as
+// many as one after the other: reductions of 4 x 2880 fp16 tokens 74.52 ->
+// 74.07 us, of 12 ragged images 424.4 -> 422.6; more chunks in flight (four)
+// were no faster.
 template <int kDt>
 __device__ __noinline__ bool df_row_block(const SelectArgs &a, long long row, int mode, ExactRec *rec, PartDf &part,
                                           const Group g) {
   constexpr int kPer = kDt == TR_F32 ? 4 : 8;  // elements per 16-byte chunk
   const int nchunks = a.d / kPer;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  bool ok = true;
-  float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
+  ValueRange<kDt> range;
+  DfPair s0, s1, s2;
   const uint4 *p0 = static_cast<const uint4 *>(mode == 0 ? a.x : (a.x_pre ? a.x_pre : a.x)) + row * nchunks;
   const uint4 *p1 = mode == 0 ? p0 : static_cast<const uint4 *>(a.x_post) + row * nchunks;
   uint4 n0 = make_uint4(0u, 0u, 0u, 0u), n1 = n0;
@@ -721,35 +767,27 @@ __device__ __noinline__ bool df_row_block(const SelectArgs &a, long long row, in
       n1 = __ldg(p1 + c + g.size);
     }
 #pragma unroll 1
-    for (int w = 0; w < 4; ++w) {
-      float v0[2], v1[2];
-      unpack_word<kDt>(u0.x, v0);
-      unpack_word<kDt>(u1.x, v1);
-#pragma unroll
-      for (int i = 0; i < (kDt == TR_F32 ? 1 : 2); ++i) {
-        const float p = v0[i], q = v1[i];  // mode 0: both x
-        ok &= df_value_ok(p) && df_value_ok(q);
-        // the terms |x|, x^2 (mode 0) or x'^2, x''^2, x'x'', products exact
-        // (fp32: as TwoProd pairs)
-        const df::F2 pp = kDt == TR_F32 ? df::two_prod(p, p) : df::F2{__fmul_rn(p, p), 0.f};
-        const df::F2 qq = kDt == TR_F32 ? df::two_prod(q, q) : df::F2{__fmul_rn(q, q), 0.f};
-        df_term(h0, l0, mode == 0 ? fabsf(p) : pp.h);
-        df_term(h1, l1, qq.h);
-        if (kDt == TR_F32) {
-          if (mode != 0) l0 = __fadd_rn(l0, pp.l);
-          l1 = __fadd_rn(l1, qq.l);
-        }
-        if (mode != 0) {
-          const df::F2 pq = kDt == TR_F32 ? df::two_prod(p, q) : df::F2{__fmul_rn(p, q), 0.f};
-          df_term(h2, l2, pq.h);
-          if (kDt == TR_F32) l2 = __fadd_rn(l2, pq.l);
-        }
+    for (int w = 0; w < kPer / 2; ++w) {
+      const float2 p = first_pair<kDt>(u0), q = first_pair<kDt>(u1);  // mode 0: both x
+      range.add_pair(u0);
+      range.add_pair(u1);
+      // the terms |x|, x^2 (mode 0) or x'^2, x''^2, x'x''
+      df_product<kDt>(s1, q, q);
+      if (mode == 0) {
+        df_term(s0, make_float2(fabsf(p.x), fabsf(p.y)));
+      } else {
+        df_product<kDt>(s0, p, p);
+        df_product<kDt>(s2, p, q);
       }
-      u0 = make_uint4(u0.y, u0.z, u0.w, 0u);  // the next word
-      u1 = make_uint4(u1.y, u1.z, u1.w, 0u);
+      u0 = after_pair<kDt>(u0);
+      u1 = after_pair<kDt>(u1);
     }
   }
-  if (!g.all(ok)) return false;
+  if (!g.all(range.ok())) return false;
+  float h0 = s0.hi.x, l0 = s0.lo.x, h1 = s1.hi.x, l1 = s1.lo.x, h2 = s2.hi.x, l2 = s2.lo.x;
+  df_join(h0, l0, s0.hi.y, s0.lo.y);
+  df_join(h1, l1, s1.hi.y, s1.lo.y);
+  df_join(h2, l2, s2.hi.y, s2.lo.y);
 #pragma unroll 1
   for (int o = 16; o > 0; o >>= 1) {
     df_join(h0, l0, __shfl_xor_sync(0xffffffffu, h0, o), __shfl_xor_sync(0xffffffffu, l0, o));
