@@ -134,3 +134,22 @@ def test_left_to_select_image(n):
     run(equal)
     run(crowded)
     run(outside, expect_nonfinite=True)
+
+
+@pytest.mark.parametrize("edge,exact", [(2.0 ** -50, False), (2.0 ** -51, True)], ids=["least", "below"])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16, torch.float32], ids=["bf16", "f16", "f32"])
+def test_near_ties_at_the_value_range(dtype, edge, exact):
+    # the double-float keys take rows of zeros and of values down to 2^-50,
+    # and leave rows with a smaller one to exact sums; fp16's least value is
+    # inside.  129 (bf16, fp16) or 258 chunks a row: partial rounds of a warp
+    # group.
+    if dtype == torch.float16:
+        edge, exact = 2.0 ** -24, False
+    x, xp, xq, *_ = _near_tie_triples(32, 1032, dtype, 8)
+    for col, v in ((100, edge), (101, -edge), (102, 0.0), (103, -0.0), (1031, edge)):
+        for t in (x, xp, xq):
+            t[:, col] = v
+    n = x.shape[0]
+    for k, k1 in [(40, 31), (60, 0), (45, 16)]:
+        st = check_reduce(x, xp, xq, [n], _budget([k], [k1]))
+        assert (st[2] > 0) == exact, st
