@@ -475,9 +475,10 @@ __device__ __forceinline__ void publish_rows(float *dst, const Acc2 &acc2) {
 // rows, warp w of its kRowWarps merging parts w, w + kRowWarps, ... in turn
 // and a warp for each of the five sums then the warps' (one warp for all five:
 // passes of 576 rows 32.06 us against 31.78), so that the record does not
-// depend on which CTA made which part; four parts' loads are in flight at a time (one
-// warp walking all parts with its loads one part ahead of their use took 19 us on
-// 36,864 rows and 34 us on 576 rows of a split GEMM).  A kernel of its own,
+// depend on which CTA made which part; four parts' loads are in flight at a
+// time (one warp walking all parts with its loads one part ahead of their use
+// took 19 us on 36,864 rows and 34 us on 576 rows of a split GEMM).  A kernel of
+// its own,
 // begun while the GEMM drains: arrival counters inside the GEMM cost each
 // tile a fence over its stores, an atomic and, for the last warp, this same
 // merge in series (about 5,000 clocks a tile, and a memset before every
@@ -861,11 +862,10 @@ EncodeTiled encode_fn() {
   return fn;
 }
 
-// Row-major bf16 [rows, cols] read in boxes of box_rows x 64 columns with the
-// 128-byte swizzle; out-of-range rows and columns read as zeros.
 // A bf16 [rows, cols] row-major tensor in boxes of box_rows x box_cols
 // (box_cols x 2 bytes = the swizzle span: 64 columns with the 128-byte
-// swizzle for operands, 32 with the 64-byte swizzle for the output staging).
+// swizzle for operands, 32 with the 64-byte swizzle for the output staging);
+// out-of-range rows and columns read as zeros.
 bool make_map(CUtensorMap *map, const void *base, long long rows, long long cols, int box_rows, int box_cols = kBK,
               CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
   EncodeTiled fn = encode_fn();
