@@ -478,10 +478,9 @@ __device__ __forceinline__ void publish_rows(float *dst, const Acc2 &acc2) {
 // depend on which CTA made which part; four parts' loads are in flight at a
 // time (one warp walking all parts with its loads one part ahead of their use
 // took 19 us on 36,864 rows and 34 us on 576 rows of a split GEMM).  A kernel of
-// its own,
-// begun while the GEMM drains: arrival counters inside the GEMM cost each
-// tile a fence over its stores, an atomic and, for the last warp, this same
-// merge in series (about 5,000 clocks a tile, and a memset before every
+// its own, begun while the GEMM drains: arrival counters inside the GEMM cost
+// each tile a fence over its stores, an atomic and, for the last warp, this
+// same merge in series (about 5,000 clocks a tile, and a memset before every
 // launch).
 constexpr int kRowWarps = 8;
 __device__ __forceinline__ void merge_part(Acc &tot, const float (&w)[kPartWords]) {
