@@ -349,14 +349,18 @@ typedef struct {
   int32_t act;         /* sigma: TR_ACT_GELU, TR_ACT_QUICK_GELU or TR_ACT_NONE          */
 } tr_mlp;
 
-/* H = sigma(x' W1^T + b1): h is device bf16 [t, d_hidden]. */
+/*
+ * H = sigma(x' W1^T + b1): h is device bf16 [t, d_hidden].  K is summed in one
+ * order whatever t: a row's H, and in tr_mlp_score its x'' and x, are the same
+ * bit for bit alone and in any batch.
+ */
 tr_status tr_mlp_hidden(const tr_mlp *m, void *h, int32_t *d_error, void *stream);
 
 /*
  * Scratch bytes of tr_mlp_score (256-byte aligned device memory); 0 on invalid
  * input.  A call given fewer (scratch sized for a larger t, whose GEMM is laid
  * out differently) still runs, in 256-column tiles, from 10 KiB per 128 rows
- * and 256 channels (begun ones counted whole) on.
+ * and 256 channels (begun ones counted whole) on, with the same x'' and x.
  */
 size_t tr_mlp_workspace_bytes(const tr_mlp *m);
 
@@ -364,7 +368,11 @@ size_t tr_mlp_workspace_bytes(const tr_mlp *m);
  * x'' = H W2^T + b2 and x = resid + x'' (both stored, bf16 [t, d]) with the
  * scoring of every row in the same pass: stats is device fp32
  * [t, TR_STATS_WORDS] laid out as in tr_score, h2 / s optional fp32 [t].
- * x_post and x must not overlap the inputs.
+ * x_post and x must not overlap the inputs.  The records' double-float sums
+ * are grouped by the GEMM's tile columns, which follow t and the scratch: from
+ * one t to another they agree to within the certified bound (about 2^-34 of
+ * the sums of |terms|), so an fp32 rounding may differ in its last bit; the
+ * selection, exact on the stored tensors, does not.
  */
 tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, float *stats, float *h2, float *s,
                        void *ws, size_t ws_bytes, int32_t *d_error, void *stream);

@@ -13,24 +13,24 @@
 //
 // One kernel serves both GEMMs (C[m, n] = A[m, k] B[n, k]^T, bf16 operands,
 // fp32 accumulation): a persistent grid of one CTA per SM, in pairs, walks
-// 256 x 256 output tiles (tile t: row block t / n_tiles, column block
-// t % n_tiles, so the pairs running at one time share row blocks of A in
-// L2).  Per CTA:
+// output tiles of 256 rows x bn columns, bn 64 to 256 by size (gemm_shape;
+// tile t: row block t / n_tiles, column block t % n_tiles, so the pairs
+// running at one time share row blocks of A in L2).  Per CTA:
 //   warp 0      TMA producer: A and B k-blocks (64 wide, 128-byte swizzle)
 //               into a 6-stage shared-memory ring;
-//   warp 1      allocates 512 TMEM columns (two 128 x 256 fp32
-//               accumulators); in the pair's even CTA it issues tcgen05.mma
-//               (M 256, N 256, K 16) from one thread, committing each stage
-//               back to the producers and each finished accumulator to the
-//               epilogues;
+//   warp 1      allocates 512 TMEM columns (two fp32 accumulators of 128 rows
+//               and up to 256 columns); in the pair's even CTA it issues
+//               tcgen05.mma (M 256, N bn, K 16) from one thread, committing
+//               each stage back to the producers and each finished
+//               accumulator to the epilogues;
 //   warps 2-    epilogue: one thread per accumulator row (TMEM lane: a
-//               warp reads the lane quarter warp % 4); the tile's eight
-//               32-column blocks are dealt to the two or four warps of each
-//               quarter in turn.  Outputs leave through TMA stores of 32 x 32 blocks
-//               staged in shared memory; the score mode's x' and residual
-//               come in the same way.
-// When the tiles are few, clusters of two or four pairs share each tile's K
-// range and exchange the partial accumulators (kSplit, see below).
+//               warp reads the lane quarter warp % 4); the tile's bn / 32
+//               blocks of 32 columns are dealt to the two or four warps of
+//               each quarter in turn.  Outputs leave through TMA stores of
+//               32 x 32 blocks staged in shared memory; the score mode's x'
+//               and residual come in the same way.
+// K is summed in one order whatever the number of rows, the tile width and the
+// mode, so a row's outputs do not depend on the batch it is in.
 // The projector mode (tr_project_kept) is the hidden GEMM with its A rows
 // gathered: A row j is token idx[j] of the image that owns kept slot j, so
 // the first projector layer reads X* = X_imp union X_div (Eq. 7) straight
@@ -62,21 +62,18 @@ namespace {
 
 constexpr int kBM = 128, kBN = 256, kBK = 64;  // a CTA's rows, a tile's columns at most, a k-block
 enum { kModeHidden = 0, kModeScore = 1, kModeProject = 2 };
-// Epilogue warps per mode: four per lane quarter where the epilogue is on the
-// critical path (the hidden GEMM, whose main loop is short, and split tiles),
-// so that they hide the latencies of one another's TMEM loads and arithmetic;
-// two for the score GEMM's unsplit tiles (64 images x 576 tokens, D 1024,
-// hidden 4096, both GEMMs: 437 us, with four 446 us -- the main loop covers
-// this epilogue, and the staging it saves is a sixth operand stage) and for
-// the projector, whose threads include its row loaders.
-__host__ __device__ constexpr int epi_warps(int mode, int split) {
-  return mode == kModeHidden || (mode == kModeScore && split > 1) ? 16 : 8;
-}
-__host__ __device__ constexpr int epi_parts(int mode, int split) { return epi_warps(mode, split) / 4; }
+// Epilogue warps per mode: four per lane quarter for the hidden GEMM, whose
+// main loop is short, so that they hide the latencies of one another's TMEM
+// loads and arithmetic; two for the score GEMM (64 images x 576 tokens, D
+// 1024, hidden 4096, both GEMMs: 437 us, with four 446 us -- the main loop
+// covers this epilogue, and the staging it saves is a sixth operand stage) and
+// for the projector, whose threads include its row loaders.
+__host__ __device__ constexpr int epi_warps(int mode) { return mode == kModeHidden ? 16 : 8; }
+__host__ __device__ constexpr int epi_parts(int mode) { return epi_warps(mode) / 4; }
 // producer, MMA issuer, epilogue (+ the A-row loader warps of the projector mode)
 constexpr int kLoadWarps = 4;  // projector: loader warps, 32 of a CTA's 128 rows each
-__host__ __device__ constexpr int gemm_threads(int mode, int split) {
-  return 64 + 32 * epi_warps(mode, split) + (mode == kModeProject ? 32 * kLoadWarps : 0);
+__host__ __device__ constexpr int gemm_threads(int mode) {
+  return 64 + 32 * epi_warps(mode) + (mode == kModeProject ? 32 * kLoadWarps : 0);
 }
 constexpr int kTmemCols = 2 * kBN;                // two accumulators
 constexpr int kPartWords = 10;                    // hi, lo of L1, S2, A, B, P
@@ -91,17 +88,9 @@ constexpr int kBlkBytes = 32 * kBlk * 2;
 // ahead of their use and overwritten in place by x'' and x.
 __host__ __device__ constexpr int stage_blks(int mode) { return mode == kModeHidden ? 1 : 2; }
 __host__ __device__ constexpr int stage_bytes(int mode) { return stage_blks(mode) * kBlkBytes; }
-// Splits of K over the pairs of a cluster: pair p of kSplit sums its k-blocks
-// into its own accumulators and finishes the tile's blocks [p, p + 1) * own,
-// own = tile blocks / kSplit, whose partial sums the other pairs send it.
-// The score mode's partial row sums per tile and lane quarter: one for each
-// warp that has blocks.
-__host__ __device__ constexpr int active_parts(int own, int split) {
-  return own < epi_parts(kModeScore, split) ? own : epi_parts(kModeScore, split);
-}
-__host__ __device__ constexpr int row_parts(int bn, int split) {
-  return split * active_parts(bn / kBlk / split, split);
-}
+// The score mode's partial row sums per tile and lane quarter: one for each of
+// its warps (a tile has at least as many blocks).
+constexpr int kRowParts = epi_parts(kModeScore);
 
 struct GemmArgs {
   int m, n, k;          // C[m, n] = A[m, k] B[n, k]^T
@@ -110,7 +99,7 @@ struct GemmArgs {
   const float *bias;    // [n] or NULL
   int act;              // hidden GEMM: TR_ACT_*
   bool has_resid;       // score: x = x'' + residual
-  float *part;          // score: [row blocks][n_tiles][row parts][4][kPartWords][32] partial sums
+  float *part;          // score: [row blocks][n_tiles][kRowParts][4][kPartWords][32] partial sums
   int32_t *err;         // optional: set when a pipeline wait timed out
   // projector mode: A row j = x[first row of the image owning kept slot j + idx[j]]
   long long total_rows;
@@ -299,7 +288,7 @@ __device__ __forceinline__ void epi_score(const GemmArgs &g, int col0, const uin
 // One epilogue warp's place: its lane quarter, its blocks of a tile (first,
 // first + parts, ... below end) and its staging.
 struct EpiWarp {
-  int first, end;      // blocks of a tile (end: past the blocks this CTA finishes)
+  int first, end;      // blocks of a tile
   uint32_t buf, bar;   // staging, and the score mode's mbarrier of its loads
   uint32_t loads;      // score: blocks requested so far
   uint32_t used;       // score: blocks waited for so far
@@ -331,36 +320,6 @@ __device__ __forceinline__ void score_load_next(const GemmArgs &g, const GemmMap
   w.blk += kParts;
 }
 
-// The partial sums of the other pairs for 8 columns are added to this pair's
-// (v), in the order of the pairs whatever pair this is, so that the result
-// does not depend on which pair owns the block.  slots: received partials,
-// [other pair][four-column unit of the owned columns][128 rows].
-template <int kSplit>
-__device__ __forceinline__ void add_partials(uint32_t slots, uint32_t slot_bytes, int pair, int unit, int row,
-                                             uint32_t (&v)[8]) {
-  float sum[8];
-#pragma unroll
-  for (int o = 0; o < kSplit; ++o) {
-    float t[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) t[i] = __uint_as_float(v[i]);
-    if (o != pair) {
-      const uint32_t src = slots + (uint32_t)(o < pair ? o : o - 1) * slot_bytes + (uint32_t)(unit * 128 + row) * 16u;
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        uint32_t r[4];
-        tc::ld_shared_v4(src + (uint32_t)u * 2048u, r[0], r[1], r[2], r[3]);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) t[4 * u + i] = __uint_as_float(r[i]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) sum[i] = o == 0 ? t[i] : __fadd_rn(sum[i], t[i]);
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __float_as_uint(sum[i]);
-}
-
 // The epilogue of one tile for this warp: for each of its blocks, the
 // accumulator columns from TMEM, the mode's arithmetic into the staged block
 // and the TMA store(s).  Rows and columns past the output are computed from
@@ -368,15 +327,13 @@ __device__ __forceinline__ void add_partials(uint32_t slots, uint32_t slot_bytes
 // timed out.  (Score: with x' and the residual loaded straight from global
 // memory, 32 rows per warp load and one chunk ahead, a tile's epilogue took
 // 24,000-33,000 clocks.)
-template <int kMode, int kSplit, typename RowOf>
+template <int kMode, typename RowOf>
 __device__ __forceinline__ bool epilogue_tile(const GemmArgs &g, const GemmMaps &maps, EpiWarp &w, uint32_t taddr,
-                                              int nt, int row0, int step, RowOf row_of, uint32_t slots, int pair,
-                                              int row_in_tile, Acc2 &acc2) {
-  constexpr int kParts = epi_parts(kMode, kSplit);
-  constexpr int kUnits = kMode == kModeScore && kSplit > 1 ? 1 : 2;  // 8-column units in flight
+                                              int nt, int row0, int step, RowOf row_of, Acc2 &acc2) {
+  constexpr int kParts = epi_parts(kMode);
+  constexpr int kUnits = 2;  // 8-column units in flight
   const int lane = threadIdx.x & 31;
   const uint32_t sw = (uint32_t)((lane >> 1) & 3);  // the 64-byte swizzle's row term
-  const int own = g.bn / kBlk / kSplit;             // blocks that each pair finishes
   for (int blk = w.first; blk < w.end; blk += kParts) {
     const int col = nt * g.bn + blk * kBlk;
     if (col >= g.n) break;
@@ -401,9 +358,6 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs &g, const GemmMaps 
 #pragma unroll
       for (int i = 0; i < kUnits; ++i) {
         const int u = u0 + i;
-        if (kSplit > 1)
-          add_partials<kSplit>(slots, 512u * (uint32_t)(own * kBlk), pair, (blk - pair * own) * 8 + 2 * u, row_in_tile,
-                               v[i]);
         const uint32_t addr = rowbuf + (((uint32_t)u ^ sw) << 4);
         if (kMode == kModeScore)
           epi_score(g, col + 8 * u, v[i], addr, acc2);
@@ -429,34 +383,10 @@ __device__ __forceinline__ bool epilogue_tile(const GemmArgs &g, const GemmMaps 
   return true;
 }
 
-// Split tiles: this pair's partial sums of the blocks the other pairs finish
-// go to them (16-byte stores into the owner's shared memory, whose operand
-// ring is idle by then; 32 lanes write 512 consecutive bytes).
-template <int kMode, int kSplit>
-__device__ __forceinline__ void send_partials(const GemmArgs &g, uint32_t slots, uint32_t taddr, int pair,
-                                              uint32_t rank, int part, int row_in_tile) {
-  const int own = g.bn / kBlk / kSplit;
-  for (int blk = part; blk < g.bn / kBlk; blk += epi_parts(kMode, kSplit)) {
-    const int owner = blk / own;
-    if (owner == pair) continue;
-    const uint32_t dst =
-        tc::map_shared(slots + (uint32_t)(pair < owner ? pair : pair - 1) * 512u * (uint32_t)(own * kBlk) +
-                           (uint32_t)((blk - owner * own) * 8 * 128 + row_in_tile) * 16u,
-                       2u * (uint32_t)owner + (rank & 1u));
-#pragma unroll 1
-    for (int u = 0; u < kBlk / 8; ++u) {
-      uint32_t v[8];
-      tc::tmem_ld8(taddr + (uint32_t)(blk * kBlk + 8 * u), v);
-      tc::st_cluster_v4(dst + (uint32_t)(2 * u) * 2048u, v[0], v[1], v[2], v[3]);
-      tc::st_cluster_v4(dst + (uint32_t)(2 * u + 1) * 2048u, v[4], v[5], v[6], v[7]);
-    }
-  }
-}
-
 // This warp's 32 rows are done for its blocks of a tile: their partial sums
 // go to the scratch; k_score_rows merges them once the GEMM has finished.
-__device__ __forceinline__ long long part_slot(const GemmArgs &g, int parts, int rb, int nt, int part, int q) {
-  return (((long long)(rb * g.n_tiles + nt) * parts + part) * 4 + q) * (kPartWords * 32);
+__device__ __forceinline__ long long part_slot(const GemmArgs &g, int rb, int nt, int part, int q) {
+  return (((long long)(rb * g.n_tiles + nt) * kRowParts + part) * 4 + q) * (kPartWords * 32);
 }
 __device__ __forceinline__ void publish_rows(float *dst, const Acc2 &acc2) {
   Acc acc{{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
@@ -477,7 +407,7 @@ __device__ __forceinline__ void publish_rows(float *dst, const Acc2 &acc2) {
 // passes of 576 rows 32.06 us against 31.78), so that the record does not
 // depend on which CTA made which part; four parts' loads are in flight at a
 // time (one warp walking all parts with its loads one part ahead of their use
-// took 19 us on 36,864 rows and 34 us on 576 rows of a split GEMM).  A kernel of
+// took 19 us on 36,864 rows).  A kernel of
 // its own, begun while the GEMM drains: arrival counters inside the GEMM cost
 // each tile a fence over its stores, an atomic and, for the last warp, this
 // same merge in series (about 5,000 clocks a tile, and a memset before every
@@ -490,15 +420,14 @@ __device__ __forceinline__ void merge_part(Acc &tot, const float (&w)[kPartWords
   df_merge(tot.b, w[6], w[7]);
   df_merge(tot.p, w[8], w[9]);
 }
-__global__ void __launch_bounds__(kRowWarps * 32) k_score_rows(const GemmArgs g, const int parts,
-                                                               float4 *__restrict__ stats, float *__restrict__ h2,
-                                                               float *__restrict__ s_out) {
+__global__ void __launch_bounds__(kRowWarps * 32) k_score_rows(const GemmArgs g, float4 *__restrict__ stats,
+                                                               float *__restrict__ h2, float *__restrict__ s_out) {
   __shared__ float sh[kRowWarps][kPartWords][32];
   pdl_trigger();
   pdl_wait();  // the partial sums come from the GEMM before this kernel
   const int rb = blockIdx.x >> 2, q = blockIdx.x & 3, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int total = parts * g.n_tiles;
-  const float *src = g.part + part_slot(g, parts, rb, 0, 0, q) + lane;
+  const int total = kRowParts * g.n_tiles;
+  const float *src = g.part + part_slot(g, rb, 0, 0, q) + lane;
   constexpr int kStep = 4 * kPartWords * 32;  // floats from one part to the next (the four quarters between)
   constexpr int kU = 4;
   Acc tot{{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
@@ -561,45 +490,37 @@ __device__ __forceinline__ long long kept_source_row(const GemmArgs &g, long lon
 }
 
 // ---------------------------------------------------------------- the SM-pair kernel
-// tcgen05's 2-SM MMA: a cluster of two CTAs shares each 256 x 256 output
-// tile (tile t: row block t / n_tiles of 256 rows).  CTA rank r loads A rows
-// 128 r .. 128 r + 127 of the tile and B rows (output columns) 128 r .. 128 r
-// + 127 into its own shared memory -- 32 KiB per k-block stage, six stages --
-// and both CTAs' loads complete on the even CTA's stage barrier.  The even
-// CTA alone issues the pair's MMAs (M 256, N 256, K 16), which read both
+// tcgen05's 2-SM MMA: a cluster of two CTAs shares each output tile of 256
+// rows x bn columns (tile t: row block t / n_tiles).  CTA rank r loads A rows
+// 128 r .. 128 r + 127 of the tile and its half of the tile's B rows (output
+// columns) into its own shared memory -- 32 KiB per k-block stage, six stages
+// -- and both CTAs' loads complete on the even CTA's stage barrier.  The even
+// CTA alone issues the pair's MMAs (M 256, N bn, K 16), which read both
 // CTAs' stages and write each CTA's 128 accumulator rows into its own TMEM;
 // its commits reach the same barriers in both CTAs (multicast).  Each CTA's
 // epilogue drains its own rows and releases the accumulator on the even
-// CTA's barrier.  Per SM a k-block brings 32 KiB of operands for a
-// 128 x 256 x 64 product, against 48 KiB on one SM.  A batch of at most 128
+// CTA's barrier.  Per SM a k-block of 256 columns brings 32 KiB of operands
+// for a 128 x 256 x 64 product, against 48 KiB on one SM.  A batch of at most 128
 // rows runs here too, the odd CTA's rows read as zeros: what such a batch
 // waits for is W, and a pair brings each half of it into its own SM (128 rows,
 // D 1024, hidden 4096, both GEMMs: 57.4 us with a one-SM kernel, 55.3 here).
-//
-// Splits: with few tiles most SMs would idle while a pair runs through all of
-// K, so a cluster of kSplit pairs shares a tile: pair p takes the k-blocks
-// [p, p + 1) * kblocks / kSplit, then the pairs exchange their partial sums
-// through distributed shared memory, each finishing 256 / kSplit of the
-// tile's columns.  One tile per cluster.
-// A split score GEMM gives one stage to its epilogue's staging.
-__host__ __device__ constexpr int gemm_stages(int mode, int split) { return mode == kModeScore && split > 1 ? 5 : 6; }
+constexpr int kStagesP = 6;
 constexpr int kHalfTile = 128 * kBK * 2;          // 128 rows of a k-block (A or B)
 constexpr int kStagePBytes = 2 * kHalfTile;       // this CTA's A rows + B rows
-__host__ __device__ constexpr int gemm_smem(int mode, int split) {  // + alignment, barriers
-  return gemm_stages(mode, split) * kStagePBytes + epi_warps(mode, split) * stage_bytes(mode) + 1024 + 512;
+__host__ __device__ constexpr int gemm_smem(int mode) {  // + alignment, barriers
+  return kStagesP * kStagePBytes + epi_warps(mode) * stage_bytes(mode) + 1024 + 512;
 }
 
-template <int kMode, int kSplit>
-__global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
+template <int kMode>
+__global__ void __launch_bounds__(gemm_threads(kMode), 1)
     k_mlp_gemm(const __grid_constant__ GemmMaps maps, const GemmArgs g) {
-  constexpr int kStagesP = gemm_stages(kMode, kSplit);
   pdl_trigger();
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                           ~static_cast<uintptr_t>(1023));
   const uint32_t out_stage = tc::smem_u32(smem + (size_t)kStagesP * kStagePBytes);  // epilogue staging
-  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)kStagesP * kStagePBytes + epi_warps(kMode, kSplit) * stage_bytes(kMode));
-  constexpr int kBlkBars = kMode == kModeScore ? epi_warps(kMode, kSplit) : 0;  // the score epilogue's staged blocks
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + (size_t)kStagesP * kStagePBytes + epi_warps(kMode) * stage_bytes(kMode));
+  constexpr int kBlkBars = kMode == kModeScore ? epi_warps(kMode) : 0;  // the score epilogue's staged blocks
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kStagesP + 5 + kBlkBars);
   const uint32_t sbase = tc::smem_u32(smem);
   const uint32_t b0 = tc::smem_u32(bars);
@@ -613,12 +534,9 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
   auto sb = [&](int s) { return sbase + (uint32_t)(s * kStagePBytes + kHalfTile); };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t crank = tc::cluster_rank();   // pair (split) crank / 2, CTA crank % 2 of it
-  const uint32_t rank = crank & 1u;
-  const int pair = kSplit > 1 ? (int)(crank >> 1) : 0;
+  const uint32_t rank = tc::cluster_rank();
   const bool leader = rank == 0;
-  const int cluster = blockIdx.x / (2 * kSplit), clusters = gridDim.x / (2 * kSplit);
-  const int kb_first = pair * g.kblocks / kSplit, kb_end = (pair + 1) * g.kblocks / kSplit;
+  const int pair = blockIdx.x / 2, pairs = gridDim.x / 2;
   // operand bytes landing on the even CTA's stage barrier per k-block (both CTAs)
   const uint32_t b_bytes = (uint32_t)g.bn * kBK * 2u;  // of B per k-block, both CTAs
   const uint32_t tx = b_bytes + (kMode == kModeProject ? 0u : 2u * kHalfTile);
@@ -630,7 +548,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
     }
     for (int a = 0; a < 2; ++a) {
       tc::mbar_init(tfull(a), 1);
-      tc::mbar_init(tempty(a), 2 * epi_warps(kMode, kSplit));  // one arrival per epilogue warp of either CTA
+      tc::mbar_init(tempty(a), 2 * epi_warps(kMode));  // one arrival per epilogue warp of either CTA
     }
     tc::mbar_init(done, 1);
     for (int i = 0; i < kBlkBars; ++i) tc::mbar_init(blk_bar(i), 1);
@@ -647,10 +565,9 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
   tc::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
   pdl_wait();  // operands come from, and outputs may still be read by, the kernels before this one
-  const uint32_t even = crank & ~1u;           // the pair's even CTA in the cluster
-  const uint16_t both = (uint16_t)(0x3u << even);
-  auto full_even = [&](int s) { return tc::map_shared(full(s), even); };
-  auto tempty_even = [&](int a) { return tc::map_shared(tempty(a), even); };
+  constexpr uint16_t both = 0x3;  // the CTAs that a commit reaches
+  auto full_even = [&](int s) { return tc::map_shared(full(s), 0u); };
+  auto tempty_even = [&](int a) { return tc::map_shared(tempty(a), 0u); };
   const int tiles = g.tiles;
 
   if (warp == 0) {
@@ -659,9 +576,9 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
       int stage = 0;
       uint32_t phase = 0, filled = 0, last_parity = 0;
       bool ok = true;
-      for (int tile = cluster; tile < tiles && ok; tile += clusters) {
+      for (int tile = pair; tile < tiles && ok; tile += pairs) {
         const int rb = tile / g.n_tiles, nt = tile - rb * g.n_tiles;
-        for (int kb = kb_first; kb < kb_end; ++kb) {
+        for (int kb = 0; kb < g.kblocks; ++kb) {
           if (!tc::mbar_wait(empty(stage), phase ^ 1u)) {
             ok = false;
             break;
@@ -693,14 +610,14 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
-      for (int tile = cluster; tile < tiles && ok; tile += clusters) {
+      for (int tile = pair; tile < tiles && ok; tile += pairs) {
         if (!tc::mbar_wait(tempty(acc), acc_phase ^ 1u)) {
           ok = false;
           break;
         }
         tc::fence_after_sync();
         const uint32_t d = tmem + (uint32_t)(acc * kBN);
-        for (int kb = kb_first; kb < kb_end; ++kb) {
+        for (int kb = 0; kb < g.kblocks; ++kb) {
           if (!tc::mbar_wait(full(stage), phase)) {
             ok = false;
             break;
@@ -709,7 +626,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
           const uint64_t da = tc::sw128_desc(sa(stage)), db = tc::sw128_desc(sb(stage));
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
-            tc::mma_bf16_pair(d, da + 2u * k, db + 2u * k, idesc, kb != kb_first || k != 0);
+            tc::mma_bf16_pair(d, da + 2u * k, db + 2u * k, idesc, (kb | k) != 0);
           tc::mma_commit_pair(empty(stage), both);  // both CTAs' stage is free once these MMAs read it
           if (++stage == kStagesP) {
             stage = 0;
@@ -726,7 +643,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
     }
     __syncwarp();
     tc::mbar_wait_warp(done, 0);  // every pair MMA has completed (both CTAs' TMEM)
-  } else if (kMode == kModeProject && warp >= 2 + epi_warps(kMode, kSplit)) {
+  } else if (kMode == kModeProject && warp >= 2 + epi_warps(kMode)) {
     // ---------------------------------------------------------------- A rows (projector mode)
     // loader warp w brings rows 32 w .. 32 w + 31 of this CTA's half of the
     // pair's rows of each A k-block with eight tile::gather4 loads; a group
@@ -735,11 +652,11 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
     // -1, which reads zeros.  The loads land on the even CTA's barrier, whose
     // loader warps expect both CTAs' bytes (the odd CTA's loader warps do not
     // arrive).  Each lane looks up one row; one thread issues.
-    const int lw = warp - 2 - epi_warps(kMode, kSplit);
+    const int lw = warp - 2 - epi_warps(kMode);
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
-    for (int tile = cluster; tile < tiles && ok; tile += clusters) {
+    for (int tile = pair; tile < tiles && ok; tile += pairs) {
       const int rb = tile / g.n_tiles;
       const long long src = kept_source_row(g, (long long)rb * 2 * kBM + (long long)rank * kBM + 32 * lw + lane);
       const int mine = src >= 0 ? (int)src : -1;
@@ -748,7 +665,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
 #pragma unroll
       for (int i = 0; i < 32; ++i) srow[i] = __shfl_sync(0xffffffffu, mine, i);
       if (tc::elect_one()) {
-        for (int kb = kb_first; kb < kb_end; ++kb) {
+        for (int kb = 0; kb < g.kblocks; ++kb) {
           if (!tc::mbar_wait(empty(stage), phase ^ 1u)) {
             ok = false;
             break;
@@ -768,7 +685,7 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
                 tc::tma_load_2d_pair(dst + (uint32_t)(i * kBK * 2), &maps.a, kb * kBK, srow[i], bar);
             }
           }
-          if (++stage == gemm_stages(kMode, kSplit)) {
+          if (++stage == kStagesP) {
             stage = 0;
             phase ^= 1u;
           }
@@ -783,31 +700,22 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
     const int part = (warp - 2) >> 2;  // which of the quadrant's warps
     // first of this warp's 32 rows in row tile rb
     auto row_of = [&](int rb) { return (2 * rb + (int)rank) * kBM + 32 * q; };
-    const int own = g.bn / kBlk / kSplit, own0 = pair * own;
-    EpiWarp w{own0 + part, own0 + own, out_stage + (uint32_t)((warp - 2) * stage_bytes(kMode)),
-              blk_bar(warp - 2), 0u, 0u, cluster, own0 + part};
-    if (kMode == kModeScore) score_load_next<epi_parts(kMode, kSplit)>(g, maps, w, clusters, row_of);
+    EpiWarp w{part, g.bn / kBlk, out_stage + (uint32_t)((warp - 2) * stage_bytes(kMode)),
+              blk_bar(warp - 2), 0u, 0u, pair, part};
+    if (kMode == kModeScore) score_load_next<epi_parts(kMode)>(g, maps, w, pairs, row_of);
     int acc = 0;
     uint32_t acc_phase = 0;
-    for (int tile = cluster; tile < tiles; tile += clusters) {
+    for (int tile = pair; tile < tiles; tile += pairs) {
       const int rb = tile / g.n_tiles, nt = tile - rb * g.n_tiles;
       if (g.bias)  // the first blocks' bias on its way to L1 while the main loop runs
-        for (int blk = w.first; blk < w.end; blk += epi_parts(kMode, kSplit))
+        for (int blk = w.first; blk < w.end; blk += epi_parts(kMode))
           if (nt * g.bn + blk * kBlk + lane < g.n) tc::touch(g.bias + nt * g.bn + blk * kBlk + lane);
       bool ok = tc::mbar_wait_warp(tfull(acc), acc_phase);
       if (!ok && lane == 0) flag_error(g, 4);
       tc::fence_after_sync();
       const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc * kBN);
-      if (kSplit > 1) {  // every pair's MMAs are done: the operand rings may take the partial sums
-        __syncwarp();
-        tc::cluster_sync();
-        if (ok) send_partials<kMode, kSplit>(g, sbase, taddr, pair, rank, part, 32 * q + lane);
-        __syncwarp();
-        tc::cluster_sync();
-      }
       Acc2 sums{};
-      if (ok && !epilogue_tile<kMode, kSplit>(g, maps, w, taddr, nt, row_of(rb), clusters, row_of, sbase, pair,
-                                              32 * q + lane, sums)) {
+      if (ok && !epilogue_tile<kMode>(g, maps, w, taddr, nt, row_of(rb), pairs, row_of, sums)) {
         ok = false;
         if (lane == 0) flag_error(g, 16);
       }
@@ -816,9 +724,8 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
       __syncwarp();
       if (lane == 0) tc::mbar_arrive_cluster(tempty_even(acc));  // this warp is done with the accumulator
       const int rb128 = 2 * rb + (int)rank;
-      const int active = active_parts(own, kSplit);
-      if (kMode == kModeScore && rb128 * kBM < g.m && part < active)
-        publish_rows(g.part + part_slot(g, kSplit * active, rb128, nt, pair * active + part, q) + lane, sums);
+      if (kMode == kModeScore && rb128 * kBM < g.m)
+        publish_rows(g.part + part_slot(g, rb128, nt, part, q) + lane, sums);
       acc ^= 1;
       if (acc == 0) acc_phase ^= 1u;
     }
@@ -830,10 +737,6 @@ __global__ void __launch_bounds__(gemm_threads(kMode, kSplit), 1)
     __syncwarp();
   }
 
-  if (kSplit > 1 && (warp < 2 || warp >= 2 + epi_warps(kMode, kSplit))) {  // the two barriers around the exchange
-    tc::cluster_sync();
-    tc::cluster_sync();
-  }
   tc::fence_before_sync();
   tc::cluster_sync();  // neither CTA leaves while the other may still signal its barriers
   if (warp == 1) {
@@ -878,123 +781,86 @@ bool make_map(CUtensorMap *map, const void *base, long long rows, long long cols
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Per device (index & 63): bit mode * 3 + log2(split) set once the variant's
-// shared-memory limit is raised and its co-resident clusters are counted.
+// Per device (index & 63): bit `mode` set once the mode's shared-memory limit
+// is raised and its co-resident pairs are counted.
 std::atomic<int> g_gemm_set[64];
-std::atomic<int> g_gemm_clusters[64][9];
+std::atomic<int> g_gemm_pairs[64][3];
 
-template <int kMode, int kSplit>
+template <int kMode>
 cudaError_t launch_gemm(const GemmMaps &maps, const GemmArgs &g, cudaStream_t st) {
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
-  constexpr int kVariant = kMode * 3 + (kSplit == 4 ? 2 : kSplit - 1);
   cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(gemm_threads(kMode, kSplit));
-  cfg.dynamicSmemBytes = gemm_smem(kMode, kSplit);
+  cfg.blockDim = dim3(gemm_threads(kMode));
+  cfg.dynamicSmemBytes = gemm_smem(kMode);
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2 * kSplit;
+  attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (!(g_gemm_set[dev & 63].load() & (1 << kVariant))) {
-    err = cudaFuncSetAttribute(k_mlp_gemm<kMode, kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               gemm_smem(kMode, kSplit));
+  if (!(g_gemm_set[dev & 63].load() & (1 << kMode))) {
+    err = cudaFuncSetAttribute(k_mlp_gemm<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(kMode));
     if (err != cudaSuccess) return err;
-    int clusters = 0;
-    cfg.gridDim = dim3(2 * kSplit * 64);
-    err = cudaOccupancyMaxActiveClusters(&clusters, k_mlp_gemm<kMode, kSplit>, &cfg);
+    int pairs = 0;
+    cfg.gridDim = dim3(2 * 64);
+    err = cudaOccupancyMaxActiveClusters(&pairs, k_mlp_gemm<kMode>, &cfg);
     if (err != cudaSuccess) return err;
-    if (clusters <= 0) return cudaErrorInvalidConfiguration;
-    g_gemm_clusters[dev & 63][kVariant].store(clusters);
-    g_gemm_set[dev & 63].fetch_or(1 << kVariant);
+    if (pairs <= 0) return cudaErrorInvalidConfiguration;
+    g_gemm_pairs[dev & 63][kMode].store(pairs);
+    g_gemm_set[dev & 63].fetch_or(1 << kMode);
   }
-  const int max_clusters = g_gemm_clusters[dev & 63][kVariant].load();
-  // split tiles: one per cluster (the grid may be larger than what runs at once)
-  const int clusters = kSplit > 1 || g.tiles < max_clusters ? g.tiles : max_clusters;
-  cfg.gridDim = dim3(2 * kSplit * clusters);
+  cfg.gridDim = dim3(2 * std::min(g.tiles, g_gemm_pairs[dev & 63][kMode].load()));
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, k_mlp_gemm<kMode, kSplit>, maps, g);
+  return cudaLaunchKernelEx(&cfg, k_mlp_gemm<kMode>, maps, g);
 }
 
 inline int row_tiles(int m) { return (int)(((long long)m + 2 * kBM - 1) / (2 * kBM)); }
 
-// How a GEMM is laid out on the 76 SM pairs: tile columns and splits of K.
+// How a GEMM is laid out on the 76 SM pairs: its tile columns.
 struct GemmShape {
-  int bn, split, n_tiles, kblocks;
+  int bn, n_tiles, kblocks;
 };
-// The cheapest of the layouts by a model in clocks, fitted to the measured
-// kernels; a function of the sizes alone (it also sizes tr_mlp_score's
-// scratch), whatever the device has free.
+// The cheapest width by a model in clocks, fitted to the measured kernels; a
+// function of the sizes alone (it also sizes tr_mlp_score's scratch), whatever
+// the device has free.
 //   A k-block takes the larger of its MMAs (2 clocks a column) and the operands
 //   into each SM at 63 bytes a clock, A's 16 KiB and B's 64 bytes a column:
 //   520 clocks for 256 columns, 455, 390 and 325 for 192, 128 and 64; the
 //   projector's row gather 1065 whatever the columns.  A tile's epilogue takes
 //   80 (score), 30 (hidden) or 65 (projector) clocks a column, overlapped with
 //   the next tile's main loop where there is one.
-//   Splitting K over two or four pairs (while all clusters run at once: 64
-//   pairs) divides the main loop and the epilogue and adds the exchange: two
-//   cluster barriers and the partial sums into each SM at 14 bytes a clock (96
-//   KiB for 256 columns in four, 7,000 clocks in all).
-// Measured: 192 rows, 1024 -> 4096, 16 tiles of 256 columns 12.3 us a pass, 64
-// of 64 columns 8.4; both GEMMs of 2885 rows, 1152 -> 4304 -> 1152, 63.4 us
-// with 60 score tiles of 256 columns, 58.9 with 72 of 192; the score GEMM of
-// 576 rows, 4096 -> 1024, 45 us in 256 columns, 21 with K split in four; both
-// GEMMs of 48 and 128 rows (1024 -> 4096 -> 1024) 28.7 and 27.0 us with 256
-// columns in four, 25.2 and 23.5 with 128.
-// The sums of an output element are the same for every mode (tr_project and
-// tr_project_kept agree bit for bit): they depend on the split alone.
+// Measured, with 256 columns throughout and with the width chosen: 192 rows,
+// 1024 -> 4096, 12.3 and 8.4 us a pass (16 tiles, 64 of 64 columns); both GEMMs
+// of 2885 rows, 1152 -> 4304 -> 1152, 63.4 and 58.9 (60 score tiles, 72 of 192
+// columns); both of 576 rows, 1024 -> 4096 -> 1024, 53.7 and 33.5 (12 score
+// tiles, 48 of 64), of 48 rows 51 and 27.7.
+// K is not shared among pairs where tiles are few: clusters that split it and
+// exchanged partial accumulators took 32.3 us for the 576 rows and 24.5 for the
+// 48, but then the order of an output element's sum, and so its last bits,
+// followed the number of rows; in one order a row gives the same H, x'' and z
+// alone, in any batch and with any scratch.
 inline GemmShape gemm_shape(int m, int n, int k, bool score, bool gather) {
   constexpr long long kPairs = 76;
   const int kb = (k + kBK - 1) / kBK;
   const long long rows = row_tiles(m);
-  auto tiles_of = [&](int bn) { return (n + bn - 1) / bn; };
-  auto epi = [&](int bn, bool g) { return (long long)bn * (score ? 80 : (g ? 65 : 30)); };
-  auto cost = [&](int bn, bool g) {
-    const long long waves = (rows * tiles_of(bn) + kPairs - 1) / kPairs;
-    const long long main = (long long)kb * (g ? 1065 : std::max(2 * bn + 8, (16384 + 64 * bn) / 63));
-    return waves * std::max(main, epi(bn, g)) + epi(bn, g);
+  auto cost = [&](int bn) {
+    const long long waves = (rows * ((n + bn - 1) / bn) + kPairs - 1) / kPairs;
+    const long long main = (long long)kb * (gather ? 1065 : std::max(2 * bn + 8, (16384 + 64 * bn) / 63));
+    const long long epi = (long long)bn * (score ? 80 : (gather ? 65 : 30));
+    return waves * std::max(main, epi) + epi;
   };
-  auto narrowest = [&](bool g, long long *least) {  // the cheapest width
-    int best = kBN;
-    *least = cost(kBN, g);
-    for (const int bn : {192, 128, 64})
-      if (cost(bn, g) < *least) {
-        *least = cost(bn, g);
-        best = bn;
-      }
-    return best;
-  };
-  long long least = 0;
-  int bn = narrowest(false, &least), split = 1;
-  for (const int s : {2, 4})  // the same for gathered rows
-    for (const int w : {256, 192, 128, 64})
-      if (w / kBlk % s == 0 && kb >= 4 * s && rows * tiles_of(w) * s <= 64) {
-        const long long c = (long long)((kb + s - 1) / s) * std::max(2 * w + 8, (16384 + 64 * w) / 63) +
-                            std::max(2500LL, epi(w, false) / s) + 1000 + 512LL * (s - 1) * (w / s) / 14;
-        if (c < least) {
-          least = c;
-          bn = w;
-          split = s;
-        }
-      }
-  if (gather && split == 1) bn = narrowest(true, &least);
-  return GemmShape{bn, split, tiles_of(bn), kb};
+  int best = kBN;
+  for (const int bn : {192, 128, 64})
+    if (cost(bn) < cost(best)) best = bn;
+  return GemmShape{best, (n + best - 1) / best, kb};
 }
 
-template <int kMode>
-cudaError_t launch_shape(const GemmMaps &maps, const GemmArgs &g, int split, cudaStream_t st) {
-  switch (split) {
-    case 4: return launch_gemm<kMode, 4>(maps, g, st);
-    case 2: return launch_gemm<kMode, 2>(maps, g, st);
-    default: return launch_gemm<kMode, 1>(maps, g, st);
-  }
-}
 inline void set_shape(GemmArgs &g, const GemmShape &sh) {
   g.bn = sh.bn;
   g.n_tiles = sh.n_tiles;
@@ -1020,15 +886,15 @@ tr_status check_mlp(const tr_mlp *m) {
 
 // Bytes of the score mode's partial sums in one layout, and the layout that
 // tr_mlp_score takes with `bytes` of them: the one gemm_shape chooses, or with
-// fewer (a workspace sized for another batch: a split or narrow layout of few
-// rows may want more than 256-column tiles of many) 256-column tiles.
+// fewer (a workspace sized for another batch: the narrow tiles of few rows may
+// want more than the 256-column tiles of many) 256-column tiles.
 size_t part_bytes(const tr_mlp *m, const GemmShape &sh) {
   const long long rblocks = ((long long)m->t + kBM - 1) / kBM;
-  return align_up((size_t)rblocks * sh.n_tiles * row_parts(sh.bn, sh.split) * 4 * kPartWords * 32 * sizeof(float), 256);
+  return align_up((size_t)rblocks * sh.n_tiles * kRowParts * 4 * kPartWords * 32 * sizeof(float), 256);
 }
 GemmShape score_shape(const tr_mlp *m, size_t bytes) {
   const GemmShape sh = gemm_shape(m->t, m->d, m->d_hidden, true, false);
-  return part_bytes(m, sh) <= bytes ? sh : GemmShape{kBN, 1, (m->d + kBN - 1) / kBN, sh.kblocks};
+  return part_bytes(m, sh) <= bytes ? sh : GemmShape{kBN, (m->d + kBN - 1) / kBN, sh.kblocks};
 }
 
 // out = act(a W^T + bias) for dense bf16 rows a [rows, k] and W [n, k]: the
@@ -1050,7 +916,7 @@ tr_status dense_act_gemm(const void *a, int rows, int k, const void *w, const fl
   if (!make_map(&maps.a, a, rows, k, kBM) || !make_map(&maps.b, w, n, k, sh.bn / 2) ||
       !make_map(&maps.out, out, rows, n, 32, kBlk, CU_TENSOR_MAP_SWIZZLE_64B))
     return TR_ERR_CUDA;
-  return launch_shape<kModeHidden>(maps, g, sh.split, st) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
+  return launch_gemm<kModeHidden>(maps, g, st) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 
 }  // namespace
@@ -1114,10 +980,9 @@ tr_status tr_mlp_score(const tr_mlp *m, const void *h, void *x_post, void *x, fl
       !block_map(&maps.p, m->x_pre) || (m->resid && !block_map(&maps.r, m->resid)) || !block_map(&maps.out, x_post) ||
       !block_map(&maps.x, x))
     return TR_ERR_CUDA;
-  if (launch_shape<kModeScore>(maps, g, sh.split, st) != cudaSuccess) return TR_ERR_CUDA;
-  const int parts = row_parts(sh.bn, sh.split);
+  if (launch_gemm<kModeScore>(maps, g, st) != cudaSuccess) return TR_ERR_CUDA;
   const cudaError_t err = launch_kernel(k_score_rows, dim3((g.m + kBM - 1) / kBM * 4), dim3(kRowWarps * 32), 0, st, true,
-                                        g, parts, reinterpret_cast<float4 *>(stats), h2, s);
+                                        g, reinterpret_cast<float4 *>(stats), h2, s);
   return err == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 
@@ -1165,7 +1030,7 @@ tr_status tr_project_kept(const tr_tokens *in, const int32_t *d_cu_k, const int3
   if (!make_map(&maps.a, in->x, total_rows, in->d, 1) || !make_map(&maps.b, w, d_out, in->d, sh.bn / 2) ||
       !make_map(&maps.out, z, total_k, d_out, 32, kBlk, CU_TENSOR_MAP_SWIZZLE_64B))
     return TR_ERR_CUDA;
-  return launch_shape<kModeProject>(maps, g, sh.split, static_cast<cudaStream_t>(stream)) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
+  return launch_gemm<kModeProject>(maps, g, static_cast<cudaStream_t>(stream)) == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 
 }  // extern "C"

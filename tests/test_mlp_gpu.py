@@ -242,28 +242,27 @@ def test_project_kept_index_outside_its_image():
     _check_close(z, _sigma(v, "gelu"), mag, slope=1.13)
 
 
-# The layouts a GEMM may take (gemm_shape): tile columns x pairs that split K,
-# with ragged rows, columns and k-blocks and k-blocks that do not divide
-# evenly.  Named by the score GEMM's layout.
-SPLIT_CASES = [
-    ("256x4", 1000, 1024, 16400, "none", True, True),            # 16 tiles, 256.25 k-blocks
-    ("128x4_one_row", 1, 256, 6144, "none", False, True),        # 2 tiles, 96 k-blocks
-    ("128x4_uneven_k", 300, 528, 4464, "gelu", True, True),      # 10 tiles, 69.75 k-blocks
-    ("256x2_uneven_k", 1500, 1024, 4400, "gelu", True, True),    # 24 tiles, 68.75 k-blocks
-    ("256x2_most_tiles", 2048, 784, 4112, "gelu", False, True),  # 32 tiles, 64.25 k-blocks
-    ("192x2", 1200, 1024, 4096, "quick_gelu", True, True),       # 5 x 6 tiles, the last 64 columns
-    ("128x2", 1000, 1024, 4160, "quick_gelu", True, False),      # 32 tiles, 65 k-blocks
-    ("64x2", 129, 1056, 1472, "quick_gelu", True, True),         # 17 tiles, the last half empty
-    ("192x1", 2885, 1152, 4304, "gelu", True, True),             # 12 x 6 tiles
-    ("128x1", 2048, 784, 2064, "gelu", False, True),             # 8 x 7 tiles, the last 16 columns
-    ("64x1", 2049, 1152, 1600, "none", True, True),              # 9 x 18 tiles
+# The layouts a GEMM may take (gemm_shape), by size: tile columns of the hidden
+# and the score GEMM, with ragged rows, columns and k-blocks.
+LAYOUT_CASES = [
+    ("256_64_long_k", 1000, 1024, 16400, "none", True, True),      # 4 x 16 score tiles, 256.25 k-blocks
+    ("64_64_one_row", 1, 256, 6144, "none", False, True),          # 4 score tiles, 96 k-blocks
+    ("128_64", 300, 528, 4464, "gelu", True, True),                # 2 x 9 score tiles, the last 16 columns
+    ("192_128", 1500, 1024, 4400, "gelu", True, True),             # 6 x 8 score tiles, 68.75 k-blocks
+    ("256_128", 2048, 784, 4112, "gelu", False, True),             # 8 x 7 score tiles, the last 16 columns
+    ("192_128_ragged_rows", 1200, 1024, 4096, "quick_gelu", True, True),  # 5 row tiles
+    ("256_64", 1000, 1024, 4160, "quick_gelu", True, False),       # 4 x 16 score tiles, 65 k-blocks
+    ("64_64", 129, 1056, 1472, "quick_gelu", True, True),          # 17 score tiles, the last half empty
+    ("256_192", 2885, 1152, 4304, "gelu", True, True),             # 12 x 6 score tiles
+    ("128_128", 2048, 784, 2064, "gelu", False, True),             # 8 x 7 score tiles, the last 16 columns
+    ("256_64_many", 2049, 1152, 1600, "none", True, True),         # 9 x 18 score tiles
 ]
 
 
-@pytest.mark.parametrize("name,t,d,dh,act,resid,bias", SPLIT_CASES, ids=[c[0] for c in SPLIT_CASES])
-def test_mlp_split(name, t, d, dh, act, resid, bias):
+@pytest.mark.parametrize("name,t,d,dh,act,resid,bias", LAYOUT_CASES, ids=[c[0] for c in LAYOUT_CASES])
+def test_mlp_layouts(name, t, d, dh, act, resid, bias):
     test_mlp_outputs_and_records(name, t, d, dh, act, resid, bias)
-    # a second call reproduces every bit: the partial sums are added in a fixed order
+    # a second call reproduces every bit: the row partials are merged in a fixed order
     altr = _alt()
     xp, w1, w2, b1, b2, r = _inputs(t, d, dh, seed=3, resid=resid, bias=bias)
     m = altr.Mlp(t, w1, w2, b1, b2, act=act)
@@ -291,9 +290,9 @@ def _project_direct(x, idx, cu_k, w, bias, seqlens):
 
 @pytest.mark.parametrize("d,d_out,k,n,b", [(8208, 528, 40, 300, 3), (4096, 2560, 200, 300, 3), (784, 1296, 50, 300, 3),
                                            (272, 528, 200, 300, 16), (256, 272, 1025, 1300, 3)],
-                         ids=["128x4", "256x2", "64x1", "gathered", "gathered_few"])
-def test_project_split(d, d_out, k, n, b):
-    # K split, or narrow tiles: the dense projector within the GEMM tolerance
+                         ids=["64_long_k", "128", "64", "gathered", "gathered_few"])
+def test_project_layouts(d, d_out, k, n, b):
+    # tiles of few columns: the dense projector within the GEMM tolerance
     # of float64, and the rows read by index bit for bit the same
     altr = _alt()
     g = torch.Generator(device="cuda").manual_seed(9)
@@ -350,3 +349,34 @@ def test_mlp_score_with_a_smaller_workspace(t, d, dh):
     m._ws_bytes = least - 256
     with pytest.raises(Exception, match="tr_mlp_score"):
         m.run(xp, r)
+
+
+@pytest.mark.parametrize("t,d,dh", [(576, 1024, 4096), (48, 1024, 4096), (129, 1056, 1472), (1, 256, 6144)])
+def test_rows_do_not_depend_on_the_batch(t, d, dh):
+    # An image's rows alone, in a batch whose GEMMs are laid out differently,
+    # and with the least scratch: K is summed in one order, so H, x'' and x are
+    # the same bit for bit, and so is the projector's z.  The records' sums are
+    # grouped by the tile columns: the same to their fp32 rounding, and the
+    # certified selection the same.
+    altr = _alt()
+    most = 12 * t if t > 1 else 3000
+    xp, w1, w2, b1, b2, r = _inputs(most, d, dh, seed=12)
+    m = altr.Mlp(most, w1, w2, b1, b2, act="quick_gelu")
+    whole = m.run(xp, r)
+    alone = altr.Mlp(t, w1, w2, b1, b2, act="quick_gelu")
+    rows = [(a.clone(), b[:t].clone()) for o in [alone.run(xp[:t].contiguous(), r[:t].contiguous())]
+            for a, b in ((o.h, whole.h), (o.x_post, whole.x_post), (o.x, whole.x), (o.stats, whole.stats))]
+    alone._ws_bytes = -(-t // 128) * -(-d // 256) * 10240
+    least = alone.run(xp[:t].contiguous(), r[:t].contiguous())
+    torch.cuda.synchronize()
+    for a, b in rows[:3]:
+        assert torch.equal(a.view(torch.int16), b.view(torch.int16))
+    for a, b in zip((least.x_post, least.x), (rows[1][0], rows[2][0])):
+        assert torch.equal(a.view(torch.int16), b.view(torch.int16))
+    sa, sb = rows[3]
+    assert torch.allclose(sa[:, :4], sb[:, :4], rtol=2.0 ** -23, atol=0)
+    z, _ = altr.project(whole.x, w1, b1)
+    za, _ = altr.project(whole.x[:t].contiguous(), w1, b1)
+    zk, _ = altr.project_kept(whole.x, torch.arange(t, dtype=torch.int32, device="cuda"), [0, t], w1, b1)
+    assert torch.equal(z[:t].view(torch.int16), za.view(torch.int16))
+    assert torch.equal(z[:t].view(torch.int16), zk.view(torch.int16))
