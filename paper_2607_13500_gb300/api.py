@@ -136,12 +136,11 @@ class _Tokens:
         self._ref = ctypes.byref(self.s)
 
     def rebind(self, x, x_pre, x_post):
-        """The same images in other tensors."""
+        """The same images in other tensors of the same shape and type."""
         self.x, self.x_pre, self.x_post = x, x_pre, x_post
         s = self.s
         s.x, s.x_post = x.data_ptr(), x_post.data_ptr()
         s.x_pre = None if x_pre is None else x_pre.data_ptr()
-        s.dtype, s.d, s.total = _dtype_code(x), x.shape[1], x.shape[0]
         return self
 
     def ref(self):
@@ -182,9 +181,15 @@ class _Bound:
         return views[0]
 
     def _bind(self, x, x_pre, x_post):
-        if x.dim() == 2:
-            if x.shape[0] != self._total:
-                raise ValueError("seqlens must sum to the number of rows of x")
+        # the outputs and the scratch were allocated for these rows and no others
+        dim = x.dim()
+        if dim != 2 and dim != 3:
+            raise ValueError("x must be [B, N, D] or [T, D]")
+        if (x.shape[0] if dim == 2 else x.shape[0] * x.shape[1]) != self._total:
+            raise ValueError("seqlens must sum to the number of rows of x")
+        if x.shape[-1] != self.d or x.dtype != self.dtype or x.device != self.d_k.device:
+            raise ValueError(f"this object reduces [{self._total}, {self.d}] {self.dtype} tokens on {self.d_k.device}")
+        if dim == 2:
             _check_tokens(x, x_pre, x_post)
         else:
             x, x_pre, x_post, _ = _flatten(x, x_pre, x_post, self.seqlens)

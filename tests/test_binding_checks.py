@@ -1,0 +1,56 @@
+"""What the binding refuses before any launch: tensors that do not match the
+shape, type or device that the kernels will read or write.  No GPU needed: the
+checks come before the one for a CUDA device, or are called on their own."""
+import pytest
+import torch
+
+from paper_2607_13500_gb300 import api
+
+
+def _bound(seqlens=(3, 4), d=16, dtype=torch.bfloat16):
+    b = object.__new__(api._Bound)
+    b.seqlens, b._total, b.d, b.dtype = list(seqlens), sum(seqlens), d, dtype
+    b.d_k = torch.zeros(len(seqlens), dtype=torch.int32)
+    b.stride, b._cu, b._tok = "alg1", None, None
+    return b
+
+
+@pytest.mark.parametrize("shape,dtype", [
+    ((7, 32), torch.bfloat16), ((7, 8), torch.bfloat16), ((7, 16), torch.float32), ((7, 16), torch.float16),
+    ((6, 16), torch.bfloat16), ((8, 16), torch.bfloat16), ((1, 6, 16), torch.bfloat16), ((2, 4, 16), torch.bfloat16),
+    ((1, 7, 32), torch.bfloat16), ((1, 7, 16), torch.float32), ((16,), torch.bfloat16), ((), torch.bfloat16)])
+def test_bound_tokens_of_another_shape_or_type(shape, dtype):
+    # outputs and scratch were allocated for [7, 16] bf16
+    x = torch.zeros(shape, dtype=dtype)
+    with pytest.raises(ValueError, match=r"sum to|\[7, 16\]|\[B, N, D\]"):
+        _bound()._bind(x, None, x)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("cls", ["Reducer", "Pipeline"])
+def test_refused_before_any_launch(cls):
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    import paper_2607_13500_gb300 as altr
+    obj = getattr(altr, cls)([40, 24], 64, torch.bfloat16, "cuda", k=4)
+    call = obj.run if cls == "Reducer" else obj.submit
+    mk = lambda *s, dt=torch.bfloat16: torch.randn(*s, device="cuda").to(dt)
+    for bad in (mk(64, 128), mk(64, 32), mk(64, 64, dt=torch.float32), mk(1, 60, 64), mk(2, 32, 128)):
+        with pytest.raises(ValueError):
+            call(bad, bad, bad)
+    good = mk(64, 64)
+    r = call(good, good, good)
+    torch.cuda.synchronize()
+    assert r.status.tolist()[3] == 0 and r.y.shape == (8, 64)
+
+
+def test_bound_tokens_on_another_device():
+    x = torch.zeros(7, 16, dtype=torch.bfloat16, device="meta")
+    with pytest.raises(ValueError, match=r"\[7, 16\]"):
+        _bound()._bind(x, None, x)
+
+
+def test_bound_tokens_that_match():
+    x = torch.zeros(7, 16, dtype=torch.bfloat16)
+    with pytest.raises(ValueError, match="CUDA device"):  # the next check
+        _bound()._bind(x, None, x)
