@@ -733,6 +733,19 @@ def mlp(x_pre, w1, w2, b1=None, b2=None, resid=None, act="gelu", scores=False) -
     return Mlp(x_pre.shape[0], w1, w2, b1, b2, act, scores).run(x_pre, resid)
 
 
+def _check_kept(batch, d, device, idx, cu_k, w, bias, error):
+    """project_kept's operands against its ``batch`` images of D = ``d``: what the
+    kernels read and write lies inside them."""
+    if w.dim() != 2 or w.shape[1] != d:
+        raise ValueError(f"w must be [d_out, {d}]")
+    if len(cu_k) != batch + 1:
+        raise ValueError(f"cu_k must hold {batch + 1} offsets")
+    _check_buf(idx, device, torch.int32, int(cu_k[-1]), "idx")
+    if bias is not None and bias.numel() < w.shape[0]:
+        raise ValueError(f"bias must hold {w.shape[0]} values")
+    _check_buf(error, device, torch.int32, 1, "error")
+
+
 def project_kept(x, idx, cu_k, w, bias=None, act="gelu", seqlens=None, error=None):
     """z = sigma(X* W^T + bias) for the kept tokens X* (tr_project_kept's result),
     their rows named by the selection's ``idx`` (local per image, image b
@@ -747,6 +760,7 @@ def project_kept(x, idx, cu_k, w, bias=None, act="gelu", seqlens=None, error=Non
     if w.device != x2.device or idx.device != x2.device or (bias is not None and bias.device != x2.device) or \
             (error is not None and error.device != x2.device):
         raise ValueError("w, idx, bias and error must live on x's device")
+    _check_kept(len(seqlens), x2.shape[1], x2.device, idx, cu_k, w, bias, error)
     tok = _Tokens(x2, None, x2, seqlens)
     total_k = int(cu_k[-1])
     d, d_out = int(x2.shape[1]), int(w.shape[0])

@@ -54,3 +54,55 @@ def test_bound_tokens_that_match():
     x = torch.zeros(7, 16, dtype=torch.bfloat16)
     with pytest.raises(ValueError, match="CUDA device"):  # the next check
         _bound()._bind(x, None, x)
+
+
+def _kept(**over):
+    a = dict(idx=torch.arange(9, dtype=torch.int32), cu_k=[0, 4, 9], w=torch.zeros(48, 32, dtype=torch.bfloat16),
+             bias=torch.zeros(48), error=torch.zeros(1, dtype=torch.int32))
+    a.update(over)
+    return a
+
+
+KEPT_REFUSED = {
+    "narrow_w": dict(w=torch.zeros(48, 16, dtype=torch.bfloat16)),
+    "wide_w": dict(w=torch.zeros(48, 64, dtype=torch.bfloat16)),
+    "flat_w": dict(w=torch.zeros(48 * 32, dtype=torch.bfloat16)),
+    "int64_idx": dict(idx=torch.arange(9)),
+    "short_idx": dict(idx=torch.arange(8, dtype=torch.int32)),
+    "strided_idx": dict(idx=torch.arange(18, dtype=torch.int32)[::2]),
+    "short_bias": dict(bias=torch.zeros(47)),
+    "short_offsets": dict(cu_k=[0, 9]),
+    "long_offsets": dict(cu_k=[0, 4, 9, 9]),
+    "float_error": dict(error=torch.zeros(1)),
+    "empty_error": dict(error=torch.zeros(0, dtype=torch.int32)),
+}
+
+
+@pytest.mark.parametrize("name", KEPT_REFUSED)
+def test_project_kept_operands(name):
+    api._check_kept(2, 32, torch.device("cpu"), **_kept())
+    api._check_kept(2, 32, torch.device("cpu"), **_kept(bias=None, error=None))
+    with pytest.raises(ValueError):
+        api._check_kept(2, 32, torch.device("cpu"), **_kept(**KEPT_REFUSED[name]))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("k", [9, 4000], ids=["few_rows", "many_rows"])
+def test_project_kept_refuses_before_any_launch(k):
+    # on either side of the number of rows from which they are copied first
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    import paper_2607_13500_gb300 as altr
+    n = 2500
+    x = torch.randn(2 * n, 32, device="cuda").to(torch.bfloat16)
+    good = _kept(idx=torch.arange(k, dtype=torch.int32) % n, cu_k=[0, k // 2, k], w=torch.zeros(1024, 32, dtype=torch.bfloat16),
+                 bias=torch.zeros(1024))
+    on = lambda a: {n: v.cuda() if isinstance(v, torch.Tensor) else v for n, v in a.items()}
+    call = lambda a: altr.project_kept(x, a["idx"], a["cu_k"], a["w"], a["bias"], seqlens=[n, n], error=a["error"])
+    for bad in (dict(w=torch.zeros(1024, 16, dtype=torch.bfloat16)), dict(idx=good["idx"].long()), dict(idx=good["idx"][1:]),
+                dict(bias=torch.zeros(1000)), dict(cu_k=[0, k]), dict(error=torch.zeros(1))):
+        with pytest.raises(ValueError):
+            call(on({**good, **bad}))
+    z, err = call(on(good))
+    torch.cuda.synchronize()
+    assert z.shape == (k, 1024) and err.item() == 0 and not bool(z.any())
