@@ -42,6 +42,11 @@ def _check_buf(t, device, dtype, min_numel, name):
         raise ValueError(f"{name} must be a contiguous {dtype} tensor of at least {min_numel} elements on {device}")
 
 
+def _check_bias(bias, n, name):
+    if bias is not None and bias.numel() < n:
+        raise ValueError(f"{name} must hold {n} values")
+
+
 def _stream(device) -> int:
     """The raw handle of torch's current stream on ``device``."""
     index = device.index
@@ -674,6 +679,8 @@ class Mlp:
             raise ValueError("w2 must be [D, d_hidden] for w1 [d_hidden, D]")
         if act not in TR_ACT:
             raise ValueError(f"act must be one of {sorted(TR_ACT)}")
+        _check_bias(b1, dh, "b1")
+        _check_bias(b2, d, "b2")
         self.t, self.d, self.dh, self.act = int(t), int(d), int(dh), act
         self.device = w1.device
         dev = self.device
@@ -741,8 +748,7 @@ def _check_kept(batch, d, device, idx, cu_k, w, bias, error):
     if len(cu_k) != batch + 1:
         raise ValueError(f"cu_k must hold {batch + 1} offsets")
     _check_buf(idx, device, torch.int32, int(cu_k[-1]), "idx")
-    if bias is not None and bias.numel() < w.shape[0]:
-        raise ValueError(f"bias must hold {w.shape[0]} values")
+    _check_bias(bias, w.shape[0], "bias")
     _check_buf(error, device, torch.int32, 1, "error")
 
 
@@ -801,6 +807,8 @@ def project(y, w, bias=None, act="gelu", error=None, out=None):
         raise ValueError(f"act must be one of {sorted(TR_ACT)}")
     if y.dim() != 2 or not y.is_contiguous() or w.dim() != 2 or w.shape[1] != y.shape[1]:
         raise ValueError("y must be contiguous [rows, D] and w [d_out, D]")
+    _check_bias(bias, w.shape[0], "bias")
+    _check_buf(error, y.device, torch.int32, 1, "error")
     rows, d = int(y.shape[0]), int(y.shape[1])
     d_out = int(w.shape[0])
     dev = y.device

@@ -106,3 +106,27 @@ def test_project_kept_refuses_before_any_launch(k):
     z, err = call(on(good))
     torch.cuda.synchronize()
     assert z.shape == (k, 1024) and err.item() == 0 and not bool(z.any())
+
+
+def test_bias_length():
+    api._check_bias(None, 8, "b")
+    api._check_bias(torch.zeros(8), 8, "b")
+    with pytest.raises(ValueError, match="b must hold 8"):
+        api._check_bias(torch.zeros(7), 8, "b")
+
+
+@pytest.mark.gpu
+def test_dense_layers_refuse_short_biases_and_other_error_buffers():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    import paper_2607_13500_gb300 as altr
+    w = torch.randn(64, 32, device="cuda").to(torch.bfloat16)
+    b64, b32, y = torch.zeros(64, device="cuda"), torch.zeros(32, device="cuda"), torch.ones_like(w)
+    for b1, b2 in ((b32, b32), (b64, b32[1:])):
+        with pytest.raises(ValueError):
+            altr.Mlp(64, w, w.t(), b1, b2)
+    for kw in (dict(bias=b32), dict(error=torch.zeros(1, device="cuda")), dict(error=torch.zeros(1, dtype=torch.int32))):
+        with pytest.raises(ValueError):
+            altr.project(y, w, **kw)
+    assert altr.Mlp(64, w, w.t(), b64, b32).run(y).error.item() == 0
+    assert altr.project(y, w, b64)[1].item() == 0
