@@ -162,7 +162,7 @@ class _Bound:
         self.seqlens = [int(v) for v in seqlens]
         self.device = torch.device(device)
         self.d, self.dtype, self.alias_pre, self.stride = d, dtype, alias_pre, stride
-        self.ks, self.k1s, self.cu_k = budget if budget is not None else budgets(self.seqlens, k, ratio, lam)
+        self.ks, self.k1s, self.cu_k = _budget_of(budget, self.seqlens, k, ratio, lam)
         self.total_k = self.cu_k[-1]
         self._total = sum(self.seqlens)
         self._tok = None
@@ -174,13 +174,8 @@ class _Bound:
             self._cu = None if offsets is None else mk(offsets)
             return torch.zeros(TR_STATUS_WORDS, dtype=torch.int32, device=dev)
         # used on the current stream only: one launch writes everything
-        b = len(self.seqlens)
         parts = [[0] * TR_STATUS_WORDS, self.ks, self.k1s, self.cu_k] + ([] if offsets is None else [offsets])
-        if len(self.ks) != b or len(self.k1s) != b or len(self.cu_k) != b + 1:
-            mk = lambda v: torch.tensor(v, dtype=torch.int32, device=dev)
-            views = [mk(v) for v in parts]
-        else:
-            views = _device_words([w for v in parts for w in v], dev).split([len(v) for v in parts])
+        views = _device_words([w for v in parts for w in v], dev).split([len(v) for v in parts])
         self.d_k, self.d_k1, self.d_cu = views[1:4]
         self._cu = None if offsets is None else views[4]
         return views[0]
@@ -203,6 +198,20 @@ class _Bound:
         else:
             self._tok.rebind(x, x_pre, x_post)
         return self._tok
+
+
+def _budget_of(budget, seqlens, k, ratio, lam):
+    """(ks, k1s, cu_k): the caller's explicit lists, which must give every image
+    its entries and its own slots of the outputs, or tr_budgets' of the rest."""
+    if budget is None:
+        return budgets(seqlens, k, ratio, lam)
+    ks, k1s, cu_k = budget
+    b = len(seqlens)
+    if len(ks) != b or len(k1s) != b or len(cu_k) != b + 1:
+        raise ValueError(f"budget must hold {b} ks, {b} k1s and {b + 1} offsets")
+    if any(k > 0 and not 0 <= c <= cu_k[-1] - k for k, c in zip(ks, cu_k)):
+        raise ValueError("budget: an image's slots lie outside cu_k[0]..cu_k[-1]")
+    return ks, k1s, cu_k
 
 
 def budgets(seqlens, k=None, ratio=None, lam=(1, 3)):
@@ -256,7 +265,7 @@ def select(x, x_pre, x_post, stats, k=None, ratio=None, lam=(1, 3), seqlens=None
     _check_buf(h2, x.device, torch.float32, t, "h2")
     _check_buf(s, x.device, torch.float32, t, "s")
     tok = _Tokens(x, x_pre, x_post, seqlens, stride)
-    ks, k1s, cu_k = budget if budget is not None else budgets(seqlens, k, ratio, lam)
+    ks, k1s, cu_k = _budget_of(budget, seqlens, k, ratio, lam)
     dev = x.device
     d_k, d_k1, d_cu = _device_words(ks, dev), _device_words(k1s, dev), _device_words(cu_k, dev)
     idx = torch.empty(max(cu_k[-1], 1), dtype=torch.int32, device=dev)

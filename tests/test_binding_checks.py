@@ -130,3 +130,16 @@ def test_dense_layers_refuse_short_biases_and_other_error_buffers():
             altr.project(y, w, **kw)
     assert altr.Mlp(64, w, w.t(), b64, b32).run(y).error.item() == 0
     assert altr.project(y, w, b64)[1].item() == 0
+
+
+@pytest.mark.parametrize("budget", [
+    ([2], [0, 1], [0, 2, 5]), ([2, 3], [0], [0, 2, 5]), ([2, 3], [0, 1], [0, 5]), ([2, 3], [0, 1], [0, 2, 5, 5]),
+    ([2, 4], [0, 1], [0, 2, 5]), ([2, 3], [0, 1], [-1, 2, 5]), ([6, 0], [0, 0], [0, 0, 5])])
+def test_explicit_budgets_keep_to_the_outputs(budget):
+    with pytest.raises(ValueError, match="budget"):
+        api._budget_of(budget, [7, 7], None, None, (1, 3))
+
+
+def test_explicit_budgets_that_fit():
+    for budget in (([2, 3], [0, 1], [0, 2, 5]), ([0, 5], [0, 5], [0, 0, 5]), ([2, 3], [0, 1], [0, 4, 9])):
+        assert api._budget_of(budget, [7, 7], None, None, (1, 3)) == budget
