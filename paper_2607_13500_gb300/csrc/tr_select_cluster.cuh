@@ -124,22 +124,23 @@ struct ClusterShared {
 };
 
 // Double-float keys of rows[0..cnt) (mode 0: R, 1: s) into their records, up
-// to four rows at a time by groups of warps; false (block-uniform) when a row
-// does not qualify.  Called by the whole block; ends with a barrier.
-__device__ __noinline__ bool refine_df(const SelectArgs &a, long long off, const uint16_t *rows, int cnt, int mode,
+// to four rows at a time by groups of warps.  A row that does not qualify gets
+// a NaN key, which compares as undecided with any other, so its run, and no
+// other, is left open.  Called by the whole block; ends with a barrier.
+__device__ __noinline__ void refine_df(const SelectArgs &a, long long off, const uint16_t *rows, int cnt, int mode,
                                        ExactRec *rec) {
   __shared__ PartDf pdf;
   const int groups = cnt >= 4 ? 4 : (cnt >= 2 ? 2 : 1);
   const int gsize = (int)blockDim.x / groups;
   const int gi = (int)threadIdx.x / gsize;
   const Group g{gi * gsize, gsize, 1 + gi};
-  bool ok = true;
   for (int base = 0; base < cnt; base += groups)
     if (base + gi < cnt) {
       const int row = rows[base + gi];
-      ok &= df_row_any(a, off + row, mode, rec + row, pdf, g);
+      if (!df_row_any(a, off + row, mode, rec + row, pdf, g) && g.tid() == 0)
+        (mode == 0 ? rec[row].r_hi : rec[row].s_hi) = __int_as_float(0x7fc00000);
     }
-  return !__syncthreads_or(!ok);
+  __syncthreads();
 }
 
 // Exact sums of rows[0..cnt) into their records, in the same way, with the H2
@@ -354,19 +355,17 @@ __device__ __forceinline__ bool cluster_stage_one(const SelectArgs &a, const Spl
         for (int q = lo + tid; q < hi; q += nthr) sh.list[q - lo] = sh.win_row[sh.win_ord[q]];
         __syncthreads();
         const int len = hi - lo;
-        bool open = !refine_df(a, im.off, sh.list, len, 0, im.rec);  // uniform
+        refine_df(a, im.off, sh.list, len, 0, im.rec);
+        bool open = false;
         int rank = 0;
-        if (!open) {
-          if (tid < len)
-            for (int j = 0; j < len; ++j) {
-              if (j == tid) continue;
-              const int c = df_cmp_r(im.rec[sh.list[j]], im.rec[sh.list[tid]], a.bounds);
-              open |= c == 0;
-              rank += c > 0;
-            }
-          open = __syncthreads_or(open) != 0;
-        }
-        if (open) {
+        if (tid < len)
+          for (int j = 0; j < len; ++j) {
+            if (j == tid) continue;
+            const int c = df_cmp_r(im.rec[sh.list[j]], im.rec[sh.list[tid]], a.bounds);
+            open |= c == 0;
+            rank += c > 0;
+          }
+        if (__syncthreads_or(open)) {
           ok = refine_exact(a, im.off, sh.list, len, 0, im.rec, im.primary);
           rank = 0;
           if (ok && tid < len) {
@@ -512,13 +511,13 @@ __device__ __forceinline__ bool cluster_stage_two(const SelectArgs &a, const Spl
   bad = __syncthreads_or(bad) != 0;
   if (__syncthreads_or(marked) && !bad) {
     const int runs = sh.runs;
-    // a run that the double-float keys leave open anywhere (or, for all runs,
-    // a row that does not qualify for them) is ranked by exact sums as a whole
-    const bool df = runs > 0 && refine_df(a, im.off, sh.list, sh.run_rows, 1, im.rec);
+    // a run that the double-float keys leave open anywhere (a pair they do not
+    // separate, or a row that does not qualify) is ranked by exact sums as a whole
+    if (runs > 0) refine_df(a, im.off, sh.list, sh.run_rows, 1, im.rec);
     for (int r = tid; r < runs; r += nthr) {
       const int len = (int)(sh.run[r] & 0xffffu) - (int)(sh.run[r] >> 16);
       const uint16_t *rows = sh.list + sh.first[r];
-      bool open = !df;
+      bool open = false;
       for (int i = 0; i < len && !open; ++i)
         for (int j = i + 1; j < len && !open; ++j) open = df_cmp_s(im.rec[rows[j]], im.rec[rows[i]], a.bounds) == 0;
       if (open) {

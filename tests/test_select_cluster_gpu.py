@@ -153,3 +153,21 @@ def test_near_ties_at_the_value_range(dtype, edge, exact):
     for k, k1 in [(40, 31), (60, 0), (45, 16)]:
         st = check_reduce(x, xp, xq, [n], _budget([k], [k1]))
         assert (st[2] > 0) == exact, st
+
+
+@pytest.mark.parametrize("rows", [1500, 5500])
+def test_exact_sums_only_for_the_run_that_needs_them(rows):
+    # every row a pick: a row outside the double-float keys' value range sends
+    # its own near-tie run to exact sums, and no other
+    d = 1024
+    tx, tp, tq, shuffle, *_ = _near_tie_triples(32, d, torch.float32, 3)
+    where = torch.argsort(shuffle)  # where[i]: the place of row i
+    for t in (tp, tq):
+        t[:, 7] = 0.0
+        t[where[15:18], 7] = 2.0 ** -60  # below 2^-50, and far below what moves a key
+    x, xp, xq = (torch.cat([a, b]) for a, b in zip((tx, tp, tq), _rows(rows, d, 4, torch.float32)))
+    perm = torch.randperm(x.shape[0], generator=torch.Generator().manual_seed(6))
+    x, xp, xq = x[perm], xp[perm], xq[perm]
+    n = x.shape[0]
+    st = check_reduce(x, xp, xq, [n], _budget([n - 1], [0]))
+    assert 3 <= st[2] <= 8, st
