@@ -357,6 +357,14 @@ typedef struct {
 tr_status tr_mlp_hidden(const tr_mlp *m, void *h, int32_t *d_error, void *stream);
 
 /*
+ * The tile width (64, 128, 192 or 256 columns) that a GEMM of `rows` rows, `n`
+ * output columns and inner extent `k` is laid out with; kind 0: tr_mlp_hidden
+ * and tr_project, 1: tr_mlp_score (given its full scratch), 2:
+ * tr_project_kept.  Host only; 0 on invalid input.  Results do not depend on it.
+ */
+int32_t tr_gemm_columns(int32_t rows, int32_t n, int32_t k, int32_t kind);
+
+/*
  * Scratch bytes of tr_mlp_score (256-byte aligned device memory); 0 on invalid
  * input.  A call given fewer (scratch sized for a larger t, whose GEMM is laid
  * out differently) still runs, in 256-column tiles, from 10 KiB per 128 rows

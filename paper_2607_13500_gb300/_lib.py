@@ -97,6 +97,7 @@ def load() -> ctypes.CDLL:
     lib.tr_reduce.restype = I32
     mlp = P(TrMlp)
     lib.tr_mlp_hidden.argtypes, lib.tr_mlp_hidden.restype = [mlp, VP, VP, VP], I32
+    lib.tr_gemm_columns.argtypes, lib.tr_gemm_columns.restype = [I32, I32, I32, I32], I32
     lib.tr_mlp_workspace_bytes.argtypes, lib.tr_mlp_workspace_bytes.restype = [mlp], SZ
     lib.tr_mlp_score.argtypes = [mlp, VP, VP, VP, VP, VP, VP, VP, SZ, VP, VP]
     lib.tr_mlp_score.restype = I32

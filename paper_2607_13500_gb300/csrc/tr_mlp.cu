@@ -826,18 +826,27 @@ inline int row_tiles(int m) { return (int)(((long long)m + 2 * kBM - 1) / (2 * k
 struct GemmShape {
   int bn, n_tiles, kblocks;
 };
-// The cheapest width by a model in clocks, fitted to the measured kernels; a
-// function of the sizes alone (it also sizes tr_mlp_score's scratch), whatever
-// the device has free.
+// The cheapest width by a model in clocks; a function of the sizes alone (it
+// also sizes tr_mlp_score's scratch), whatever the device has free: the waves
+// of tiles times the longer of a tile's main loop and its epilogue, and among
+// equals the narrowest, whose last epilogue ends sooner.
 //   A k-block takes the larger of its MMAs (2 clocks a column) and the operands
 //   into each SM at 63 bytes a clock, A's 16 KiB and B's 64 bytes a column:
 //   520 clocks for 256 columns, 455, 390 and 325 for 192, 128 and 64; the
-//   projector's row gather 1065 whatever the columns.  A tile's epilogue takes
-//   80 (score), 30 (hidden) or 65 (projector) clocks a column, overlapped with
-//   the next tile's main loop where there is one.
-// Measured, with 256 columns throughout and with the width chosen: 192 rows,
-// 1024 -> 4096, 12.3 and 8.4 us a pass (16 tiles, 64 of 64 columns); both GEMMs
-// of 2885 rows, 1152 -> 4304 -> 1152, 63.4 and 58.9 (60 score tiles, 72 of 192
+//   projector's row gather 1065 whatever the columns.  An epilogue takes a
+//   fixed part and one for each round of blocks over its warps: score 18,500
+//   clocks for 256 columns and 9,500 for 64, projector 7,500 and 3,750.  The
+//   hidden GEMM's, shared by twice the warps, shrinks with the width no more
+//   than its main loop does (5,400 to 8,700 clocks by activation for 256
+//   columns, 3,200 to 4,000 for 64), so the main loop ranks the widths at any K.
+// Against the best of the four widths, each measured on 1419 sizes (K 64 to
+// 4096, 256 to 4096 columns, 192 to 36,864 rows, three modes): within 0.1 % on
+// average and 5.2 % at most.  (An epilogue in proportion to the columns gave
+// few k-blocks narrow tiles whatever the rows: 36,864 rows, K 64, 4096 columns
+// 255 us in 64-column tiles, 138 in 256.)
+// With 256 columns throughout and with the width chosen: 192 rows, 1024 ->
+// 4096, 12.3 and 8.4 us a pass (16 tiles, 64 of 64 columns); both GEMMs of 2885
+// rows, 1152 -> 4304 -> 1152, 63.4 and 58.9 (60 score tiles, 72 of 192
 // columns); both of 576 rows, 1024 -> 4096 -> 1024, 53.7 and 33.5 (12 score
 // tiles, 48 of 64), of 48 rows 51 and 27.7.
 // K is not shared among pairs where tiles are few: clusters that split it and
@@ -845,19 +854,19 @@ struct GemmShape {
 // 48, but then the order of an output element's sum, and so its last bits,
 // followed the number of rows; in one order a row gives the same H, x'' and z
 // alone, in any batch and with any scratch.
-inline GemmShape gemm_shape(int m, int n, int k, bool score, bool gather) {
+inline GemmShape gemm_shape(int m, int n, int k, int mode) {
   constexpr long long kPairs = 76;
   const int kb = (k + kBK - 1) / kBK;
   const long long rows = row_tiles(m);
   auto cost = [&](int bn) {
     const long long waves = (rows * ((n + bn - 1) / bn) + kPairs - 1) / kPairs;
-    const long long main = (long long)kb * (gather ? 1065 : std::max(2 * bn + 8, (16384 + 64 * bn) / 63));
-    const long long epi = (long long)bn * (score ? 80 : (gather ? 65 : 30));
-    return waves * std::max(main, epi) + epi;
+    const int main = kb * (mode == kModeProject ? 1065 : std::max(2 * bn + 8, (16384 + 64 * bn) / 63));
+    const int epi = mode == kModeScore ? 6500 + 3000 * bn / 64 : (mode == kModeProject ? 2500 + 1250 * bn / 64 : 0);
+    return waves * std::max(main, epi);
   };
   int best = kBN;
   for (const int bn : {192, 128, 64})
-    if (cost(bn) < cost(best)) best = bn;
+    if (cost(bn) <= cost(best)) best = bn;
   return GemmShape{best, (n + best - 1) / best, kb};
 }
 
@@ -893,7 +902,7 @@ size_t part_bytes(const tr_mlp *m, const GemmShape &sh) {
   return align_up((size_t)rblocks * sh.n_tiles * kRowParts * 4 * kPartWords * 32 * sizeof(float), 256);
 }
 GemmShape score_shape(const tr_mlp *m, size_t bytes) {
-  const GemmShape sh = gemm_shape(m->t, m->d, m->d_hidden, true, false);
+  const GemmShape sh = gemm_shape(m->t, m->d, m->d_hidden, kModeScore);
   return part_bytes(m, sh) <= bytes ? sh : GemmShape{kBN, (m->d + kBN - 1) / kBN, sh.kblocks};
 }
 
@@ -907,7 +916,7 @@ tr_status dense_act_gemm(const void *a, int rows, int k, const void *w, const fl
   g.m = rows;
   g.n = n;
   g.k = k;
-  const GemmShape sh = gemm_shape(g.m, g.n, g.k, false, false);
+  const GemmShape sh = gemm_shape(g.m, g.n, g.k, kModeHidden);
   set_shape(g, sh);
   g.bias = bias;
   g.act = act;
@@ -944,6 +953,11 @@ tr_status tr_project(const void *y, int32_t rows, int32_t d, const void *w, cons
   if (((long long)rows + kBM - 1) / kBM * ((d_out + kBN - 1) / kBN) > INT_MAX) return TR_ERR_UNSUPPORTED;
   if (misaligned16(y) || misaligned16(w) || misaligned16(bias) || misaligned16(z)) return TR_ERR_ALIGN;
   return dense_act_gemm(y, rows, d, w, bias, d_out, act, z, d_error, static_cast<cudaStream_t>(stream));
+}
+
+int32_t tr_gemm_columns(int32_t rows, int32_t n, int32_t k, int32_t kind) {
+  if (rows <= 0 || n <= 0 || k <= 0 || kind < kModeHidden || kind > kModeProject) return 0;
+  return gemm_shape(rows, n, k, kind).bn;
 }
 
 size_t tr_mlp_workspace_bytes(const tr_mlp *m) {
@@ -1014,7 +1028,7 @@ tr_status tr_project_kept(const tr_tokens *in, const int32_t *d_cu_k, const int3
   g.m = total_k;
   g.n = d_out;
   g.k = in->d;
-  const GemmShape sh = gemm_shape(g.m, g.n, g.k, false, true);
+  const GemmShape sh = gemm_shape(g.m, g.n, g.k, kModeProject);
   set_shape(g, sh);
   g.bias = bias;
   g.act = act;

@@ -178,3 +178,14 @@ def test_binding_refuses_bad_buffers_before_any_launch(lib, monkeypatch):
     monkeypatch.setattr(api, "_workspace", lambda lib_, tok, device: (torch.empty(256, dtype=torch.uint8), 256))
     idx, role, cu_k, status = api.select(x, x, x, good, k=4, h2=torch.zeros(16), s=torch.zeros(16))
     assert calls == [13] and cu_k == [0, 4] and idx.shape == (4,) and role.shape == (16,)
+
+
+@pytest.mark.parametrize("rows,n,k,kind,columns", [
+    (192, 4096, 1024, 0, 64), (36864, 4096, 1024, 0, 256), (2885, 1152, 4304, 1, 192), (576, 1024, 4096, 1, 64),
+    (36864, 1024, 4096, 1, 256), (12288, 4096, 1024, 2, 256),
+    # few k-blocks and many rows: the epilogues set the pace, not narrow tiles' waves
+    (36864, 4096, 64, 0, 256), (36864, 2048, 256, 0, 256), (12288, 1024, 384, 0, 256), (36864, 2048, 64, 1, 256),
+    (36864, 1024, 256, 2, 256), (576, 1024, 64, 0, 64),
+    (0, 64, 64, 0, 0), (64, 0, 64, 0, 0), (64, 64, 0, 0, 0), (64, 64, 64, 3, 0), (64, 64, 64, -1, 0)])
+def test_gemm_columns(lib, rows, n, k, kind, columns):
+    assert lib.tr_gemm_columns(rows, n, k, kind) == columns

@@ -242,26 +242,34 @@ def test_project_kept_index_outside_its_image():
     _check_close(z, _sigma(v, "gelu"), mag, slope=1.13)
 
 
-# The layouts a GEMM may take (gemm_shape), by size: tile columns of the hidden
-# and the score GEMM, with ragged rows, columns and k-blocks.
+def _columns(rows, n, k, kind):
+    from paper_2607_13500_gb300 import _lib
+    return _lib.load().tr_gemm_columns(rows, n, k, kind)
+
+
+# The layouts a GEMM may take, by size: tile columns of the hidden and the
+# score GEMM (asserted), with ragged rows, columns and k-blocks.
 LAYOUT_CASES = [
-    ("256_64_long_k", 1000, 1024, 16400, "none", True, True),      # 4 x 16 score tiles, 256.25 k-blocks
-    ("64_64_one_row", 1, 256, 6144, "none", False, True),          # 4 score tiles, 96 k-blocks
-    ("128_64", 300, 528, 4464, "gelu", True, True),                # 2 x 9 score tiles, the last 16 columns
-    ("192_128", 1500, 1024, 4400, "gelu", True, True),             # 6 x 8 score tiles, 68.75 k-blocks
-    ("256_128", 2048, 784, 4112, "gelu", False, True),             # 8 x 7 score tiles, the last 16 columns
-    ("192_128_ragged_rows", 1200, 1024, 4096, "quick_gelu", True, True),  # 5 row tiles
-    ("256_64", 1000, 1024, 4160, "quick_gelu", True, False),       # 4 x 16 score tiles, 65 k-blocks
-    ("64_64", 129, 1056, 1472, "quick_gelu", True, True),          # 17 score tiles, the last half empty
-    ("256_192", 2885, 1152, 4304, "gelu", True, True),             # 12 x 6 score tiles
-    ("128_128", 2048, 784, 2064, "gelu", False, True),             # 8 x 7 score tiles, the last 16 columns
-    ("256_64_many", 2049, 1152, 1600, "none", True, True),         # 9 x 18 score tiles
+    ((256, 64), 1000, 1024, 16400, "none", True, True),     # 4 x 16 score tiles, 256.25 k-blocks
+    ((128, 64), 1, 256, 6144, "none", False, True),         # one row, 4 score tiles, 96 k-blocks
+    ((128, 64), 300, 528, 4464, "gelu", True, True),        # 2 x 9 score tiles, the last 16 columns
+    ((192, 128), 1500, 1024, 4400, "gelu", True, True),     # 6 x 8 score tiles, 68.75 k-blocks
+    ((256, 128), 2048, 784, 4112, "gelu", False, True),     # 8 x 7 score tiles, the last 16 columns
+    ((192, 128), 1200, 1024, 4096, "quick_gelu", True, True),  # 5 row tiles
+    ((256, 64), 1000, 1024, 4160, "quick_gelu", True, False),  # 4 x 16 score tiles, 65 k-blocks
+    ((64, 64), 129, 1056, 1472, "quick_gelu", True, True),  # 17 score tiles, the last half empty
+    ((256, 192), 2885, 1152, 4304, "gelu", True, True),     # 12 x 6 score tiles
+    ((256, 128), 2048, 784, 2064, "gelu", False, True),     # 8 x 7 score tiles, the last 16 columns
+    ((256, 192), 2049, 1152, 1600, "none", True, True),     # 9 x 6 score tiles
+    ((128, 256), 3000, 1296, 528, "gelu", True, True),      # 12 x 6 score tiles, the last 16 columns
 ]
 
 
-@pytest.mark.parametrize("name,t,d,dh,act,resid,bias", LAYOUT_CASES, ids=[c[0] for c in LAYOUT_CASES])
-def test_mlp_layouts(name, t, d, dh, act, resid, bias):
-    test_mlp_outputs_and_records(name, t, d, dh, act, resid, bias)
+@pytest.mark.parametrize("columns,t,d,dh,act,resid,bias", LAYOUT_CASES,
+                         ids=["%d-%d-%d" % c[1:4] for c in LAYOUT_CASES])
+def test_mlp_layouts(columns, t, d, dh, act, resid, bias):
+    assert columns == (_columns(t, dh, d, 0), _columns(t, d, dh, 1))
+    test_mlp_outputs_and_records("%d-%d" % columns, t, d, dh, act, resid, bias)
     # a second call reproduces every bit: the row partials are merged in a fixed order
     altr = _alt()
     xp, w1, w2, b1, b2, r = _inputs(t, d, dh, seed=3, resid=resid, bias=bias)
@@ -288,12 +296,14 @@ def _project_direct(x, idx, cu_k, w, bias, seqlens):
     return z, err
 
 
-@pytest.mark.parametrize("d,d_out,k,n,b", [(8208, 528, 40, 300, 3), (4096, 2560, 200, 300, 3), (784, 1296, 50, 300, 3),
-                                           (272, 528, 200, 300, 16), (256, 272, 1025, 1300, 3)],
-                         ids=["64_long_k", "128", "64", "gathered", "gathered_few"])
-def test_project_layouts(d, d_out, k, n, b):
-    # tiles of few columns: the dense projector within the GEMM tolerance
-    # of float64, and the rows read by index bit for bit the same
+@pytest.mark.parametrize("columns,d,d_out,k,n,b", [
+    (64, 8208, 528, 40, 300, 3), (128, 4096, 2560, 200, 300, 3), (64, 784, 1296, 50, 300, 3), (128, 272, 528, 200, 300, 16),
+    (64, 256, 272, 1025, 1300, 3), (192, 272, 528, 350, 400, 12), (256, 272, 1040, 1025, 1300, 3),
+    (256, 784, 1040, 1025, 1300, 3)])
+def test_project_layouts(columns, d, d_out, k, n, b):
+    # every tile width: the dense projector within the GEMM tolerance of
+    # float64, and the rows read by index bit for bit the same
+    assert columns == _columns(b * k, d_out, d, 0) == _columns(b * k, d_out, d, 2)
     altr = _alt()
     g = torch.Generator(device="cuda").manual_seed(9)
     x = torch.randn(b * n, d, generator=g, device="cuda").to(torch.bfloat16)
