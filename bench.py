@@ -706,7 +706,7 @@ def measure_mlp(args, dev, altr, reps=20, batch=None):
                                                   "tr_project_kept": tf(flop_p, med["tr_project_kept"]) / peak}},
         "projector_note": "the step projects the gathered rows y (tr_project); tr_project_kept, timed outside the "
                           "step, is the binding's project_kept on the same rows, named by index (from 3072 rows "
-                          "on it copies them first), and gives the same z bit for bit",
+                          "and 1024 columns on it copies them first), and gives the same z bit for bit",
         "scoring_bytes": {"fused_extra_reads": t * d * e, "separate_pass_reads": 3 * t * d * e,
                           "note": "the fused epilogue reads x' (its P and A terms); x'' and x are written by the "
                                   "MLP in both routes; the separate pass reads x, x', x'' again"},

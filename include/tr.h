@@ -416,9 +416,10 @@ tr_status tr_project_kept(const tr_tokens *in, const int32_t *d_cu_k, const int3
  * z = sigma(y W^T + bias) by the kernel of tr_mlp_hidden; for y = the rows
  * that tr_project_kept reads, the two give the same z bit for bit (the same
  * MMA order and epilogue arithmetic).  Gathering first and projecting the
- * dense rows is the faster route on GB300: tr_project_kept's row loads are
- * TMA gathers whose issue rate sets its pace, while the copy costs one write
- * and one read of rows * d * 2 bytes.  d and d_out multiples of 16, pointers
+ * dense rows is the faster route on GB300 from about 1024 output columns on:
+ * tr_project_kept's row loads are TMA gathers whose issue rate sets its pace
+ * tile by tile, while the copy costs one write and one read of rows * d * 2
+ * bytes.  d and d_out multiples of 16, pointers
  * 16-byte aligned; rows = 0 does nothing.  d_error as for tr_mlp_hidden.
  */
 tr_status tr_project(const void *y, int32_t rows, int32_t d, const void *w, const float *bias, int32_t d_out,

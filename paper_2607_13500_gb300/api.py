@@ -765,7 +765,9 @@ def project_kept(x, idx, cu_k, w, bias=None, act="gelu", seqlens=None, error=Non
     """z = sigma(X* W^T + bias) for the kept tokens X* (tr_project_kept's result),
     their rows named by the selection's ``idx`` (local per image, image b
     owning slots cu_k[b]..cu_k[b+1]) in ``x``.  ``w`` bf16
-    [d_out, D], ``bias`` fp32 [d_out] or None; returns z bf16 [sum K, d_out]."""
+    [d_out, D], ``bias`` fp32 [d_out] or None; returns z bf16 [sum K, d_out].
+    From 3072 rows and 1024 output columns on the rows are first copied (a
+    temporary bf16 [sum K, D])."""
     lib = load()
     if x.dtype != torch.bfloat16 or w.dtype != torch.bfloat16:
         raise TypeError("x and w must be bf16")
@@ -786,12 +788,17 @@ def project_kept(x, idx, cu_k, w, bias=None, act="gelu", seqlens=None, error=Non
     z = torch.empty(max(total_k, 1), d_out, dtype=torch.bfloat16, device=dev)
     err = torch.zeros(1, dtype=torch.int32, device=dev) if error is None else error
     st = _stream(dev)
-    if 3072 <= total_k <= x2.shape[0] and max(seqlens, default=0) <= TR_MAX_N:
+    if 3072 <= total_k <= x2.shape[0] and d_out >= 1024 and max(seqlens, default=0) <= TR_MAX_N:
         # A copy of the rows and the dense layer on it, the same z bit for bit:
-        # the row-gathering TMA loads of the direct kernel set its pace (1024 ->
-        # 4096, 12288 rows: 84 us on the GPU against 107, 3072 rows 30 against
-        # 38).  Fewer rows: one launch, for the host's sake (a pass of 64 rows
-        # takes 25 us with it and 35 with two).
+        # the row-gathering TMA loads of the direct kernel set its pace, tile by
+        # tile, and the copy costs a write and a read of the rows once.  GPU us,
+        # direct and copied, D 128 to 4096, 3072 to 49152 rows: 4096 columns 1.2
+        # to 1.45x (1024 -> 4096, 12288 rows 106 and 81), 2048 columns 1.04 to
+        # 1.45x, 1280 and 1536 columns 0.96 to 1.28x, 1024 columns 0.90 to 1.39x
+        # (2048 -> 1024, 6144 rows 40.8 and 29.3; 49152 rows 186 and 190); 768
+        # and fewer 0.48 to 1.25x (4096 -> 256, 49152 rows 103 and 216), so those
+        # stay with the direct kernel.  So do fewer rows: one launch, for the
+        # host's sake (a pass of 64 rows takes 25 us with it and 35 with two).
         y = torch.empty(max(total_k, 1), d, dtype=torch.bfloat16, device=dev)
         check("tr_project_kept", lib.tr_gather(tok.ref(), _ptr(d_cu), _ptr(idx), total_k, _ptr(y), st))
         check("tr_project_kept", lib.tr_project(_ptr(y), total_k, d, _ptr(w), _ptr(b), d_out, TR_ACT[act], _ptr(z),

@@ -323,6 +323,43 @@ def test_project_layouts(columns, d, d_out, k, n, b):
     _check_close(z, _sigma(v, "gelu"), mag, slope=1.13)
 
 
+@pytest.mark.parametrize("d_out,copied", [(1008, False), (1024, True)])
+def test_project_kept_of_many_rows_of_a_ragged_batch(d_out, copied, monkeypatch):
+    # both routes on either side of the width from which the rows are copied
+    # first: images of several sizes, one empty and one that keeps nothing,
+    # and indices outside their images, which feed rows of zeros
+    altr = _alt()
+    from paper_2607_13500_gb300 import _lib
+    lib, copies = _lib.load(), []
+    gather = lib.tr_gather
+    monkeypatch.setattr(lib, "tr_gather", lambda *a: copies.append(a) or gather(*a))
+    seqlens, ks, d = [1500, 0, 2600, 7, 900], [1200, 0, 1900, 0, 200], 272
+    g = torch.Generator(device="cuda").manual_seed(4)
+    x = torch.randn(sum(seqlens), d, generator=g, device="cuda").to(torch.bfloat16)
+    w = (torch.randn(d_out, d, generator=g, device="cuda") / math.sqrt(d)).to(torch.bfloat16)
+    bias = 0.05 * torch.randn(d_out, generator=g, device="cuda")
+    idx, rows, cu, off = [], [], [0], 0
+    for n, k in zip(seqlens, ks):
+        i = torch.randperm(max(n, 1), generator=g, device="cuda")[:k].sort().values
+        idx.append(i)
+        rows.append(off + i)
+        off += n
+        cu.append(cu[-1] + k)
+    idx, rows = torch.cat(idx).to(torch.int32), torch.cat(rows)
+    y = x[rows]
+    for slot, bad in ((0, -1), (1199, 1500), (1200, 2600), (3099, 2 ** 31 - 1), (3100, -2 ** 31), (3299, 900)):
+        idx[slot] = bad
+        y[slot] = 0
+    z, err = altr.project_kept(x, idx, cu, w, bias, act="gelu", seqlens=seqlens)
+    assert bool(copies) == copied
+    zd, err_d = _project_direct(x, idx, cu, w, bias, seqlens)
+    zy, err_y = altr.project(y, w, bias, act="gelu")
+    torch.cuda.synchronize()
+    assert err.item() == 0 and err_d.item() == 0 and err_y.item() == 0
+    assert torch.equal(z.view(torch.int16), zd.view(torch.int16))
+    assert torch.equal(z.view(torch.int16), zy.view(torch.int16))
+
+
 def test_project_kept_of_an_image_past_the_gather_limit():
     # more tokens in an image than tr_gather takes: the direct kernel
     altr = _alt()
