@@ -115,7 +115,7 @@ struct ClusterShared {
   uint32_t win_count;
   int lo, hi;
   float wr[kWarps][4];
-  // runs around picks: [lo, hi) packed, and their rows (listed from `first`)
+  // runs around picks (RunPlace, where this CTA's rows are few)
   uint32_t run[kMaxRuns];
   int first[kMaxRuns];
   int runs, run_rows, exact_rows, exact_total;
@@ -388,6 +388,28 @@ __device__ __forceinline__ bool cluster_stage_one(const SelectArgs &a, const Spl
   return sh.fail[kFailCut] == 0u;
 }
 
+// Where a CTA lists the runs around its picks: [lo, hi) packed, the place of
+// their rows in the list, the list, and that of the rows for exact sums.  A CTA
+// with many rows lists them in the memory of its R keys, which Stage I was the
+// last to read (half of it is taken): an eighth as many runs as rows, and twice
+// as many rows of runs.  Keys of a narrow band have some hundred near-ties at
+// one pick in two (8192 tokens of 1544 channels, half of them kept: 191 runs),
+// and an image with more runs than are listed is selected anew by select_image.
+constexpr int kWideRows = 2048;
+struct RunPlace {
+  uint32_t *run;
+  int *first;
+  uint16_t *list, *xlist;
+  int max_runs, max_rows;
+};
+template <bool kMany>
+__device__ __forceinline__ RunPlace run_place(const SplitImage<kMany> &im, ClusterShared &sh) {
+  if (im.cap < kWideRows) return RunPlace{sh.run, sh.first, sh.list, sh.xlist, kMaxRuns, kPendCap};
+  const int w = im.cap / 8;
+  uint16_t *list = reinterpret_cast<uint16_t *>(im.keyr + 2 * w);
+  return RunPlace{im.keyr, reinterpret_cast<int *>(im.keyr + w), list, list + 2 * w, w, 2 * w};
+}
+
 // Element q of X_rem sorted by s, wherever it is.
 struct SortedRow {
   float s;
@@ -477,6 +499,7 @@ __device__ __forceinline__ bool cluster_stage_two(const SelectArgs &a, const Spl
   }
   im.barrier();
   // the picks inside this CTA's stretch
+  const RunPlace place = run_place(im, sh);
   bool bad = false, marked = false;
   for (int j = tid; j < im.k2; j += nthr) {
     const int p = pick_position(j, m, im.k2, t, a.stride_interval);
@@ -499,10 +522,10 @@ __device__ __forceinline__ bool cluster_stage_two(const SelectArgs &a, const Spl
     if (j == 0 || pick_position(j - 1, m, im.k2, t, a.stride_interval) < lo) {
       const int slot = atomicAdd(&sh.runs, 1);
       const int at = atomicAdd(&sh.run_rows, hi - lo);
-      if (slot < kMaxRuns && at + (hi - lo) <= kPendCap) {
-        sh.run[slot] = ((uint32_t)lo << 16) | (uint32_t)hi;
-        sh.first[slot] = at;
-        for (int q = lo; q < hi; ++q) sh.list[at + q - lo] = (uint16_t)sorted_row(im, sh, q).row;
+      if (slot < place.max_runs && at + (hi - lo) <= place.max_rows) {
+        place.run[slot] = ((uint32_t)lo << 16) | (uint32_t)hi;
+        place.first[slot] = at;
+        for (int q = lo; q < hi; ++q) place.list[at + q - lo] = (uint16_t)sorted_row(im, sh, q).row;
       } else {
         bad = true;
       }
@@ -513,26 +536,26 @@ __device__ __forceinline__ bool cluster_stage_two(const SelectArgs &a, const Spl
     const int runs = sh.runs;
     // a run that the double-float keys leave open anywhere (a pair they do not
     // separate, or a row that does not qualify) is ranked by exact sums as a whole
-    if (runs > 0) refine_df(a, im.off, sh.list, sh.run_rows, 1, im.rec);
+    if (runs > 0) refine_df(a, im.off, place.list, sh.run_rows, 1, im.rec);
     for (int r = tid; r < runs; r += nthr) {
-      const int len = (int)(sh.run[r] & 0xffffu) - (int)(sh.run[r] >> 16);
-      const uint16_t *rows = sh.list + sh.first[r];
+      const int len = (int)(place.run[r] & 0xffffu) - (int)(place.run[r] >> 16);
+      const uint16_t *rows = place.list + place.first[r];
       bool open = false;
       for (int i = 0; i < len && !open; ++i)
         for (int j = i + 1; j < len && !open; ++j) open = df_cmp_s(im.rec[rows[j]], im.rec[rows[i]], a.bounds) == 0;
       if (open) {
         const int at = atomicAdd(&sh.exact_rows, len);
-        for (int i = 0; i < len; ++i) sh.xlist[at + i] = rows[i];
-        sh.first[r] |= kRunExact;
+        for (int i = 0; i < len; ++i) place.xlist[at + i] = rows[i];
+        place.first[r] |= kRunExact;
       }
     }
     __syncthreads();
-    if (sh.exact_rows > 0) bad = !refine_exact(a, im.off, sh.xlist, sh.exact_rows, 1, im.rec, im.primary);
+    if (sh.exact_rows > 0) bad = !refine_exact(a, im.off, place.xlist, sh.exact_rows, 1, im.rec, im.primary);
     if (!bad) {
       for (int r = tid; r < runs; r += nthr) {
-        const int lo = (int)(sh.run[r] >> 16), len = (int)(sh.run[r] & 0xffffu) - lo;
-        const bool exact = (sh.first[r] & kRunExact) != 0;
-        const uint16_t *rows = sh.list + (sh.first[r] & ~kRunExact);
+        const int lo = (int)(place.run[r] >> 16), len = (int)(place.run[r] & 0xffffu) - lo;
+        const bool exact = (place.first[r] & kRunExact) != 0;
+        const uint16_t *rows = place.list + (place.first[r] & ~kRunExact);
         for (int i = 0; i < len; ++i) {
           int rank = 0;
           for (int j = 0; j < len; ++j) {

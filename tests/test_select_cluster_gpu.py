@@ -99,6 +99,29 @@ def test_near_ties(dtype, rows):
         assert 0 < st[2] <= 4 * len(pairs) + 8, st
 
 
+@pytest.mark.parametrize("groups,rows,exact", [(40, 1900, True), (150, 1700, False), (150, 1700, True), (300, 1500, False),
+                                               (300, 6000, True)],
+                         ids=["40", "150", "150_exact", "300", "300_exact"])
+def test_many_runs(groups, rows, exact):
+    # every row a pick and hundreds of near-tie runs: in the small list, in the
+    # large one (an eighth as many runs as rows) and more than it holds; some
+    # with an exact tie, which alone take exact sums
+    d = 1024
+    t3 = _near_tie_triples(groups, d, torch.float32, 5)
+    where = torch.argsort(t3[3])
+    tx, tp, tq = t3[:3]
+    ties = range(0, 3 * groups, 36) if exact else ()
+    for i in ties:
+        for t in (tx, tp, tq):
+            t[where[i + 1]] = t[where[i]]
+    x, xp, xq = (torch.cat([a, b]) for a, b in zip((tx, tp, tq), _rows(rows, d, 4, torch.float32)))
+    perm = torch.randperm(x.shape[0], generator=torch.Generator().manual_seed(6))
+    x, xp, xq = x[perm], xp[perm], xq[perm]
+    n = x.shape[0]
+    st = check_reduce(x, xp, xq, [n], _budget([n - 1], [0]))
+    assert 2 * len(ties) <= st[2] <= 8 * len(ties), st
+
+
 @pytest.mark.parametrize("n", [2600, 6000])
 def test_left_to_select_image(n):
     d = 64
