@@ -82,6 +82,10 @@ struct Bounds {
   float df_r, df_s_abs, df_s_rel;
 };
 
+// The row partials of tr_mlp_score's epilogue: kMlpRowParts per tile, each of
+// an equal share of the tile's columns, kMlpMinColumns to kMlpMaxColumns.
+constexpr int kMlpRowParts = 2, kMlpMinColumns = 64, kMlpMaxColumns = 256;
+
 inline Bounds certification_bounds(int d, int dtype) {
   const double u = 1.0 / 16777216.0;  // fp32 unit roundoff 2^-24
   const int h = score_depth(d, dtype);
@@ -99,15 +103,17 @@ inline Bounds certification_bounds(int d, int dtype) {
   double ep = 2.0 * u * u * (lane_terms * lane_terms + 12.0 * d) + 0x1p-52;
   if (dtype == TR_F32) ep *= 2.0;  // bf16 and fp16 products are exact in fp32
   // The encoder-MLP GEMM's epilogue (tr_mlp_score, bf16) writes the same
-  // records: each term enters its double-float sum through TwoSum, over at
-  // most c = 128 columns per partial (low-part roundings below u^2 c (c + 1) /
-  // 2 of the partial's sum|x'x''|), and at most j = 8 ceil(d / 256) partials
-  // are merged, each merge two low-part additions whose sums stay below
-  // (c + j) u of the total: 2 j (c + j) u^2.  The bounds cover both producers
-  // of a record.  Its L1, S2, A and B are within that same tiny relative
-  // error, far inside g above.
+  // records: each term enters its double-float sum through TwoSum, over the c
+  // columns of a partial (low-part roundings below u^2 c (c + 1) / 2 of the
+  // partial's sum|x'x''|), and j partials are merged, each merge two low-part
+  // additions whose sums stay below (c + j) u of the total: 2 j (c + j) u^2.
+  // Tiles of bn columns have c = bn / 2 and j = 2 ceil(d / bn); the sum grows
+  // with both, so the widest tile's c and the narrowest's j cover every layout.
+  // The bounds cover both producers of a record.  Its L1, S2, A and B are
+  // within that same tiny relative error, far inside g above.
   if (dtype == TR_BF16) {
-    const double c = 128.0, j = 8.0 * (double)((d + 255) / 256);
+    const double c = (double)(kMlpMaxColumns / kMlpRowParts);
+    const double j = (double)kMlpRowParts * (double)((d + kMlpMinColumns - 1) / kMlpMinColumns);
     const double ep_mlp = u * u * (c * (c + 1.0) / 2.0 + 2.0 * j * (c + j)) + 0x1p-52;
     if (ep_mlp > ep) ep = ep_mlp;
   }

@@ -89,8 +89,14 @@ constexpr int kBlkBytes = 32 * kBlk * 2;
 __host__ __device__ constexpr int stage_blks(int mode) { return mode == kModeHidden ? 1 : 2; }
 __host__ __device__ constexpr int stage_bytes(int mode) { return stage_blks(mode) * kBlkBytes; }
 // The score mode's partial row sums per tile and lane quarter: one for each of
-// its warps (a tile has at least as many blocks).
-constexpr int kRowParts = epi_parts(kModeScore);
+// its warps, of an equal share of the tile's blocks.  certification_bounds
+// counts on these numbers.
+constexpr int kRowParts = kMlpRowParts;
+constexpr int kWidths[] = {kMlpMaxColumns, 192, 128, kMlpMinColumns};  // a tile's columns
+static_assert(kRowParts == epi_parts(kModeScore) && kBN == kMlpMaxColumns, "layout of the row partials");
+static_assert(kWidths[1] % (kRowParts * kBlk) == 0 && kWidths[2] % (kRowParts * kBlk) == 0 &&
+                  kMlpMinColumns == kRowParts * kBlk,
+              "equal shares of every tile's blocks");
 
 struct GemmArgs {
   int m, n, k;          // C[m, n] = A[m, k] B[n, k]^T
@@ -865,7 +871,7 @@ inline GemmShape gemm_shape(int m, int n, int k, int mode) {
     return waves * std::max(main, epi);
   };
   int best = kBN;
-  for (const int bn : {192, 128, 64})
+  for (const int bn : kWidths)
     if (cost(bn) <= cost(best)) best = bn;
   return GemmShape{best, (n + best - 1) / best, kb};
 }
