@@ -101,7 +101,7 @@ tr_status select_capped(const tr_tokens *in, const float *stats, const int32_t *
 }
 
 tr_status gather_impl(const tr_tokens *in, const int32_t *d_cu_k, const int32_t *idx, int32_t total_k, void *y,
-                      void *stream, bool pdl) {
+                      void *stream, bool pdl, bool beside_scoring) {
   Shape sh;
   tr_status rc = check_tokens(in, &sh);
   if (rc != TR_OK) return rc;
@@ -109,7 +109,8 @@ tr_status gather_impl(const tr_tokens *in, const int32_t *d_cu_k, const int32_t 
   if (total_k > 0 && (!d_cu_k || !idx || !y || in->batch == 0)) return TR_ERR_ARG;
   if (misaligned(y, 16)) return TR_ERR_ALIGN;
   cudaError_t err = launch_gather(in->x, sh.total, in->dtype, in->d, in->batch, in->cu_seqlens ? 0 : in->n,
-                                  in->cu_seqlens, d_cu_k, idx, total_k, y, static_cast<cudaStream_t>(stream), pdl);
+                                  in->cu_seqlens, d_cu_k, idx, total_k, y, static_cast<cudaStream_t>(stream), pdl,
+                                  beside_scoring);
   return err == cudaSuccess ? TR_OK : TR_ERR_CUDA;
 }
 
@@ -252,7 +253,7 @@ tr_status tr_reduce(const tr_tokens *in, const int32_t *d_k, const int32_t *d_k1
 
 tr_status tr_gather(const tr_tokens *in, const int32_t *d_cu_k, const int32_t *idx, int32_t total_k, void *y,
                     void *stream) {
-  return gather_impl(in, d_cu_k, idx, total_k, y, stream, true);
+  return gather_impl(in, d_cu_k, idx, total_k, y, stream, true, false);
 }
 
 // ---------------------------------------------------------------- pipeline
@@ -363,7 +364,7 @@ tr_status tr_pipeline_submit(tr_pipeline *p, const tr_tokens *in, const int32_t 
     if ((rc = select_capped(in, stats, d_k, d_k1, d_cu_k, idx, nullptr, h2, s, ws, p->ws_bytes, d_status, b, cap,
                             false)) != TR_OK)
       return rc;
-    if ((rc = gather_impl(in, d_cu_k, idx, total_k, y, b, false)) != TR_OK) return rc;
+    if ((rc = gather_impl(in, d_cu_k, idx, total_k, y, b, false, true)) != TR_OK) return rc;
     p->kernels += (sh.total > 0) + (in->batch > 0) + (total_k > 0);
   }
   if (cudaEventRecord(p->done[slot], b) != cudaSuccess) return TR_ERR_CUDA;

@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kGatherWarps * 32)
 
 cudaError_t launch_gather(const void *x, long long total_rows, int dtype, int d, int batch, int n_uniform,
                           const int32_t *cu_seqlens, const int32_t *cu_k, const int32_t *idx, int total_k, void *y,
-                          cudaStream_t st, bool pdl) {
+                          cudaStream_t st, bool pdl, bool beside_scoring) {
   if (total_k == 0) return cudaSuccess;
   const int nchunks = d * elem_bytes(dtype) / 16;
   const int grid = (total_k + kGatherWarps - 1) / kGatherWarps;
@@ -77,12 +77,12 @@ cudaError_t launch_gather(const void *x, long long total_rows, int dtype, int d,
   // (14 per lane: two of seven), none alone: what a round costs is its latency.
   // (Four a round and the rest one by one took 55.5 us on 12 ragged images of
   // 3584 bf16 channels, 322 MB, against 51.8, and 10.2 against 8.2 for a clip's
-  // 784 rows, launch included.)  Beside another batch's scoring (the pipeline,
-  // pdl false) four loads a round: there its own latency is hidden and its
+  // 784 rows, launch included.)  Beside another batch's scoring (the pipeline)
+  // four loads a round: there its own latency is hidden and its
   // bursts hold the scoring up (64 images of 576 x 4096 bf16, a third kept,
   // 168.2 us a batch against 168.6; 32 images, a third kept, 85.6 against 85.9).
   const int per_lane = (nchunks + 31) / 32;
-  const int most = pdl ? 8 : 4;
+  const int most = beside_scoring ? 4 : 8;
   const int rounds = (per_lane + most - 1) / most;
   switch ((per_lane + rounds - 1) / rounds) {
     case 1: return launch(k_gather<1>);

@@ -259,8 +259,9 @@ int select_cluster_ctas(int batch, int max_n);
 cudaError_t launch_select(const SelectArgs &a, cudaStream_t st, int max_ctas, bool pdl);
 int sm_count();  // SMs of the current device (cached), 0 on error
 cudaError_t launch_select_gather(const SelectArgs &a, void *y, cudaStream_t st, bool pdl);
+// beside_scoring: another batch's scoring kernel runs at the same time.
 cudaError_t launch_gather(const void *x, long long total_rows, int dtype, int d, int batch, int n_uniform,
                           const int32_t *cu_seqlens, const int32_t *cu_k, const int32_t *idx, int total_k, void *y,
-                          cudaStream_t st, bool pdl);
+                          cudaStream_t st, bool pdl, bool beside_scoring);
 
 }  // namespace tr
