@@ -31,8 +31,9 @@ cudaError_t launch_score(const void *x, const void *x_pre, const void *x_post, i
   float4 *ps = reinterpret_cast<float4 *>(stats);
   // Programmatic dependent launch (single calls): the launch of one call's
   // scoring overlaps the end of the call before it on the stream -- passes of
-  // one 576-token fp32 image 22.1 -> 19.7 us, of a 6272-token clip 58.3 ->
-  // 55.9, of 4 x 2880 fp16 74.2 -> 72.3, of 64 x 576 bf16 191.8 -> 189.8.
+  // one 576-token fp32 image 16.4 us without and 13.6 with it, of a 6272-token
+  // clip 59.5 and 57.8, of 4 x 2880 fp16 71.9 and 70.2, of 64 x 576 bf16 185.9
+  // and 183.8.
   // One row per warp and no more, in small CTAs: CTAs retire as they
   // finish, so kernels on other streams (the selection of an earlier batch)
   // can take SMs while this one still runs, and an SM's slots refill row by

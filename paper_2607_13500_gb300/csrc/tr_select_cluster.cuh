@@ -29,8 +29,9 @@
 // shared memory): the selection of every image up to kSoloMaxN tokens that no
 // cluster takes.  It beats select_image's fast path by keeping the s keys from
 // the one load of the records, by ranking buckets instead of sorting, and by
-// fewer passes: passes of one 576-token fp32 image 19.5 -> 14.7 us, k_select on
-// 64 x 576 tokens 25.6 -> 20.5, a 2880-token image (bf16, D 512) 26.7 -> 19.8.
+// fewer passes: passes of one 576-token fp32 image 17.1 us with select_image
+// alone and 13.6 with the fast path before it, tr_select on 64 x 576 tokens 11.8
+// and 9.5, on a 2880-token image 20.0 and 15.2.
 //
 // What bounds it: a chain of about ten short phases, each ending in a cluster
 // barrier (0.5-0.6 us) and spending as much on its own latencies; a run to

@@ -39,9 +39,6 @@ __device__ __forceinline__ void mbar_fence_init() { asm volatile("fence.mbarrier
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 // True when the phase of parity `parity` has completed.
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -79,9 +76,8 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
 
 // ---------------------------------------------------------------- TMA
 // 2-D tiled load of the box at (c0 = innermost coordinate, c1) into shared
-// memory; completes `bytes` transactions on the barrier.  c0 * 2 bytes is a
-// multiple of 128 at every call site (16-byte rule for the innermost
-// coordinate).
+// memory; completes the box's bytes on the barrier.  c0 is a multiple of 32
+// elements (64 bytes) at every call site; the hardware wants 16 bytes.
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
@@ -90,7 +86,7 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
       : "memory");
 }
 // 2-D tiled store of a shared-memory box to global memory at (c0, c1) (c0 a
-// multiple of 64 elements at every call site; rows and columns past the
+// multiple of 32 elements at every call site; rows and columns past the
 // tensor's extent are not written), tracked by this thread's bulk groups.
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, int c0, int c1, uint32_t src) {
   asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
@@ -177,11 +173,11 @@ __device__ __forceinline__ uint32_t map_shared(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-// All threads of both CTAs (a hardware barrier; every path of the kernel reaches it).
+// All threads of the cluster's CTAs (a hardware barrier; every path of the kernel reaches it).
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// Arrive on a barrier given by its shared::cluster address (this CTA's or the peer's).
+// Arrive on a barrier given by its shared::cluster address (this CTA's or another's).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }

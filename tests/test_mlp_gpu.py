@@ -122,7 +122,7 @@ def test_mlp_outputs_and_records(name, t, d, dh, act, resid, bias):
     torch.cuda.synchronize()
     rs = ref_stats.double().cpu().numpy()
     assert np.allclose(st[:, :4], rs[:, :4], rtol=4e-7, atol=0)
-    # a second call gives the same bits (the arrival counters start again at zero)
+    # a second call gives the same bits
     h0, q0, x0, s0 = (v.clone() for v in (out.h, out.x_post, out.x, out.stats))
     out2 = m.run(xp, r)
     torch.cuda.synchronize()
