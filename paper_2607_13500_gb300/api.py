@@ -482,7 +482,8 @@ class Pipeline(_Bound):
         kernel.  With
         ``after_current`` the scoring waits for the work already queued on
         the caller's current stream (where the inputs were written); pass
-        False when the inputs are known to be ready."""
+        False when the inputs are known to be ready.  The inputs must stay as
+        they are until the submission is done (``wait``)."""
         if self._graphed and not torch.cuda.is_current_stream_capturing():
             raise RuntimeError("this pipeline was captured by Pipeline.graph: replay the graph instead")
         tok = self._bind(x, x_pre, x_post)
@@ -499,6 +500,10 @@ class Pipeline(_Bound):
         check("tr_pipeline_submit", self.lib.tr_pipeline_submit(
             self._handle, tok.ref(), _ptr(self.d_k), _ptr(self.d_k1), _ptr(self.d_cu), self.total_k, _ptr(o["y"]),
             _ptr(o["idx"]), _ptr(o["h2"]), _ptr(o["s"]), _ptr(o["status"]), ev[0], ev[1]))
+        for t, given in ((tok.x, x), (tok.x_pre, x_pre), (tok.x_post, x_post)):
+            if t is not None and t.data_ptr() != given.data_ptr():  # a contiguous copy made by the binding
+                t.record_stream(sst)
+                t.record_stream(self.select_stream)
         self.submitted += 1
         y, idx = (o["y"], o["idx"]) if self.total_k else (o["y"][:0], o["idx"][:0])
         return ReduceResult(y, idx, self.cu_k, o["h2"], o["s"], o["status"])
