@@ -193,6 +193,10 @@ class _Bound:
             _check_tokens(x, x_pre, x_post)
         else:
             x, x_pre, x_post, _ = _flatten(x, x_pre, x_post, self.seqlens)
+        return self._take(x, x_pre, x_post)
+
+    def _take(self, x, x_pre, x_post):
+        """The token struct of packed, checked tensors."""
         if self._tok is None:
             self._tok = _Tokens(x, x_pre, x_post, self.seqlens, self.stride, self._cu)
         else:
@@ -305,8 +309,8 @@ class Reducer(_Bound):
         self.s = torch.empty(t, dtype=torch.float32, device=dev) if scores else None
         self._ws = None
 
-    def _bind(self, x, x_pre, x_post):
-        tok = super()._bind(x, x_pre, x_post)
+    def _take(self, x, x_pre, x_post):
+        tok = super()._take(x, x_pre, x_post)
         if self._ws is None:
             self._ws, self._ws_bytes = _workspace(self.lib, tok, self.device)
         return tok
@@ -457,8 +461,8 @@ class Pipeline(_Bound):
         self._graphed = False
         self.submitted = 0
 
-    def _bind(self, x, x_pre, x_post):
-        super()._bind(x, x_pre, x_post)
+    def _take(self, x, x_pre, x_post):
+        super()._take(x, x_pre, x_post)
         if self._handle is None:
             nbytes = self.lib.tr_workspace_bytes(self._tok.ref())
             if nbytes == 0:
@@ -658,7 +662,7 @@ def reduce(x, x_pre, x_post, k=None, ratio=None, lam=(1, 3), seqlens=None, score
     x2, p2, q2, seqlens = _flatten(x, x_pre, x_post, seqlens)
     r = Reducer(seqlens, x2.shape[1], x2.dtype, x2.device, k=k, ratio=ratio, lam=lam, alias_pre=p2 is None,
                 scores=scores, budget=budget, stride=stride, _sync=False)
-    return r.run(x2, p2, q2)
+    return r._run(r._take(x2, p2, q2))  # made for these tensors: nothing to check again
 
 
 # ---------------------------------------------------------------- encoder MLP with fused scoring
@@ -819,25 +823,28 @@ def project(y, w, bias=None, act="gelu", error=None, out=None):
     y, bf16 [rows, D]); ``w`` bf16 [d_out, D], ``bias`` fp32 [d_out] or None;
     ``out`` an optional bf16 [rows, d_out] buffer.  Returns (z, error)."""
     lib = load()
-    if y.device.type != "cuda" or w.device != y.device or (bias is not None and bias.device != y.device) or \
-            (out is not None and out.device != y.device):
+    dev = y.device  # few attribute reads from here on: a pass of some rows is as long as this host code
+    if dev.type != "cuda" or w.device != dev or (bias is not None and bias.device != dev) or \
+            (out is not None and out.device != dev):
         raise ValueError("y, w, bias and out must live on one CUDA device (libtr has no CPU path)")
     if y.dtype != torch.bfloat16 or w.dtype != torch.bfloat16:
         raise TypeError("y and w must be bf16")
     if act not in TR_ACT:
         raise ValueError(f"act must be one of {sorted(TR_ACT)}")
-    if y.dim() != 2 or not y.is_contiguous() or w.dim() != 2 or w.shape[1] != y.shape[1]:
+    ys, ws = y.shape, w.shape
+    if len(ys) != 2 or not y.is_contiguous() or len(ws) != 2 or ws[1] != ys[1]:
         raise ValueError("y must be contiguous [rows, D] and w [d_out, D]")
-    _check_bias(bias, w.shape[0], "bias")
-    _check_buf(error, y.device, torch.int32, 1, "error")
-    rows, d = int(y.shape[0]), int(y.shape[1])
-    d_out = int(w.shape[0])
-    dev = y.device
-    b = None if bias is None else bias.float().contiguous()
+    (rows, d), d_out = ys, ws[0]
+    _check_bias(bias, d_out, "bias")
+    _check_buf(error, dev, torch.int32, 1, "error")
+    b = bias
+    if b is not None and (b.dtype != torch.float32 or not b.is_contiguous()):
+        b = b.float().contiguous()
     z = out if out is not None else torch.empty(max(rows, 1), d_out, dtype=torch.bfloat16, device=dev)
-    if z.dtype != torch.bfloat16 or not z.is_contiguous() or z.shape[1] != d_out or z.shape[0] < rows:
+    zs = z.shape
+    if z.dtype != torch.bfloat16 or not z.is_contiguous() or zs[1] != d_out or zs[0] < rows:
         raise ValueError(f"out must be contiguous bf16 [>= {rows}, {d_out}]")
     err = torch.zeros(1, dtype=torch.int32, device=dev) if error is None else error
     check("tr_project", lib.tr_project(_ptr(y), rows, d, _ptr(w.contiguous()), _ptr(b), d_out, TR_ACT[act], _ptr(z),
                                        _ptr(err), _stream(dev)))
-    return z if z.shape[0] == rows else z[:rows], err
+    return z if zs[0] == rows else z[:rows], err
